@@ -453,8 +453,8 @@ CG_API cg_status cg_offsets_noalloc(const int32_t* lengths, int64_t count, int64
  * one that lays out contigs and read pieces (Sec. 4.4 offsets) -- over
  * `tiles` tiles (2..4096) of zeros on the context's stream, with the ticket
  * of tile 0 never handed out, so the tiles after it wait on a descriptor that
- * no block publishes. Their wait is bounded (2^22 polls with a 200 ns back-off,
- * about one to two seconds); it then gives up, the kernel records the timeout
+ * no block publishes. Their wait is bounded (2^20 polls with a 200 ns back-off,
+ * about a second); it then gives up, the kernel records the timeout
  * in the context's error word and returns. Nothing faults or hangs. Returns
  * CG_ETIMEOUT, after which the context refuses all work until cg_destroy as
  * after any device timeout; CG_EKERNEL if the wait did not run out. Waits

@@ -460,21 +460,23 @@ cg_status finish_load(cg_graph* g, uint32_t flags) {
   S.wfirst = galloc<int32_t>(g, N, &st);
   if (G.no_reads) S.wread = galloc<int32_t>(g, N, &st);
   S.contig_off = galloc<int64_t>(g, N + 1, &st);
-  S.scan_tiles_cap = (int64_t)(N + 2047) / 2048 + 1;
-  S.scan_state[0] = galloc<unsigned long long>(g, 3 * ((size_t)S.scan_tiles_cap + 1), &st);
-  if (S.scan_state[0]) {
-    S.scan_state[1] = S.scan_state[0] + (S.scan_tiles_cap + 1);
-    S.scan_state[2] = S.scan_state[1] + (S.scan_tiles_cap + 1);
-    // zeroed once; afterwards each offsets-stage scan zeroes the other's descriptors
-    CK(cudaMemsetAsync(S.scan_state[0], 0, 3 * ((size_t)S.scan_tiles_cap + 1) * sizeof(unsigned long long),
-                       c->stream), "clear scan descriptors");
-  }
-  S.ctr = galloc<cg::Counters>(g, 1, &st);
+  // tiles of the heads bitmap: 8192 reads, more for graphs of over 16.7M reads
+  // (at most 2048 tiles, as every block of the scan adds up the sums before its own)
+  S.h_shift = 13;
+  while ((N >> S.h_shift) >= 2048) ++S.h_shift;
+  S.h_tiles = (int)((N + ((size_t)1 << S.h_shift) - 1) >> S.h_shift);
+  // the counters, and behind them the lone reads' tile sums (cleared together by the mask stage)
+  unsigned char* ctr = galloc<unsigned char>(g, sizeof(cg::Counters) + 8 * (size_t)S.h_tiles, &st);
+  S.ctr = reinterpret_cast<cg::Counters*>(ctr);
+  S.hsum_mask = ctr ? reinterpret_cast<unsigned long long*>(ctr + sizeof(cg::Counters)) : nullptr;
+  S.hsum = galloc<unsigned long long>(g, (size_t)S.h_tiles, &st);
+  S.scan_tiles_cap = (int64_t)(N + cg::kPieceTile - 1) / cg::kPieceTile;
+  S.scan_state = galloc<unsigned long long>(g, (size_t)S.scan_tiles_cap + 1, &st);
   S.tickets = galloc<unsigned long long>(g, cg::kTicketSets * cg::kTicketStride, &st);
   g->d_sum = galloc<unsigned long long>(g, 1, &st);
   S.derr = c->derr;
   if (st != CG_OK) return st;
-  CK(cudaMemsetAsync(S.ctr, 0, sizeof(cg::Counters), c->stream), "clear counters");
+  CK(cudaMemsetAsync(S.ctr, 0, sizeof(cg::Counters) + 8 * (size_t)S.h_tiles, c->stream), "clear counters");
   CK(cudaMemsetAsync(g->d_sum, 0, 8, c->stream), "clear sum");
 
   if (!(flags & CG_NO_VALIDATE) && n > 0) CK(cg::launch_validate(G, c->derr, c->env), "validation kernels");

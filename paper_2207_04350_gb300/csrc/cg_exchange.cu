@@ -256,7 +256,7 @@ cudaError_t launch_x_scan_pairs(const Scratch& s, const XchgArgs& x, long long n
   const long long tiles = (n_pairs + kTileItems - 1) / kTileItems;
   if (tiles > state_cap) return cudaErrorInvalidValue;
   cudaMemsetAsync(state, 0, (size_t)(state_cap + 1) * sizeof(unsigned long long), env.stream);
-  k_scan<<<scan_grid(tiles, env), kBlock, 0, env.stream>>>(XPairLoad{s, x}, XPairStore{slot}, n_pairs, nullptr, state,
+  k_scan<<<scan_grid(tiles, env), kBlock, 0, env.stream>>>(XPairLoad{s, x}, XPairStore{slot}, n_pairs, state,
                                                            state_cap, s.derr, (int)K_SCAN_OFFSETS);
   mark(env, "k_scan_exchange_pairs");
   return cudaGetLastError();
@@ -271,7 +271,7 @@ cudaError_t launch_x_scan(const Scratch& s, const XchgArgs& x, long long j0, lon
   if (tiles > state_cap) return cudaErrorInvalidValue;
   cudaMemsetAsync(state, 0, (size_t)(state_cap + 1) * sizeof(unsigned long long), env.stream);
   k_scan<<<scan_grid(tiles, env), kBlock, 0, env.stream>>>(XLoad{s, x, j0, who}, XStore{s, x, j0, who, slot}, count,
-                                                           nullptr, state, state_cap, s.derr, (int)K_SCAN_OFFSETS);
+                                                           state, state_cap, s.derr, (int)K_SCAN_OFFSETS);
   mark(env, "k_scan_exchange");
   return cudaGetLastError();
 }

@@ -52,6 +52,7 @@ __device__ __forceinline__ int sampled(int v, int ruler_log2) {
 __device__ __forceinline__ void mark_head(const Scratch& s, int32_t m, int32_t q) {
   atomicOr(&s.hb[m >> 5], 1u << (m & 31));
   s.headq[m] = q;
+  atomicAdd(&s.hsum[m >> s.h_shift], (1ull << kHeadShift) | (unsigned)q);
 }
 
 // Software grid barrier for kernels launched cooperatively (all blocks
@@ -307,12 +308,10 @@ __global__ void __launch_bounds__(kBlock, CG_MASK_MIN_BLOCKS) k_mask(DevGraph g,
       kl += nl;
 #pragma unroll
       for (int j = 0; j < kMaskLane; ++j)
-        if ((lone >> j) & 1u) {
-          const int32_t v = (int32_t)(wbase + p0 + j);
-          bl[kl++] = v;
-          s.headq[v] = 1;
-        }
+        if ((lone >> j) & 1u) bl[kl++] = (int32_t)(wbase + p0 + j);
       nl += L;
+      // a pass lies inside one tile of the heads bitmap (tiles hold 2^13 reads or more)
+      if (lane == 0 && L) atomicAdd(&s.hsum_mask[wbase >> s.h_shift], L * ((1ull << kHeadShift) | 1ull));
     } else if (lane < kMaskSpan / 32 && 32 * lane < cnt) {
       s.hb_mask[(wbase >> 5) + lane] = 0u;
     }
@@ -432,7 +431,9 @@ __global__ void __launch_bounds__(kBlock) k_succ(DevGraph g, Scratch s, int rule
   uint32_t* const bs = b_start[wib];
   unsigned ns = 0, nh = 0;                           // buffered starts (warp-uniform), and the heads among them
   // the chain stage's heads bitmap starts from the mask stage's words (lone reads)
+  // and so do the tile sums of it
   for (long long w = grid_tid(); w < (g.n + 31) / 32; w += grid_threads()) s.hb[w] = s.hb_mask[w];
+  for (long long t = grid_tid(); t < s.h_tiles; t += grid_threads()) s.hsum[t] = s.hsum_mask[t];
   const long long Nw = (N + 31) / 32 * 32;           // whole warps iterate together
   for (long long ci = grid_tid(); ci < Nw; ci += grid_threads()) {
     int s0 = -1, s1 = -1;
@@ -673,6 +674,7 @@ __global__ void k_final(DevGraph g, Scratch s) {
   const long long n = (N + 31) & ~31ll;
   const int4* pj = s.pj[fb];
   const long long T = grid_threads();
+  unsigned heads = 0;                      // contig heads this thread marked
   for (long long k0 = grid_tid(); k0 < n; k0 += kFinalItems * T) {   // warp-uniform trip count
     bool in[kFinalItems];
     int32_t v[kFinalItems];
@@ -749,18 +751,20 @@ __global__ void k_final(DevGraph g, Scratch s) {
         s.prd[ci] = make_int4(m[j], rk[j], len, o[j]);
         if (v[j] == m[j]) {
           mark_head(s, m[j], q[j]);
-          atomicAdd(&c->n_heads, 1u);
+          ++heads;
         }
       } else if (in[j] && !cyc[j]) {
         s.prd[ci] = make_int4(-1, -1, 0, 255);
       } else if (!in[j] && ci < N && g.min_chain <= 1) {   // cut off by branch reads: its own contig
         mark_head(s, v[j], 1);
-        atomicAdd(&c->n_heads, 1u);
+        ++heads;
       }
       const unsigned slot = warp_append(&c->n_cycle_reads, cyc[j]);
       if (cyc[j]) s.cyc[slot] = (int32_t)ci;
     }
   }
+  heads = __reduce_add_sync(0xffffffffu, heads);
+  if ((threadIdx.x & 31) == 0 && heads) atomicAdd(&c->n_heads, heads);
 }
 
 // Closed chains (rare). Over their oriented candidates: pointer jumping for
@@ -935,7 +939,10 @@ cudaError_t launch_sum_len(const DevGraph& g, unsigned long long* out, const Lau
 }
 
 cudaError_t launch_mask(const DevGraph& g, const Scratch& s, const LaunchEnv& env) {
-  cudaMemsetAsync(&s.ctr->n_branch, 0, sizeof(Counters) - offsetof(Counters, n_branch), env.stream);
+  // the counters and, right behind them, the tile sums of the lone reads
+  cudaMemsetAsync(&s.ctr->n_branch, 0,
+                  sizeof(Counters) - offsetof(Counters, n_branch) + (size_t)s.h_tiles * sizeof(unsigned long long),
+                  env.stream);
   const bool al = (reinterpret_cast<uintptr_t>(g.row_ptr) & 15) == 0;   // 16-byte row_ptr loads
   if (g.rp64) {
     if (al) launch_mask_kernel<int64_t, true>(g, s, env);

@@ -8,6 +8,8 @@
 namespace cg {
 
 constexpr int kBlock = 256;
+constexpr int kPieceTile = 1024; // walk positions per tile of the piece scan
+constexpr int kHeadShift = 31;   // heads-bitmap sums: the count of heads above, their contigs' reads below (both < 2^30)
 
 // First device-side error wins (atomicCAS from 0).
 enum : int32_t {
@@ -123,7 +125,12 @@ struct Scratch {
   // part[c] != part_p add no bases, so the layout holds that part's contigs only
   const int32_t* part;  // n_contigs, or nullptr for the whole layout
   int32_t part_p;
-  unsigned long long* scan_state[3];  // look-back tile descriptors (+1 ticket word) of the three scans
+  // sums over tiles of the heads bitmap, added up by the kernels that mark the
+  // heads, so that the scan of the heads starts from them (cg_scan.cu)
+  unsigned long long* hsum_mask;  // h_tiles: the lone reads of each tile of 2^h_shift reads (heads << 31 | reads)
+  unsigned long long* hsum;       // h_tiles: all contig heads of the tile and their contigs' reads
+  int h_shift, h_tiles;
+  unsigned long long* scan_state; // look-back descriptors of the piece scan (+1 ticket word)
   int64_t scan_tiles_cap;
   Counters* ctr;
   DevError* derr;

@@ -104,7 +104,7 @@ extern "C" CG_API cg_status cg_offsets_noalloc(const int32_t* lengths, int64_t c
     cg::LaunchEnv env = {};
     env.num_sms = su.num_sms;
     const unsigned grid = cg::scan_grid(tiles, env);
-    cg::k_scan<LenLoad, OffStore><<<grid, cg::kBlock, 0, s>>>(LenLoad{lengths}, OffStore{offsets}, count, nullptr,
+    cg::k_scan<LenLoad, OffStore><<<grid, cg::kBlock, 0, s>>>(LenLoad{lengths}, OffStore{offsets}, count,
                                                               state, tiles, derr, (int)cg::K_SCAN_OFFSETS);
     if (cudaGetLastError() != cudaSuccess) return CG_ECUDA;
   }

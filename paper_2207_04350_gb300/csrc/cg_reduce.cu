@@ -177,7 +177,7 @@ cudaError_t launch_transitive(const DevGraph& g, int fuzz, const TrBuffers& t, c
   if (tiles > t.state_cap) return cudaErrorInvalidValue;
   if (g.n > 0) {
     k_scan<<<scan_grid(tiles, env), kBlock, 0, env.stream>>>(RowCntLoad{t.row_cnt}, RowPtrStore{t.out_rp, t.total}, g.n,
-                                                       nullptr, t.state, t.state_cap, t.derr, K_TRANSITIVE);
+                                                       t.state, t.state_cap, t.derr, K_TRANSITIVE);
     mark(env, "k_scan_rows");
   } else {
     cudaMemsetAsync(t.out_rp, 0, sizeof(int64_t), env.stream);

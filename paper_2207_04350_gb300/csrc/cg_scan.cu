@@ -5,8 +5,7 @@
 //   1. scan over the words of the heads bitmap (bit m set when read m is the
 //      smallest read of a contig) of their heads and those heads' read
 //      counts: the contig index of every head, listing contigs by smallest
-//      read id, and every contig's first walk position; the store step lays
-//      the read counts out in contig order;
+//      read id, and every contig's first walk position and read count;
 //   2. scatter every spelled read to walk position first(contig) + rank: the
 //      on-device compaction that replaces the induced-subgraph exchange;
 //   3. scan over walk positions of the bases each read adds: the output
@@ -17,11 +16,12 @@
 // the reads of other parts' contigs empty pieces, so step 3 lays out that
 // part's contigs alone, back to back.
 //
-// The scans are single-pass decoupled look-back scans: tiles take tickets in
-// order, publish their aggregate, then look back over predecessors with one
-// warp (32 descriptors at a time) until an inclusive prefix is found. The
-// wait on a predecessor is bounded; on timeout the kernel records
-// DERR_TIMEOUT and stops.
+// The scan of step 1 takes a block per tile, and whoever marks a head also adds
+// it to the sum of its tile (mark_head, and the mask's lone reads): a tile's
+// start is the sum of the tile sums before it, read by its own block, and no
+// block waits for another. There are at most 2048 tiles; larger graphs have
+// larger ones. The scan of step 3 is a single-pass decoupled look-back scan
+// (cg_lookback.cuh), whose wait on a predecessor is bounded.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -33,84 +33,116 @@ namespace cg {
 
 namespace {
 
-// ---- scan 1: contig index and first walk position of every head ----
-// The value of bitmap word w packs the contigs headed in it (their count,
-// above bit kHeadShift) and their reads (below): both stay under 2^30, so
-// one scan gives every head its contig index and its contig's first walk
-// position at once.
-constexpr int kHeadShift = 31;
-constexpr unsigned long long kHeadLow = (1ull << kHeadShift) - 1;
+// Block-wide exclusive prefix of one 64-bit value per thread; the sum of all in
+// *total. `tot` is shared memory of kBlock / 32 words, free again after a barrier.
+__device__ __forceinline__ unsigned long long block_exclusive(unsigned long long v, unsigned long long* tot,
+                                                              unsigned long long* total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned long long inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long t = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += t;
+  }
+  if (lane == 31) tot[warp] = inc;
+  __syncthreads();
+  unsigned long long before = 0, all = 0;
+#pragma unroll
+  for (int w = 0; w < kBlock / 32; ++w) {
+    if (w < warp) before += tot[w];
+    all += tot[w];
+  }
+  *total = all;
+  return before + inc - v;
+}
 
-struct HeadWordLoad {
-  const unsigned* hb;
-  const int32_t* headq;
-  // the word's bits and the read count of its first head
-  using Item = int2;
-  __device__ int2 fetch(long long w) const {
-    const unsigned bits = hb[w];
-    return make_int2((int)bits, bits ? headq[32 * w + __ffs(bits) - 1] : 0);
-  }
-  __device__ unsigned long long value(long long w, const int2& it) const {
-    unsigned bits = (unsigned)it.x;
-    const unsigned long long heads = (unsigned long long)__popc(bits);
-    unsigned long long reads = (unsigned)it.y;
-    if (bits) bits &= bits - 1;
-    while (bits) {                     // a second head in one word: rare
-      reads += (unsigned)headq[32 * w + __ffs(bits) - 1];
-      bits &= bits - 1;
+// Block-wide sum, the same scratch.
+__device__ __forceinline__ unsigned long long block_sum(unsigned long long v, unsigned long long* tot) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) tot[threadIdx.x >> 5] = v;
+  __syncthreads();
+  unsigned long long all = 0;
+#pragma unroll
+  for (int w = 0; w < kBlock / 32; ++w) all += tot[w];
+  return all;
+}
+
+// Contig index and first walk position of every head, a block per tile of the
+// heads bitmap (256 words or more). The value of a word packs the contigs
+// headed in it (their count, above bit kHeadShift) and their reads (below):
+// both stay under 2^30, so one scan gives every head its contig index and its
+// contig's first walk position at once. A lone read's contig has one read; only
+// the chain heads' read counts are loaded. The kernels that marked the heads
+// added up every tile's sum (hsum), so a block adds the sums before its tile,
+// a load or a few per thread, and waits for no other block: what bounds it is
+// three dependent loads and the block scan: 14.3 us by events on the 3.1 Gb
+// graph. With tiles of 2048 words that looked back over their predecessors it
+// took 30.7 us there (95 tiles in flight at once, each waiting for the one
+// before), and 131 us on 94 thousand lone reads, whose 32 heads per word one
+// thread then loaded in turn (the whole step: 397 us before, 283 now).
+__global__ void __launch_bounds__(kBlock) k_heads(Scratch s, long long n, int64_t* user_off, long long user_cap) {
+  pdl_enter();
+  __shared__ unsigned long long tot[2][kBlock / 32];   // the prefix's sums, the words' sums
+  for (long long i = grid_tid(); i <= s.scan_tiles_cap; i += grid_threads()) s.scan_state[i] = 0ull;   // of the piece scan
+  const int tile = (int)blockIdx.x, tid = threadIdx.x;
+  unsigned long long run = 0;
+  for (int i = tid; i < tile; i += kBlock) run += s.hsum[i];
+  const long long per = 1ll << (s.h_shift - 5);
+  const long long w_end = min((n + 31) / 32, (tile + 1) * per);
+  bool first = true;
+  for (long long wb = tile * per; wb < w_end; wb += kBlock) {
+    const long long w = wb + tid;
+    unsigned bits = w < w_end ? s.hb[w] : 0u;
+    const unsigned lone = w < w_end ? s.hb_mask[w] : 0u, chain = bits & ~lone;
+    const int32_t* const hq = s.headq + 32 * w;
+    const unsigned q0 = chain ? (unsigned)hq[__ffs(chain) - 1] : 0u;
+    unsigned long long reads = __popc(lone) + q0;
+    for (unsigned c = chain & (chain - 1); c; c &= c - 1) reads += (unsigned)hq[__ffs(c) - 1];   // rare
+    if (first) {
+      run = block_sum(run, tot[1]);
+      first = false;
     }
-    return (heads << kHeadShift) | reads;
-  }
-};
-struct HeadWordStore {
-  unsigned* wp;
-  const int32_t* headq;
-  int32_t* qd;
-  unsigned long long* cbase;
-  int64_t* contig_off;
-  int64_t* user_off;           // the caller's contig offsets, written by the piece scan (or nullptr)
-  long long user_cap;
-  Counters* c;
-  __device__ void item(long long w, unsigned long long e, const int2& it) const {
-    unsigned k = (unsigned)(e >> kHeadShift);
-    wp[w] = k;
-    unsigned bits = (unsigned)it.x;
-    if (!bits) return;
-    unsigned long long r = e & kHeadLow;
-    int32_t q = it.y;
-    for (;;) {                         // contigs in order of their smallest read
-      qd[k] = q;
-      cbase[k] = r;
-      r += (unsigned)q;
-      ++k;
-      bits &= bits - 1;
-      if (!bits) break;
-      q = headq[32 * w + __ffs(bits) - 1];
+    unsigned long long all;
+    const unsigned long long e =
+        run + block_exclusive(((unsigned long long)__popc(bits) << kHeadShift) | reads, tot[0], &all);
+    if (w < w_end) {
+      unsigned k = (unsigned)(e >> kHeadShift);
+      unsigned long long r = e & ((1ull << kHeadShift) - 1);
+      s.wp[w] = k;
+      for (; bits; bits &= bits - 1, ++k) {            // contigs in order of their smallest read
+        const int b = __ffs(bits) - 1;
+        const unsigned q = (lone >> b) & 1u ? 1u : (b == __ffs(chain) - 1 ? q0 : (unsigned)hq[b]);
+        s.qd[k] = (int32_t)q;
+        s.cbase[k] = r;
+        r += q;
+      }
     }
+    run += all;
+    __syncthreads();                                   // tot is reused by the next words
   }
-  __device__ void last(long long, unsigned long long total) const {
-    const unsigned C = (unsigned)(total >> kHeadShift);
+  if (tile == (int)gridDim.x - 1 && tid == 0) {
+    Counters* c = s.ctr;
+    unsigned C = (unsigned)(run >> kHeadShift);
+    unsigned long long W = run & ((1ull << kHeadShift) - 1);
+    if (W > (unsigned long long)n) {                   // contigs of more reads than there are: not a string graph
+      set_error(s.derr, DERR_KERNEL, K_SCAN_HEADS, (long long)W);
+      C = 0;
+      W = 0;
+    }
     c->n_contigs = C;
-    cbase[C] = total & kHeadLow;
-    c->n_walk = (unsigned)(total & kHeadLow);
-    if (C == 0) {                      // no contigs: the piece scan has nothing to scan
-      contig_off[0] = 0;
+    s.cbase[C] = W;
+    c->n_walk = (unsigned)W;
+    if (C == 0) {                                      // no contigs: the piece scan has nothing to scan
+      s.contig_off[0] = 0;
       if (user_off && user_cap >= 1) user_off[0] = 0;
       c->total_bases = 0;
       c->n_tiles = 0;
     }
   }
-};
+}
 
-// ---- scan 3: piece offsets over walk positions ----
-struct PieceLoad {
-  const int32_t* wlen;
-  const int32_t* wfirst;
-  // the piece's length and the contig it starts, or -1
-  using Item = int2;
-  __device__ int2 fetch(long long j) const { return make_int2(wlen[j], wfirst[j]); }
-  __device__ unsigned long long value(long long, const int2& it) const { return (unsigned long long)(unsigned)it.x; }
-};
+// What the piece scan writes for walk position j: a piece of L bases from
+// output offset o on, the first of contig `starts` (or -1).
 struct PieceStore {
   int64_t* out_off;
   int64_t* contig_off;
@@ -127,12 +159,11 @@ struct PieceStore {
   __device__ bool user_fits() const {
     return user_off && (long long)*(const volatile unsigned*)&c->n_contigs + 1 <= user_cap;
   }
-  __device__ void item(long long j, unsigned long long e, const int2& it) const {
-    long long o = (long long)e, L = it.x;
+  __device__ void item(long long j, long long o, long long L, int32_t starts) const {
     out_off[j] = o;
-    if (it.y >= 0) {
-      contig_off[it.y] = o;
-      if (user_fits()) user_off[it.y] = o;
+    if (starts >= 0) {
+      contig_off[starts] = o;
+      if (user_fits()) user_off[starts] = o;
     }
     // tile_bytes is a power of two: the first tile starting at or after o, and after o + L
     const int sh = __ffsll(tile_bytes) - 1;
@@ -156,6 +187,55 @@ struct PieceStore {
     else set_error(derr, DERR_KERNEL, K_SCAN_OFFSETS, nt);
   }
 };
+
+// Piece offsets over the walk positions, in tiles of kPieceTile positions, four
+// per thread, with a decoupled look-back (cg_lookback.cuh). Adding up every
+// tile's bases in the scatter instead, as the heads' sums are, cost the scatter
+// 30 us on the 3.1 Gb graph (a thousand additions to each of 410 words).
+constexpr int kPieceItems = kPieceTile / kBlock;
+static_assert(kPieceItems == 4, "one 16-byte load per thread and array");
+
+__global__ void __launch_bounds__(kBlock) k_pieces(Scratch s, PieceStore ps) {
+  pdl_enter();
+  __shared__ unsigned long long tot[kBlock / 32];
+  __shared__ long long s_tile;
+  const int tid = threadIdx.x;
+  const long long W = *(const volatile unsigned*)&s.ctr->n_walk;
+  const long long tiles = (W + kPieceTile - 1) / kPieceTile;
+  if ((long long)blockIdx.x >= tiles) return;
+  for (;;) {
+    if (tid == 0) s_tile = (long long)atomicAdd(&s.scan_state[s.scan_tiles_cap], 1ull);
+    __syncthreads();
+    const long long tile = s_tile;
+    if (tile >= tiles) return;                         // block-uniform
+    const long long i0 = tile * kPieceTile + kPieceItems * tid;
+    int32_t L[kPieceItems], f[kPieceItems];
+    if (i0 + kPieceItems <= W) {
+      const int4 a = *reinterpret_cast<const int4*>(s.wlen + i0), b = *reinterpret_cast<const int4*>(s.wfirst + i0);
+      L[0] = a.x; L[1] = a.y; L[2] = a.z; L[3] = a.w;
+      f[0] = b.x; f[1] = b.y; f[2] = b.z; f[3] = b.w;
+    } else {
+#pragma unroll
+      for (int k = 0; k < kPieceItems; ++k) {
+        L[k] = i0 + k < W ? s.wlen[i0 + k] : 0;
+        f[k] = i0 + k < W ? s.wfirst[i0 + k] : -1;
+      }
+    }
+    unsigned long long sum = 0;
+#pragma unroll
+    for (int k = 0; k < kPieceItems; ++k) sum += (unsigned)L[k];
+    unsigned long long all, e = block_exclusive(sum, tot, &all);
+    e += lookback(s.scan_state, tile, all, s.derr, (int)K_SCAN_OFFSETS);
+#pragma unroll
+    for (int k = 0; k < kPieceItems; ++k) {
+      if (i0 + k >= W) break;
+      ps.item(i0 + k, (long long)e, L[k], f[k]);
+      e += (unsigned)L[k];
+      if (i0 + k == W - 1) ps.last(W, e);
+    }
+    __syncthreads();                                   // s_tile and tot are reused by the next tile
+  }
+}
 
 // Every spelled read goes to walk position first(contig) + rank, with the
 // stored-base address of its piece (for one part's layout, an empty piece
@@ -255,40 +335,24 @@ __global__ void k_export_contig_off(Scratch s, int64_t* out, long long cap) {
 
 cudaError_t launch_offsets(const DevGraph& g, const Scratch& s, const Tuning& t, const LaunchEnv& env,
                            int64_t* user_off, long long user_cap) {
-  // No memset: the scans' last steps assign every counter of this stage, and
-  // each scan zeroes the other one's descriptors (the heads scan the piece
-  // scan's, the piece scan the heads scan's, for the next run); the graph
-  // load zeroes both once.
-  const long long words = (g.n + 31) / 32;
-  const long long tiles_w = (words + kTileItems - 1) / kTileItems;
-  const long long tiles_n = (g.n + kTileItems - 1) / kTileItems;
-  if (tiles_n > s.scan_tiles_cap || tiles_w > s.scan_tiles_cap) return cudaErrorInvalidValue;
-  const long long state_words = s.scan_tiles_cap + 1;
   if (g.n == 0) {
     k_contig_off<<<1, kBlock, 0, env.stream>>>(s);
     mark(env, "k_contig_off");
     return cudaGetLastError();
   }
-  HeadWordLoad hl{s.hb, s.headq};
-  HeadWordStore hs{s.wp, s.headq, s.qd, s.cbase, s.contig_off, user_off, user_cap, s.ctr};
-  cudaError_t e = launch_k(k_scan<HeadWordLoad, HeadWordStore>, scan_grid(tiles_w, env), env, env.pdl_first, hl, hs,
-                           words, (const unsigned*)nullptr, s.scan_state[0], s.scan_tiles_cap, s.derr,
-                           (int)K_SCAN_HEADS, s.scan_state[2], state_words);
+  cudaError_t e = launch_k(k_heads, s.h_tiles, env, env.pdl_first, s, (long long)g.n, user_off, user_cap);
   if (e != cudaSuccess) return e;
-  mark(env, "k_scan_heads");
+  mark(env, "k_heads");
   static const int scatter_resident = resident_blocks(k_scatter);   // a persistent grid
   const long long scatter_need = (g.n + (long long)kBlock * kScatterItems - 1) / ((long long)kBlock * kScatterItems);
   e = launch_k(k_scatter, (int)std::max(1LL, std::min((long long)env.num_sms * scatter_resident, scatter_need)), env,
                true, g, s);
   if (e != cudaSuccess) return e;
   mark(env, "k_scatter");
-  PieceLoad pl{s.wlen, s.wfirst};
   PieceStore ps{s.out_off, s.contig_off, s.tile_seg, s.tiles_cap, t.tile_bytes, s.ctr, s.derr, user_off, user_cap};
-  e = launch_k(k_scan<PieceLoad, PieceStore>, scan_grid(tiles_n, env), env, true, pl, ps, 0ll,
-               (const unsigned*)&s.ctr->n_walk, s.scan_state[2], s.scan_tiles_cap, s.derr, (int)K_SCAN_OFFSETS,
-               s.scan_state[0], state_words);
+  e = launch_k(k_pieces, (int)std::min((long long)s.scan_tiles_cap, (long long)env.num_sms * 4), env, true, s, ps);
   if (e != cudaSuccess) return e;
-  mark(env, "k_scan_pieces");
+  mark(env, "k_pieces");
   return cudaGetLastError();
 }
 
@@ -303,7 +367,7 @@ struct NoStore {
 }  // namespace
 
 cudaError_t launch_selftest_wait(unsigned long long* state, long long tiles, DevError* derr, const LaunchEnv& env) {
-  k_scan<<<scan_grid(tiles, env), kBlock, 0, env.stream>>>(ZeroLoad{}, NoStore{}, tiles * kTileItems, nullptr, state,
+  k_scan<<<scan_grid(tiles, env), kBlock, 0, env.stream>>>(ZeroLoad{}, NoStore{}, tiles * kTileItems, state,
                                                            tiles, derr, (int)K_SELFTEST_WAIT);
   mark(env, "k_scan_selftest");
   return cudaGetLastError();
@@ -487,7 +551,7 @@ cudaError_t launch_partition(const Scratch& s, long long C, int weight, long lon
       k_sort_hist<<<grid, kBlock, 0, env.stream>>>(b.key[cur], C, pass, b.hist, tiles);
       mark(env, "k_sort_hist");
       cudaMemsetAsync(b.state, 0, (size_t)(b.state_cap + 1) * sizeof(unsigned long long), env.stream);
-      k_scan<<<scan_grid(scan_tiles, env), kBlock, 0, env.stream>>>(HistLoad{b.hist}, HistStore{b.base}, nh, nullptr,
+      k_scan<<<scan_grid(scan_tiles, env), kBlock, 0, env.stream>>>(HistLoad{b.hist}, HistStore{b.base}, nh,
                                                               b.state, b.state_cap, s.derr, K_SORT);
       mark(env, "k_scan_digits");
       k_sort_scatter<<<grid, kBlock, 0, env.stream>>>(b.key[cur], b.val[cur], b.key[cur ^ 1], b.val[cur ^ 1], C,

@@ -1,0 +1,46 @@
+"""The layout's scans at the edges of their tiles, against the oracle: contig
+heads in tiles of 8,192 reads (lone reads fill whole words of the heads bitmap,
+chain heads sit between them), pieces in tiles of 1,024 walk positions, and
+more pieces than one look (256 tiles) of the look-back covers."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2207_04350_gb300 import cg
+from tests._gpu import assert_parity, run_gpu
+from tests._graphs import structured
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import torch
+    from paper_2207_04350_gb300 import _build
+    _build.build()
+    assert torch.cuda.is_available()
+    c = cg.cg_create(0)
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("sizes,lone,mcr", [
+    ([], 1, 1), ([], 31, 1), ([], 33, 1),                               # a word of heads
+    ([], 8191, 1), ([], 8192, 1), ([], 8193, 1), ([2, 5], 16384, 1),    # a tile of the heads bitmap
+    ([1023], 0, 2), ([1024], 0, 2), ([1025], 0, 2),                     # a tile of pieces
+    ([2] * 512, 9000, 2), ([2] * 513, 9000, 2),                         # heads in every other word
+    ([3, 1, 2, 40, 1], 270_000, 1),                                     # 264 tiles of pieces
+])
+def test_tile_edges(ctx, sizes, lone, mcr):
+    G = structured(len(sizes) + lone, sizes, lone=lone)
+    assert_parity(run_gpu(ctx, G, min_chain_reads=mcr, inputs="device", outputs="device"),
+                  oracle.run(G, min_chain_reads=mcr))
+
+
+def test_heads_in_one_word(ctx):
+    """Chains whose smallest reads are neighbours: several chain heads per word,
+    with lone reads between them, in both minimum chain lengths."""
+    G = structured(21, [2] * 3000, lone=50)
+    for mcr in (1, 2):
+        assert_parity(run_gpu(ctx, G, min_chain_reads=mcr), oracle.run(G, min_chain_reads=mcr))
+    assert np.count_nonzero(oracle.run(G).contig_off) == 3000
