@@ -68,8 +68,9 @@ struct cg_graph {
   int32_t* part_buf = nullptr;         // device copy of a host part assignment (cg_emit_part)
   int64_t part_buf_cap = 0;
   unsigned long long* d_sum = nullptr;
-  StageExec execs[8];                  // mask, chains, offsets, emission, contig_off export, 2-bit emission,
-                                       // offsets + emission + export in one graph, all stages in one graph
+  StageExec execs[12];                 // mask, chains, offsets, emission, contig_off export, 2-bit emission; then for
+                                       // contigs, 2-bit contigs and a share of them (Form): offsets + emission +
+                                       // export in one graph, all stages in one graph
   int batch_k = 0;                     // graphs of a batch (0: a single graph)
   int64_t* batch_R = nullptr;          // device: first read of each graph, batch_k + 1 entries
   // a batch whose reads stay in pinned host memory: per graph its stream's
@@ -415,6 +416,71 @@ void* pinned_device_alias(const void* p) {
   if (a.type != cudaMemoryTypeHost || !a.devicePointer || !a.hostPointer) return nullptr;
   // the alias of p itself (p may lie inside a larger pinned allocation)
   return (char*)a.devicePointer + ((const char*)p - (const char*)a.hostPointer);
+}
+
+// The layout, the spelling into a device buffer and the caller's contig offsets
+// replayed as one graph; with the mask and chain launches too when both wait (a
+// whole step in one). Each graph launch of its own leaves the GPU idle a few
+// microseconds, and so does each memset between two kernels: the 2-bit step of a
+// 1.2 Gb genome took 246 us as four graphs and a copy kernel and takes 225 as one,
+// the step of a 1 Mb genome 51.5 and 43.
+enum class Form { kAscii, k2Bit, kShare };
+
+cg_status spell_device(cg_graph* g, Form form, int64_t* contig_off, int64_t contig_off_cap, uint8_t* out, int64_t cap,
+                       int share, int n_shares) {
+  cg_ctx* c = g->ctx;
+  cg_status st = CG_OK;
+  const bool whole = g->want == 2 && g->stage == 0 && defer_ok(c);
+  if (!whole) {
+    if (g->want) {
+      st = flush(g);
+      if (st != CG_OK) return st;
+    }
+    if (g->stage < 2) {
+      st = run_chains(g);
+      if (st != CG_OK) return st;
+    }
+  }
+  g->want = 0;
+  const bool timing = c->timing != 0, stages = timing && !c->timing_emit_only;
+  uint64_t key = mix_key(mix_key(mix_key(mix_key((uint64_t)(uintptr_t)out, (uint64_t)cap),
+                                         (uint64_t)(uintptr_t)g->g.packed), (uint64_t)gt(g).tile_bytes),
+                         (uint64_t)cg::emit_launch_key(gt(g)));
+  key = mix_key(mix_key(mix_key(key, (uint64_t)(uintptr_t)contig_off), (uint64_t)contig_off_cap),
+                stages ? 3 : (timing ? 5 : 4));
+  key = mix_key(mix_key(key, (uint64_t)share), (uint64_t)n_shares);
+  if (whole) key = mix_key(key, (uint64_t)gt(g).ruler_log2);
+  // the caller's contig offsets come from the piece scan itself (no copy kernel)
+  const bool fold_off = contig_off && g->g.n > 0;
+  st = run_stage(g, 6 + 2 * (int)form + (whole ? 1 : 0), key, [&]() -> cg_status {
+    cg::LaunchEnv env = c->env;
+    if (whole) {
+      CK(cg::launch_mask(g->g, g->s, c->env), "mask kernels");
+      CK(cg::launch_chains(g->g, g->s, gt(g), c->env, true), "chain kernels");
+      env.pdl_first = true;
+    }
+    if (stages) record_stage_event(c, 4);
+    CK(cg::launch_offsets(g->g, g->s, gt(g), env, fold_off ? contig_off : nullptr, fold_off ? contig_off_cap : 0),
+       "offset kernels");
+    if (stages) record_stage_event(c, 5);
+    if (timing) record_stage_event(c, 6);
+    env.pdl_first = !timing;           // no event node between these kernels and the ones before
+    const bool after_layout = g->g.n > 0;
+    if (form != Form::k2Bit)
+      CK(cg::launch_emit(g->g, g->s, gt(g), out, cap, env, 0, 1ll << 62, share, n_shares, after_layout),
+         "emission kernel");
+    else
+      CK(cg::launch_emit2(g->g, g->s, gt(g), out, cap, env, 0, 1ll << 62, after_layout), "2-bit emission kernel");
+    if (timing) record_stage_event(c, 7);
+    if (contig_off && !fold_off)
+      CK(cg::launch_export_contig_off(g->s, contig_off, contig_off_cap, env), "export contig_off");
+    return CG_OK;
+  });
+  if (st != CG_OK) return st;
+  if (stages) c->recorded[2] = true;
+  if (timing) c->recorded[3] = true;
+  g->stage = 3;
+  return CG_OK;
 }
 
 // Scratch, input checks and output bounds of a graph whose inputs are in place.
@@ -1139,52 +1205,9 @@ cg_status cg_emit_contigs(cg_graph* g, int64_t* contig_off, int64_t contig_off_c
   if (mem != CG_MEM_HOST && mem != CG_MEM_DEVICE) return fail(c, CG_EINVAL, "bad mem");
   if ((bases && bases_cap < 0) || (contig_off && contig_off_cap < 1)) return fail(c, CG_EINVAL, "bad capacity");
   if (mem == CG_MEM_DEVICE && bases && !g->host_batch) {
-    // the layout, the spelling and the offsets export replayed as one graph;
-    // with the mask and chain launches too when both wait (a whole step in one)
     if (!aligned(bases, 16)) return fail(c, CG_EINVAL, "device bases buffer must be 16-byte aligned");
-    const bool whole = g->want == 2 && g->stage == 0 && defer_ok(c);
-    if (!whole) {
-      if (g->want) {
-        st = flush(g);
-        if (st != CG_OK) return st;
-      }
-      if (g->stage < 2) {
-        st = run_chains(g);
-        if (st != CG_OK) return st;
-      }
-    }
-    g->want = 0;
-    const bool timing = c->timing != 0, stages = timing && !c->timing_emit_only;
-    uint64_t key = mix_key(mix_key(mix_key(mix_key((uint64_t)(uintptr_t)bases, (uint64_t)bases_cap),
-                                           (uint64_t)(uintptr_t)g->g.packed), (uint64_t)gt(g).tile_bytes),
-                           (uint64_t)cg::emit_launch_key(gt(g)));
-    key = mix_key(mix_key(mix_key(key, (uint64_t)(uintptr_t)contig_off), (uint64_t)contig_off_cap),
-                  stages ? 3 : (timing ? 5 : 4));
-    if (whole) key = mix_key(key, (uint64_t)gt(g).ruler_log2);
-    // the caller's contig offsets come from the piece scan itself (no copy kernel)
-    const bool fold_off = contig_off && g->g.n > 0;
-    st = run_stage(g, whole ? 7 : 6, key, [&]() -> cg_status {
-      if (whole) {
-        CK(cg::launch_mask(g->g, g->s, c->env), "mask kernels");
-        CK(cg::launch_chains(g->g, g->s, gt(g), c->env), "chain kernels");
-      }
-      if (stages) record_stage_event(c, 4);
-      CK(cg::launch_offsets(g->g, g->s, gt(g), c->env, fold_off ? contig_off : nullptr,
-                            fold_off ? contig_off_cap : 0), "offset kernels");
-      if (stages) record_stage_event(c, 5);
-      if (timing) record_stage_event(c, 6);
-      cg::LaunchEnv env = c->env;
-      env.pdl_first = !timing;           // no event node between these kernels and the ones before
-      CK(cg::launch_emit(g->g, g->s, gt(g), bases, bases_cap, env), "emission kernel");
-      if (timing) record_stage_event(c, 7);
-      if (contig_off && !fold_off)
-        CK(cg::launch_export_contig_off(g->s, contig_off, contig_off_cap, env), "export contig_off");
-      return CG_OK;
-    });
+    st = spell_device(g, Form::kAscii, contig_off, contig_off_cap, bases, bases_cap, 0, 1);
     if (st != CG_OK) return st;
-    if (stages) c->recorded[2] = true;
-    if (timing) c->recorded[3] = true;
-    g->stage = 3;
     if (n_contigs || total_bases) {
       st = wait_and_read(g);
       if (st != CG_OK) return st;
@@ -1369,20 +1392,34 @@ cg_status cg_emit_share(cg_graph* g, int32_t share, int32_t n_shares, int64_t* c
   if (n_shares < 1 || share < 0 || share >= n_shares)
     return fail(c, CG_EINVAL, "share %d of %d shares", (int)share, (int)n_shares);
   if ((bases && bases_cap < 0) || (contig_off && contig_off_cap < 1)) return fail(c, CG_EINVAL, "bad capacity");
-  st = run_offsets(g);
-  if (st != CG_OK) return st;
-  if (bases) {
-    st = prepare_emit(g);
-    if (st != CG_OK) return st;
-  }
-  // the share's stream range, from the stream's size (known on the host after a wait)
   const int64_t tb = gt(g).tile_bytes;
+  // the share's stream range, from the stream's size (known on the host after a wait)
   auto range = [&](int64_t total, int64_t* fb, int64_t* nb) {
     const int64_t T = (total + tb - 1) / tb;
     const int64_t t0 = (int64_t)share * T / n_shares, t1 = (int64_t)(share + 1) * T / n_shares;
     *fb = t0 * tb;
     *nb = std::max<int64_t>(0, std::min(total, t1 * tb) - t0 * tb);
   };
+  if (mem == CG_MEM_DEVICE && bases && !g->host_batch) {
+    if (!aligned(bases, 16)) return fail(c, CG_EINVAL, "device bases buffer must be 16-byte aligned");
+    st = spell_device(g, Form::kShare, contig_off, contig_off_cap, bases, bases_cap, share, n_shares);
+    if (st != CG_OK) return st;
+    if (first_base || n_bases) {
+      st = wait_and_read(g);
+      if (st != CG_OK) return st;
+      int64_t fb = 0, nb = 0;
+      range(c->h_ctr->total_bases, &fb, &nb);
+      if (first_base) *first_base = fb;
+      if (n_bases) *n_bases = nb;
+    }
+    return CG_OK;
+  }
+  st = run_offsets(g);
+  if (st != CG_OK) return st;
+  if (bases) {
+    st = prepare_emit(g);
+    if (st != CG_OK) return st;
+  }
   auto spell = [&](uint8_t* dst, int64_t cap) -> cg_status {
     StageTimer tm(c, 3);
     uint64_t key = mix_key(mix_key(mix_key(mix_key((uint64_t)(uintptr_t)dst, (uint64_t)cap),
@@ -1685,6 +1722,18 @@ cg_status cg_emit_contigs_2bit(cg_graph* g, int64_t* contig_off, int64_t contig_
     return fail(c, CG_EINVAL, "the graph was loaded without its reads: spell a share with cg_emit_share_received");
   if (mem != CG_MEM_HOST && mem != CG_MEM_DEVICE) return fail(c, CG_EINVAL, "bad mem");
   if ((packed_out && packed_cap < 0) || (contig_off && contig_off_cap < 1)) return fail(c, CG_EINVAL, "bad capacity");
+  if (mem == CG_MEM_DEVICE && packed_out && !g->host_batch) {
+    if (!aligned(packed_out, 16)) return fail(c, CG_EINVAL, "device output buffer must be 16-byte aligned");
+    st = spell_device(g, Form::k2Bit, contig_off, contig_off_cap, packed_out, packed_cap, 0, 1);
+    if (st != CG_OK) return st;
+    if (n_contigs || total_bases) {
+      st = wait_and_read(g);
+      if (st != CG_OK) return st;
+    }
+    if (n_contigs) *n_contigs = (int64_t)c->h_ctr->n_contigs;
+    if (total_bases) *total_bases = c->h_ctr->total_bases;
+    return CG_OK;
+  }
   st = run_offsets(g);
   if (st != CG_OK) return st;
   if (packed_out) {

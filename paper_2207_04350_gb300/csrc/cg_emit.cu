@@ -221,12 +221,15 @@ namespace {
 // at once (the function-local static is initialised once, safely across threads).
 template <int BT>
 cudaError_t launch_emit_bt(const DevGraph& g, const Scratch& s, const Tuning& t, uint8_t* out, int64_t cap,
-                           const LaunchEnv& env, long long t_begin, long long t_end, int share, int n_shares) {
+                           const LaunchEnv& env, long long t_begin, long long t_end, int share, int n_shares,
+                           bool after_layout) {
   static const int resident = resident_blocks(k_emit<4, BT>, BT);
   const int per_sm = t.emit_blocks_per_sm < resident ? t.emit_blocks_per_sm : resident;
-  cudaError_t e = cudaMemsetAsync(s.tickets, 0, kTicketSets * kTicketStride * sizeof(unsigned long long), env.stream);
-  if (e != cudaSuccess) return e;
-  const bool chained = false;                     // a memset, not a kernel, comes right before
+  if (!after_layout) {
+    cudaError_t e = cudaMemsetAsync(s.tickets, 0, kTicketSets * kTicketStride * sizeof(unsigned long long), env.stream);
+    if (e != cudaSuccess) return e;
+  }
+  const bool chained = after_layout && env.pdl_first;   // otherwise a memset or an event, not a kernel, comes right before
   return launch_kb(k_emit<4, BT>, env.num_sms * per_sm, BT, env, chained, s, g.packed,
                    (long long)g.packed_bytes, (long long)(g.packed_readable / 4), out, (long long)cap, t.tile_bytes,
                    t.emit_tile, t_begin, t_end, share, n_shares);
@@ -235,12 +238,13 @@ cudaError_t launch_emit_bt(const DevGraph& g, const Scratch& s, const Tuning& t,
 }  // namespace
 
 cudaError_t launch_emit(const DevGraph& g, const Scratch& s, const Tuning& t, uint8_t* out, int64_t cap,
-                        const LaunchEnv& env, long long t_begin, long long t_end, int share, int n_shares) {
+                        const LaunchEnv& env, long long t_begin, long long t_end, int share, int n_shares,
+                        bool after_layout) {
   cudaError_t e = t.emit_block_threads == 128
-                      ? launch_emit_bt<128>(g, s, t, out, cap, env, t_begin, t_end, share, n_shares)
+                      ? launch_emit_bt<128>(g, s, t, out, cap, env, t_begin, t_end, share, n_shares, after_layout)
                   : t.emit_block_threads == 512
-                      ? launch_emit_bt<512>(g, s, t, out, cap, env, t_begin, t_end, share, n_shares)
-                      : launch_emit_bt<256>(g, s, t, out, cap, env, t_begin, t_end, share, n_shares);
+                      ? launch_emit_bt<512>(g, s, t, out, cap, env, t_begin, t_end, share, n_shares, after_layout)
+                      : launch_emit_bt<256>(g, s, t, out, cap, env, t_begin, t_end, share, n_shares, after_layout);
   if (e != cudaSuccess) return e;
   mark(env, "k_emit");
   return cudaGetLastError();

@@ -447,7 +447,7 @@ namespace {
 
 template <int BT>
 cudaError_t launch_emit2_bt(const DevGraph& g, const Scratch& s, const Tuning& t, uint8_t* out, int64_t cap,
-                            const LaunchEnv& env, long long t_begin, long long t_end) {
+                            const LaunchEnv& env, long long t_begin, long long t_end, bool after_layout) {
   const bool aligned16 = (reinterpret_cast<uintptr_t>(g.packed) & 15) == 0;
   // the L2 prefetch pays for HBM-resident reads only: with the reads in pinned
   // host memory it did not help (the 3.1 Gb end-to-end 2-bit step took 10.7 ms
@@ -455,9 +455,11 @@ cudaError_t launch_emit2_bt(const DevGraph& g, const Scratch& s, const Tuning& t
   const bool prefetch = aligned16 && !g.packed_host;
   static const int resident = resident_blocks(k_emit2<BT>, BT);   // once, safely across threads
   const int per_sm = t.emit_blocks_per_sm < resident ? t.emit_blocks_per_sm : resident;
-  cudaError_t e = cudaMemsetAsync(s.tickets, 0, kTicketSets * kTicketStride * sizeof(unsigned long long), env.stream);
-  if (e != cudaSuccess) return e;
-  const bool chained = false;                     // a memset, not a kernel, comes right before
+  if (!after_layout) {
+    cudaError_t e = cudaMemsetAsync(s.tickets, 0, kTicketSets * kTicketStride * sizeof(unsigned long long), env.stream);
+    if (e != cudaSuccess) return e;
+  }
+  const bool chained = after_layout && env.pdl_first;   // otherwise a memset or an event, not a kernel, comes right before
   return launch_kb(k_emit2<BT>, env.num_sms * per_sm, BT, env, chained, s, g.packed,
                    (long long)g.packed_bytes, (long long)(g.packed_readable / 4), aligned16, prefetch,
                    reinterpret_cast<uint4*>(out), (long long)cap, t.tile_bytes, t.emit_tile, t_begin, t_end);
@@ -466,10 +468,10 @@ cudaError_t launch_emit2_bt(const DevGraph& g, const Scratch& s, const Tuning& t
 }  // namespace
 
 cudaError_t launch_emit2(const DevGraph& g, const Scratch& s, const Tuning& t, uint8_t* out, int64_t cap,
-                         const LaunchEnv& env, long long t_begin, long long t_end) {
-  cudaError_t e = t.emit_block_threads == 128 ? launch_emit2_bt<128>(g, s, t, out, cap, env, t_begin, t_end)
-                  : t.emit_block_threads == 512 ? launch_emit2_bt<512>(g, s, t, out, cap, env, t_begin, t_end)
-                                                : launch_emit2_bt<256>(g, s, t, out, cap, env, t_begin, t_end);
+                         const LaunchEnv& env, long long t_begin, long long t_end, bool after_layout) {
+  cudaError_t e = t.emit_block_threads == 128 ? launch_emit2_bt<128>(g, s, t, out, cap, env, t_begin, t_end, after_layout)
+                  : t.emit_block_threads == 512 ? launch_emit2_bt<512>(g, s, t, out, cap, env, t_begin, t_end, after_layout)
+                                                : launch_emit2_bt<256>(g, s, t, out, cap, env, t_begin, t_end, after_layout);
   if (e != cudaSuccess) return e;
   mark(env, "k_emit2");
   return cudaGetLastError();

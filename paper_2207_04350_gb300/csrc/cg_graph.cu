@@ -955,10 +955,12 @@ cudaError_t launch_mask(const DevGraph& g, const Scratch& s, const LaunchEnv& en
   return cudaGetLastError();
 }
 
-cudaError_t launch_chains(const DevGraph& g, const Scratch& s, const Tuning& t, const LaunchEnv& env) {
+cudaError_t launch_chains(const DevGraph& g, const Scratch& s, const Tuning& t, const LaunchEnv& env,
+                          bool after_mask) {
   // restart the chain-stage counters; the head bitmap restarts from the mask
   // stage's words (lone reads; k_succ copies them) and gains the chain heads
-  cudaMemsetAsync(&s.ctr->n_rulers, 0, offsetof(Counters, n_contigs) - offsetof(Counters, n_rulers), env.stream);
+  if (!after_mask)
+    cudaMemsetAsync(&s.ctr->n_rulers, 0, offsetof(Counters, n_contigs) - offsetof(Counters, n_rulers), env.stream);
   static const int succ_resident = resident_blocks(k_succ);   // persistent grids
   static const int final_resident = resident_blocks(k_final);
   // a persistent grid, but no more blocks than the reads can use (a small
@@ -967,9 +969,11 @@ cudaError_t launch_chains(const DevGraph& g, const Scratch& s, const Tuning& t, 
     const long long need = (g.n + items_per_block - 1) / items_per_block;
     return (int)std::max(1LL, std::min(resident_grid, need));
   };
-  k_succ<<<cap((long long)env.num_sms * succ_resident, kBlock), kBlock, 0, env.stream>>>(g, s, t.ruler_log2);
+  cudaError_t e = launch_k(k_succ, cap((long long)env.num_sms * succ_resident, kBlock), env, after_mask, g, s,
+                           t.ruler_log2);
+  if (e != cudaSuccess) return e;
   mark(env, "k_succ");
-  cudaError_t e = launch_k(k_walk, grid_for(2 * g.n, env), env, true, s, t.ruler_log2, (int64_t)(2 * g.n + 1));
+  e = launch_k(k_walk, grid_for(2 * g.n, env), env, true, s, t.ruler_log2, (int64_t)(2 * g.n + 1));
   if (e != cudaSuccess) return e;
   mark(env, "k_walk");
   e = launch_k(k_listwalk, grid_for(2 * g.n, env), env, true, s);

@@ -240,23 +240,29 @@ inline void mark(const LaunchEnv& env, const char* name) {
 // ---- launchers (each returns cudaGetLastError()) ----
 cudaError_t launch_validate(const DevGraph& g, DevError* derr, const LaunchEnv& env);
 cudaError_t launch_mask(const DevGraph& g, const Scratch& s, const LaunchEnv& env);
-cudaError_t launch_chains(const DevGraph& g, const Scratch& s, const Tuning& t, const LaunchEnv& env);
+// after_mask: the mask's launch comes right before on the stream, and has just
+// cleared the chain stage's counters too.
+cudaError_t launch_chains(const DevGraph& g, const Scratch& s, const Tuning& t, const LaunchEnv& env,
+                          bool after_mask = false);
 // With user_off, the piece scan also writes the caller's contig offsets
 // (user_cap entries; a capacity error and nothing written when too small).
 cudaError_t launch_offsets(const DevGraph& g, const Scratch& s, const Tuning& t, const LaunchEnv& env,
                            int64_t* user_off = nullptr, long long user_cap = 0);
 // Spells the output tiles [t_begin, t_end) (all of them by default); with
 // n_shares > 1, share `share` of the tiles cut into n_shares equal runs,
-// written from out[0] on (out and cap hold that share only).
+// written from out[0] on (out and cap hold that share only). after_layout: the
+// offsets stage comes right before on the stream; its last kernel has cleared the
+// tile queue's counters, so that nothing stands between the two kernels.
 cudaError_t launch_emit(const DevGraph& g, const Scratch& s, const Tuning& t, uint8_t* out, int64_t cap,
                         const LaunchEnv& env, long long t_begin = 0, long long t_end = 1ll << 62, int share = 0,
-                        int n_shares = 1);
+                        int n_shares = 1, bool after_layout = false);
 cudaError_t launch_export_reads(const DevGraph& g, const Scratch& s, int32_t* cid, int32_t* rank, uint8_t* orient,
                                 const LaunchEnv& env);
 // 2-bit spelling: cap = bytes of `out`, which must hold 16 * ceil(total / 64).
 // The 2-bit form of the tiles [t_begin, t_end) (tiles of tile_bytes bases; all by default).
 cudaError_t launch_emit2(const DevGraph& g, const Scratch& s, const Tuning& t, uint8_t* out, int64_t cap,
-                         const LaunchEnv& env, long long t_begin = 0, long long t_end = 1ll << 62);
+                         const LaunchEnv& env, long long t_begin = 0, long long t_end = 1ll << 62,
+                         bool after_layout = false);
 cudaError_t launch_export_contig_off(const Scratch& s, int64_t* out, int64_t cap, const LaunchEnv& env);
 cudaError_t launch_sum_len(const DevGraph& g, unsigned long long* out, const LaunchEnv& env);
 // One copy of a batched load: `bytes` bytes from src (device memory, or the

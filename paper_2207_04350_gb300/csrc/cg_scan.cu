@@ -202,6 +202,7 @@ __global__ void __launch_bounds__(kBlock) k_pieces(Scratch s, PieceStore ps) {
   const int tid = threadIdx.x;
   const long long W = *(const volatile unsigned*)&s.ctr->n_walk;
   const long long tiles = (W + kPieceTile - 1) / kPieceTile;
+  if (blockIdx.x == 0 && tid < kTicketSets) s.tickets[kTicketStride * tid] = 0ull;   // for a spelling right after
   if ((long long)blockIdx.x >= tiles) return;
   for (;;) {
     if (tid == 0) s_tile = (long long)atomicAdd(&s.scan_state[s.scan_tiles_cap], 1ull);
