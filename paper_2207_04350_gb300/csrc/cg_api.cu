@@ -1966,33 +1966,33 @@ cg_status cg_partition_contigs(cg_graph* g, int32_t n_parts, int32_t weight, int
   const long long C = c->h_ctr->n_contigs;
   const long long max_w = weight == CG_WEIGHT_READS ? (long long)c->h_ctr->n_walk : (long long)c->h_ctr->total_bases;
   if (C > 0 && (!part || part_cap < C)) return fail(c, CG_EINVAL, "part capacity %lld < %lld", (long long)part_cap, C);
-  // temporaries: the sort buffers, and staging for host outputs
+  // temporaries: the sort buffers, and staging for host outputs, in one allocation
   const size_t N = (size_t)(C > 0 ? C : 1);
-  const long long tiles = (long long)(N + 2047) / 2048;
+  const bool one_block = C <= cg::kSortBlockMax;
   cg::SortBuffers b{};
-  b.tiles_cap = tiles;
-  b.state_cap = (256 * tiles + 2047) / 2048 + 1;
-  const size_t bytes[8] = {8 * N, 8 * N, 4 * N, 4 * N, 4 * 256 * (size_t)tiles, 8 * 256 * (size_t)tiles,
-                           8 * ((size_t)b.state_cap + 1), mem == CG_MEM_HOST ? 4 * N + 8 * (size_t)n_parts : 0};
-  void* p[8] = {};
-  for (int k = 0; k < 8 && st == CG_OK; ++k)
-    if (bytes[k]) p[k] = dalloc(c, bytes[k], &st);
-  auto release = [&]() {
-    for (int k = 0; k < 8; ++k) dfree(c, p[k]);
+  b.tiles_cap = one_block ? 0 : (long long)(N + 2047) / 2048;
+  b.state_cap = one_block ? 0 : (256 * b.tiles_cap + 2047) / 2048 + 1;
+  size_t bytes = 0;
+  auto place = [&](size_t want) {                    // 256-byte aligned, like allocations of their own
+    const size_t at = bytes;
+    bytes += (want + 255) & ~size_t(255);
+    return at;
   };
-  if (st != CG_OK) {
-    release();
-    return st;
-  }
-  b.key[0] = (unsigned long long*)p[0];
-  b.key[1] = (unsigned long long*)p[1];
-  b.val[0] = (int32_t*)p[2];
-  b.val[1] = (int32_t*)p[3];
-  b.hist = (unsigned*)p[4];
-  b.base = (unsigned long long*)p[5];
-  b.state = (unsigned long long*)p[6];
-  int64_t* d_w = mem == CG_MEM_HOST ? (int64_t*)p[7] : part_weight;
-  int32_t* d_part = mem == CG_MEM_HOST ? (int32_t*)((char*)p[7] + 8 * (size_t)n_parts) : part;
+  const size_t o_key0 = place(8 * N), o_key1 = place(8 * N), o_val0 = place(4 * N), o_val1 = place(4 * N);
+  const size_t o_hist = place(4 * 256 * (size_t)b.tiles_cap), o_base = place(8 * 256 * (size_t)b.tiles_cap);
+  const size_t o_state = place(one_block ? 0 : 8 * ((size_t)b.state_cap + 1));
+  const size_t o_w = place(mem == CG_MEM_HOST ? 8 * (size_t)n_parts : 0), o_part = place(mem == CG_MEM_HOST ? 4 * N : 0);
+  char* tmp = (char*)dalloc(c, bytes, &st);
+  if (!tmp) return st;
+  b.key[0] = (unsigned long long*)(tmp + o_key0);
+  b.key[1] = (unsigned long long*)(tmp + o_key1);
+  b.val[0] = (int32_t*)(tmp + o_val0);
+  b.val[1] = (int32_t*)(tmp + o_val1);
+  b.hist = (unsigned*)(tmp + o_hist);
+  b.base = (unsigned long long*)(tmp + o_base);
+  b.state = (unsigned long long*)(tmp + o_state);
+  int64_t* d_w = mem == CG_MEM_HOST ? (int64_t*)(tmp + o_w) : part_weight;
+  int32_t* d_part = mem == CG_MEM_HOST ? (int32_t*)(tmp + o_part) : part;
   if (c->marks.on) {                   // per-kernel marks cover the partition alone
     c->marks.n = 0;
     cudaEventRecord(c->marks.ev[0], c->stream);
@@ -2003,7 +2003,7 @@ cg_status cg_partition_contigs(cg_graph* g, int32_t n_parts, int32_t weight, int
     if (e == cudaSuccess && C > 0) e = cudaMemcpyAsync(part, d_part, 4 * (size_t)C, cudaMemcpyDeviceToHost, c->stream);
   }
   if (e == cudaSuccess) st = wait_and_read(g);
-  release();
+  dfree(c, tmp);
   if (e != cudaSuccess) return cuda_fail(c, e, "partition kernels");
   if (st != CG_OK) return st;
   if (n_contigs) *n_contigs = C;

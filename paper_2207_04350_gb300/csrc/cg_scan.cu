@@ -388,8 +388,9 @@ cudaError_t launch_export_contig_off(const Scratch& s, int64_t* out, int64_t cap
 // reads (the size estimate of Sec. 4.3) or by their spelled bases, sorted by
 // weight, largest first, equal weights in contig order, and each in turn goes
 // to the part whose weight sum is smallest so far, the lowest part on ties.
-// The sort is a stable LSD radix sort, 8-bit digits, of kmax - weight; the
-// assignment is sequential by definition and runs in one warp.
+// The sort is a stable LSD radix sort, 8-bit digits, of kmax - weight, in one
+// block for up to 65,536 contigs; the assignment is sequential by definition
+// and runs in one block, a round of up to one contig per part at a time.
 namespace cg {
 
 namespace {
@@ -477,59 +478,368 @@ __global__ void k_sort_scatter(const unsigned long long* key_in, const int32_t* 
   }
 }
 
-// One warp. A part is the key (weight sum << part_bits) | part index, so that
-// the smallest key is the least-loaded part, the lowest index on ties, and no
-// two keys are equal. Lane l holds the keys of parts l + 32 j, j < KPL, in
-// registers. Per contig the warp takes the smallest key overall with the
-// redux unit (one 32-bit minimum when every key fits in 32 bits, else the
-// high halves, then the low halves at that high half) and the part holding
-// it adds the contig's weight; no branch depends on the data.
-template <int KPL, bool Narrow>
-__global__ void __launch_bounds__(32) k_lpt_assign(const unsigned long long* key, const int32_t* val, long long C,
-                                                   unsigned long long kmax, int P, int part_bits, int32_t* part,
-                                                   int64_t* psum) {
+// The same sort by one block, for at most kSortBlockMax contigs, where the
+// launches and round trips of the kernels above are what a pass costs. Each of
+// the 32 warps takes a run of the keys, counts its digits, and after one scan
+// over digits and warps writes its keys in order, so the sort is stable; eight
+// keys per lane are loaded before any is used. It sorts by wmax - weight, wmax
+// the largest weight there is, so that small weights (reads per contig) need
+// fewer passes than the bound kmax. Results in key[0], val[0]. The 3.1 Gb
+// graph's contigs, two passes: 40 us by events, and 100 for the ten launches above;
+// the line lies where a block's passes, growing with the contigs, meet them.
+constexpr int kSortBlock = 1024;
+constexpr int kSortLoad = 8;
+
+__global__ void __launch_bounds__(kSortBlock) k_sort_block(const Scratch s, int C, int weight, unsigned long long kmax,
+                                                           unsigned long long* key0, unsigned long long* key1,
+                                                           int32_t* val0, int32_t* val1) {
+  pdl_enter();
+  __shared__ unsigned cnt[kSortBlock / 32][256];
+  __shared__ unsigned long long red[kSortBlock / 32];
+  __shared__ unsigned warp_tot[kSortBlock / 32];
   const unsigned full = 0xffffffffu;
-  const unsigned long long idx_mask = (1ull << part_bits) - 1;
-  const int lane = threadIdx.x;
-  unsigned long long K[KPL];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const unsigned lt = (1u << lane) - 1u;
+  auto weight_of = [&](int i) -> unsigned long long {
+    return weight == 0 ? (unsigned long long)s.qd[i] : (unsigned long long)(s.contig_off[i + 1] - s.contig_off[i]);
+  };
+  unsigned long long wmax = 0;
+#pragma unroll 8
+  for (int i = tid; i < C; i += kSortBlock) wmax = max(wmax, weight_of(i));
+  for (int o = 16; o > 0; o >>= 1) wmax = max(wmax, __shfl_xor_sync(full, wmax, o));
+  if (lane == 0) red[warp] = wmax;
+  __syncthreads();
+  wmax = red[lane];
+  for (int o = 16; o > 0; o >>= 1) wmax = max(wmax, __shfl_xor_sync(full, wmax, o));
+  int passes = 1;
+  while (passes < 8 && (wmax >> (8 * passes)) != 0) ++passes;
+  const int seg = (C + kSortBlock - 1) / kSortBlock * 32;          // keys per warp, whole rounds of 32
+  const int i_begin = warp * seg, i_end = min(C, i_begin + seg);
+  for (int pass = 0; pass < passes; ++pass) {
+    const bool to0 = ((passes - pass) & 1) != 0;                   // the last pass writes buffer 0
+    const unsigned long long* kin = to0 ? key1 : key0;
+    const int32_t* vin = to0 ? val1 : val0;
+    unsigned long long* kout = to0 ? key0 : key1;
+    int32_t* vout = to0 ? val0 : val1;
+    // a key as sorted; the last pass stores kmax - weight
+    auto load = [&](int i) -> unsigned long long { return pass == 0 ? wmax - weight_of(i) : kin[i]; };
+    const unsigned long long shift = pass == passes - 1 ? kmax - wmax : 0ull;
+    for (int x = tid; x < (kSortBlock / 32) * 256; x += kSortBlock) (&cnt[0][0])[x] = 0;
+    __syncthreads();
+    for (int i0 = i_begin; i0 < i_begin + seg; i0 += 32 * kSortLoad) {   // warp-uniform
+      unsigned long long k[kSortLoad];
 #pragma unroll
-  for (int j = 0; j < KPL; ++j) K[j] = lane + 32 * j < P ? (unsigned long long)(lane + 32 * j) : ~0ull;
-  for (long long i0 = 0; i0 < C; i0 += 32) {
-    const long long ii = i0 + lane;
-    const int32_t ci = ii < C ? val[ii] : -1;
-    const unsigned long long w = ii < C ? (kmax - key[ii]) << part_bits : 0ull;
-    unsigned long long mine = 0;
-    const int cnt = (int)min(32ll, C - i0);
-    for (int q = 0; q < cnt; ++q) {
-      const unsigned long long wq = __shfl_sync(full, w, q);
-      unsigned long long my = K[0];
+      for (int j = 0; j < kSortLoad; ++j) k[j] = i0 + 32 * j + lane < i_end ? load(i0 + 32 * j + lane) : 0ull;
 #pragma unroll
-      for (int j = 1; j < KPL; ++j) my = min(my, K[j]);
-      unsigned long long m;
-      if (Narrow) {
-        m = __reduce_min_sync(full, (unsigned)min(my, 0xffffffffull));
-      } else {
-        const unsigned hi = (unsigned)(my >> 32);
-        const unsigned mhi = __reduce_min_sync(full, hi);
-        const unsigned mlo = __reduce_min_sync(full, hi == mhi ? (unsigned)my : 0xffffffffu);
-        m = ((unsigned long long)mhi << 32) | mlo;
-      }
-      mine = lane == q ? m : mine;
-#pragma unroll
-      for (int j = 0; j < KPL; ++j) K[j] += K[j] == m ? wq : 0ull;
+      for (int j = 0; j < kSortLoad; ++j)
+        if (i0 + 32 * j + lane < i_end) atomicAdd(&cnt[warp][digit_of(k[j], pass)], 1u);
     }
-    if (ii < C) part[ci] = (int32_t)(mine & idx_mask);
-  }
+    __syncthreads();
+    {                                                              // exclusive sums by digit, then by warp
+      const int d = tid >> 2, w0 = (tid & 3) * 8;
+      unsigned c[8], sum = 0;
 #pragma unroll
-  for (int j = 0; j < KPL; ++j)
-    if (lane + 32 * j < P) psum[lane + 32 * j] = (int64_t)(K[j] >> part_bits);
+      for (int w = 0; w < 8; ++w) { c[w] = cnt[w0 + w][d]; sum += c[w]; }
+      unsigned inc = sum;
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned x = __shfl_up_sync(full, inc, o);
+        if (lane >= o) inc += x;
+      }
+      if (lane == 31) warp_tot[warp] = inc;
+      __syncthreads();
+      unsigned run = inc - sum;
+      for (int w = 0; w < warp; ++w) run += warp_tot[w];
+#pragma unroll
+      for (int w = 0; w < 8; ++w) { cnt[w0 + w][d] = run; run += c[w]; }
+    }
+    __syncthreads();
+    for (int i0 = i_begin; i0 < i_begin + seg; i0 += 32 * kSortLoad) {
+      unsigned long long k[kSortLoad];
+      int32_t v[kSortLoad];
+#pragma unroll
+      for (int j = 0; j < kSortLoad; ++j) {
+        const int i = i0 + 32 * j + lane;
+        k[j] = i < i_end ? load(i) : 0ull;
+        v[j] = i < i_end ? (pass == 0 ? i : vin[i]) : 0;
+      }
+#pragma unroll
+      for (int j = 0; j < kSortLoad; ++j) {
+        const bool valid = i0 + 32 * j + lane < i_end;
+        const unsigned d = digit_of(k[j], pass);
+        // the lanes with this digit: a ballot per bit (a match instruction per 32
+        // keys and phase made the two passes 48 us)
+        unsigned peers = __ballot_sync(full, valid);
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+          const unsigned set = __ballot_sync(full, (d >> b) & 1u);
+          peers &= (d >> b) & 1u ? set : ~set;
+        }
+        const unsigned at = valid ? cnt[warp][d] + __popc(peers & lt) : 0u;
+        __syncwarp();
+        if (valid && (peers & lt) == 0) cnt[warp][d] += __popc(peers);
+        __syncwarp();
+        if (valid) {
+          kout[at] = k[j] + shift;
+          vout[at] = v[j];
+        }
+      }
+    }
+    __syncthreads();
+  }
 }
 
-template <int KPL>
-void lpt_launch(bool narrow, const unsigned long long* key, const int32_t* val, long long C, unsigned long long kmax,
-                int P, int part_bits, int32_t* part, int64_t* psum, cudaStream_t st) {
-  if (narrow) k_lpt_assign<KPL, true><<<1, 32, 0, st>>>(key, val, C, kmax, P, part_bits, part, psum);
-  else k_lpt_assign<KPL, false><<<1, 32, 0, st>>>(key, val, C, kmax, P, part_bits, part, psum);
+// The assignment, a round of contigs at a time. A part is the key (weight sum
+// << part_bits) | part index, so that the smallest key is the least-loaded
+// part, the lowest index on ties, and no two keys are equal. Taken one by one,
+// the next contigs go to the parts of rank 0, 1, 2, ... for as long as no part
+// that has just received one is below the next rank's key: mostly for a whole
+// round of P contigs, since the weights come in descending order and a round
+// levels the sums. So a round ranks the P keys, hands contig r to the part of
+// rank r and keeps the longest prefix for which that holds: all of it when every
+// raised key is above the largest old one, else up to the first rank whose old
+// key is above a raised key of a lower rank. When only the first is kept, the
+// least-loaded part stays so for a while, and takes every further contig that
+// leaves it below the second. The parts are those of the rule taken literally.
+// Up to 32 parts: a warp, a part per lane, ranked by P shuffles. More: a block,
+// G threads per part, each comparing its key with a G-th of the P keys in shared
+// memory. What bounds both is the chain of ranks and barriers of each round.
+// The 3.1 Gb graph's contigs into 72 parts: 121 us by events, and 776 one contig
+// at a time in one warp.
+constexpr int kLptSmem = 160 << 10;  // bytes of weights and parts staged at a time; kMaxParts contigs at least
+
+// The smallest value of the lanes before this one.
+template <typename K>
+__device__ __forceinline__ K warp_min_before(K m, int lane) {
+  const K none = ~(K)0;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const K x = __shfl_up_sync(0xffffffffu, m, o);
+    if (lane >= o) m = min(m, x);
+  }
+  const K e = __shfl_up_sync(0xffffffffu, m, 1);
+  return lane == 0 ? none : e;
+}
+
+// How many of the weights w[0..n), at most 32, the part with key `lowest` takes
+// one after another while it stays below `second`; their sum in *added. All
+// lanes of a warp.
+template <typename K>
+__device__ __forceinline__ int lpt_run(const K* w, int n, K lowest, K second, K* added, int lane) {
+  const unsigned full = 0xffffffffu;
+  const K wl = lane < n ? w[lane] : (K)0;
+  K sum = wl;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const K x = __shfl_up_sync(full, sum, o);
+    if (lane >= o) sum += x;
+  }
+  const unsigned ok = __ballot_sync(full, lane < n && (lane == 0 || lowest + (sum - wl) < second));
+  const int run = __popc(ok);                          // sums never decrease: the first `run` lanes
+  *added = __shfl_sync(full, sum, run - 1);
+  return run;
+}
+
+// Rounds over the staged weights w[cur..n) for P <= 32, by one warp; `mine` is
+// the lane's key. Returns where it stopped: at n, or (unless `last`) with fewer
+// than P left. byrank: shared, 2 x 32 keys.
+template <typename K>
+__device__ __forceinline__ int lpt_rounds_warp(const K* w, short* to, int n, bool last, int P, int part_bits, K& mine,
+                                               K* byrank, int lane) {
+  const unsigned full = 0xffffffffu;
+  const K none = ~(K)0;
+  int cur = 0;
+  while (cur < n && (last || n - cur >= P)) {          // warp-uniform
+    const int cnt = min(P, n - cur);
+    int r = 0;
+#pragma unroll 8
+    for (int j = 0; j < P; ++j) r += __shfl_sync(full, mine, j) < mine;
+    if (lane >= P) r = 32;
+    const K raised = r < cnt ? mine + w[cur + r] : none;
+    const K top = __shfl_sync(full, mine, __ffs(__ballot_sync(full, r == cnt - 1)) - 1);
+    int kept = cnt;
+    if (__any_sync(full, r < cnt - 1 && raised < top)) {
+      if (lane < P) {
+        byrank[r] = mine;
+        byrank[32 + r] = raised;
+      }
+      __syncwarp();
+      const K old_key = lane < P ? byrank[lane] : none, new_key = lane < cnt ? byrank[32 + lane] : none;
+      const K before = warp_min_before(new_key, lane);
+      const unsigned bad = __ballot_sync(full, lane > 0 && lane < cnt && old_key > before);
+      if (bad) kept = __ffs(bad) - 1;
+      if (kept == 1) {
+        const K lowest = __shfl_sync(full, old_key, 0), second = __shfl_sync(full, old_key, 1);
+        K added;
+        const int run = lpt_run(w + cur, min(32, n - cur), lowest, second, &added, lane);
+        if (r == 0) mine += added;
+        if (lane < run) to[cur + lane] = (short)(lowest & (((K)1 << part_bits) - 1));
+        cur += run;
+        __syncwarp();
+        continue;
+      }
+      __syncwarp();
+    }
+    if (r < kept) {
+      to[cur + r] = (short)lane;
+      mine = raised;
+    }
+    cur += kept;
+  }
+  return cur;
+}
+
+template <typename K>
+__device__ __forceinline__ int keys_below(const K* keys, int n4, int g, int G, K mine);
+template <>
+__device__ __forceinline__ int keys_below<uint32_t>(const uint32_t* keys, int n4, int g, int G, uint32_t mine) {
+  int r0 = 0, r1 = 0;
+#pragma unroll 4
+  for (int j = 4 * g; j < n4; j += 4 * G) {
+    const uint4 x = *reinterpret_cast<const uint4*>(keys + j);
+    r0 += (x.x < mine) + (x.y < mine);
+    r1 += (x.z < mine) + (x.w < mine);
+  }
+  return r0 + r1;
+}
+template <>
+__device__ __forceinline__ int keys_below<unsigned long long>(const unsigned long long* keys, int n4, int g, int G,
+                                                              unsigned long long mine) {
+  int r0 = 0, r1 = 0;
+#pragma unroll 4
+  for (int j = 2 * g; j < n4; j += 2 * G) {
+    const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(keys + j);
+    r0 += x.x < mine;
+    r1 += x.y < mine;
+  }
+  return r0 + r1;
+}
+
+// G threads per part (a power of two, 32 at most); P * G threads or more. Up to
+// 32 parts (G = 0): warp 0 assigns, the others only stage weights and write parts.
+template <typename K>
+__global__ void __launch_bounds__(kMaxParts) k_lpt_assign(const unsigned long long* key, const int32_t* val, long long C,
+                                                          unsigned long long kmax, int P, int G, int part_bits,
+                                                          int chunk, int32_t* part, int64_t* psum) {
+  pdl_enter();
+  __shared__ __align__(16) K keys[kMaxParts];              // by part
+  __shared__ K old_key[kMaxParts], new_key[kMaxParts];     // by rank
+  extern __shared__ __align__(16) unsigned char staged[];
+  K* const w = reinterpret_cast<K*>(staged);               // chunk weights
+  short* const to = reinterpret_cast<short*>(w + chunk);   // and the parts they go to
+  __shared__ K warp_min[32], top;
+  __shared__ int first_bad, stop;
+  const unsigned full = 0xffffffffu;
+  const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, warp = tid >> 5;
+  const K none = ~(K)0;
+  const int me = G ? tid / G : tid, g = G ? tid & (G - 1) : 0;
+  const bool act = me < P, lead = act && g == 0;
+  const int n4 = (P + 3) & ~3;
+  if (tid >= P && tid < n4) keys[tid] = none;              // the last vector's empty places
+  K mine = act ? (K)me : none;
+  for (long long c0 = 0; c0 < C;) {
+    const int n = (int)min((long long)chunk, C - c0);
+#pragma unroll 8
+    for (int i = tid; i < n; i += T) w[i] = (K)((kmax - key[c0 + i]) << part_bits);
+    __syncthreads();
+    const bool last = c0 + n == C;
+    int cur = 0;
+    if (G == 0) {
+      if (warp == 0) {
+        cur = lpt_rounds_warp(w, to, n, last, P, part_bits, mine, old_key, lane);
+        if (lane == 0) stop = cur;
+      }
+      __syncthreads();
+      cur = stop;
+    }
+    while (G && cur < n && (last || n - cur >= P)) {       // block-uniform
+      const int cnt = min(P, n - cur);
+      if (lead) keys[me] = mine;
+      __syncthreads();
+      int r = act ? keys_below<K>(keys, n4, g, G, mine) : 0;
+      for (int o = G >> 1; o > 0; o >>= 1) r += __shfl_xor_sync(full, r, o);
+      if (!act) r = P;
+      const K raised = r < cnt ? mine + w[cur + r] : none;
+      if (lead && r == cnt - 1) top = mine;
+      __syncthreads();
+      if (!__syncthreads_or(r < cnt - 1 && raised < top)) {
+        if (r < cnt) {
+          if (lead) to[cur + r] = (short)me;
+          mine = raised;
+        }
+        cur += cnt;
+        continue;
+      }
+      if (lead) {
+        old_key[r] = mine;
+        if (r < cnt) new_key[r] = raised;
+      }
+      if (tid == 0) first_bad = cnt;
+      __syncthreads();
+      const K m = tid < cnt ? new_key[tid] : none;         // thread t now looks at rank t
+      K before = warp_min_before(m, lane);
+      if (lane == 31) warp_min[warp] = min(before, m);
+      __syncthreads();
+      for (int x = 0; x < warp; ++x) before = min(before, warp_min[x]);
+      if (tid > 0 && tid < cnt && old_key[tid] > before) atomicMin(&first_bad, tid);
+      __syncthreads();
+      const int kept = first_bad;
+      if (kept > 1) {
+        if (r < kept) {
+          if (lead) to[cur + r] = (short)me;
+          mine = raised;
+        }
+        cur += kept;
+      } else {                                             // every warp computes the run
+        K added;
+        const int run = lpt_run(w + cur, min(32, n - cur), old_key[0], old_key[1], &added, lane);
+        if (r == 0) mine += added;
+        if (tid < run) to[cur + tid] = (short)(old_key[0] & (((K)1 << part_bits) - 1));
+        cur += run;
+      }
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int i = tid; i < cur; i += T) part[val[c0 + i]] = to[i];
+    c0 += cur;
+    __syncthreads();
+  }
+  if (lead) psum[me] = (int64_t)(mine >> part_bits);
+}
+
+// As many contigs staged at a time as fit kLptSmem: all of them for most graphs,
+// since each chunk costs two round trips to memory.
+template <typename K>
+cudaError_t lpt_launch(const unsigned long long* key, const int32_t* val, long long C, unsigned long long kmax, int P, int G,
+                       int part_bits, int threads, int32_t* part, int64_t* psum, const LaunchEnv& env) {
+  const int per = (int)(sizeof(K) + sizeof(short)), most = kLptSmem / per / 64 * 64;
+  const int chunk = C < most ? (int)((C + 63) / 64 * 64) : most;
+  const size_t smem = (size_t)std::max(chunk, kMaxParts) * per;
+  cudaError_t e = cudaFuncSetAttribute(k_lpt_assign<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLptSmem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(1);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = env.stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = env.pdl && !(env.marks && env.marks->on) ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k_lpt_assign<K>, key, val, C, kmax, P, G, part_bits, std::max(chunk, kMaxParts), part,
+                            psum);
+}
+
+// One part takes every contig.
+__global__ void __launch_bounds__(kBlock) k_lpt_one(const Scratch s, long long C, int weight, int32_t* part,
+                                                    int64_t* psum) {
+  unsigned long long sum = 0;
+  for (long long i = grid_tid(); i < C; i += grid_threads()) {
+    part[i] = 0;
+    sum += weight == 0 ? (unsigned long long)s.qd[i] : (unsigned long long)(s.contig_off[i + 1] - s.contig_off[i]);
+  }
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0 && sum) atomicAdd(reinterpret_cast<unsigned long long*>(psum), sum);
 }
 
 }  // namespace
@@ -539,7 +849,19 @@ cudaError_t launch_partition(const Scratch& s, long long C, int weight, long lon
   int bits = 8;
   while (bits < 63 && (max_weight >> bits) != 0) bits += 8;
   const unsigned long long kmax = bits >= 64 ? ~0ull : (1ull << bits) - 1;
-  if (C > 0) {
+  if (C <= 0 || P == 1) cudaMemsetAsync(psum, 0, (size_t)P * sizeof(int64_t), env.stream);
+  if (C <= 0) return cudaGetLastError();
+  if (P == 1) {
+    k_lpt_one<<<grid_for(C, env), kBlock, 0, env.stream>>>(s, C, weight, part, psum);
+    mark(env, "k_lpt_one");
+    return cudaGetLastError();
+  }
+  int cur = 0;
+  const bool small = C <= kSortBlockMax;
+  if (small) {
+    k_sort_block<<<1, kSortBlock, 0, env.stream>>>(s, (int)C, weight, kmax, b.key[0], b.key[1], b.val[0], b.val[1]);
+    mark(env, "k_sort_block");
+  } else {
     const long long tiles = (C + kSortTile - 1) / kSortTile;
     const long long nh = 256 * tiles;
     const long long scan_tiles = (nh + kTileItems - 1) / kTileItems;
@@ -547,7 +869,6 @@ cudaError_t launch_partition(const Scratch& s, long long C, int weight, long lon
     k_sort_keys<<<grid_for(C, env), kBlock, 0, env.stream>>>(s, C, weight, kmax, b.key[0], b.val[0]);
     mark(env, "k_sort_keys");
     const int grid = (int)std::min<long long>(tiles, (long long)env.num_sms * 4);
-    int cur = 0;
     for (int pass = 0; pass < bits / 8; ++pass) {
       k_sort_hist<<<grid, kBlock, 0, env.stream>>>(b.key[cur], C, pass, b.hist, tiles);
       mark(env, "k_sort_hist");
@@ -560,23 +881,22 @@ cudaError_t launch_partition(const Scratch& s, long long C, int weight, long lon
       mark(env, "k_sort_scatter");
       cur ^= 1;
     }
-    int part_bits = 0;
-    while ((1 << part_bits) < P) ++part_bits;
-    if (part_bits + bits > 63) return cudaErrorInvalidValue;
-    // narrow: the largest key, max_weight << part_bits | (P - 1), stays below 2^32 - 1
-    const bool narrow = (((unsigned long long)max_weight << part_bits) | (unsigned long long)(P - 1)) < 0xffffffffull;
-    const unsigned long long* kk = b.key[cur];
-    const int32_t* vv = b.val[cur];
-    if (P <= 32) lpt_launch<1>(narrow, kk, vv, C, kmax, P, part_bits, part, psum, env.stream);
-    else if (P <= 64) lpt_launch<2>(narrow, kk, vv, C, kmax, P, part_bits, part, psum, env.stream);
-    else if (P <= 128) lpt_launch<4>(narrow, kk, vv, C, kmax, P, part_bits, part, psum, env.stream);
-    else if (P <= 256) lpt_launch<8>(narrow, kk, vv, C, kmax, P, part_bits, part, psum, env.stream);
-    else if (P <= 512) lpt_launch<16>(narrow, kk, vv, C, kmax, P, part_bits, part, psum, env.stream);
-    else lpt_launch<32>(narrow, kk, vv, C, kmax, P, part_bits, part, psum, env.stream);
-    mark(env, "k_lpt_assign");
-  } else {
-    cudaMemsetAsync(psum, 0, (size_t)P * sizeof(int64_t), env.stream);
   }
+  int part_bits = 0;
+  while ((1 << part_bits) < P) ++part_bits;
+  if (part_bits + bits > 63) return cudaErrorInvalidValue;
+  // narrow: the largest key, max_weight << part_bits | (P - 1), stays below 2^32 - 1
+  const bool narrow = (((unsigned long long)max_weight << part_bits) | (unsigned long long)(P - 1)) < 0xffffffffull;
+  // threads per part: as many as 512 threads allow (1024 from 129 parts on), and no more than there are vectors of keys
+  int G = 1;
+  while (2 * G * P <= (P > 128 ? kMaxParts : 512) && 2 * G <= (P + 3) / 4) G *= 2;
+  if (P <= 32) G = 0;
+  const int threads = std::max(256, (P * G + 31) & ~31);  // enough of them to stage the weights
+  cudaError_t e = narrow ? lpt_launch<uint32_t>(b.key[cur], b.val[cur], C, kmax, P, G, part_bits, threads, part, psum, env)
+                         : lpt_launch<unsigned long long>(b.key[cur], b.val[cur], C, kmax, P, G, part_bits, threads, part,
+                                                          psum, env);
+  if (e != cudaSuccess) return e;
+  mark(env, "k_lpt_assign");
   return cudaGetLastError();
 }
 

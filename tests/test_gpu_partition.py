@@ -128,6 +128,18 @@ def test_many_contigs_few_parts(ctx):
     check(ctx, G, [8, 16, 32])
 
 
+@pytest.mark.parametrize("sizes,parts", [
+    # a few contigs above everything else: rounds that keep one part, or some, at a time
+    ([3000, 2900, 40] + [2] * 300, [2, 3, 4, 33, 40]),
+    ([900, 500, 300, 200, 100, 60, 30, 20, 10, 5, 3, 2, 2, 2] + [2, 3, 4] * 60, [2, 5, 8, 31, 33, 64, 130]),
+    # more contigs than one block sorts (65,536) and than are staged at a time (27,264 or 16,384)
+    ([2, 3, 4, 5, 9] * 14_000, [2, 8, 72, 1024]),
+])
+def test_uneven_and_many(ctx, sizes, parts):
+    G = structured(len(sizes), list(sizes), lone=5)
+    check(ctx, G, parts)
+
+
 def test_one_contig_of_80mb(ctx):
     """A contig of about 80 Mb with 3 and 32 parts: part sums beyond 32 bits
     once shifted above the part index, so the assignment takes wide keys."""
