@@ -1886,33 +1886,36 @@ cg_status cg_transitive_reduction(cg_ctx* c, const cg_graph_desc* d, int32_t fuz
   G.suf = (const int32_t*)in(d->suf, (size_t)m * 4);
   G.len = (const int32_t*)in(d->len, (size_t)n * 4);
   cg::TrBuffers t{};
-  t.row_of = (int32_t*)alloc((size_t)m * 4);
+  const size_t tiles = (size_t)cg::transitive_tiles(m);
+  t.rows_cap = std::min(n, m);
+  t.rows = (int4*)alloc((size_t)t.rows_cap * sizeof(int4));
+  t.info = (int4*)alloc((size_t)n * sizeof(int4));
+  t.has = (unsigned*)alloc(((size_t)n + 31) / 32 * 4);
+  t.ent = (uint2*)alloc((size_t)m * sizeof(uint2));
   t.trans = (uint8_t*)alloc((size_t)m);
-  t.keep = (uint8_t*)alloc((size_t)m);
-  t.row_cnt = (int32_t*)alloc((size_t)n * 4);
-  t.out_rp = (int64_t*)alloc((size_t)(n + 1) * 8);
-  t.total = (unsigned long long*)alloc(8);
-  t.state_cap = (n + 2047) / 2048 + 1;
-  t.state = (unsigned long long*)alloc((size_t)(t.state_cap + 1) * 8);
+  t.mir = (int32_t*)alloc((size_t)m * 4);
+  t.keep = (unsigned*)alloc(tiles * 64 * 4);
+  t.before = (unsigned*)alloc(tiles * 64 * 4);
+  t.tile_cnt = (unsigned*)alloc(tiles * 4);
+  t.total = (unsigned long long*)alloc(16);
+  t.n_rows = t.total ? (unsigned*)(t.total + 1) : nullptr;
   t.derr = c->derr;
+  // device outputs are written in place; an offset array that is not 8-byte aligned gets a copy
+  const bool device_out = want && mem == CG_MEM_DEVICE;
+  int64_t* out_rp = row_ptr;
+  if (want && !(device_out && aligned(row_ptr, 8))) out_rp = (int64_t*)alloc((size_t)(n + 1) * 8);
   if (st != CG_OK) return done(st);
   if (c->marks.on) {                   // per-kernel marks cover this call alone
     c->marks.n = 0;
     cudaEventRecord(c->marks.ev[0], c->stream);
   }
-  // the rows (offsets, order), then the entries (columns, codes, suffixes,
-  // mirrors), each waited for: the reduction indexes rows by column values
   cg_graph probe{};
   probe.ctx = c;
-  cudaError_t e = cg::launch_transitive_check(G, c->derr, c->env);
-  if (e != cudaSuccess) return done(cuda_fail(c, e, "row checks"));
-  st = wait_and_read(&probe);
-  if (st != CG_OK) return done(st);
-  e = cg::launch_transitive_entries(G, t, c->env);
-  if (e != cudaSuccess) return done(cuda_fail(c, e, "entry checks"));
-  st = wait_and_read(&probe);
-  if (st != CG_OK) return done(st);
-  e = cg::launch_transitive(G, fuzz, t, c->env);
+  cudaError_t e = cg::launch_transitive(G, fuzz, t, c->env);
+  // with device outputs the whole call is queued before its one wait: the last
+  // kernel writes nothing when a check failed or the entries do not fit
+  if (e == cudaSuccess && device_out)
+    e = cg::launch_transitive_scatter(G, t, cap_entries, out_rp, col, code, suf, c->env, m > 0);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->h_u64, t.total, 8, cudaMemcpyDeviceToHost, c->stream);
   if (e != cudaSuccess) return done(cuda_fail(c, e, "transitive reduction kernels"));
   st = wait_and_read(&probe);
@@ -1922,23 +1925,21 @@ cg_status cg_transitive_reduction(cg_ctx* c, const cg_graph_desc* d, int32_t fuz
   if (!want) return done(CG_OK);
   if (cap_entries < total) return done(fail(c, CG_EINVAL, "capacity %lld < %lld entries", (long long)cap_entries,
                                             (long long)total));
-  int32_t* oc = col;
-  uint8_t* ok = code;
-  int32_t* os = suf;
-  if (mem == CG_MEM_HOST) {
-    oc = (int32_t*)alloc((size_t)total * 4);
-    ok = (uint8_t*)alloc((size_t)total);
-    os = (int32_t*)alloc((size_t)total * 4);
-    if (st != CG_OK) return done(st);
-  }
-  e = cg::launch_transitive_scatter(G, t, oc, ok, os, c->env);
+  if (device_out && out_rp == row_ptr) return done(CG_OK);
   const cudaMemcpyKind k = mem == CG_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(row_ptr, t.out_rp, (size_t)(n + 1) * 8, k, c->stream);
-  if (mem == CG_MEM_HOST && total > 0) {
-    if (e == cudaSuccess) e = cudaMemcpyAsync(col, oc, (size_t)total * 4, k, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(code, ok, (size_t)total, k, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(suf, os, (size_t)total * 4, k, c->stream);
+  if (mem == CG_MEM_HOST) {
+    int32_t* oc = (int32_t*)alloc((size_t)total * 4);
+    uint8_t* ok = (uint8_t*)alloc((size_t)total);
+    int32_t* os = (int32_t*)alloc((size_t)total * 4);
+    if (st != CG_OK) return done(st);
+    e = cg::launch_transitive_scatter(G, t, total, out_rp, oc, ok, os, c->env, false);
+    if (total > 0) {
+      if (e == cudaSuccess) e = cudaMemcpyAsync(col, oc, (size_t)total * 4, k, c->stream);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(code, ok, (size_t)total, k, c->stream);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(suf, os, (size_t)total * 4, k, c->stream);
+    }
   }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(row_ptr, out_rp, (size_t)(n + 1) * 8, k, c->stream);
   if (e != cudaSuccess) return done(cuda_fail(c, e, "write the reduced graph"));
   st = wait_and_read(&probe);
   return done(st);

@@ -302,25 +302,28 @@ struct SortBuffers {
 };
 // Buffers of the transitive reduction (m entries, n rows).
 struct TrBuffers {
-  int32_t* row_of;             // m: row of every entry
+  int4* rows;                  // rows with entries: (read, first entry, entries)
+  long long rows_cap;          // at most min(n, m)
+  unsigned* n_rows;
+  int4* info;                  // n, set for rows with entries: first entry, first of the second run, end, read length
+  unsigned* has;               // n bits: the read has entries
+  uint2* ent;                  // m: each row in two runs by the end its entries leave through, (column << 2 | code, suffix)
   uint8_t* trans;              // m: entry is transitive
-  uint8_t* keep;               // m: entry kept (its pair is not transitive)
-  int32_t* row_cnt;            // n: kept entries per row
-  int64_t* out_rp;             // n + 1: the reduced graph's row offsets
+  int32_t* mir;                // m: the entry's mirror
+  unsigned* keep;              // transitive_tiles(m) x 64 words: a bit per kept entry (its pair is not transitive)
+  unsigned* before;            // per word: the kept entries before it in its tile
+  unsigned* tile_cnt;          // per tile: the kept entries before it
   unsigned long long* total;   // kept entries
-  unsigned long long* state;   // look-back descriptors of the row scan, + 1 ticket
-  long long state_cap;
   DevError* derr;
 };
-// TransitiveReduction: row checks (launch_transitive_check, then the entry
-// checks), marks, keeps, scans (launch_transitive), then writes the kept
-// entries (launch_transitive_scatter). Each step needs the checks before it
-// to have passed: the later kernels index rows by column values.
-cudaError_t launch_transitive_check(const DevGraph& g, DevError* derr, const LaunchEnv& env);
-cudaError_t launch_transitive_entries(const DevGraph& g, const TrBuffers& t, const LaunchEnv& env);
+long long transitive_tiles(long long m);
+// TransitiveReduction: checks, marks, keeps and counts (launch_transitive), then
+// writes the kept entries and the new row offsets, unless they are more than
+// `cap` (launch_transitive_scatter). After a failed check the later kernels do
+// nothing.
 cudaError_t launch_transitive(const DevGraph& g, int fuzz, const TrBuffers& t, const LaunchEnv& env);
-cudaError_t launch_transitive_scatter(const DevGraph& g, const TrBuffers& t, int32_t* col, uint8_t* code, int32_t* suf,
-                                      const LaunchEnv& env);
+cudaError_t launch_transitive_scatter(const DevGraph& g, const TrBuffers& t, long long cap, int64_t* row_ptr, int32_t* col,
+                                      uint8_t* code, int32_t* suf, const LaunchEnv& env, bool chained);
 constexpr int kMaxParts = 1024;
 // GreedyPartitioning of the C contigs of the last offsets stage into P parts
 // (weight 0: reads per contig, 1: bases); max_weight bounds every part sum.

@@ -7,188 +7,471 @@
 // and whose suffixes add up to x's within a tolerance. A pair of reads keeps
 // both entries only when neither is transitive.
 //
-// Rows hold a few entries and most reads none, so after one pass that writes
-// every entry's row, the work takes one thread per entry: the entry (u->v)
-// walks v's row and looks each w up in u's row (rows are sorted by column) by
-// binary search; an entry is kept when neither it nor its mirror is
-// transitive; per-row counts and a look-back scan give the new row offsets;
-// every kept entry goes to its row's offset plus the kept entries before it.
+// Rows hold a few entries and most reads none, so the rows with entries are
+// listed first, and every row's entries are copied in two runs, those that leave
+// the read through its 5' end and those that leave through the other, each packed
+// into eight bytes. Then a block takes a batch of listed rows, stages them in
+// shared memory and gives every entry (u->v) a thread, which walks the run of
+// v's row that leaves v through the other end: every entry of it is a walk u ->
+// v -> w, whose w is looked up in u's staged row. Everything after that is per
+// entry: an entry is kept when neither it nor its mirror is transitive; the kept
+// entries are bits of one map over all entries with the count of those before
+// each word, and since entries lie in row order that count places both the kept
+// entries and the new row offsets.
+//
+// Nothing waits for the host in between: an invalid graph sets the error word,
+// and every later kernel reads it first and returns. The kernels that follow
+// an entry to another row run only once all row offsets have passed.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "cg_internal.cuh"
-#include "cg_lookback.cuh"
 
 namespace cg {
 
 namespace {
 
+constexpr int kTrTile = 2048;        // entries of one tile of the map: 64 words
+constexpr int kTrRows = 4;           // rows per thread of the row pass
+constexpr int kTrBatch = 120;        // listed rows a block takes at a time, at most
+constexpr int kTrAim = 960;          // entries a batch aims at: just under four per thread
+constexpr int kTrStage = 2048;       // entries of a batch staged in shared memory
+
+__device__ __forceinline__ bool failed(const DevError* e) { return *(const volatile int*)&e->err != 0; }
+
 // Position of column w in the sorted row [a, b), or -1.
-__device__ __forceinline__ int64_t find_col(const int32_t* col, int64_t a, int64_t b, int32_t w) {
-  int64_t lo = a, hi = b;
+__device__ __forceinline__ int32_t find_col(const int32_t* col, int32_t a, int32_t b, int32_t w) {
+  int32_t lo = a, hi = b;
   while (lo < hi) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (__ldg(col + mid) < w) lo = mid + 1;
+    const int32_t mid = (lo + hi) >> 1;
+    if (col[mid] < w) lo = mid + 1;
     else hi = mid;
   }
-  return lo < b && __ldg(col + lo) == w ? lo : -1;
+  return lo < b && col[lo] == w ? lo : -1;
 }
 
-// Rows: offsets in [0, m] and increasing, columns strictly increasing (sorted,
-// no repeated pair), every read at least one base long.
-__global__ void k_tr_check(DevGraph g, DevError* e) {
-  for (long long u = grid_tid(); u < g.n; u += grid_threads()) {
-    const int64_t a = rowp(g, u), b = rowp(g, u + 1);
-    if (a < 0 || b < a || b > g.m || g.len[u] < 1) {
-      set_error(e, DERR_GRAPH, K_TRANSITIVE, u);
-      continue;
+// Rows: offsets from 0 to m that never decrease, every read at least one base
+// long. Lists the rows with entries (read, first entry, entries), one
+// reservation per block, with a record per such read and a bit in a map of them.
+// Reads every row offset and length once, 12 B per read.
+__global__ void __launch_bounds__(kBlock, 6) k_tr_check(DevGraph g, TrBuffers t) {
+  __shared__ unsigned cnt, base;
+  const long long u0 = (long long)blockIdx.x * (kTrRows * kBlock) + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) cnt = 0;
+  __syncthreads();
+  int64_t a[kTrRows], b[kTrRows];
+  int32_t len[kTrRows];
+#pragma unroll
+  for (int k = 0; k < kTrRows; ++k) {
+    const long long u = u0 + k * kBlock;
+    a[k] = u < g.n ? rowp(g, u) : 0;
+    b[k] = u < g.n ? rowp(g, u + 1) : 0;
+    len[k] = u < g.n ? g.len[u] : 1;
+  }
+  unsigned slot[kTrRows];
+#pragma unroll
+  for (int k = 0; k < kTrRows; ++k) {
+    const long long u = u0 + k * kBlock;
+    const bool ok = a[k] >= 0 && b[k] >= a[k] && b[k] <= g.m && len[k] >= 1;
+    if (!ok) {
+      set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, u);
+      b[k] = a[k];
     }
-    for (int64_t x = a + 1; x < b; ++x)
-      if (g.col[x] <= g.col[x - 1]) set_error(e, DERR_GRAPH, K_TRANSITIVE, x);
-  }
-  if (grid_tid() == 0 && (rowp(g, 0) != 0 || rowp(g, g.n) != g.m)) set_error(e, DERR_GRAPH, K_TRANSITIVE, -1);
-}
-
-// Row of every entry (one thread per row), so that the kernels below can
-// take one thread per entry: rows hold few entries and most reads none.
-__global__ void k_tr_rowof(DevGraph g, int32_t* row_of) {
-  for (long long u = grid_tid(); u < g.n; u += grid_threads()) {
-    const int64_t a = rowp(g, u), b = rowp(g, u + 1);
-    for (int64_t x = a; x < b; ++x) row_of[x] = (int32_t)u;
-  }
-}
-
-// Entries, once the rows are known sorted: column in range and not the row
-// itself, code 0..3, suffix in [1, len-1], and exactly one mirror entry (found
-// by binary search) with the swapped code.
-__global__ void k_tr_entries(DevGraph g, const int32_t* row_of, DevError* e) {
-  for (long long x = grid_tid(); x < g.m; x += grid_threads()) {
-    const int32_t u = row_of[x], w = g.col[x];
-    const int cd = g.code[x];
-    if (w < 0 || w >= g.n || w == u || cd > 3) {
-      set_error(e, DERR_GRAPH, K_TRANSITIVE, x);
-      continue;
-    }
-    const int32_t sf = g.suf[x];
-    if (sf < 1 || sf > g.len[w] - 1) set_error(e, DERR_GRAPH, K_TRANSITIVE, x);
-    const int64_t y = find_col(g.col, rowp(g, w), rowp(g, w + 1), u);
-    if (y < 0 || g.code[y] != (((cd & 1) << 1) | (cd >> 1))) set_error(e, DERR_GRAPH, K_TRANSITIVE, x);
-  }
-}
-
-// One thread per entry y = (u->v): every walk u -> v -> w through v's row,
-// each w looked up in u's sorted row; marks the transitive (u->w).
-__global__ void __launch_bounds__(kBlock) k_tr_mark(DevGraph g, const int32_t* row_of, int fuzz, uint8_t* trans) {
-  for (long long y = grid_tid(); y < g.m; y += grid_threads()) {
-    const int32_t u = row_of[y], v = g.col[y];
-    const int cy = g.code[y];
-    const int32_t sy = g.suf[y];
-    const int eu = cy & 1, ev_in = (cy >> 1) & 1;
-    const int64_t a = rowp(g, u), b = rowp(g, u + 1);
-    const int64_t va = rowp(g, v), vb = rowp(g, v + 1);
-    for (int64_t z = va; z < vb; ++z) {
-      const int cz = g.code[z];
-      if ((cz & 1) != 1 - ev_in) continue;        // leave v through its other end
-      const int32_t w = g.col[z];
-      if (w == u) continue;
-      const int64_t x = find_col(g.col, a, b, w);
-      if (x < 0) continue;
-      const int cx = g.code[x];
-      if ((cx & 1) != eu || ((cx >> 1) & 1) != ((cz >> 1) & 1)) continue;   // the ends of x
-      const long long d = (long long)sy + g.suf[z] - g.suf[x];
-      if (d <= fuzz && d >= -fuzz) trans[x] = 1;
+    const bool full = b[k] > a[k];
+    const unsigned bits = __ballot_sync(0xffffffffu, full);
+    if (lane == 0 && u < g.n) t.has[u >> 5] = bits;
+    slot[k] = 0;
+    if (bits) {                                        // warp-uniform
+      unsigned at = 0;
+      if (lane == 0) at = atomicAdd(&cnt, (unsigned)__popc(bits));
+      slot[k] = __shfl_sync(0xffffffffu, at, 0) + __popc(bits & ((1u << lane) - 1u));
     }
   }
-}
-
-// One thread per entry: kept when neither it nor its mirror is transitive.
-__global__ void k_tr_keep(DevGraph g, const int32_t* row_of, const uint8_t* trans, uint8_t* keep) {
-  for (long long x = grid_tid(); x < g.m; x += grid_threads()) {
-    const int32_t u = row_of[x], w = g.col[x];
-    const int64_t y = find_col(g.col, rowp(g, w), rowp(g, w + 1), u);
-    keep[x] = !trans[x] && !(y >= 0 && trans[y]);
+  if (u0 == 0 && (rowp(g, 0) != 0 || rowp(g, g.n) != g.m)) set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, -1);
+  __syncthreads();
+  if (threadIdx.x == 0) base = cnt ? atomicAdd(t.n_rows, cnt) : 0;
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < kTrRows; ++k) {
+    if (b[k] <= a[k]) continue;
+    const long long u = u0 + k * kBlock, at = (long long)base + slot[k];
+    if (at < t.rows_cap) t.rows[at] = make_int4((int)u, (int)a[k], (int)(b[k] - a[k]), 0);
+    else set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, u);   // more rows with entries than entries: rows that overlap
+    t.info[u] = make_int4((int)a[k], 0, (int)b[k], len[k]);
   }
 }
 
-// One thread per row: its kept entries.
-__global__ void k_tr_rowcnt(DevGraph g, const uint8_t* keep, int32_t* row_cnt) {
-  for (long long u = grid_tid(); u < g.n; u += grid_threads()) {
-    const int64_t a = rowp(g, u), b = rowp(g, u + 1);
-    int cnt = 0;
-    for (int64_t x = a; x < b; ++x) cnt += keep[x];
-    row_cnt[u] = cnt;
+// A batch of listed rows: their records and the places of their entries in the
+// batch, row[j].w the first of row j. Returns the number of entries. Whole block.
+__device__ __forceinline__ int load_batch(const TrBuffers& t, long long b0, int rows, long long R, int4* row,
+                                          int* warp_tot) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int4 mine = make_int4(0, 0, 0, 0);
+  if (tid < rows && b0 + tid < R) mine = t.rows[b0 + tid];
+  int inc = mine.z;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int x = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += x;
+  }
+  if (lane == 31) warp_tot[warp] = inc;
+  __syncthreads();
+  int total = 0;
+  mine.w = inc - mine.z;
+  for (int w = 0; w < (kTrBatch + 31) / 32; ++w) {
+    if (w < warp) mine.w += warp_tot[w];
+    total += warp_tot[w];
+  }
+  if (tid < kTrBatch) row[tid] = mine;
+  __syncthreads();
+  return total;
+}
+
+// The row of the batch's entry i (places past the last listed row start at the
+// batch's end).
+__device__ __forceinline__ int find_row(const int4* row, int i) {
+  int j = 0;
+#pragma unroll
+  for (int step = 64; step > 0; step >>= 1)
+    if (j + step < kTrBatch && row[j + step].w <= i) j += step;
+  return j;
+}
+
+// Rows per batch: as many as hold about kTrAim entries.
+__device__ __forceinline__ int batch_rows(long long m, long long R) {
+  return (int)max(1ll, min((long long)kTrBatch, kTrAim * R / max(m, 1ll)));
+}
+
+// Entries: columns in range, increasing in the row, not the row's own read and a
+// read with entries; codes 0..3. Copies every row in two runs by the end its
+// entries leave through, each run in the row's order: 9 B read and 12 written per
+// entry. An entry's place in its run is the count of entries of that end before
+// it, from the ballots of the block's entries.
+__global__ void __launch_bounds__(kBlock) k_tr_pack(DevGraph g, TrBuffers t) {
+  pdl_enter();
+  __shared__ int4 row[kTrBatch];
+  __shared__ unsigned zeros[kTrStage / 32];            // per word of staged entries: entries leaving through end 0
+  __shared__ int before[kTrStage / 32 + 1];            // the same before each word
+  __shared__ int warp_tot[kBlock / 32];
+  if (__syncthreads_or(failed(t.derr))) return;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const long long R = *t.n_rows;
+  const int rows = batch_rows(g.m, R);
+  for (long long b0 = (long long)blockIdx.x * rows; b0 < R; b0 += (long long)gridDim.x * rows) {
+    const int total = load_batch(t, b0, rows, R, row, warp_tot);
+    constexpr int kPer = kTrStage / kBlock;
+    unsigned cd[kPer];                                 // this thread's staged entries
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const int i = k * kBlock + tid;
+      cd[k] = 4;
+      if (i < total) {
+        const int j = find_row(row, i);
+        cd[k] = g.code[row[j].y + (i - row[j].w)];
+      }
+      const unsigned z = __ballot_sync(0xffffffffu, i < total && (cd[k] & 1) == 0);
+      if (lane == 0) zeros[(k * kBlock + tid) >> 5] = z;
+    }
+    __syncthreads();
+    if (tid < 32) {                                    // two words per lane
+      const int z0 = __popc(zeros[2 * lane]), z1 = __popc(zeros[2 * lane + 1]);
+      int inc = z0 + z1;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += x;
+      }
+      before[2 * lane] = inc - z0 - z1;
+      before[2 * lane + 1] = inc - z1;
+      if (lane == 31) before[kTrStage / 32] = inc;
+    }
+    __syncthreads();
+    auto zeros_before = [&](int i) {                   // among the staged entries
+      return before[i >> 5] + (i < kTrStage ? __popc(zeros[i >> 5] & ((1u << (i & 31)) - 1u)) : 0);
+    };
+    for (int i = tid; i < total; i += kBlock) {
+      const int j = find_row(row, i);
+      const int u = row[j].x, a = row[j].y, n = row[j].z, s0 = row[j].w, x = a + (i - s0);
+      const int32_t w = g.col[x];
+      const unsigned c = g.code[x];
+      const bool ok = w >= 0 && w < g.n && w != u && c <= 3 && (i == s0 || g.col[x - 1] < w) &&
+                      ((t.has[w >> 5] >> (w & 31)) & 1u);
+      if (!ok) set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, x);
+      int z, nz;                                       // entries of end 0 before this one and in the row
+      if (s0 + n <= kTrStage) {
+        z = zeros_before(i) - zeros_before(s0);
+        nz = zeros_before(s0 + n) - zeros_before(s0);
+      } else {
+        z = nz = 0;
+        for (int y = a; y < a + n; ++y) {
+          const int end0 = (g.code[y] & 1) == 0;
+          nz += end0;
+          z += y < x ? end0 : 0;
+        }
+      }
+      if (i == s0) t.info[u].y = a + nz;
+      const int at = (c & 1) == 0 ? a + z : a + nz + (x - a - z);
+      t.ent[at] = make_uint2(((unsigned)w << 2) | (c & 3u), (unsigned)g.suf[x]);
+      if (w < u) t.mir[x] = -1;                        // found from the other side, or missing
+    }
+    __syncthreads();
   }
 }
 
-struct RowCntLoad {
-  const int32_t* cnt;
-  __device__ unsigned long long operator()(long long i) const { return (unsigned long long)cnt[i]; }
-};
-struct RowPtrStore {
-  int64_t* rp;
-  unsigned long long* total;
-  __device__ void item(long long i, unsigned long long e) const { rp[i] = (int64_t)e; }
-  __device__ void last(long long n, unsigned long long t) const {
-    rp[n] = (int64_t)t;
-    *total = t;
-  }
-};
+// One entry z = (v->w) of a walk u -> v -> w: whether it makes the entry x of
+// u's row that leads to w transitive (codes and suffixes of the three).
+__device__ __forceinline__ bool closes(unsigned cx, unsigned cy, unsigned cz, int32_t sx, int32_t sy, int32_t sz,
+                                       int fuzz) {
+  if (((cx ^ cy) & 1) != 0 || ((cx ^ cz) & 2) != 0) return false;   // the ends of x
+  const long long d = (long long)sy + sz - sx;
+  return d <= fuzz && d >= -fuzz;
+}
 
-// One thread per kept entry: its row's new offset plus the kept entries
-// before it in the row (rows keep their order).
-__global__ void k_tr_scatter(DevGraph g, const int32_t* row_of, const uint8_t* keep, const int64_t* out_rp,
-                             int32_t* col, uint8_t* code, int32_t* suf) {
-  for (long long x = grid_tid(); x < g.m; x += grid_threads()) {
-    if (!keep[x]) continue;
-    const int32_t u = row_of[x];
-    int64_t o = out_rp[u];
-    for (int64_t y = rowp(g, u); y < x; ++y) o += keep[y];
-    col[o] = g.col[x];
-    code[o] = g.code[x];
-    suf[o] = g.suf[x];
+// A block per batch of listed rows, a thread per entry y = (u->v): suffix in
+// [1, len-1]; from the smaller read's side, the pair's mirrors; and the entries
+// of u's row that a walk through v makes transitive. The look-ups are binary
+// searches in shared memory, except in rows past the staged entries of a batch,
+// which are searched in place. What bounds it is the records, runs and columns
+// of the rows v, which lie at random (a sector or two each), and issuing the
+// searches, in warps whose lanes walk runs of unequal length. 3.38M entries of
+// 420 thousand rows, by events: 178 us, and 56 for the packing before it; a
+// thread per entry walking whole rows and searching u's row in memory took 283,
+// after 93 for mirrors found by a search of their own; eight lanes per row, four
+// rows of a warp in step, took 476, most of its lanes waiting for longer rows.
+__global__ void __launch_bounds__(kBlock) k_tr_rows(DevGraph g, TrBuffers t, int fuzz) {
+  pdl_enter();
+  __shared__ int4 row[kTrBatch];                       // read, first entry, entries, first of the batch's entries
+  __shared__ unsigned key[kTrStage];                   // column << 2 | code
+  __shared__ int32_t suf[kTrStage];
+  __shared__ uint8_t row_of[kTrStage], hit[kTrStage];
+  __shared__ int warp_tot[kBlock / 32];
+  if (__syncthreads_or(failed(t.derr))) return;
+  const int tid = threadIdx.x;
+  const long long R = *t.n_rows;
+  const int rows = batch_rows(g.m, R);
+  for (long long b0 = (long long)blockIdx.x * rows; b0 < R; b0 += (long long)gridDim.x * rows) {
+    const int total = load_batch(t, b0, rows, R, row, warp_tot);
+    for (int i = tid; i < total; i += kBlock) {
+      const int j = find_row(row, i);
+      const int x = row[j].y + (i - row[j].w);
+      if (row[j].w + row[j].z <= kTrStage) {
+        key[i] = ((unsigned)g.col[x] << 2) | g.code[x];
+        suf[i] = g.suf[x];
+        row_of[i] = (uint8_t)j;
+        hit[i] = 0;
+      } else {
+        t.trans[x] = 0;
+      }
+    }
+    __syncthreads();
+    for (int i = tid; i < total; i += kBlock) {
+      // entry i is staged when its whole row is: then it lies below kTrStage with row_of set
+      int j = i < kTrStage ? row_of[i] : kTrBatch;
+      if (j >= kTrBatch || i < row[j].w || i >= row[j].w + row[j].z || row[j].w + row[j].z > kTrStage)
+        j = find_row(row, i);
+      const int u = row[j].x, a = row[j].y, n = row[j].z, s0 = row[j].w, y = a + (i - s0);
+      const bool staged = s0 + n <= kTrStage;
+      const unsigned e = staged ? key[i] : ((unsigned)g.col[y] << 2) | g.code[y];
+      const int32_t sy = staged ? suf[i] : g.suf[y];
+      const int v = (int)(e >> 2);
+      const unsigned cy = e & 3u;
+      const int4 iv = t.info[v];                       // first entry, first of the second run, end, length
+      if (sy < 1 || sy > iv.w - 1) set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, y);
+      // v is left through its other end: the first run when it was entered through end 1
+      const int z1 = cy & 2u ? iv.y : iv.z;
+      int z = cy & 2u ? iv.x : iv.y;
+      if (u < v) {
+        const int32_t back = find_col(g.col, iv.x, iv.z, u);
+        if (back < 0 || g.code[back] != (((cy & 1) << 1) | (cy >> 1))) {
+          set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, y);
+        } else {
+          t.mir[back] = y;
+        }
+        t.mir[y] = back;
+      }
+      for (; z < z1; z += 4) {
+        uint2 q[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (z + k < z1) q[k] = t.ent[z + k];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          if (z + k >= z1) break;
+          const unsigned ez = q[k].x;
+          if (staged) {
+            int lo = s0;                               // the last column <= w, or the first one
+            for (int len = n; len > 1;) {
+              const int half = len >> 1;
+              if (key[lo + half] <= (ez | 3u)) lo += half;
+              len -= half;
+            }
+            const unsigned kx = key[lo];
+            if ((kx ^ ez) < 4u && closes(kx, cy, ez, suf[lo], sy, (int32_t)q[k].y, fuzz)) hit[lo] = 1;
+          } else {
+            const int32_t x = find_col(g.col, a, a + n, (int32_t)(ez >> 2));
+            if (x >= 0 && closes(g.code[x], cy, ez, g.suf[x], sy, (int32_t)q[k].y, fuzz)) t.trans[x] = 1;
+          }
+        }
+      }
+    }
+    __syncthreads();
+    for (int i = tid; i < min(total, kTrStage); i += kBlock) {
+      const int j = row_of[i];                         // set when i is staged
+      if (j < kTrBatch && i >= row[j].w && i < row[j].w + row[j].z && row[j].w + row[j].z <= kTrStage)
+        t.trans[row[j].y + (i - row[j].w)] = hit[i];
+    }
+    __syncthreads();
+  }
+}
+
+// Per entry: its mirror must have been found; kept when neither is transitive. A block per
+// tile of the map writes the tile's words, the kept entries of the tile before
+// each word, and the tile's count.
+__global__ void __launch_bounds__(kBlock) k_tr_keep(long long m, const uint8_t* trans, const int32_t* mir, unsigned* keep,
+                                                    unsigned* before, unsigned* tile_cnt, DevError* e) {
+  pdl_enter();
+  if (__syncthreads_or(failed(e))) return;
+  constexpr int kPer = kTrTile / kBlock;
+  __shared__ unsigned cnt[kTrTile / 32];
+  const long long tile = blockIdx.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint8_t t[kPer];
+  int32_t y[kPer];
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const long long x = tile * kTrTile + k * kBlock + threadIdx.x;
+    t[k] = x < m ? trans[x] : 1;
+    y[k] = x < m ? mir[x] : 0;
+  }
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    if (y[k] < 0) {                                    // an entry whose pair has no entry back
+      set_error(e, DERR_GRAPH, K_TRANSITIVE, tile * kTrTile + k * kBlock + threadIdx.x);
+      y[k] = 0;
+    }
+    t[k] |= trans[y[k]];
+  }
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const unsigned bits = __ballot_sync(0xffffffffu, t[k] == 0);
+    const int w = k * (kBlock / 32) + warp;
+    if (lane == 0) {
+      keep[tile * (kTrTile / 32) + w] = bits;
+      cnt[w] = __popc(bits);
+    }
+  }
+  __syncthreads();
+  if (warp == 0) {
+    unsigned c[2], inc;
+    c[0] = cnt[2 * lane];
+    c[1] = cnt[2 * lane + 1];
+    inc = c[0] + c[1];
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned x = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += x;
+    }
+    const unsigned ex = inc - c[0] - c[1];
+    unsigned* const b = before + tile * (kTrTile / 32) + 2 * lane;
+    b[0] = ex;
+    b[1] = ex + c[0];
+    if (lane == 31) tile_cnt[tile] = inc;
+  }
+}
+
+// One block: the kept entries before every tile, and all of them in *total.
+__global__ void __launch_bounds__(1024) k_tr_tiles(unsigned* tile_cnt, long long tiles, unsigned long long* total,
+                                                   const DevError* e) {
+  pdl_enter();
+  if (failed(e)) return;
+  __shared__ unsigned warp_tot[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned run = 0;
+  for (long long t0 = 0; t0 < tiles; t0 += 1024) {
+    const long long t = t0 + threadIdx.x;
+    const unsigned v = t < tiles ? tile_cnt[t] : 0u;
+    unsigned inc = v;
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned x = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += x;
+    }
+    if (lane == 31) warp_tot[warp] = inc;
+    __syncthreads();
+    unsigned all = 0, lower = 0;
+    for (int w = 0; w < 32; ++w) {
+      if (w < warp) lower += warp_tot[w];
+      all += warp_tot[w];
+    }
+    if (t < tiles) tile_cnt[t] = run + lower + inc - v;
+    run += all;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) *total = run;
+}
+
+// The kept entries before entry p.
+__device__ __forceinline__ unsigned kept_before(const TrBuffers& t, int64_t p) {
+  return t.tile_cnt[p / kTrTile] + t.before[p >> 5] + __popc(t.keep[p >> 5] & ((1u << (p & 31)) - 1u));
+}
+
+// The reduced graph: every kept entry to its place, and every row's offset;
+// nothing when the entries do not fit.
+__global__ void __launch_bounds__(kBlock) k_tr_scatter(DevGraph g, TrBuffers t, long long cap, int64_t* row_ptr,
+                                                       int32_t* col, uint8_t* code, int32_t* suf) {
+  pdl_enter();
+  if (failed(t.derr)) return;
+  const unsigned long long total = *t.total;
+  if ((long long)total > cap) return;
+  const long long most = max((long long)g.n + 1, (long long)g.m);
+  for (long long i = grid_tid(); i < most; i += grid_threads()) {
+    if (i <= g.n) {
+      const int64_t p = rowp(g, i);
+      row_ptr[i] = p < g.m ? (int64_t)kept_before(t, p) : (int64_t)total;
+    }
+    if (i < g.m && ((t.keep[i >> 5] >> (i & 31)) & 1u)) {
+      const unsigned o = kept_before(t, i);
+      col[o] = g.col[i];
+      code[o] = g.code[i];
+      suf[o] = g.suf[i];
+    }
   }
 }
 
 }  // namespace
 
-cudaError_t launch_transitive_check(const DevGraph& g, DevError* derr, const LaunchEnv& env) {
-  k_tr_check<<<grid_for(g.n, env), kBlock, 0, env.stream>>>(g, derr);
-  mark(env, "k_tr_check");
-  return cudaGetLastError();
-}
-
-cudaError_t launch_transitive_entries(const DevGraph& g, const TrBuffers& t, const LaunchEnv& env) {
-  k_tr_rowof<<<grid_for(g.n, env), kBlock, 0, env.stream>>>(g, t.row_of);
-  mark(env, "k_tr_rowof");
-  k_tr_entries<<<grid_for(g.m, env), kBlock, 0, env.stream>>>(g, t.row_of, t.derr);
-  mark(env, "k_tr_entries");
-  return cudaGetLastError();
-}
+long long transitive_tiles(long long m) { return (m + kTrTile - 1) / kTrTile; }
 
 cudaError_t launch_transitive(const DevGraph& g, int fuzz, const TrBuffers& t, const LaunchEnv& env) {
-  cudaMemsetAsync(t.trans, 0, (size_t)(g.m > 0 ? g.m : 1), env.stream);
-  k_tr_mark<<<grid_for(g.m, env), kBlock, 0, env.stream>>>(g, t.row_of, fuzz, t.trans);
-  mark(env, "k_tr_mark");
-  k_tr_keep<<<grid_for(g.m, env), kBlock, 0, env.stream>>>(g, t.row_of, t.trans, t.keep);
-  mark(env, "k_tr_keep");
-  k_tr_rowcnt<<<grid_for(g.n, env), kBlock, 0, env.stream>>>(g, t.keep, t.row_cnt);
-  mark(env, "k_tr_rowcnt");
-  cudaMemsetAsync(t.state, 0, (size_t)(t.state_cap + 1) * sizeof(unsigned long long), env.stream);
-  const long long tiles = (g.n + kTileItems - 1) / kTileItems;
-  if (tiles > t.state_cap) return cudaErrorInvalidValue;
-  if (g.n > 0) {
-    k_scan<<<scan_grid(tiles, env), kBlock, 0, env.stream>>>(RowCntLoad{t.row_cnt}, RowPtrStore{t.out_rp, t.total}, g.n,
-                                                       t.state, t.state_cap, t.derr, K_TRANSITIVE);
-    mark(env, "k_scan_rows");
-  } else {
-    cudaMemsetAsync(t.out_rp, 0, sizeof(int64_t), env.stream);
-    cudaMemsetAsync(t.total, 0, sizeof(unsigned long long), env.stream);
+  cudaMemsetAsync(t.n_rows, 0, sizeof(unsigned), env.stream);
+  cudaMemsetAsync(t.total, 0, sizeof(unsigned long long), env.stream);
+  const long long blocks = std::max(1ll, ((long long)g.n + kTrRows * kBlock - 1) / (kTrRows * kBlock));
+  k_tr_check<<<(unsigned)blocks, kBlock, 0, env.stream>>>(g, t);
+  mark(env, "k_tr_check");
+  if (g.m > 0) {
+    static const int pack_resident = resident_blocks(k_tr_pack), rows_resident = resident_blocks(k_tr_rows);
+    // persistent grids; no more batches than rows with entries
+    const long long need = std::min((long long)g.n, (long long)g.m);
+    cudaError_t e = launch_k(k_tr_pack, (int)std::min(need, (long long)env.num_sms * pack_resident), env, true, g, t);
+    if (e != cudaSuccess) return e;
+    mark(env, "k_tr_pack");
+    e = launch_k(k_tr_rows, (int)std::min(need, (long long)env.num_sms * rows_resident), env, true, g, t, fuzz);
+    if (e != cudaSuccess) return e;
+    mark(env, "k_tr_rows");
+    const long long tiles = transitive_tiles(g.m);
+    e = launch_k(k_tr_keep, (int)tiles, env, true, (long long)g.m, t.trans, t.mir, t.keep, t.before, t.tile_cnt, t.derr);
+    if (e != cudaSuccess) return e;
+    mark(env, "k_tr_keep");
+    e = launch_kb(k_tr_tiles, 1, 1024, env, true, t.tile_cnt, tiles, t.total, t.derr);
+    if (e != cudaSuccess) return e;
+    mark(env, "k_tr_tiles");
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_transitive_scatter(const DevGraph& g, const TrBuffers& t, int32_t* col, uint8_t* code, int32_t* suf,
-                                      const LaunchEnv& env) {
-  k_tr_scatter<<<grid_for(g.m, env), kBlock, 0, env.stream>>>(g, t.row_of, t.keep, t.out_rp, col, code, suf);
+cudaError_t launch_transitive_scatter(const DevGraph& g, const TrBuffers& t, long long cap, int64_t* row_ptr, int32_t* col,
+                                      uint8_t* code, int32_t* suf, const LaunchEnv& env, bool chained) {
+  cudaError_t e = launch_k(k_tr_scatter, grid_for(std::max((long long)g.n + 1, (long long)g.m), env), env, chained, g, t,
+                           cap, row_ptr, col, code, suf);
+  if (e != cudaSuccess) return e;
   mark(env, "k_tr_scatter");
   return cudaGetLastError();
 }

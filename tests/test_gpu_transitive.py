@@ -100,6 +100,67 @@ def test_on_device_to_contigs(ctx):
     assert np.array_equal(off, orc.contig_off) and np.array_equal(bases, orc.bases)
 
 
+def random_overlaps(seed, n, pairs, hub=0):
+    """Overlaps of random pairs among n reads, codes at random, suffixes of 1 to 4
+    bases (so that many two-step walks add up); with `hub`, read 0 overlaps that
+    many others."""
+    rng = np.random.default_rng(seed)
+    u, v = rng.integers(0, n, size=(2, pairs))
+    if hub:
+        u, v = np.concatenate([u, np.zeros(hub, np.int64)]), np.concatenate([v, np.arange(1, hub + 1)])
+    keep = u != v
+    key = np.unique(np.minimum(u, v)[keep] * n + np.maximum(u, v)[keep])
+    u, v = key // n, key % n
+    code = rng.integers(0, 4, size=len(u))
+    suf = rng.integers(1, 5, size=(2, len(u)))
+    rows, cols = np.concatenate([u, v]), np.concatenate([v, u])
+    codes = np.concatenate([code, ((code & 1) << 1) | (code >> 1)])
+    sufs = np.concatenate(suf)
+    o = np.lexsort((cols, rows))
+    rp = np.zeros(n + 1, np.int64)
+    np.add.at(rp, rows + 1, 1)
+    G = type("R", (), {})()
+    G.row_ptr, G.col, G.code = np.cumsum(rp), cols[o].astype(np.int32), codes[o].astype(np.uint8)
+    G.suf, G.len = sufs[o].astype(np.int32), np.full(n, 400, np.int32)
+    G.off, G.packed, G.n, G.m = np.arange(n, dtype=np.int64) * 400, np.zeros(100 * n, np.uint8), n, len(cols)
+    return G
+
+
+@pytest.mark.parametrize("n,pairs,hub", [
+    (1, 0, 0), (31, 15, 0), (33, 300, 0),       # no entries; a word of reads; dense rows
+    (121, 2000, 0), (240, 3600, 0),             # batches of rows: 30 entries a row, so fewer rows than a batch holds
+    (5000, 900, 0), (9000, 60, 0),              # mostly empty rows, batches that are not full
+    (300, 12000, 0),                            # 80 entries a row
+    (2600, 4000, 2040), (2600, 4000, 2500),     # a row about as long as, and longer than, what is staged
+])
+def test_row_shapes(ctx, n, pairs, hub):
+    G = random_overlaps(n + hub, n, pairs, hub)
+    for fuzz in (0, 1):
+        assert same_csr(cg.cg_transitive_reduction(ctx, G, fuzz), oracle.transitive_reduction(G, fuzz))
+
+
+def test_missing_or_foreign_mirrors(ctx):
+    """An entry whose pair lacks the entry back, seen from the smaller and from the
+    larger read, and one that leads to a read without entries."""
+    G = random_overlaps(5, 200, 900)
+    rows = np.repeat(np.arange(200), np.diff(G.row_ptr))
+    for x in (np.flatnonzero(rows < G.col)[7], np.flatnonzero(rows > G.col)[11]):
+        H = type("R", (), dict(vars(G)))()
+        keep = np.arange(G.m) != x
+        H.row_ptr = G.row_ptr - (np.arange(201) > rows[x])
+        H.col, H.code, H.suf, H.m = G.col[keep], G.code[keep], G.suf[keep], G.m - 1
+        with pytest.raises(cg.CgError) as e:
+            cg.cg_transitive_reduction(ctx, H)
+        assert e.value.status == cg.CG_EGRAPH
+    H = type("R", (), dict(vars(G)))()
+    H.row_ptr, H.col = np.append(G.row_ptr, G.m), G.col.copy()
+    H.col[G.row_ptr[200] - 1], H.len = 200, np.full(201, 400, np.int32)
+    H.off = np.arange(201, dtype=np.int64) * 400
+    with pytest.raises(cg.CgError) as e:
+        cg.cg_transitive_reduction(ctx, H)
+    assert e.value.status == cg.CG_EGRAPH
+
+
 def test_invalid_and_capacity(ctx):
     G = _pins._tr_triangle(1, 1, 1, 10, 15, 25, 30, 20, 50)
     bad = []
