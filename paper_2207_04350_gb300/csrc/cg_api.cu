@@ -454,14 +454,20 @@ cg_status spell_device(cg_graph* g, Form form, int64_t* contig_off, int64_t cont
   const bool fold_off = contig_off && g->g.n > 0;
   st = run_stage(g, 6 + 2 * (int)form + (whole ? 1 : 0), key, [&]() -> cg_status {
     cg::LaunchEnv env = c->env;
-    if (whole) {
-      CK(cg::launch_mask(g->g, g->s, c->env), "mask kernels");
-      CK(cg::launch_chains(g->g, g->s, gt(g), c->env, true), "chain kernels");
-      env.pdl_first = true;
+    int64_t* user_off = fold_off ? contig_off : nullptr;
+    const int64_t user_cap = fold_off ? contig_off_cap : 0;
+    if (whole && g->s.small) {
+      CK(cg::launch_small(g->g, g->s, gt(g), cg::kStageMask | cg::kStageChains | cg::kStageOffsets, user_off, user_cap,
+                          env, false), "stages of a small graph");
+    } else {
+      if (whole) {
+        CK(cg::launch_mask(g->g, g->s, c->env), "mask kernels");
+        CK(cg::launch_chains(g->g, g->s, gt(g), c->env, true), "chain kernels");
+        env.pdl_first = true;
+      }
+      if (stages) record_stage_event(c, 4);
+      CK(cg::launch_offsets(g->g, g->s, gt(g), env, user_off, user_cap), "offset kernels");
     }
-    if (stages) record_stage_event(c, 4);
-    CK(cg::launch_offsets(g->g, g->s, gt(g), env, fold_off ? contig_off : nullptr, fold_off ? contig_off_cap : 0),
-       "offset kernels");
     if (stages) record_stage_event(c, 5);
     if (timing) record_stage_event(c, 6);
     env.pdl_first = !timing;           // no event node between these kernels and the ones before
@@ -540,6 +546,7 @@ cg_status finish_load(cg_graph* g, uint32_t flags) {
   S.scan_state = galloc<unsigned long long>(g, (size_t)S.scan_tiles_cap + 1, &st);
   S.tickets = galloc<unsigned long long>(g, cg::kTicketSets * cg::kTicketStride, &st);
   g->d_sum = galloc<unsigned long long>(g, 1, &st);
+  S.small = cg::small_graph(n, G.m, G.min_chain);
   S.derr = c->derr;
   if (st != CG_OK) return st;
   CK(cudaMemsetAsync(S.ctr, 0, sizeof(cg::Counters) + 8 * (size_t)S.h_tiles, c->stream), "clear counters");

@@ -31,6 +31,7 @@
 #include <cuda_runtime.h>
 
 #include "cg_internal.cuh"
+#include "cg_stage.cuh"
 
 namespace cg {
 
@@ -46,13 +47,6 @@ __device__ __forceinline__ int sampled(int v, int ruler_log2) {
   h *= 0x85EBCA77u;
   h ^= h >> 13;
   return (h & ((1u << ruler_log2) - 1u)) == 0u;
-}
-
-// Read m is the smallest read of a contig of q reads.
-__device__ __forceinline__ void mark_head(const Scratch& s, int32_t m, int32_t q) {
-  atomicOr(&s.hb[m >> 5], 1u << (m & 31));
-  s.headq[m] = q;
-  atomicAdd(&s.hsum[m >> s.h_shift], (1ull << kHeadShift) | (unsigned)q);
 }
 
 // Software grid barrier for kernels launched cooperatively (all blocks
@@ -439,45 +433,8 @@ __global__ void __launch_bounds__(kBlock) k_succ(DevGraph g, Scratch s, int rule
     int s0 = -1, s1 = -1;
     bool r0 = false, r1 = false;
     if (ci < N) {
-      const int32_t v = s.cand[ci];
-      const int64_t a = rowp(g, v);
-      const bool two = rowp(g, v + 1) - a == 2;
-      const int32_t w0 = g.col[a], w1 = two ? g.col[a + 1] : 0;
-      const int cd0 = g.code[a], cd1 = two ? g.code[a + 1] : 0;
-      int32_t q0, q1 = 0, p0 = 0, p1 = 0;
-      if (g.pre) {
-        q0 = g.post[a]; p0 = g.pre[a];
-        if (two) { q1 = g.post[a + 1]; p1 = g.pre[a + 1]; }
-      } else {
-        q0 = g.suf[a];
-        if (two) q1 = g.suf[a + 1];
-      }
-      // a neighbour's candidate index, -1 for a branch read; an entry without its
-      // mirror (a graph loaded unvalidated) may reach a read whose index the mask
-      // stage never wrote: an out-of-range value counts as a branch read, so the
-      // successor and suffix stores below stay inside their arrays
-      int32_t c0 = s.cidx[w0], c1 = two ? s.cidx[w1] : -1;
-      if ((uint32_t)c0 >= (uint32_t)N) c0 = -1;
-      if ((uint32_t)c1 >= (uint32_t)N) c1 = -1;
-      const int32_t u0 = 2 * (int32_t)ci;
-      if (c0 >= 0) {                     // (v, 1-ev) leaves through end ev
-        const int ev = cd0 & 1, to = 2 * c0 + (cd0 >> 1);
-        if (ev == 1) s0 = to; else s1 = to;
-        s.sufin[to] = q0;
-        if (g.pre) s.preout[u0 + 1 - ev] = p0;
-      }
-      if (c1 >= 0) {
-        const int ev = cd1 & 1, to = 2 * c1 + (cd1 >> 1);
-        if (ev == 1) s0 = to; else s1 = to;
-        s.sufin[to] = q1;
-        if (g.pre) s.preout[u0 + 1 - ev] = p1;
-      }
-      s.succ[ci] = make_int4(s0, s1, v, 0);
-      if (s0 < 0 && s1 < 0) {            // every overlap leads to a branch read: spelled alone, or in no contig
-        const bool lone = g.min_chain <= 1;
-        s.prd[ci] = make_int4(lone ? v : -1, lone ? 0 : -1, lone ? g.len[v] : 0, lone ? 0 : 255);
-        if (g.pre) s.pfirst[ci] = 0;   // its contig head is marked by k_final
-      } else {
+      int32_t v;
+      if (link_candidate(g, s, ci, N, s0, s1, v)) {
         reinterpret_cast<int4*>(s.rr)[ci] = make_int4(-1, 0, -1, 0);   // not yet reached by a sublist walk
         const bool smp = sampled(v, ruler_log2) != 0;
         r0 = s1 < 0 || smp;              // (c,0) has no predecessor when (c,1) has no successor
@@ -629,32 +586,6 @@ __global__ void k_jump(Scratch s) {
   if (grid_tid() == 0) c->final_buf = (unsigned)cur;
 }
 
-// x-drop form (Sec. 4.4): read v (candidate ci), walked as oriented
-// candidate u at rank rk of a contig of q reads, contributes
-// l_v[post(e_in) : pre(e_out)] with alpha (its first base in walk direction)
-// for the first read and beta (its last) for the last one; a piece whose end
-// comes before its start is empty. Returns the piece's length; its first
-// stored base goes to pfirst.
-__device__ __forceinline__ int32_t set_piece(const DevGraph& g, const Scratch& s, int32_t v, int32_t ci, int32_t u,
-                                             int32_t rk, int32_t q) {
-  const int o = u & 1;
-  const int32_t L = g.len[v];
-  const int32_t first = rk == 0 ? (o == 0 ? 0 : L - 1) : s.sufin[u];
-  const int32_t last = rk == q - 1 ? (o == 0 ? L - 1 : 0) : s.preout[u];
-  const int32_t cnt = o == 0 ? last - first + 1 : first - last + 1;
-  s.pfirst[ci] = first;
-  return cnt > 0 ? cnt : 0;
-}
-
-// The bases a chain read adds: the first read whole, each later one the
-// suffix of the overlap it is entered through (or, in the x-drop form, its
-// piece).
-__device__ __forceinline__ int32_t piece_len(const DevGraph& g, const Scratch& s, int32_t v, int32_t ci, int32_t u,
-                                             int32_t rk, int32_t q) {
-  if (g.pre) return set_piece(g, s, v, ci, u, rk, q);
-  return rk == 0 ? g.len[v] : s.sufin[u];
-}
-
 // Per chain candidate: combine its two oriented copies. head(list of (c,0))
 // is the reverse of tail(list of (c,1)). The contig starts at the
 // smaller-id end read, so (c,0) is the walk orientation when that end heads
@@ -767,94 +698,12 @@ __global__ void k_final(DevGraph g, Scratch s) {
   if ((threadIdx.x & 31) == 0 && heads) atomicAdd(&c->n_heads, heads);
 }
 
-// Closed chains (rare). Over their oriented candidates: pointer jumping for
-// the smallest oriented read 2v + o of each directed cycle, carried with the
-// oriented candidate that holds it (the copy holding (m,0) is the walk, m the
-// smallest read), then cut the walk before (m,0) and rank by pointer jumping
-// again.
 __global__ void k_cycles(DevGraph g, Scratch s) {
   pdl_enter();
   Counters* c = s.ctr;
-  unsigned C = *(volatile unsigned*)&c->n_cycle_reads;
+  const unsigned C = *(volatile unsigned*)&c->n_cycle_reads;
   if (C == 0) return;
-  long long N = 2ll * C;
-  for (long long i = grid_tid(); i < N; i += grid_threads()) {
-    const int32_t ci = s.cyc[i >> 1], u = 2 * ci + (int)(i & 1);
-    const int4 sv = s.succ[ci];
-    const int32_t z = (u & 1) ? sv.y : sv.x;
-    if (z < 0) set_error(s.derr, DERR_KERNEL, K_CYCLE, u);
-    s.c_ptr[0][u] = z;
-    s.c_val[0][u] = ((long long)(2 * sv.z + (u & 1)) << 32) | (unsigned)u;
-  }
-  int rounds = 1;
-  while ((1ll << rounds) < N + 1 && rounds < 31) ++rounds;
-  ++rounds;
-  int cur = 0;
-  if (!grid_sync(c, s.derr)) return;
-  for (int r = 0; r < rounds; ++r) {
-    int nxt = cur ^ 1;
-    for (long long i = grid_tid(); i < N; i += grid_threads()) {
-      const int32_t u = 2 * s.cyc[i >> 1] + (int)(i & 1);
-      const int32_t p = s.c_ptr[cur][u];
-      if (p < 0) continue;
-      s.c_val[nxt][u] = min(s.c_val[cur][u], s.c_val[cur][p]);
-      s.c_ptr[nxt][u] = s.c_ptr[cur][p];
-    }
-    cur = nxt;
-    if (!grid_sync(c, s.derr)) return;
-  }
-  // cut: on the walk copy, the oriented candidate before the start has no successor
-  for (long long i = grid_tid(); i < N; i += grid_threads()) {
-    const int32_t ci = s.cyc[i >> 1], u = 2 * ci + (int)(i & 1);
-    const int32_t head = (int32_t)(s.c_val[cur][u] & 0xffffffffll);   // the oriented candidate holding the smallest read
-    s.c_head[u] = head;
-    if ((head & 1) == 0) {
-      const int4 sv = s.succ[ci];
-      const int32_t z = (u & 1) ? sv.y : sv.x;
-      const int32_t p = (z == head) ? -1 : z;
-      s.c_ptr[0][u] = p;
-      s.c_val[0][u] = p < 0 ? 0 : 1;
-    }
-  }
-  cur = 0;
-  if (!grid_sync(c, s.derr)) return;
-  for (int r = 0; r < rounds; ++r) {
-    int nxt = cur ^ 1;
-    for (long long i = grid_tid(); i < N; i += grid_threads()) {
-      const int32_t u = 2 * s.cyc[i >> 1] + (int)(i & 1);
-      if (s.c_head[u] & 1) continue;
-      const int32_t p = s.c_ptr[cur][u];
-      if (p >= 0) {
-        s.c_val[nxt][u] = s.c_val[cur][u] + s.c_val[cur][p];
-        s.c_ptr[nxt][u] = s.c_ptr[cur][p];
-      } else {
-        s.c_val[nxt][u] = s.c_val[cur][u];
-        s.c_ptr[nxt][u] = -1;
-      }
-    }
-    cur = nxt;
-    if (!grid_sync(c, s.derr)) return;
-  }
-  for (long long i = grid_tid(); i < N; i += grid_threads()) {
-    const int32_t ci = s.cyc[i >> 1];
-    const int32_t u = 2 * ci + (int)(i & 1);
-    const int32_t head = s.c_head[u];
-    if (head & 1) continue;
-    const int32_t L = (int32_t)s.c_val[cur][head] + 1;      // distance from the start to the cut, plus one
-    const int32_t rk = L - 1 - (int32_t)s.c_val[cur][u];
-    const int32_t m = s.cand[head >> 1];
-    const int32_t v = s.cand[ci];
-    if (L >= g.min_chain) {
-      s.prd[ci] = make_int4(m, rk, piece_len(g, s, v, ci, u, rk, L), u & 1);
-      if (rk == 0) {
-        mark_head(s, m, L);
-        atomicAdd(&c->n_heads, 1u);
-      }
-    } else {
-      s.prd[ci] = make_int4(-1, -1, 0, 255);
-    }
-    if (rk == 0) atomicAdd(&c->n_cycles, 1u);
-  }
+  close_cycles(g, s, C, grid_tid(), grid_threads(), [&] { return grid_sync(c, s.derr); });
 }
 
 // Per-read chain outputs: first every read's default (a lone read, when
@@ -939,6 +788,7 @@ cudaError_t launch_sum_len(const DevGraph& g, unsigned long long* out, const Lau
 }
 
 cudaError_t launch_mask(const DevGraph& g, const Scratch& s, const LaunchEnv& env) {
+  if (s.small) return launch_small(g, s, Tuning{}, kStageMask, nullptr, 0, env, false);
   // the counters and, right behind them, the tile sums of the lone reads
   cudaMemsetAsync(&s.ctr->n_branch, 0,
                   sizeof(Counters) - offsetof(Counters, n_branch) + (size_t)s.h_tiles * sizeof(unsigned long long),
@@ -957,6 +807,7 @@ cudaError_t launch_mask(const DevGraph& g, const Scratch& s, const LaunchEnv& en
 
 cudaError_t launch_chains(const DevGraph& g, const Scratch& s, const Tuning& t, const LaunchEnv& env,
                           bool after_mask) {
+  if (s.small) return launch_small(g, s, t, kStageChains, nullptr, 0, env, after_mask);
   // restart the chain-stage counters; the head bitmap restarts from the mask
   // stage's words (lone reads; k_succ copies them) and gains the chain heads
   if (!after_mask)

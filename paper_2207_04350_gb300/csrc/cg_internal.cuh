@@ -134,6 +134,7 @@ struct Scratch {
   int64_t scan_tiles_cap;
   Counters* ctr;
   DevError* derr;
+  bool small;                   // one kernel runs the mask, chain and offsets stages (cg_small.cu)
   unsigned long long* tickets;  // kTicketSets counters, one 128-byte line each: a spelling launch's tiles
 };
 
@@ -238,6 +239,22 @@ inline void mark(const LaunchEnv& env, const char* name) {
 }
 
 // ---- launchers (each returns cudaGetLastError()) ----
+// The stages of a small graph, any of them in one kernel (cg_small.cu); the
+// launchers of the single stages below use it for such graphs too.
+enum : int { kStageMask = 1, kStageChains = 2, kStageOffsets = 4 };
+// A small graph: one block beats ten kernels while a few reads and candidates per
+// thread are all there is. Steps in us, one block against ten kernels: 750 reads
+// 26.7 / 39.0, 5,000 31.5 / 44.0, 10,000 38.1 / 45.2, 20,000 51.7 / 49.6, 40,000
+// 84 / 56; with the lone reads spelled too, which one block also scatters, 2,500
+// 42.7 / 49.5 and 5,000 68.5 / 64.9. The bound on the entries is that of an
+// overlap graph of so many reads after the reduction; 8 entries a read would cost
+// what 20,000 reads do.
+constexpr int64_t kSmallReads = 16384, kSmallLoneReads = 4096, kSmallEntries = 8192;
+inline bool small_graph(int64_t n, int64_t m, int min_chain) {
+  return n > 0 && n <= (min_chain <= 1 ? kSmallLoneReads : kSmallReads) && m <= kSmallEntries;
+}
+cudaError_t launch_small(const DevGraph& g, const Scratch& s, const Tuning& t, int stages, int64_t* user_off,
+                         long long user_cap, const LaunchEnv& env, bool chained);
 cudaError_t launch_validate(const DevGraph& g, DevError* derr, const LaunchEnv& env);
 cudaError_t launch_mask(const DevGraph& g, const Scratch& s, const LaunchEnv& env);
 // after_mask: the mask's launch comes right before on the stream, and has just

@@ -28,44 +28,11 @@
 
 #include "cg_internal.cuh"
 #include "cg_lookback.cuh"
+#include "cg_stage.cuh"
 
 namespace cg {
 
 namespace {
-
-// Block-wide exclusive prefix of one 64-bit value per thread; the sum of all in
-// *total. `tot` is shared memory of kBlock / 32 words, free again after a barrier.
-__device__ __forceinline__ unsigned long long block_exclusive(unsigned long long v, unsigned long long* tot,
-                                                              unsigned long long* total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned long long inc = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned long long t = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += t;
-  }
-  if (lane == 31) tot[warp] = inc;
-  __syncthreads();
-  unsigned long long before = 0, all = 0;
-#pragma unroll
-  for (int w = 0; w < kBlock / 32; ++w) {
-    if (w < warp) before += tot[w];
-    all += tot[w];
-  }
-  *total = all;
-  return before + inc - v;
-}
-
-// Block-wide sum, the same scratch.
-__device__ __forceinline__ unsigned long long block_sum(unsigned long long v, unsigned long long* tot) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) tot[threadIdx.x >> 5] = v;
-  __syncthreads();
-  unsigned long long all = 0;
-#pragma unroll
-  for (int w = 0; w < kBlock / 32; ++w) all += tot[w];
-  return all;
-}
 
 // Contig index and first walk position of every head, a block per tile of the
 // heads bitmap (256 words or more). The value of a word packs the contigs
@@ -99,12 +66,12 @@ __global__ void __launch_bounds__(kBlock) k_heads(Scratch s, long long n, int64_
     unsigned long long reads = __popc(lone) + q0;
     for (unsigned c = chain & (chain - 1); c; c &= c - 1) reads += (unsigned)hq[__ffs(c) - 1];   // rare
     if (first) {
-      run = block_sum(run, tot[1]);
+      run = block_sum<kBlock / 32>(run, tot[1]);
       first = false;
     }
     unsigned long long all;
     const unsigned long long e =
-        run + block_exclusive(((unsigned long long)__popc(bits) << kHeadShift) | reads, tot[0], &all);
+        run + block_exclusive<kBlock / 32>(((unsigned long long)__popc(bits) << kHeadShift) | reads, tot[0], &all);
     if (w < w_end) {
       unsigned k = (unsigned)(e >> kHeadShift);
       unsigned long long r = e & ((1ull << kHeadShift) - 1);
@@ -140,53 +107,6 @@ __global__ void __launch_bounds__(kBlock) k_heads(Scratch s, long long n, int64_
     }
   }
 }
-
-// What the piece scan writes for walk position j: a piece of L bases from
-// output offset o on, the first of contig `starts` (or -1).
-struct PieceStore {
-  int64_t* out_off;
-  int64_t* contig_off;
-  int32_t* tile_seg;
-  long long tiles_cap;
-  long long tile_bytes;
-  Counters* c;
-  DevError* derr;
-  // The caller's contig offsets, when the offsets are spelled for a caller
-  // buffer in the same replayed stage: written here instead of by a copy kernel
-  // afterwards, and only when all n_contigs + 1 fit (else a capacity error).
-  int64_t* user_off;
-  long long user_cap;
-  __device__ bool user_fits() const {
-    return user_off && (long long)*(const volatile unsigned*)&c->n_contigs + 1 <= user_cap;
-  }
-  __device__ void item(long long j, long long o, long long L, int32_t starts) const {
-    out_off[j] = o;
-    if (starts >= 0) {
-      contig_off[starts] = o;
-      if (user_fits()) user_off[starts] = o;
-    }
-    // tile_bytes is a power of two: the first tile starting at or after o, and after o + L
-    const int sh = __ffsll(tile_bytes) - 1;
-    long long t0 = (o + tile_bytes - 1) >> sh, t1 = (o + L + tile_bytes - 1) >> sh;
-    for (long long t = t0; t < t1; ++t) {
-      if (t < tiles_cap) tile_seg[t] = (int32_t)j;
-      else set_error(derr, DERR_KERNEL, K_SCAN_OFFSETS, t);
-    }
-  }
-  __device__ void last(long long count, unsigned long long total) const {
-    out_off[count] = (long long)total;
-    contig_off[c->n_contigs] = (long long)total;
-    if (user_off) {
-      if (user_fits()) user_off[c->n_contigs] = (long long)total;
-      else set_error(derr, DERR_CAPACITY, K_CONTIG_OFF, (long long)c->n_contigs + 1);
-    }
-    c->total_bases = (long long)total;
-    long long nt = ((long long)total + tile_bytes - 1) / tile_bytes;
-    c->n_tiles = (unsigned)nt;
-    if (nt <= tiles_cap) tile_seg[nt] = (int32_t)(count - 1);
-    else set_error(derr, DERR_KERNEL, K_SCAN_OFFSETS, nt);
-  }
-};
 
 // Piece offsets over the walk positions, in tiles of kPieceTile positions, four
 // per thread, with a decoupled look-back (cg_lookback.cuh). Adding up every
@@ -225,7 +145,7 @@ __global__ void __launch_bounds__(kBlock) k_pieces(Scratch s, PieceStore ps) {
     unsigned long long sum = 0;
 #pragma unroll
     for (int k = 0; k < kPieceItems; ++k) sum += (unsigned)L[k];
-    unsigned long long all, e = block_exclusive(sum, tot, &all);
+    unsigned long long all, e = block_exclusive<kBlock / 32>(sum, tot, &all);
     e += lookback(s.scan_state, tile, all, s.derr, (int)K_SCAN_OFFSETS);
 #pragma unroll
     for (int k = 0; k < kPieceItems; ++k) {
@@ -238,75 +158,9 @@ __global__ void __launch_bounds__(kBlock) k_pieces(Scratch s, PieceStore ps) {
   }
 }
 
-// Every spelled read goes to walk position first(contig) + rank, with the
-// stored-base address of its piece (for one part's layout, an empty piece
-// when its contig belongs to another part): forward reads add stored bases
-// [len-contrib, len), reverse-complement reads the complement of stored
-// bases contrib-1 down to 0. The spelled reads are the lone reads of the mask
-// stage (each its own contig, whole and forward) and the candidates with a
-// contig in their record (chains long enough, and reads cut off by branch
-// reads when those are spelled alone). A thread takes two reads at a time and
-// issues each level of their dependent loads together, before any store.
-constexpr int kScatterItems = 2;
-
 __global__ void k_scatter(DevGraph g, Scratch s) {
   pdl_enter();
-  Counters* c = s.ctr;
-  const long long L1 = *(volatile unsigned*)&c->n_lone, NC = *(volatile unsigned*)&c->n_cand;
-  const long long W = *(volatile unsigned*)&c->n_walk;
-  const long long total = L1 + NC;
-  const long long T = grid_threads();
-  for (long long k0 = grid_tid(); k0 < total; k0 += kScatterItems * T) {
-    long long k[kScatterItems];
-    int32_t v[kScatterItems];
-    int4 p[kScatterItems];
-    bool ok[kScatterItems];
-#pragma unroll
-    for (int j = 0; j < kScatterItems; ++j) {
-      k[j] = k0 + j * T;
-      v[j] = k[j] >= total ? 0 : (k[j] < L1 ? s.lone[k[j]] : s.cand[k[j] - L1]);
-      // a lone read: its own contig, rank 0, whole and forward (its length is filled in below)
-      p[j] = k[j] >= total ? make_int4(-1, 0, 0, 0) : (k[j] < L1 ? make_int4(v[j], 0, -1, 0) : s.prd[k[j] - L1]);
-      ok[j] = p[j].x >= 0;                 // not a chain shorter than min_chain
-    }
-    unsigned word[kScatterItems], wpv[kScatterItems];
-    int32_t L[kScatterItems], pf[kScatterItems];
-    int64_t base[kScatterItems];
-#pragma unroll
-    for (int j = 0; j < kScatterItems; ++j) {
-      const int32_t m = ok[j] ? p[j].x : 0;
-      word[j] = ok[j] ? s.hb[m >> 5] : 0u;
-      wpv[j] = ok[j] ? s.wp[m >> 5] : 0u;
-      L[j] = ok[j] ? g.len[v[j]] : 0;
-      base[j] = ok[j] ? g.off[v[j]] : 0;
-      pf[j] = ok[j] && g.pre && k[j] >= L1 ? s.pfirst[k[j] - L1] : 0;
-    }
-    long long cidx[kScatterItems], pos[kScatterItems];
-#pragma unroll
-    for (int j = 0; j < kScatterItems; ++j) {
-      const int32_t m = p[j].x;
-      cidx[j] = (long long)wpv[j] + __popc(word[j] & ((1u << (m & 31)) - 1u));
-      pos[j] = ok[j] ? (long long)s.cbase[cidx[j]] + p[j].y : 0;
-    }
-#pragma unroll
-    for (int j = 0; j < kScatterItems; ++j) {
-      if (!ok[j]) continue;
-      const int32_t m = p[j].x, rk = p[j].y;
-      if (!((word[j] >> (m & 31)) & 1u) || pos[j] >= W) { set_error(s.derr, DERR_KERNEL, K_SCATTER, v[j]); continue; }
-      const int o = p[j].w;
-      const int32_t cb = p[j].z < 0 ? L[j] : p[j].z;
-      // stored index of the piece's first base: suffix form, the last cb bases
-      // of the oriented read; x-drop form, set by the chain stage (a read spelled
-      // alone is whole and forward)
-      const int64_t first = !g.pre ? (o == 0 ? L[j] - cb : cb - 1) : pf[j];
-      const unsigned long long src = o == 0 ? (unsigned long long)(base[j] + first)
-                                            : ((unsigned long long)(base[j] + first) | (1ull << 63));
-      s.wsrc[pos[j]] = src;
-      s.wlen[pos[j]] = s.part && s.part[cidx[j]] != s.part_p ? 0 : cb;   // another part's contig: empty
-      s.wfirst[pos[j]] = rk == 0 ? (int32_t)cidx[j] : -1;
-      if (s.wread) s.wread[pos[j]] = v[j];           // a graph without its reads: for the read exchange
-    }
-  }
+  scatter_reads(g, s, grid_tid(), grid_threads());
 }
 
 // An empty graph: no contigs, and the one offset 0.
@@ -341,6 +195,7 @@ cudaError_t launch_offsets(const DevGraph& g, const Scratch& s, const Tuning& t,
     mark(env, "k_contig_off");
     return cudaGetLastError();
   }
+  if (s.small) return launch_small(g, s, t, kStageOffsets, user_off, user_cap, env, env.pdl_first);
   cudaError_t e = launch_k(k_heads, s.h_tiles, env, env.pdl_first, s, (long long)g.n, user_off, user_cap);
   if (e != cudaSuccess) return e;
   mark(env, "k_heads");
