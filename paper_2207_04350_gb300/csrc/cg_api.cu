@@ -1490,24 +1490,27 @@ cg_status cg_emit_share(cg_graph* g, int32_t share, int32_t n_shares, int64_t* c
 }
 
 // ------------------------------------------------------------ read exchange
-// Device state of one exchange call: the read bounds, the shares' walk
-// ranges, the first pair of each share's range.
+// One exchange call: its device arrays (one allocation) and, on the host, what
+// the kernels counted.
 struct Xchg {
   cg::XchgArgs x{};
-  std::vector<long long> range, pair0;   // host copies
-  long long n_pairs = 0;
-  void* mem[3] = {nullptr, nullptr, nullptr};
+  std::vector<int64_t> counted;          // range (2 N), pair0 (N + 1), send words (N), receive words (N)
+  uint32_t* mine = nullptr;
+  void* mem = nullptr;
+  const int64_t* range() const { return counted.data(); }
+  const int64_t* pair0() const { return counted.data() + 2 * x.n_shares; }
+  const int64_t* send() const { return counted.data() + 3 * x.n_shares + 1; }
+  const int64_t* recv() const { return counted.data() + 4 * x.n_shares + 1; }
+  static int64_t sum(const int64_t* w, int n) {
+    int64_t t = 0;
+    for (int k = 0; k < n; ++k) t += w[k];
+    return t;
+  }
 };
 
-static void x_release(cg_ctx* c, Xchg& X) {
-  for (void*& p : X.mem) {
-    dfree(c, p);
-    p = nullptr;
-  }
-}
-
-// Checks the arguments, lays out the graph if needed and fills X (waits).
-static cg_status x_prepare(cg_graph* g, int32_t n_shares, const int64_t* read_first, int32_t rank, Xchg& X) {
+// Checks the arguments, lays out the graph if needed and fills X; with want_mine
+// also every pair's words (X.mine). Waits once.
+static cg_status x_count(cg_graph* g, int32_t n_shares, const int64_t* read_first, int32_t rank, bool want_mine, Xchg& X) {
   cg_ctx* c = g->ctx;
   if (!g->g.no_reads) return fail(c, CG_EINVAL, "the read exchange is for graphs loaded with CG_NO_READS");
   if (n_shares < 1 || n_shares > CG_MAX_PARTS || rank < 0 || rank >= n_shares || !read_first)
@@ -1520,64 +1523,24 @@ static cg_status x_prepare(cg_graph* g, int32_t n_shares, const int64_t* read_fi
     st = run_offsets(g);
     if (st != CG_OK) return st;
   }
-  const int N = n_shares;
-  int64_t* rf = (int64_t*)dalloc(c, (size_t)(N + 1) * 8, &st);
-  long long* range = st == CG_OK ? (long long*)dalloc(c, (size_t)2 * N * 8, &st) : nullptr;
-  long long* pair0 = st == CG_OK ? (long long*)dalloc(c, (size_t)(N + 1) * 8, &st) : nullptr;
-  X.mem[0] = rf;
-  X.mem[1] = range;
-  X.mem[2] = pair0;
-  if (st != CG_OK) return st;
-  CK(cudaMemcpyAsync(rf, read_first, (size_t)(N + 1) * 8, cudaMemcpyHostToDevice, c->stream), "copy read bounds");
-  CK(cg::launch_x_ranges(g->s, N, gt(g).tile_bytes, range, c->env), "share ranges");
-  X.range.assign((size_t)2 * N, 0);
-  CK(cudaMemcpyAsync(X.range.data(), range, (size_t)2 * N * 8, cudaMemcpyDeviceToHost, c->stream), "read ranges");
-  st = wait_and_read(g);
-  if (st != CG_OK) return st;
-  X.pair0.assign((size_t)N + 1, 0);
-  for (int p = 0; p < N; ++p)
-    X.pair0[p + 1] = X.pair0[p] + std::max(0ll, X.range[2 * p + 1] - X.range[2 * p] + 1);
-  X.n_pairs = X.pair0[N];
-  CK(cudaMemcpyAsync(pair0, X.pair0.data(), (size_t)(N + 1) * 8, cudaMemcpyHostToDevice, c->stream), "copy pairs");
-  X.x.rf = rf;
-  X.x.n_shares = N;
-  X.x.rank = rank;
-  X.x.range = range;
-  X.x.pair0 = pair0;
-  return CG_OK;
-}
-
-// Words sent to each share and received from each rank (host vectors; waits).
-static cg_status x_sizes(cg_graph* g, Xchg& X, std::vector<unsigned long long>& send_w,
-                         std::vector<unsigned long long>& recv_w) {
-  cg_ctx* c = g->ctx;
-  const int N = X.x.n_shares;
-  cg_status st = CG_OK;
-  unsigned long long* d = (unsigned long long*)dalloc(c, (size_t)2 * N * 8, &st);
+  const size_t N = (size_t)n_shares, counts = 5 * N + 1;
+  const size_t pairs = want_mine ? (size_t)g->g.n + N : 0;    // a share's first piece may be the last of the one before
+  int64_t* d = (int64_t*)dalloc(c, (counts + N + 1) * 8 + pairs * 4, &st);
   if (!d) return st;
-  send_w.assign((size_t)N, 0);
-  recv_w.assign((size_t)N, 0);
-  cudaError_t e = cg::launch_x_sizes(g->s, X.x, d, d + N, X.n_pairs, c->env);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(send_w.data(), d, (size_t)N * 8, cudaMemcpyDeviceToHost, c->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(recv_w.data(), d + N, (size_t)N * 8, cudaMemcpyDeviceToHost, c->stream);
-  if (e == cudaSuccess) st = wait_and_read(g);
-  dfree(c, d);
-  if (e != cudaSuccess) return cuda_fail(c, e, "exchange sizes");
-  return st;
-}
-
-// Per-owner exclusive scans over walk ranges: slot arrays of `count` entries.
-static cg_status x_scan(cg_graph* g, Xchg& X, long long j0, long long count, int who, long long* slot) {
-  cg_ctx* c = g->ctx;
-  if (count <= 0) return CG_OK;
-  cg_status st = CG_OK;
-  const long long cap = (count + 2047) / 2048 + 1;
-  unsigned long long* state = (unsigned long long*)dalloc(c, (size_t)(cap + 1) * 8, &st);
-  if (!state) return st;
-  cudaError_t e = cg::launch_x_scan(g->s, X.x, j0, count, who, slot, state, cap, c->env);
-  dfree(c, state);                    // stream-ordered: freed after the scan
-  if (e != cudaSuccess) return cuda_fail(c, e, "exchange scan");
-  return CG_OK;
+  X.mem = d;
+  X.x.n_shares = n_shares;
+  X.x.rank = rank;
+  X.x.range = (long long*)d;
+  X.x.pair0 = X.x.range + 2 * N;
+  X.x.send_words = (unsigned long long*)(X.x.pair0 + N + 1);
+  X.x.recv_words = X.x.send_words + N;
+  X.x.rf = (int64_t*)(X.x.recv_words + N);
+  X.mine = want_mine ? (uint32_t*)(d + counts + N + 1) : nullptr;
+  CK(cudaMemcpyAsync((void*)X.x.rf, read_first, (N + 1) * 8, cudaMemcpyHostToDevice, c->stream), "copy read bounds");
+  CK(cg::launch_x_sizes(g->s, X.x, gt(g).tile_bytes, g->g.n + n_shares, X.mine, c->env), "exchange sizes");
+  X.counted.assign(counts, 0);
+  CK(cudaMemcpyAsync(X.counted.data(), d, counts * 8, cudaMemcpyDeviceToHost, c->stream), "read exchange sizes");
+  return wait_and_read(g);
 }
 
 cg_status cg_exchange_sizes(cg_graph* g, int32_t n_shares, const int64_t* read_first, int32_t rank,
@@ -1588,14 +1551,12 @@ cg_status cg_exchange_sizes(cg_graph* g, int32_t n_shares, const int64_t* read_f
   cg_status st = check_ctx(c);
   if (st != CG_OK) return st;
   Xchg X;
-  st = x_prepare(g, n_shares, read_first, rank, X);
-  std::vector<unsigned long long> sw, rw;
-  if (st == CG_OK) st = x_sizes(g, X, sw, rw);
-  x_release(c, X);
+  st = x_count(g, n_shares, read_first, rank, false, X);
+  dfree(c, X.mem);
   if (st != CG_OK) return st;
   for (int p = 0; p < n_shares; ++p) {
-    if (send_bytes) send_bytes[p] = (int64_t)(4 * sw[p]);
-    if (recv_bytes) recv_bytes[p] = (int64_t)(4 * rw[p]);
+    if (send_bytes) send_bytes[p] = 4 * X.send()[p];
+    if (recv_bytes) recv_bytes[p] = 4 * X.recv()[p];
   }
   return CG_OK;
 }
@@ -1612,43 +1573,27 @@ cg_status cg_exchange_pack(cg_graph* g, int32_t n_shares, const int64_t* read_fi
       !aligned(my_off, 8))
     return fail(c, CG_EINVAL, "bad exchange buffers");
   Xchg X;
-  st = x_prepare(g, n_shares, read_first, rank, X);
-  std::vector<unsigned long long> sw, rw;
-  if (st == CG_OK) st = x_sizes(g, X, sw, rw);
-  long long* seg = nullptr;
-  long long* slot = nullptr;
+  st = x_count(g, n_shares, read_first, rank, true, X);
+  char* tmp = nullptr;
   if (st == CG_OK) {
-    std::vector<long long> seg_h((size_t)n_shares + 1, 0);
-    for (int p = 0; p < n_shares; ++p) seg_h[p + 1] = seg_h[p] + (long long)sw[p];
-    if (4 * seg_h[n_shares] > send_cap)
-      st = fail(c, CG_EINVAL, "send capacity %lld < %lld", (long long)send_cap, 4 * seg_h[n_shares]);
-    const long long my_reads = read_first[rank + 1] - read_first[rank];
-    if (st == CG_OK && my_reads > 0 && !my_off) st = fail(c, CG_EINVAL, "my_off is required");
-    if (st == CG_OK) seg = (long long*)dalloc(c, (size_t)(n_shares + 1) * 8, &st);
-    if (st == CG_OK) slot = (long long*)dalloc(c, (size_t)std::max(1ll, X.n_pairs) * 8, &st);
-    if (st == CG_OK && seg_h[n_shares] > 0) {
-      cudaError_t e = cudaMemcpyAsync(seg, seg_h.data(), (size_t)(n_shares + 1) * 8, cudaMemcpyHostToDevice, c->stream);
-      if (e != cudaSuccess) st = cuda_fail(c, e, "copy segments");
-      if (st == CG_OK) {               // one scan over every share's pairs
-        const long long cap = (X.n_pairs + 2047) / 2048 + 1;
-        unsigned long long* state = (unsigned long long*)dalloc(c, (size_t)(cap + 1) * 8, &st);
-        if (state) {
-          e = cg::launch_x_scan_pairs(g->s, X.x, X.n_pairs, slot, state, cap, c->env);
-          dfree(c, state);
-          if (e != cudaSuccess) st = cuda_fail(c, e, "exchange scan");
-        }
+    const int64_t words = Xchg::sum(X.send(), n_shares), pairs = X.pair0()[n_shares];
+    if (4 * words > send_cap)
+      st = fail(c, CG_EINVAL, "send capacity %lld < %lld", (long long)send_cap, (long long)(4 * words));
+    else if (read_first[rank + 1] > read_first[rank] && !my_off)
+      st = fail(c, CG_EINVAL, "my_off is required");
+    else if (words > 0) {
+      const long long cap = (pairs + 2047) / 2048 + 1;   // the places of the pairs, and the scan's descriptors
+      tmp = (char*)dalloc(c, (size_t)pairs * 8 + (size_t)(cap + 1) * 8, &st);
+      if (tmp) {
+        cudaError_t e = cg::launch_x_pack(g->g, g->s, X.x, my_packed, my_packed_bytes, my_off, X.mine, (long long*)tmp,
+                                          (unsigned long long*)(tmp + 8 * (size_t)pairs), cap,
+                                          reinterpret_cast<uint32_t*>(send_buf), pairs, c->env);
+        st = e != cudaSuccess ? cuda_fail(c, e, "exchange pack") : wait_and_read(g);
       }
-      if (st == CG_OK) {
-        e = cg::launch_x_pack(g->g, g->s, X.x, my_packed, my_packed_bytes, my_off, seg, slot,
-                              reinterpret_cast<uint32_t*>(send_buf), X.n_pairs, c->env);
-        if (e != cudaSuccess) st = cuda_fail(c, e, "exchange pack");
-      }
-      if (st == CG_OK) st = wait_and_read(g);
     }
   }
-  dfree(c, seg);
-  dfree(c, slot);
-  x_release(c, X);
+  dfree(c, tmp);
+  dfree(c, X.mem);
   return st;
 }
 
@@ -1665,28 +1610,19 @@ cg_status cg_emit_share_received(cg_graph* g, int32_t n_shares, const int64_t* r
       (bases && bases_cap < 0) || (contig_off && contig_off_cap < 1))
     return fail(c, CG_EINVAL, "bad receive or output buffers");
   Xchg X;
-  st = x_prepare(g, n_shares, read_first, rank, X);
-  std::vector<unsigned long long> sw, rw;
-  if (st == CG_OK) st = x_sizes(g, X, sw, rw);
-  long long* seg = nullptr;
-  long long* slot = nullptr;
-  const long long j0 = X.range.empty() ? 0 : X.range[2 * rank];
-  const long long count = st == CG_OK ? X.pair0[rank + 1] - X.pair0[rank] : 0;
+  st = x_count(g, n_shares, read_first, rank, false, X);
+  unsigned long long* state = nullptr;
   if (st == CG_OK) {
-    std::vector<long long> seg_h((size_t)n_shares + 1, 0);
-    for (int r = 0; r < n_shares; ++r) seg_h[r + 1] = seg_h[r] + (long long)rw[r];
-    if (4 * seg_h[n_shares] != recv_bytes)
-      st = fail(c, CG_EINVAL, "received %lld bytes, the layout needs %lld", (long long)recv_bytes, 4 * seg_h[n_shares]);
-    if (st == CG_OK) seg = (long long*)dalloc(c, (size_t)(n_shares + 1) * 8, &st);
-    if (st == CG_OK) slot = (long long*)dalloc(c, (size_t)std::max(1ll, count) * 8, &st);
-    if (st == CG_OK) {
-      cudaError_t e = cudaMemcpyAsync(seg, seg_h.data(), (size_t)(n_shares + 1) * 8, cudaMemcpyHostToDevice, c->stream);
-      if (e != cudaSuccess) st = cuda_fail(c, e, "copy segments");
-    }
-    for (int r = 0; r < n_shares && st == CG_OK; ++r) st = x_scan(g, X, j0, count, r, slot);
-    if (st == CG_OK && count > 0) {
-      cudaError_t e = cg::launch_x_rewrite(g->s, X.x, seg, slot, c->env);
-      if (e != cudaSuccess) st = cuda_fail(c, e, "exchange rewrite");
+    const int64_t words = Xchg::sum(X.recv(), n_shares), count = X.pair0()[rank + 1] - X.pair0()[rank];
+    if (4 * words != recv_bytes)
+      st = fail(c, CG_EINVAL, "received %lld bytes, the layout needs %lld", (long long)recv_bytes, (long long)(4 * words));
+    else if (count > 0) {
+      const long long cap = (count + cg::kXchgTile - 1) / cg::kXchgTile;
+      state = (unsigned long long*)dalloc(c, (size_t)n_shares * (size_t)(cap + 1) * 8, &st);
+      if (state) {
+        cudaError_t e = cg::launch_x_place(g->s, X.x, count, state, cap, c->env);
+        if (e != cudaSuccess) st = cuda_fail(c, e, "exchange placement");
+      }
     }
   }
   if (st == CG_OK) {
@@ -1713,9 +1649,8 @@ cg_status cg_emit_share_received(cg_graph* g, int32_t n_shares, const int64_t* r
       if (n_bases) *n_bases = std::max<int64_t>(0, std::min(total, t1 * tb) - t0 * tb);
     }
   }
-  dfree(c, seg);
-  dfree(c, slot);
-  x_release(c, X);
+  dfree(c, state);
+  dfree(c, X.mem);
   return st;
 }
 

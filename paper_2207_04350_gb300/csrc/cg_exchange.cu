@@ -16,8 +16,11 @@
 // share from there.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "cg_internal.cuh"
 #include "cg_lookback.cuh"
+#include "cg_stage.cuh"
 
 namespace cg {
 
@@ -37,121 +40,125 @@ __device__ __forceinline__ int owner_of(const int64_t* rf, int n, long long v) {
 struct XPiece {
   long long W0;      // first virtual word sent
   long long words;   // words sent (0 for an empty piece)
-  int owner;
 };
 
-__device__ __forceinline__ XPiece x_piece(const Scratch& s, const XchgArgs& x, long long j) {
-  XPiece p;
-  p.owner = owner_of(x.rf, x.n_shares, s.wread[j]);
+// Walk position j: words W0 .. hi / 16 + 1 of its stored bases, the spelling's
+// two-word windows.
+__device__ __forceinline__ XPiece x_piece(const Scratch& s, long long j) {
   const long long L = s.wlen[j];
-  if (L <= 0) {
-    p.W0 = 0;
-    p.words = 0;
-    return p;
-  }
   const unsigned long long w = s.wsrc[j];
   const long long src = (long long)(w & ~(1ull << 63));
   const int rc = (int)(w >> 63);
   const long long lo = rc ? src - L + 1 : src, hi = rc ? src : src + L - 1;
-  p.W0 = lo >> 4;
-  p.words = (hi >> 4) + 2 - p.W0;              // words W0 .. hi / 16 + 1: the spelling's two-word windows
+  XPiece p;
+  p.W0 = L > 0 ? lo >> 4 : 0;
+  p.words = L > 0 ? (hi >> 4) + 2 - p.W0 : 0;
   return p;
 }
 
 // The share of pair i (pairs are the shares' ranges laid end to end).
-__device__ __forceinline__ int share_of_pair(const XchgArgs& x, long long i) {
-  int lo = 0, hi = x.n_shares - 1;
+__device__ __forceinline__ int share_of_pair(const long long* pair0, int n_shares, long long i) {
+  int lo = 0, hi = n_shares - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (x.pair0[mid] <= i) lo = mid;
+    if (pair0[mid] <= i) lo = mid;
     else hi = mid - 1;
   }
   return lo;
 }
 
-__global__ void k_x_ranges(Scratch s, int n_shares, int tile_bytes, long long* range) {
-  const int p = (int)grid_tid();
-  if (p >= n_shares) return;
-  const long long total = *(const volatile long long*)&s.ctr->total_bases;
-  const long long T = (total + tile_bytes - 1) / tile_bytes;
-  const long long t0 = (long long)p * T / n_shares, t1 = (long long)(p + 1) * T / n_shares;
-  if (t0 >= t1) {
-    range[2 * p] = 1;
-    range[2 * p + 1] = 0;
-  } else {
-    range[2 * p] = s.tile_seg[t0];
-    range[2 * p + 1] = s.tile_seg[t1];
+// One block, a thread per share: the share's walk range from the tile map, the
+// first pair of each range (their number at [n_shares]), and the counts of
+// k_x_sizes cleared.
+__global__ void __launch_bounds__(kMaxParts) k_x_ranges(Scratch s, XchgArgs x, int tile_bytes) {
+  pdl_enter();
+  __shared__ long long warp_tot[kMaxParts / 32];
+  const int p = (int)threadIdx.x, lane = p & 31, warp = p >> 5;
+  long long cnt = 0;
+  if (p < x.n_shares) {
+    const long long total = *(const volatile long long*)&s.ctr->total_bases;
+    const long long T = (total + tile_bytes - 1) / tile_bytes;
+    const long long t0 = (long long)p * T / x.n_shares, t1 = (long long)(p + 1) * T / x.n_shares;
+    long long a = 1, b = 0;                              // empty
+    if (t0 < t1) {
+      a = s.tile_seg[t0];
+      b = s.tile_seg[t1];
+    }
+    x.range[2 * p] = a;
+    x.range[2 * p + 1] = b;
+    cnt = max(0ll, b - a + 1);
+    x.send_words[p] = 0ull;
+    x.recv_words[p] = 0ull;
+  }
+  long long inc = cnt;
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long v = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += v;
+  }
+  if (lane == 31) warp_tot[warp] = inc;
+  __syncthreads();
+  for (int w = 0; w < warp; ++w) inc += warp_tot[w];
+  if (p < x.n_shares) {
+    x.pair0[p] = inc - cnt;
+    if (p == x.n_shares - 1) x.pair0[x.n_shares] = inc;
   }
 }
 
-// Words to each share (send) and from each rank (recv), summed per warp over
-// the lanes with the same share or owner before one atomic each.
-__global__ void k_x_sizes(Scratch s, XchgArgs x, unsigned long long* send_words, unsigned long long* recv_words,
-                          long long n_pairs) {
-  const long long T = grid_threads();
+// Words to each share (send) and from each rank (recv): added up per block in
+// shared memory, then one addition each (one per warp and key, found by matching
+// lanes, took 45 us for 135 thousand pieces into 8 shares). With `mine` also every
+// pair's words when this rank owns its read, else 0. A warp's pieces mostly lie
+// in one share, which takes one addition for the warp.
+__global__ void __launch_bounds__(kBlock) k_x_sizes(Scratch s, XchgArgs x, uint32_t* mine) {
+  pdl_enter();
+  __shared__ unsigned long long send[kMaxParts], recv[kMaxParts];
+  __shared__ long long pair0[kMaxParts + 1];
+  __shared__ int64_t rf[kMaxParts + 1];
+  const int N = x.n_shares, lane = threadIdx.x & 31;
+  for (int i = threadIdx.x; i <= N; i += kBlock) {
+    pair0[i] = x.pair0[i];
+    rf[i] = x.rf[i];
+    if (i < N) send[i] = recv[i] = 0ull;
+  }
+  __syncthreads();
+  const long long n_pairs = pair0[N], T = grid_threads();
   const long long n_iter = (n_pairs + T - 1) / T * T;  // whole warps iterate together
   for (long long i = grid_tid(); i < n_iter; i += T) {
-    int p = -1, owner = -1;
-    unsigned long long words = 0;
+    int p = -1;
+    unsigned long long out = 0;                        // words this rank sends
     if (i < n_pairs) {
-      p = share_of_pair(x, i);
-      const long long j = x.range[2 * p] + (i - x.pair0[p]);
-      const XPiece q = x_piece(s, x, j);
-      owner = q.owner;
-      words = (unsigned long long)q.words;
+      p = share_of_pair(pair0, N, i);
+      const long long j = x.range[2 * p] + (i - pair0[p]);
+      const long long v = s.wread[j];
+      const bool own = v >= rf[x.rank] && v < rf[x.rank + 1];
+      if (own || p == x.rank) {
+        const unsigned long long words = (unsigned long long)x_piece(s, j).words;
+        if (own) out = words;
+        if (p == x.rank && words) atomicAdd(&recv[owner_of(rf, N, v)], words);
+      }
+      if (mine) mine[i] = (uint32_t)out;
     }
-    {
-      const int key = owner == x.rank ? p : -1;
-      const unsigned peers = __match_any_sync(0xffffffffu, key);
-      unsigned long long sum = 0;
-      for (unsigned m = peers; m; m &= m - 1) sum += __shfl_sync(peers, words, __ffs(m) - 1);
-      if (key >= 0 && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&send_words[key], sum);
+    const int p0 = __shfl_sync(0xffffffffu, p, 0);
+    if (__all_sync(0xffffffffu, p == p0 || p < 0)) {   // lanes past the last pair add nothing
+      for (int o = 16; o > 0; o >>= 1) out += __shfl_down_sync(0xffffffffu, out, o);
+      if (lane == 0 && out) atomicAdd(&send[p0], out);
+    } else if (out) {
+      atomicAdd(&send[p], out);
     }
-    {
-      const int key = p == x.rank ? owner : -1;
-      const unsigned peers = __match_any_sync(0xffffffffu, key);
-      unsigned long long sum = 0;
-      for (unsigned m = peers; m; m &= m - 1) sum += __shfl_sync(peers, words, __ffs(m) - 1);
-      if (key >= 0 && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&recv_words[key], sum);
-    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < N; i += kBlock) {
+    if (send[i]) atomicAdd(&x.send_words[i], send[i]);
+    if (recv[i]) atomicAdd(&x.recv_words[i], recv[i]);
   }
 }
 
-// Scan loads: the words of a piece of one share's range when its owner is `who`.
-struct XLoad {
-  Scratch s;
-  XchgArgs x;
-  long long j0;
-  int who;
-  __device__ unsigned long long operator()(long long i) const {
-    const XPiece q = x_piece(s, x, j0 + i);
-    return q.owner == who ? (unsigned long long)q.words : 0ull;
-  }
-};
-struct XStore {
-  Scratch s;
-  XchgArgs x;
-  long long j0;
-  int who;
-  long long* slot;              // slot[i] for the items owned by `who`
-  __device__ void item(long long i, unsigned long long e) const {
-    if (x_piece(s, x, j0 + i).owner == who) slot[i] = (long long)e;
-  }
-  __device__ void last(long long, unsigned long long) const {}
-};
-
-// Scan over all pairs (the shares' ranges end to end): the words of the
-// pieces this rank owns; every pair gets its exclusive prefix, so that a
-// piece's offset in its share's segment is its prefix less the prefix at the
-// share's first pair.
+// Scan over all pairs: the words of the pieces this rank owns; every pair gets
+// its exclusive prefix, which is its offset in the send buffer, as the segments
+// lie end to end in the order of the shares.
 struct XPairLoad {
-  Scratch s;
-  XchgArgs x;
-  __device__ unsigned long long operator()(long long i) const {
-    const int p = share_of_pair(x, i);
-    const XPiece q = x_piece(s, x, x.range[2 * p] + (i - x.pair0[p]));
-    return q.owner == x.rank ? (unsigned long long)q.words : 0ull;
-  }
+  const uint32_t* mine;
+  __device__ unsigned long long operator()(long long i) const { return mine[i]; }
 };
 struct XPairStore {
   long long* slot;
@@ -171,108 +178,150 @@ __device__ __forceinline__ uint32_t word_checked(const uint32_t* words, const ui
   return r;
 }
 
-// One warp per pair this rank owns: the piece's virtual words W0 .. W0 +
-// words - 1, each built from the rank's own stream (read v's bases start at
-// my_off[v - rf[rank]] there and at off[v] in the virtual stream) with one
-// funnel shift; words outside the rank's stream read as 0.
-__global__ void k_x_pack(DevGraph g, Scratch s, XchgArgs x, const uint8_t* my_packed, long long my_bytes,
-                         const int64_t* my_off, const long long* seg, const long long* slot, uint32_t* send,
-                         long long n_pairs) {
+// The pairs this rank owns, each warp looking at eight pairs: a piece's virtual
+// words W0 .. W0 + words - 1, each built from the rank's own stream (read v's
+// bases start at my_off[v - rf[rank]] there and at off[v] in the virtual stream)
+// with one funnel shift, four words per lane in flight; words outside the rank's
+// stream read as 0. A warp per pair and one word per lane at a time took 124 us
+// for 33 MB, as seven of eight warps found nothing and the others waited for one
+// round trip per 128 bytes.
+constexpr int kPackPairs = 8;
+
+__global__ void __launch_bounds__(kBlock) k_x_pack(DevGraph g, Scratch s, XchgArgs x, const uint8_t* my_packed,
+                                                   long long my_bytes, const int64_t* my_off, const uint32_t* mine,
+                                                   const long long* slot, uint32_t* send) {
+  pdl_enter();
+  const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const uint32_t* mw = reinterpret_cast<const uint32_t*>(my_packed);
-  const long long my_first = x.rf[x.rank];
-  for (long long i = grid_tid() >> 5; i < n_pairs; i += grid_threads() >> 5) {
-    const int p = share_of_pair(x, i);
-    const long long j = x.range[2 * p] + (i - x.pair0[p]);
-    const XPiece q = x_piece(s, x, j);
-    if (q.owner != x.rank || q.words == 0) continue;        // uniform across the warp
-    const long long v = s.wread[j];
-    const long long delta = my_off[v - my_first] - g.off[v];
-    uint32_t* dst = send + seg[p] + (slot[i] - slot[x.pair0[p]]);
-    for (long long k = lane; k < q.words; k += 32) {
-      const long long b = 16 * (q.W0 + k) + delta;          // the word's first base in this rank's stream
-      const long long w = b >> 4;                            // floor, also below 0
+  const long long my_first = x.rf[x.rank], n_pairs = x.pair0[x.n_shares], safe = my_bytes / 4 - 1;
+  for (long long i0 = (grid_tid() >> 5) * kPackPairs; i0 < n_pairs; i0 += (grid_threads() >> 5) * kPackPairs) {
+    const long long i = i0 + lane;
+    const bool look = lane < kPackPairs && i < n_pairs;
+    const uint32_t words = look ? mine[i] : 0u;
+    long long first = 0, at = 0;                          // first base in this rank's stream, place in the buffer
+    if (words) {
+      const int p = share_of_pair(x.pair0, x.n_shares, i);
+      const long long j = x.range[2 * p] + (i - x.pair0[p]);
+      const long long v = s.wread[j];
+      first = 16 * x_piece(s, j).W0 + my_off[v - my_first] - g.off[v];
+      at = slot[i];
+    }
+    for (unsigned m = __ballot_sync(full, words != 0); m; m &= m - 1) {   // warp-uniform
+      const int src = __ffs(m) - 1;
+      const long long b = __shfl_sync(full, first, src), w0 = b >> 4;     // floor, also below 0
       const unsigned sh = (unsigned)(2 * (b & 15));
-      dst[k] = __funnelshift_r(word_checked(mw, my_packed, my_bytes, w), word_checked(mw, my_packed, my_bytes, w + 1),
-                               sh);
+      const long long n = (long long)__shfl_sync(full, words, src);
+      uint32_t* dst = send + __shfl_sync(full, at, src);
+      long long k = lane;
+      if (w0 >= 0 && w0 + n <= safe) {
+        for (; k + 96 < n; k += 128) {
+          uint32_t lo[4], hi[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            lo[u] = __ldg(mw + w0 + k + 32 * u);
+            hi[u] = __ldg(mw + w0 + k + 32 * u + 1);
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) dst[k + 32 * u] = __funnelshift_r(lo[u], hi[u], sh);
+        }
+      }
+      for (; k < n; k += 32)
+        dst[k] = __funnelshift_r(word_checked(mw, my_packed, my_bytes, w0 + k),
+                                 word_checked(mw, my_packed, my_bytes, w0 + k + 1), sh);
     }
   }
 }
 
 // The receiver: every piece of its range, its source moved into the receive
-// buffer (16 bases per word, the piece's phase within its first word kept).
-__global__ void k_x_rewrite(Scratch s, XchgArgs x, const long long* seg, const long long* slot) {
-  const long long j0 = x.range[2 * x.rank], j1 = x.range[2 * x.rank + 1];
-  for (long long i = grid_tid(); j0 + i <= j1; i += grid_threads()) {
-    const long long j = j0 + i;
-    const XPiece q = x_piece(s, x, j);
-    if (q.words == 0) continue;
-    const unsigned long long w = s.wsrc[j];
-    const long long src = (long long)(w & ~(1ull << 63));
-    const long long at = 16 * (seg[q.owner] + slot[i]) + (src - 16 * q.W0);
-    s.wsrc[j] = (unsigned long long)at | (w & (1ull << 63));
+// buffer (16 bases per word, the piece's phase within its first word kept). The
+// blocks of row r scan the range for the words of the pieces whose reads rank r
+// holds; r's segment starts after those of the ranks before it. One launch of all
+// scans: one per source rank, each waiting for the one before, took 18 us apiece.
+__global__ void __launch_bounds__(kBlock) k_x_place(Scratch s, XchgArgs x, unsigned long long* state, long long state_cap) {
+  pdl_enter();
+  constexpr int kPer = kXchgTile / kBlock;
+  __shared__ unsigned long long tot[kBlock / 32];
+  __shared__ long long s_tile;
+  const int who = (int)blockIdx.y, tid = threadIdx.x;
+  const long long j0 = x.range[2 * x.rank], count = x.range[2 * x.rank + 1] - j0 + 1;
+  const long long tiles = (count + kXchgTile - 1) / kXchgTile;
+  if ((long long)blockIdx.x >= tiles) return;
+  const int64_t v0 = x.rf[who], v1 = x.rf[who + 1];
+  state += (long long)who * (state_cap + 1);
+  unsigned long long seg = 0;
+  for (int r = tid; r < who; r += kBlock) seg += x.recv_words[r];
+  seg = block_sum<kBlock / 32>(seg, tot);
+  for (;;) {
+    if (tid == 0) s_tile = (long long)atomicAdd(&state[state_cap], 1ull);
+    __syncthreads();
+    const long long tile = s_tile;
+    if (tile >= tiles) return;                           // block-uniform
+    const long long i0 = tile * kXchgTile + kPer * tid;
+    XPiece q[kPer];
+    unsigned long long sum = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      q[k].words = 0;
+      if (i0 + k < count) {
+        const long long v = s.wread[j0 + i0 + k];
+        if (v >= v0 && v < v1) q[k] = x_piece(s, j0 + i0 + k);
+      }
+      sum += (unsigned long long)q[k].words;
+    }
+    unsigned long long all, e = block_exclusive<kBlock / 32>(sum, tot, &all);
+    e += seg + lookback(state, tile, all, s.derr, (int)K_SCAN_OFFSETS);
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      if (q[k].words == 0) continue;
+      const unsigned long long w = s.wsrc[j0 + i0 + k];
+      const long long src = (long long)(w & ~(1ull << 63));
+      s.wsrc[j0 + i0 + k] = (unsigned long long)(16 * (long long)e + (src - 16 * q[k].W0)) | (w & (1ull << 63));
+      e += (unsigned long long)q[k].words;
+    }
+    __syncthreads();                                     // s_tile and tot are reused by the next tile
   }
 }
 
 }  // namespace
 
-cudaError_t launch_x_ranges(const Scratch& s, int n_shares, int tile_bytes, long long* range, const LaunchEnv& env) {
-  k_x_ranges<<<(n_shares + kBlock - 1) / kBlock, kBlock, 0, env.stream>>>(s, n_shares, tile_bytes, range);
+cudaError_t launch_x_sizes(const Scratch& s, const XchgArgs& x, int tile_bytes, long long n, uint32_t* mine,
+                           const LaunchEnv& env) {
+  k_x_ranges<<<1, std::max(32, (x.n_shares + 31) & ~31), 0, env.stream>>>(s, x, tile_bytes);
   mark(env, "k_x_ranges");
-  return cudaGetLastError();
-}
-
-cudaError_t launch_x_sizes(const Scratch& s, const XchgArgs& x, unsigned long long* send_words,
-                           unsigned long long* recv_words, long long n_pairs, const LaunchEnv& env) {
-  cudaMemsetAsync(send_words, 0, (size_t)x.n_shares * 8, env.stream);
-  cudaMemsetAsync(recv_words, 0, (size_t)x.n_shares * 8, env.stream);
-  if (n_pairs > 0) {
-    k_x_sizes<<<grid_for(n_pairs, env), kBlock, 0, env.stream>>>(s, x, send_words, recv_words, n_pairs);
-    mark(env, "k_x_sizes");
-  }
+  cudaError_t e = launch_k(k_x_sizes, grid_for(n, env, 4), env, true, s, x, mine);
+  if (e != cudaSuccess) return e;
+  mark(env, "k_x_sizes");
   return cudaGetLastError();
 }
 
 cudaError_t launch_x_pack(const DevGraph& g, const Scratch& s, const XchgArgs& x, const uint8_t* my_packed,
-                          long long my_bytes, const int64_t* my_off, const long long* seg, const long long* slot,
-                          uint32_t* send, long long n_pairs, const LaunchEnv& env) {
-  if (n_pairs <= 0) return cudaSuccess;
-  k_x_pack<<<grid_for(32 * n_pairs, env), kBlock, 0, env.stream>>>(g, s, x, my_packed, my_bytes, my_off, seg, slot,
-                                                                     send, n_pairs);
-  mark(env, "k_x_pack");
-  return cudaGetLastError();
-}
-
-cudaError_t launch_x_rewrite(const Scratch& s, const XchgArgs& x, const long long* seg, const long long* slot,
-                             const LaunchEnv& env) {
-  k_x_rewrite<<<env.num_sms * 4, kBlock, 0, env.stream>>>(s, x, seg, slot);
-  mark(env, "k_x_rewrite");
-  return cudaGetLastError();
-}
-
-cudaError_t launch_x_scan_pairs(const Scratch& s, const XchgArgs& x, long long n_pairs, long long* slot,
-                                unsigned long long* state, long long state_cap, const LaunchEnv& env) {
+                          long long my_bytes, const int64_t* my_off, const uint32_t* mine, long long* slot,
+                          unsigned long long* state, long long state_cap, uint32_t* send, long long n_pairs,
+                          const LaunchEnv& env) {
   if (n_pairs <= 0) return cudaSuccess;
   const long long tiles = (n_pairs + kTileItems - 1) / kTileItems;
   if (tiles > state_cap) return cudaErrorInvalidValue;
   cudaMemsetAsync(state, 0, (size_t)(state_cap + 1) * sizeof(unsigned long long), env.stream);
-  k_scan<<<scan_grid(tiles, env), kBlock, 0, env.stream>>>(XPairLoad{s, x}, XPairStore{slot}, n_pairs, state,
-                                                           state_cap, s.derr, (int)K_SCAN_OFFSETS);
+  k_scan<<<scan_grid(tiles, env), kBlock, 0, env.stream>>>(XPairLoad{mine}, XPairStore{slot}, n_pairs, state, state_cap,
+                                                           s.derr, (int)K_SCAN_OFFSETS);
   mark(env, "k_scan_exchange_pairs");
+  cudaError_t e = launch_k(k_x_pack, grid_for(32 * ((n_pairs + kPackPairs - 1) / kPackPairs), env), env, true, g, s, x,
+                           my_packed, my_bytes, my_off, mine, (const long long*)slot, send);
+  if (e != cudaSuccess) return e;
+  mark(env, "k_x_pack");
   return cudaGetLastError();
 }
 
-// One exclusive scan over a share's range [j0, j0 + count): the word offset,
-// among the pieces owned by `who`, of each piece owned by `who`.
-cudaError_t launch_x_scan(const Scratch& s, const XchgArgs& x, long long j0, long long count, int who,
-                          long long* slot, unsigned long long* state, long long state_cap, const LaunchEnv& env) {
+cudaError_t launch_x_place(const Scratch& s, const XchgArgs& x, long long count, unsigned long long* state,
+                           long long state_cap, const LaunchEnv& env) {
   if (count <= 0) return cudaSuccess;
-  const long long tiles = (count + kTileItems - 1) / kTileItems;
+  const long long tiles = (count + kXchgTile - 1) / kXchgTile;
   if (tiles > state_cap) return cudaErrorInvalidValue;
-  cudaMemsetAsync(state, 0, (size_t)(state_cap + 1) * sizeof(unsigned long long), env.stream);
-  k_scan<<<scan_grid(tiles, env), kBlock, 0, env.stream>>>(XLoad{s, x, j0, who}, XStore{s, x, j0, who, slot}, count,
-                                                           state, state_cap, s.derr, (int)K_SCAN_OFFSETS);
-  mark(env, "k_scan_exchange");
+  cudaMemsetAsync(state, 0, (size_t)x.n_shares * (size_t)(state_cap + 1) * sizeof(unsigned long long), env.stream);
+  k_x_place<<<dim3((unsigned)std::min(tiles, (long long)env.num_sms * 2), (unsigned)x.n_shares), kBlock, 0, env.stream>>>(
+      s, x, state, state_cap);
+  mark(env, "k_x_place");
   return cudaGetLastError();
 }
 

@@ -355,29 +355,27 @@ struct XchgArgs {
   const int64_t* rf;
   int n_shares;
   int rank;
-  const long long* range;       // 2 x n_shares
-  const long long* pair0;       // n_shares + 1: first pair index of each share's range
+  long long* range;             // 2 x n_shares
+  long long* pair0;             // n_shares + 1: first pair index of each share's range, then their number
+  unsigned long long* send_words;   // n_shares: words (4 bytes) this rank sends to each share
+  unsigned long long* recv_words;   // n_shares: words it receives from each rank
 };
-// share ranges from the tile map (needs the layout's counters)
-cudaError_t launch_x_ranges(const Scratch& s, int n_shares, int tile_bytes, long long* range, const LaunchEnv& env);
-// words (4 bytes) this rank sends to each share and receives from each rank
-cudaError_t launch_x_sizes(const Scratch& s, const XchgArgs& x, unsigned long long* send_words,
-                           unsigned long long* recv_words, long long n_pairs, const LaunchEnv& env);
-// one exclusive scan over a share's walk positions [j0, j0 + count): for the
-// pieces whose read `who` owns, their word offset among those pieces (slot[i])
-cudaError_t launch_x_scan(const Scratch& s, const XchgArgs& x, long long j0, long long count, int who,
-                          long long* slot, unsigned long long* state, long long state_cap, const LaunchEnv& env);
-// the sender: one exclusive scan over all pairs of the words of the pieces it
-// owns (slot[i] for every pair; a piece's offset in its share's segment is
-// slot[i] - slot[first pair of that share])
-cudaError_t launch_x_scan_pairs(const Scratch& s, const XchgArgs& x, long long n_pairs, long long* slot,
-                                unsigned long long* state, long long state_cap, const LaunchEnv& env);
+constexpr int kXchgTile = 1024;  // walk positions per tile of the receiver's scans
+// Share ranges, pairs and word counts from the tile map (needs the layout's
+// counters); n bounds the pairs. mine: nullptr, or the words of every pair whose
+// read this rank owns (else 0), n + n_shares entries.
+cudaError_t launch_x_sizes(const Scratch& s, const XchgArgs& x, int tile_bytes, long long n, uint32_t* mine,
+                           const LaunchEnv& env);
+// the sender: one exclusive scan over all pairs of `mine` (slot[i], the pair's
+// place in the send buffer), then the owned pieces' words
 cudaError_t launch_x_pack(const DevGraph& g, const Scratch& s, const XchgArgs& x, const uint8_t* my_packed,
-                          long long my_bytes, const int64_t* my_off, const long long* seg, const long long* slot,
-                          uint32_t* send, long long n_pairs, const LaunchEnv& env);
-// the receiver: every piece's source moved into the receive buffer
-cudaError_t launch_x_rewrite(const Scratch& s, const XchgArgs& x, const long long* seg, const long long* slot,
-                             const LaunchEnv& env);
+                          long long my_bytes, const int64_t* my_off, const uint32_t* mine, long long* slot,
+                          unsigned long long* state, long long state_cap, uint32_t* send, long long n_pairs,
+                          const LaunchEnv& env);
+// the receiver: the source of every piece of its range (count of them) moved into
+// the receive buffer. state: n_shares x (state_cap + 1) words.
+cudaError_t launch_x_place(const Scratch& s, const XchgArgs& x, long long count, unsigned long long* state,
+                           long long state_cap, const LaunchEnv& env);
 // Self-test of the look-back scan's bounded wait: scans `tiles` tiles of
 // zeros with `state` (tiles descriptors + the ticket word) prepared by the
 // caller; a ticket that starts at 1 withholds tile 0, so the later tiles'

@@ -104,6 +104,19 @@ def test_exchange_gives_the_oracle_stream(ctx, name, world):
         assert np.array_equal(np.concatenate(shares), want.bases), (name, world, tile)
 
 
+@pytest.mark.parametrize("world,lens,mcr", [
+    (40, (8, 40), 1),          # more shares than a warp has lanes; pieces of a word or two, a share inside one warp
+    (2, (8, 40), 1),           # more pieces per share than one tile of the receiver's scans (1,024)
+    (5, (1500, 2700), 2),      # pieces around the 128 words a warp moves at a time
+])
+def test_many_shares_and_short_pieces(ctx, world, lens, mcr):
+    G = structured(world, [700, 300] + [2, 3, 9] * 90, min_len=lens[0], max_len=lens[1], lone=3000, align=1)
+    want = oracle.run(G, min_chain_reads=mcr)
+    shares, offs, _ = _run_all(ctx, G, world, _bounds(G.n, world, 0.4), mcr)
+    assert np.array_equal(np.concatenate(shares), want.bases)
+    assert all(np.array_equal(o, want.contig_off) for o in offs)
+
+
 def test_exchange_refusals(ctx):
     import torch
     G = gen.generate("tiny-1Mb", threads=8)
