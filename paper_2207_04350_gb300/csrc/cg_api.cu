@@ -67,7 +67,6 @@ struct cg_graph {
   void* stage_reads = nullptr;
   int32_t* part_buf = nullptr;         // device copy of a host part assignment (cg_emit_part)
   int64_t part_buf_cap = 0;
-  unsigned long long* d_sum = nullptr;
   StageExec execs[12];                 // mask, chains, offsets, emission, contig_off export, 2-bit emission; then for
                                        // contigs, 2-bit contigs and a share of them (Form): offsets + emission +
                                        // export in one graph, all stages in one graph
@@ -155,6 +154,31 @@ T* galloc(cg_graph* g, size_t count, cg_status* st) {
   if (p) g->owned.push_back(p);
   return reinterpret_cast<T*>(p);
 }
+
+// Several arrays in one allocation, each 256-byte aligned: a graph's scratch is
+// some forty arrays, and an allocation call apiece, with its free, is host time
+// that every load pays (and that the workers of a server pay one at a time, in the
+// driver). take() places them and sets their pointers.
+struct Slab {
+  std::vector<std::pair<void**, size_t>> parts;
+  template <class T>
+  void add(T** p, size_t count) {
+    parts.emplace_back(const_cast<void**>(reinterpret_cast<const void* const*>(p)), count * sizeof(T));
+  }
+  bool take(cg_graph* g, cg_status* st) {
+    auto room = [](size_t b) { return ((b > 0 ? b : 16) + 255) & ~size_t(255); };
+    size_t total = 0;
+    for (auto& p : parts) total += room(p.second);
+    char* at = (char*)dalloc(g->ctx, total, st);
+    if (!at) return false;
+    g->owned.push_back(at);
+    for (auto& p : parts) {
+      *p.first = at;
+      at += room(p.second);
+    }
+    return true;
+  }
+};
 
 // Reads the context error word and the graph counters (waits for the stream).
 cg_status flush(cg_graph* g);
@@ -498,63 +522,66 @@ cg_status finish_load(cg_graph* g, uint32_t flags) {
   // scratch
   cg::Scratch& S = g->s;
   const size_t N = (size_t)(n > 0 ? n : 1), N2 = 2 * N, NW = N / 32 + 2;
-  S.branch = galloc<uint8_t>(g, N, &st);
-  S.cand = galloc<int32_t>(g, N, &st);
-  S.cidx = galloc<int32_t>(g, N, &st);
-  S.lone = galloc<int32_t>(g, N, &st);
-  S.hb_mask = galloc<unsigned>(g, NW, &st);
-  S.hb = galloc<unsigned>(g, NW, &st);
-  S.wp = galloc<unsigned>(g, NW, &st);
-  S.succ = galloc<int4>(g, N, &st);
-  S.sufin = galloc<int32_t>(g, N2, &st);
-  if (G.pre) {
-    S.preout = galloc<int32_t>(g, N2, &st);
-    S.pfirst = galloc<int32_t>(g, N, &st);
-  }
-  S.rr = galloc<int2>(g, N2, &st);
-  S.rlist = galloc<int32_t>(g, N2, &st);
-  S.hlist = galloc<int32_t>(g, N2, &st);
-  S.rec = galloc<int4>(g, N2, &st);
-  for (int b = 0; b < 2; ++b) {
-    S.pj[b] = galloc<int4>(g, N2, &st);
-    S.c_ptr[b] = galloc<int32_t>(g, N2, &st);
-    S.c_val[b] = galloc<long long>(g, N2, &st);
-  }
-  S.c_head = galloc<int32_t>(g, N2, &st);
-  S.prd = galloc<int4>(g, N, &st);
-  S.headq = galloc<int32_t>(g, N, &st);
-  S.cyc = galloc<int32_t>(g, N, &st);
-  S.qd = galloc<int32_t>(g, N, &st);
-  S.cbase = galloc<unsigned long long>(g, N + 1, &st);
-  S.wsrc = galloc<unsigned long long>(g, N, &st);
-  S.wlen = galloc<int32_t>(g, N, &st);
-  S.out_off = galloc<int64_t>(g, N + 1, &st);
-  S.wfirst = galloc<int32_t>(g, N, &st);
-  if (G.no_reads) S.wread = galloc<int32_t>(g, N, &st);
-  S.contig_off = galloc<int64_t>(g, N + 1, &st);
   // tiles of the heads bitmap: 8192 reads, more for graphs of over 16.7M reads
   // (at most 2048 tiles, as every block of the scan adds up the sums before its own)
   S.h_shift = 13;
   while ((N >> S.h_shift) >= 2048) ++S.h_shift;
   S.h_tiles = (int)((N + ((size_t)1 << S.h_shift) - 1) >> S.h_shift);
-  // the counters, and behind them the lone reads' tile sums (cleared together by the mask stage)
-  unsigned char* ctr = galloc<unsigned char>(g, sizeof(cg::Counters) + 8 * (size_t)S.h_tiles, &st);
-  S.ctr = reinterpret_cast<cg::Counters*>(ctr);
-  S.hsum_mask = ctr ? reinterpret_cast<unsigned long long*>(ctr + sizeof(cg::Counters)) : nullptr;
-  S.hsum = galloc<unsigned long long>(g, (size_t)S.h_tiles, &st);
   S.scan_tiles_cap = (int64_t)(N + cg::kPieceTile - 1) / cg::kPieceTile;
-  S.scan_state = galloc<unsigned long long>(g, (size_t)S.scan_tiles_cap + 1, &st);
-  S.tickets = galloc<unsigned long long>(g, cg::kTicketSets * cg::kTicketStride, &st);
-  g->d_sum = galloc<unsigned long long>(g, 1, &st);
+  Slab slab;
+  slab.add(&S.branch, N);
+  slab.add(&S.cand, N);
+  slab.add(&S.cidx, N);
+  slab.add(&S.lone, N);
+  slab.add(&S.hb_mask, NW);
+  slab.add(&S.hb, NW);
+  slab.add(&S.wp, NW);
+  slab.add(&S.succ, N);
+  slab.add(&S.sufin, N2);
+  if (G.pre) {
+    slab.add(&S.preout, N2);
+    slab.add(&S.pfirst, N);
+  }
+  slab.add(&S.rr, N2);
+  slab.add(&S.rlist, N2);
+  slab.add(&S.hlist, N2);
+  slab.add(&S.rec, N2);
+  for (int b = 0; b < 2; ++b) {
+    slab.add(&S.pj[b], N2);
+    slab.add(&S.c_ptr[b], N2);
+    slab.add(&S.c_val[b], N2);
+  }
+  slab.add(&S.c_head, N2);
+  slab.add(&S.prd, N);
+  slab.add(&S.headq, N);
+  slab.add(&S.cyc, N);
+  slab.add(&S.qd, N);
+  slab.add(&S.cbase, N + 1);
+  slab.add(&S.wsrc, N);
+  slab.add(&S.wlen, N);
+  slab.add(&S.out_off, N + 1);
+  slab.add(&S.wfirst, N);
+  if (G.no_reads) slab.add(&S.wread, N);
+  slab.add(&S.contig_off, N + 1);
+  slab.add(&S.scan_state, (size_t)S.scan_tiles_cap + 1);
+  slab.add(&S.hsum, (size_t)S.h_tiles);
+  slab.add(&S.tickets, cg::kTicketSets * cg::kTicketStride);
+  // the counters, and behind them the lone reads' tile sums (cleared together by
+  // the mask stage) and the sum of the read lengths
+  unsigned char* ctr = nullptr;
+  const size_t ctr_bytes = sizeof(cg::Counters) + 8 * (size_t)S.h_tiles + 8;
+  slab.add(&ctr, ctr_bytes);
+  if (!slab.take(g, &st)) return st;
+  S.ctr = reinterpret_cast<cg::Counters*>(ctr);
+  S.hsum_mask = reinterpret_cast<unsigned long long*>(ctr + sizeof(cg::Counters));
+  unsigned long long* d_sum = S.hsum_mask + S.h_tiles;
   S.small = cg::small_graph(n, G.m, G.min_chain);
   S.derr = c->derr;
-  if (st != CG_OK) return st;
-  CK(cudaMemsetAsync(S.ctr, 0, sizeof(cg::Counters) + 8 * (size_t)S.h_tiles, c->stream), "clear counters");
-  CK(cudaMemsetAsync(g->d_sum, 0, 8, c->stream), "clear sum");
+  CK(cudaMemsetAsync(ctr, 0, ctr_bytes, c->stream), "clear counters");
 
   if (!(flags & CG_NO_VALIDATE) && n > 0) CK(cg::launch_validate(G, c->derr, c->env), "validation kernels");
-  CK(cg::launch_sum_len(G, g->d_sum, c->env), "length sum");
-  CK(cudaMemcpyAsync(c->h_u64, g->d_sum, 8, cudaMemcpyDeviceToHost, c->stream), "read sum");
+  CK(cg::launch_sum_len(G, d_sum, c->env), "length sum");
+  CK(cudaMemcpyAsync(c->h_u64, d_sum, 8, cudaMemcpyDeviceToHost, c->stream), "read sum");
   st = wait_and_read(g);
   if (st != CG_OK) return st;
   if (c->fault.hit("bad_graph")) return fail(c, CG_EGRAPH, "injected: invalid string graph");
@@ -885,39 +912,51 @@ cg_status cg_load_graph(cg_ctx* c, const cg_graph_desc* d, uint32_t flags, cg_gr
     G.off = d->off;
     G.packed = d->packed;
   } else {
-    auto copy_in = [&](const void* src, size_t bytes, size_t pad) -> const void* {
-      void* p = dalloc(c, bytes + pad, &st);
-      if (!p) return nullptr;
-      g->owned.push_back(p);
+    Slab slab;
+    uint8_t* copied = nullptr;                   // the packed reads, and 16 bytes of zeros behind them
+    slab.add((const uint8_t**)&G.row_ptr, (size_t)(n + 1) * d->row_ptr_bytes);
+    slab.add(&G.col, (size_t)m);
+    slab.add(&G.code, (size_t)m);
+    if (xdrop) {
+      slab.add(&G.pre, (size_t)m);
+      slab.add(&G.post, (size_t)m);
+    } else {
+      slab.add(&G.suf, (size_t)m);
+    }
+    slab.add(&G.len, (size_t)n);
+    slab.add(&G.off, (size_t)n);
+    if (!host_reads && !no_reads) slab.add(&copied, (size_t)d->packed_bytes + 16);
+    if (!slab.take(g, &st)) return bail(st);
+    auto copy_in = [&](const void* dst, const void* src, size_t bytes) {
+      if (st != CG_OK) return;
       if (c->fault.hit("h2d")) {
         st = fail(c, CG_ECUDA, "injected: copy graph input failed");
-        return nullptr;
+        return;
       }
-      if (bytes) {
-        cudaError_t e = cudaMemcpyAsync(p, src, bytes, kind, c->stream);
-        if (e != cudaSuccess) { st = cuda_fail(c, e, "copy graph input"); return nullptr; }
-      }
-      if (pad) cudaMemsetAsync((char*)p + bytes, 0, pad, c->stream);
-      return p;
+      if (!bytes) return;
+      cudaError_t e = cudaMemcpyAsync(const_cast<void*>(dst), src, bytes, kind, c->stream);
+      if (e != cudaSuccess) st = cuda_fail(c, e, "copy graph input");
     };
-    G.row_ptr = copy_in(d->row_ptr, (size_t)(n + 1) * d->row_ptr_bytes, 0);
-    if (st == CG_OK) G.col = (const int32_t*)copy_in(d->col, (size_t)m * 4, 0);
-    if (st == CG_OK) G.code = (const uint8_t*)copy_in(d->code, (size_t)m, 0);
+    copy_in(G.row_ptr, d->row_ptr, (size_t)(n + 1) * d->row_ptr_bytes);
+    copy_in(G.col, d->col, (size_t)m * 4);
+    copy_in(G.code, d->code, (size_t)m);
     if (xdrop) {
-      if (st == CG_OK) G.pre = (const int32_t*)copy_in(d->pre, (size_t)m * 4, 0);
-      if (st == CG_OK) G.post = (const int32_t*)copy_in(d->post, (size_t)m * 4, 0);
-    } else if (st == CG_OK) {
-      G.suf = (const int32_t*)copy_in(d->suf, (size_t)m * 4, 0);
+      copy_in(G.pre, d->pre, (size_t)m * 4);
+      copy_in(G.post, d->post, (size_t)m * 4);
+    } else {
+      copy_in(G.suf, d->suf, (size_t)m * 4);
     }
-    if (st == CG_OK) G.len = (const int32_t*)copy_in(d->len, (size_t)n * 4, 0);
-    if (st == CG_OK) G.off = (const int64_t*)copy_in(d->off, (size_t)n * 8, 0);
+    copy_in(G.len, d->len, (size_t)n * 4);
+    copy_in(G.off, d->off, (size_t)n * 8);
     if (host_reads) {
       G.packed = host_packed_dev;
       G.packed_host = true;
     } else if (no_reads) {
       G.packed = nullptr;
-    } else if (st == CG_OK) {
-      G.packed = (const uint8_t*)copy_in(d->packed, (size_t)d->packed_bytes, 16);
+    } else {
+      copy_in(copied, d->packed, (size_t)d->packed_bytes);
+      if (st == CG_OK) cudaMemsetAsync(copied + d->packed_bytes, 0, 16, c->stream);
+      G.packed = copied;
     }
     if (st != CG_OK) return bail(st);
   }
@@ -983,20 +1022,31 @@ cg_status cg_load_batch(cg_ctx* c, const cg_graph_desc* d, int k, uint32_t flags
   G.min_chain = mcr <= 0 ? 2 : mcr;
   G.packed_bytes = PB[k];
   G.packed_readable = PB[k] + 16;
-  int64_t* rp = galloc<int64_t>(g, (size_t)n + 1, &st);
-  int32_t* col = galloc<int32_t>(g, (size_t)(m > 0 ? m : 1), &st);
-  uint8_t* code = galloc<uint8_t>(g, (size_t)(m > 0 ? m : 1), &st);
-  int32_t* suf = xdrop ? nullptr : galloc<int32_t>(g, (size_t)(m > 0 ? m : 1), &st);
-  int32_t* pre = xdrop ? galloc<int32_t>(g, (size_t)(m > 0 ? m : 1), &st) : nullptr;
-  int32_t* post = xdrop ? galloc<int32_t>(g, (size_t)(m > 0 ? m : 1), &st) : nullptr;
-  int32_t* len = galloc<int32_t>(g, (size_t)(n > 0 ? n : 1), &st);
-  int64_t* off = galloc<int64_t>(g, (size_t)(n > 0 ? n : 1), &st);
-  uint8_t* packed = host_reads ? nullptr : galloc<uint8_t>(g, (size_t)PB[k] + 16, &st);
-  const uint8_t** hb_base = host_reads ? galloc<const uint8_t*>(g, (size_t)k, &st) : nullptr;
-  int64_t* hb_bytes = host_reads ? galloc<int64_t>(g, (size_t)k, &st) : nullptr;
+  Slab slab;
+  int64_t *rp = nullptr, *off = nullptr, *hb_bytes = nullptr, *tab = nullptr;
+  int32_t *col = nullptr, *suf = nullptr, *pre = nullptr, *post = nullptr, *len = nullptr;
+  uint8_t *code = nullptr, *packed = nullptr;
+  const uint8_t** hb_base = nullptr;
+  slab.add(&rp, (size_t)n + 1);
+  slab.add(&col, (size_t)m);
+  slab.add(&code, (size_t)m);
+  if (xdrop) {
+    slab.add(&pre, (size_t)m);
+    slab.add(&post, (size_t)m);
+  } else {
+    slab.add(&suf, (size_t)m);
+  }
+  slab.add(&len, (size_t)n);
+  slab.add(&off, (size_t)n);
+  if (!host_reads) slab.add(&packed, (size_t)PB[k] + 16);
+  if (host_reads) {
+    slab.add(&hb_base, (size_t)k);
+    slab.add(&hb_bytes, (size_t)k);
+  }
+  slab.add(&tab, 4 * (size_t)(k + 1));
+  if (!slab.take(g, &st)) return bail(st);
   void* stage_rp = dalloc(c, (size_t)SR[k] * rpb, &st);
-  int64_t* tab = galloc<int64_t>(g, 4 * (size_t)(k + 1), &st);
-  if (st != CG_OK) { dfree(c, stage_rp); return bail(st); }
+  if (!stage_rp) return bail(st);
   g->batch_k = k;
   g->batch_R = tab;
   if (!host_reads) CK(cudaMemsetAsync(packed, 0, (size_t)PB[k] + 16, c->stream), "clear packed");

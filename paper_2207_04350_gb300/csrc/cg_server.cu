@@ -11,8 +11,10 @@
 
 #include <chrono>
 #include <condition_variable>
+#include <cstdlib>
 #include <cstring>
 #include <deque>
+#include <iterator>
 #include <map>
 #include <mutex>
 #include <new>
@@ -31,6 +33,73 @@ int64_t now_ns() {
   return std::chrono::duration_cast<std::chrono::nanoseconds>(Clock::now().time_since_epoch()).count();
 }
 
+// Host memory of one request's result. Pinned, so that the copy engines write it
+// while other batches run; the copies into pageable memory, freshly mapped and
+// zeroed for each request, were most of what a request took. Pinned blocks are
+// expensive to make, so released ones wait in the pool for the next request: at
+// most kPinnedMost bytes of them exist, waiting or in use, until the server stops,
+// and past that results lie in ordinary memory. Any thread may take and give.
+struct HostBuf {
+  void* p = nullptr;
+  size_t cap = 0;
+  bool pinned = false;
+};
+
+class HostPool {
+ public:
+  static constexpr size_t kPinnedMost = size_t(1) << 30;
+  // A block of at least `bytes`; p is null when there is no memory.
+  HostBuf take(size_t bytes) {
+    const size_t want = (bytes + 65535) & ~size_t(65535), make = want + want / 4;
+    std::vector<void*> drop;
+    bool room = false;
+    {
+      std::lock_guard<std::mutex> lk(mu_);
+      auto it = idle_.lower_bound(want);
+      if (it != idle_.end() && it->first <= 4 * want) {
+        HostBuf b{it->second, it->first, true};
+        idle_.erase(it);
+        return b;
+      }
+      // a new block; waiting ones that did not fit make room for it
+      while (held_ + make > kPinnedMost && !idle_.empty()) {
+        auto last = std::prev(idle_.end());
+        held_ -= last->first;
+        drop.push_back(last->second);
+        idle_.erase(last);
+      }
+      room = held_ + make <= kPinnedMost;
+      if (room) held_ += make;
+    }
+    for (void* p : drop) cudaFreeHost(p);
+    if (room) {
+      void* p = nullptr;
+      if (cudaHostAlloc(&p, make, cudaHostAllocPortable) == cudaSuccess) return HostBuf{p, make, true};
+      cudaGetLastError();
+      std::lock_guard<std::mutex> lk(mu_);
+      held_ -= make;
+    }
+    return HostBuf{std::malloc(bytes > 0 ? bytes : 1), bytes, false};
+  }
+  void give(HostBuf& b) {
+    if (b.p && b.pinned) {
+      std::lock_guard<std::mutex> lk(mu_);
+      idle_.emplace(b.cap, b.p);
+    } else {
+      std::free(b.p);
+    }
+    b = HostBuf{};
+  }
+  ~HostPool() {
+    for (auto& kv : idle_) cudaFreeHost(kv.second);
+  }
+
+ private:
+  std::mutex mu_;
+  std::multimap<size_t, void*> idle_;    // by size
+  size_t held_ = 0;                      // pinned bytes, waiting or in use
+};
+
 struct Request {
   uint64_t id = 0;
   cg_graph_desc desc{};
@@ -39,8 +108,9 @@ struct Request {
   int done = 0;
   cg_status status = CG_OK;
   int64_t n_contigs = 0, total_bases = 0;
-  std::vector<int64_t> contig_off;
-  std::vector<uint8_t> bases;
+  HostBuf buf;                         // contig_off (n_contigs + 1), then the bases
+  int64_t* contig_off = nullptr;
+  uint8_t* bases = nullptr;
   int batch_size = 0;
 };
 
@@ -51,6 +121,7 @@ struct cg_server {
   cg_server_opts opts{};
   std::mutex mu;
   std::condition_variable cv_work, cv_done;
+  HostPool results;                      // destroyed last: requests give their blocks back to it
   std::deque<Request*> waiting;          // submitted, not yet admitted
   std::deque<Request*> admitted;         // within the budget, not yet taken by a worker
   std::map<uint64_t, Request*> all;
@@ -197,25 +268,32 @@ cg_status run_union(cg_server* s, Worker& w, std::vector<Request*>& batch) {
       const int64_t c0 = fc[j], c1 = fc[j + 1], b0 = fb[j], b1 = fb[j + 1];
       r->n_contigs = c1 - c0;
       r->total_bases = b1 - b0;
-      r->contig_off.resize((size_t)(c1 - c0) + 1);
-      r->bases.resize((size_t)(b1 - b0));
-      if (cudaMemcpyAsync(r->contig_off.data(), wb.off + c0, (size_t)(c1 - c0 + 1) * 8, cudaMemcpyDeviceToHost,
+      const size_t off_bytes = ((size_t)(c1 - c0 + 1) * 8 + 15) & ~size_t(15);
+      r->buf = s->results.take(off_bytes + (size_t)(b1 - b0));
+      if (!r->buf.p) {
+        st = CG_ENOMEM;
+        break;
+      }
+      r->contig_off = (int64_t*)r->buf.p;
+      r->bases = (uint8_t*)r->buf.p + off_bytes;
+      if (cudaMemcpyAsync(r->contig_off, wb.off + c0, (size_t)(c1 - c0 + 1) * 8, cudaMemcpyDeviceToHost,
                           w.stream) != cudaSuccess ||
-          (b1 > b0 && cudaMemcpyAsync(r->bases.data(), wb.bases + b0, (size_t)(b1 - b0), cudaMemcpyDeviceToHost,
+          (b1 > b0 && cudaMemcpyAsync(r->bases, wb.bases + b0, (size_t)(b1 - b0), cudaMemcpyDeviceToHost,
                                       w.stream) != cudaSuccess))
         st = CG_ECUDA;
     }
     if (cudaStreamSynchronize(w.stream) != cudaSuccess) st = CG_ECUDA;
-    for (int j = 0; j < k; ++j)
-      for (int64_t& o : batch[j]->contig_off) o -= fb[j];
+    for (int j = 0; j < k && st == CG_OK; ++j)
+      for (int64_t i = 0; i <= batch[j]->n_contigs; ++i) batch[j]->contig_off[i] -= fb[j];
   }
   if (g) cg_free_graph(g);
   cudaGetLastError();
   if (st != CG_OK)
     for (Request* r : batch) {
       r->n_contigs = r->total_bases = 0;
-      r->contig_off.clear();
-      r->bases.clear();
+      r->contig_off = nullptr;
+      r->bases = nullptr;
+      s->results.give(r->buf);             // no copy is in flight: the stream was waited for
     }
   return st;
 }
@@ -391,8 +469,8 @@ cg_status cg_server_wait(cg_server* s, uint64_t id, int64_t timeout_ms, cg_serve
   res->status = r->status;
   res->n_contigs = r->n_contigs;
   res->total_bases = r->total_bases;
-  res->contig_off = r->contig_off.data();
-  res->bases = r->bases.data();
+  res->contig_off = r->contig_off;
+  res->bases = r->bases;
   res->t_submit_ns = r->t_submit;
   res->t_start_ns = r->t_start;
   res->t_done_ns = r->t_done;
@@ -405,6 +483,7 @@ cg_status cg_server_release(cg_server* s, uint64_t id) {
   std::lock_guard<std::mutex> lk(s->mu);
   auto it = s->all.find(id);
   if (it == s->all.end() || !it->second->done) return CG_EINVAL;
+  s->results.give(it->second->buf);
   delete it->second;
   s->all.erase(it);
   return CG_OK;
@@ -450,7 +529,10 @@ cg_status cg_server_stop(cg_server* s) {
     if (c) cg_destroy(c);
   for (cudaStream_t y : s->streams) cudaStreamDestroy(y);
   if (s->pool) cudaMemPoolDestroy(s->pool);
-  for (auto& kv : s->all) delete kv.second;   // every request is in `all` until released; workers drained them
+  for (auto& kv : s->all) {                   // every request is in `all` until released; workers drained them
+    s->results.give(kv.second->buf);
+    delete kv.second;
+  }
   delete s;
   return CG_OK;
 }
