@@ -498,11 +498,11 @@ cg_status spell_device(cg_graph* g, Form form, int64_t* contig_off, int64_t cont
     } else {
       if (whole) {
         CK(cg::launch_mask(g->g, g->s, c->env), "mask kernels");
-        CK(cg::launch_chains(g->g, g->s, gt(g), c->env, true), "chain kernels");
+        CK(cg::launch_chains(g->g, g->s, gt(g), c->env, true, true), "chain kernels");
         env.pdl_first = true;
       }
       if (stages) record_stage_event(c, 4);
-      CK(cg::launch_offsets(g->g, g->s, gt(g), env, user_off, user_cap), "offset kernels");
+      CK(cg::launch_offsets(g->g, g->s, gt(g), env, user_off, user_cap, whole), "offset kernels");
     }
     if (stages) record_stage_event(c, 5);
     if (timing) record_stage_event(c, 6);

@@ -37,7 +37,6 @@ namespace cg {
 
 namespace {
 
-constexpr long long kSpinLimit = 1ll << 22;   // barrier polls before giving up (~1 s with backoff)
 constexpr int kListWalkMax = 64;              // sublists a list head follows before leaving it to jumping
 constexpr int kUnresolved = -2;               // pj next field of a sublist no list walk has finished
 
@@ -47,39 +46,6 @@ __device__ __forceinline__ int sampled(int v, int ruler_log2) {
   h *= 0x85EBCA77u;
   h ^= h >> 13;
   return (h & ((1u << ruler_log2) - 1u)) == 0u;
-}
-
-// Software grid barrier for kernels launched cooperatively (all blocks
-// co-resident). Bounded: a block that waits too long records DERR_TIMEOUT and
-// every block returns false from then on.
-__device__ bool grid_sync(Counters* c, DevError* e) {
-  __shared__ int ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    ok = 1;
-    volatile unsigned* gen = &c->bar_gen;
-    unsigned g0 = *gen;
-    __threadfence();
-    unsigned arrived = atomicAdd(&c->bar_count, 1u);
-    if (arrived == gridDim.x - 1) {
-      c->bar_count = 0;
-      __threadfence();
-      atomicAdd(&c->bar_gen, 1u);
-    } else {
-      long long spins = 0;
-      while (*gen == g0) {
-        if (++spins > kSpinLimit || *(volatile int*)&e->err == DERR_TIMEOUT) {
-          set_error(e, DERR_TIMEOUT, K_JUMP, spins);
-          ok = 0;
-          break;
-        }
-        __nanosleep(spins < 64 ? 32 : 256);
-      }
-    }
-    __threadfence();
-  }
-  __syncthreads();
-  return ok != 0;
 }
 
 // -------------------------------------------------------------- validation
@@ -547,11 +513,10 @@ __global__ void k_listwalk(Scratch s) {
 // list walk gave up (very long chains). After it, for a sublist on an open
 // list: acc = oriented reads from its start to the list tail, mn = smallest
 // read id over that span, tail = the list's last oriented read. Sublists on
-// directed cycles keep next >= 0.
-__global__ void k_jump(Scratch s) {
-  pdl_enter();
+// directed cycles keep next >= 0. Returns the buffer that holds the result, or -1
+// when a barrier gave up.
+__device__ __forceinline__ int jump_lists(const Scratch& s) {
   Counters* c = s.ctr;
-  if (*(volatile unsigned*)&c->need_jump == 0) return;   // the same for every block: written by the kernel before
   unsigned R = *(volatile unsigned*)&c->n_rulers;
   for (long long i = grid_tid(); i < R; i += grid_threads()) {
     const int4 rc = s.rec[i];
@@ -561,7 +526,7 @@ __global__ void k_jump(Scratch s) {
   while ((1u << rounds) < R + 1u && rounds < 31) ++rounds;
   ++rounds;
   int cur = 0;
-  if (!grid_sync(c, s.derr)) return;
+  if (!grid_sync(c, s.derr)) return -1;
   for (int r = 0; r < rounds; ++r) {
     int nxt = cur ^ 1;
     unsigned active = 0;
@@ -580,10 +545,10 @@ __global__ void k_jump(Scratch s) {
     active = __syncthreads_or(active);
     if (threadIdx.x == 0 && active) atomicOr(&c->round_flag[r], 1u);   // zeroed by the stage
     cur = nxt;
-    if (!grid_sync(c, s.derr)) return;
+    if (!grid_sync(c, s.derr)) return -1;
     if (*(volatile unsigned*)&c->round_flag[r] == 0) break;
   }
-  if (grid_tid() == 0) c->final_buf = (unsigned)cur;
+  return cur;
 }
 
 // Per chain candidate: combine its two oriented copies. head(list of (c,0))
@@ -597,10 +562,17 @@ __global__ void k_jump(Scratch s) {
 // any store.
 constexpr int kFinalItems = 2;
 
-__global__ void k_final(DevGraph g, Scratch s) {
+// A list the list walk gave up on is jumped first, by the same (cooperative) grid:
+// a kernel of its own for that, which mostly found nothing to do, and one for the
+// closed chains (see k_heads) made the step of a 100 Mb genome 99.1 us, not 92.6.
+__global__ void __launch_bounds__(kBlock) k_final(DevGraph g, Scratch s) {
   pdl_enter();
   Counters* c = s.ctr;
-  const int fb = (int)*(volatile unsigned*)&c->final_buf;
+  int fb = 0;
+  if (*(volatile unsigned*)&c->need_jump != 0) {   // the same for every block: written by the kernel before
+    fb = jump_lists(s);
+    if (fb < 0) return;
+  }
   const long long N = *(volatile unsigned*)&c->n_cand;
   const long long n = (N + 31) & ~31ll;
   const int4* pj = s.pj[fb];
@@ -737,35 +709,11 @@ __global__ void k_sum_len(DevGraph g, unsigned long long* out) {
   if ((threadIdx.x & 31) == 0 && acc) atomicAdd(out, acc);
 }
 
-// Cooperative launch (all blocks co-resident, as the grid barrier needs);
-// expressed as a launch attribute so that stream capture can record it.
-// A cooperative launch (every block resident at once, for the grid barrier).
-// Directly after another kernel of the stage it also carries programmatic
-// dependent launch, like launch_k: no kernel signals its dependents early, so
-// the grid is launched only once every block of the kernel before it has
-// exited (the SMs are free for all of its blocks), and each block waits for
-// that kernel's completion before it touches memory.
-cudaError_t coop(const void* fn, int blocks, void** args, const LaunchEnv& env, bool chained) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(blocks);
-  cfg.blockDim = dim3(kBlock);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = env.stream;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = chained && env.pdl && !(env.marks && env.marks->on) ? 2 : 1;
-  return cudaLaunchKernelExC(&cfg, fn, args);
-}
-
 }  // namespace
 
 int coop_blocks_for_grid_kernels(int num_sms) {
   int a = 0, b = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_jump, kBlock, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_final, kBlock, 0);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_cycles, kBlock, 0);
   int per = a < b ? a : b;
   if (per > 2) per = 2;
@@ -806,7 +754,7 @@ cudaError_t launch_mask(const DevGraph& g, const Scratch& s, const LaunchEnv& en
 }
 
 cudaError_t launch_chains(const DevGraph& g, const Scratch& s, const Tuning& t, const LaunchEnv& env,
-                          bool after_mask) {
+                          bool after_mask, bool leave_cycles) {
   if (s.small) return launch_small(g, s, t, kStageChains, nullptr, 0, env, after_mask);
   // restart the chain-stage counters; the head bitmap restarts from the mask
   // stage's words (lone reads; k_succ copies them) and gains the chain heads
@@ -830,19 +778,15 @@ cudaError_t launch_chains(const DevGraph& g, const Scratch& s, const Tuning& t, 
   e = launch_k(k_listwalk, grid_for(2 * g.n, env), env, true, s);
   if (e != cudaSuccess) return e;
   mark(env, "k_listwalk");
-  Scratch sc = s;
-  void* args[] = {&sc};
-  const int coop_grid = cap(env.coop_blocks, kBlock / 2);   // up to 2 rulers or candidates per read
-  e = coop((const void*)k_jump, coop_grid, args, env, true);
-  if (e != cudaSuccess) return e;
-  mark(env, "k_jump");
   DevGraph gg = g;
-  e = launch_k(k_final, cap((long long)env.num_sms * final_resident, (long long)kBlock * kFinalItems), env, true, gg,
-               s);
+  Scratch sc = s;
+  void* args[] = {&gg, &sc};
+  e = coop((const void*)k_final, cap((long long)env.num_sms * final_resident, (long long)kBlock * kFinalItems), args, env,
+           true);
   if (e != cudaSuccess) return e;
   mark(env, "k_final");
-  void* args2[] = {&gg, &sc};
-  e = coop((const void*)k_cycles, coop_grid, args2, env, true);
+  if (leave_cycles) return cudaGetLastError();
+  e = coop((const void*)k_cycles, cap(env.coop_blocks, kBlock / 2), args, env, true);   // up to 2 candidates per read
   if (e != cudaSuccess) return e;
   mark(env, "k_cycles");
   return cudaGetLastError();

@@ -41,7 +41,6 @@ struct Counters {
   unsigned int n_cycles;
   unsigned int n_heads;        // contigs found by the chain stage
   unsigned int need_jump;      // a list had more sublists than the list walk follows
-  unsigned int final_buf;      // which pointer-jumping buffer holds the result
   unsigned int bar_count;      // grid barrier arrival counter
   unsigned int bar_gen;        // grid barrier generation
   unsigned int round_flag[64]; // "some pointer still moves" per jumping round
@@ -49,7 +48,6 @@ struct Counters {
   unsigned int n_contigs;
   unsigned int n_walk;         // walk positions = reads spelled
   unsigned int n_tiles;        // emission tiles
-  unsigned int pad;
   long long total_bases;
 };
 
@@ -258,13 +256,14 @@ cudaError_t launch_small(const DevGraph& g, const Scratch& s, const Tuning& t, i
 cudaError_t launch_validate(const DevGraph& g, DevError* derr, const LaunchEnv& env);
 cudaError_t launch_mask(const DevGraph& g, const Scratch& s, const LaunchEnv& env);
 // after_mask: the mask's launch comes right before on the stream, and has just
-// cleared the chain stage's counters too.
+// cleared the chain stage's counters too. leave_cycles: the closed chains are left
+// to a launch_offsets with_cycles that follows.
 cudaError_t launch_chains(const DevGraph& g, const Scratch& s, const Tuning& t, const LaunchEnv& env,
-                          bool after_mask = false);
+                          bool after_mask = false, bool leave_cycles = false);
 // With user_off, the piece scan also writes the caller's contig offsets
 // (user_cap entries; a capacity error and nothing written when too small).
 cudaError_t launch_offsets(const DevGraph& g, const Scratch& s, const Tuning& t, const LaunchEnv& env,
-                           int64_t* user_off = nullptr, long long user_cap = 0);
+                           int64_t* user_off = nullptr, long long user_cap = 0, bool with_cycles = false);
 // Spells the output tiles [t_begin, t_end) (all of them by default); with
 // n_shares > 1, share `share` of the tiles cut into n_shares equal runs,
 // written from out[0] on (out and cap hold that share only). after_layout: the
@@ -445,6 +444,30 @@ inline cudaError_t launch_kb(void (*kernel)(P...), int grid, int threads, const 
 template <typename... P, typename... A>
 inline cudaError_t launch_k(void (*kernel)(P...), int grid, const LaunchEnv& env, bool chained, A&&... args) {
   return launch_kb(kernel, grid, kBlock, env, chained, static_cast<A&&>(args)...);
+}
+
+// Cooperative launch (all blocks co-resident, as the grid barrier needs);
+// expressed as a launch attribute so that stream capture can record it.
+// A cooperative launch (every block resident at once, for the grid barrier).
+// Directly after another kernel of the stage it also carries programmatic
+// dependent launch, like launch_k: no kernel signals its dependents early, so
+// the grid is launched only once every block of the kernel before it has
+// exited (the SMs are free for all of its blocks), and each block waits for
+// that kernel's completion before it touches memory.
+inline cudaError_t coop(const void* fn, int blocks, void** args, const LaunchEnv& env, bool chained) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(kBlock);
+  cfg.dynamicSmemBytes = 0;
+  cfg.stream = env.stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = chained && env.pdl && !(env.marks && env.marks->on) ? 2 : 1;
+  return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
 inline int grid_for(long long n, const LaunchEnv& env, int per_sm = 8) {

@@ -47,63 +47,77 @@ namespace {
 // took 30.7 us there (95 tiles in flight at once, each waiting for the one
 // before), and 131 us on 94 thousand lone reads, whose 32 heads per word one
 // thread then loaded in turn (the whole step: 397 us before, 283 now).
-__global__ void __launch_bounds__(kBlock) k_heads(Scratch s, long long n, int64_t* user_off, long long user_cap) {
+// with_cycles: the closed chains come first, on the same (cooperative) grid, when
+// there are any.
+__global__ void __launch_bounds__(kBlock) k_heads(DevGraph g, Scratch s, bool with_cycles, int64_t* user_off,
+                                                  long long user_cap) {
   pdl_enter();
   __shared__ unsigned long long tot[2][kBlock / 32];   // the prefix's sums, the words' sums
-  for (long long i = grid_tid(); i <= s.scan_tiles_cap; i += grid_threads()) s.scan_state[i] = 0ull;   // of the piece scan
-  const int tile = (int)blockIdx.x, tid = threadIdx.x;
-  unsigned long long run = 0;
-  for (int i = tid; i < tile; i += kBlock) run += s.hsum[i];
-  const long long per = 1ll << (s.h_shift - 5);
-  const long long w_end = min((n + 31) / 32, (tile + 1) * per);
-  bool first = true;
-  for (long long wb = tile * per; wb < w_end; wb += kBlock) {
-    const long long w = wb + tid;
-    unsigned bits = w < w_end ? s.hb[w] : 0u;
-    const unsigned lone = w < w_end ? s.hb_mask[w] : 0u, chain = bits & ~lone;
-    const int32_t* const hq = s.headq + 32 * w;
-    const unsigned q0 = chain ? (unsigned)hq[__ffs(chain) - 1] : 0u;
-    unsigned long long reads = __popc(lone) + q0;
-    for (unsigned c = chain & (chain - 1); c; c &= c - 1) reads += (unsigned)hq[__ffs(c) - 1];   // rare
-    if (first) {
-      run = block_sum<kBlock / 32>(run, tot[1]);
-      first = false;
-    }
-    unsigned long long all;
-    const unsigned long long e =
-        run + block_exclusive<kBlock / 32>(((unsigned long long)__popc(bits) << kHeadShift) | reads, tot[0], &all);
-    if (w < w_end) {
-      unsigned k = (unsigned)(e >> kHeadShift);
-      unsigned long long r = e & ((1ull << kHeadShift) - 1);
-      s.wp[w] = k;
-      for (; bits; bits &= bits - 1, ++k) {            // contigs in order of their smallest read
-        const int b = __ffs(bits) - 1;
-        const unsigned q = (lone >> b) & 1u ? 1u : (b == __ffs(chain) - 1 ? q0 : (unsigned)hq[b]);
-        s.qd[k] = (int32_t)q;
-        s.cbase[k] = r;
-        r += q;
-      }
-    }
-    run += all;
-    __syncthreads();                                   // tot is reused by the next words
-  }
-  if (tile == (int)gridDim.x - 1 && tid == 0) {
+  const long long n = g.n;
+  if (with_cycles) {
     Counters* c = s.ctr;
-    unsigned C = (unsigned)(run >> kHeadShift);
-    unsigned long long W = run & ((1ull << kHeadShift) - 1);
-    if (W > (unsigned long long)n) {                   // contigs of more reads than there are: not a string graph
-      set_error(s.derr, DERR_KERNEL, K_SCAN_HEADS, (long long)W);
-      C = 0;
-      W = 0;
+    const unsigned C = *(volatile unsigned*)&c->n_cycle_reads;   // the same for every block
+    if (C > 0) {
+      close_cycles(g, s, C, grid_tid(), grid_threads(), [&] { return grid_sync(c, s.derr); });
+      if (!grid_sync(c, s.derr)) return;
     }
-    c->n_contigs = C;
-    s.cbase[C] = W;
-    c->n_walk = (unsigned)W;
-    if (C == 0) {                                      // no contigs: the piece scan has nothing to scan
-      s.contig_off[0] = 0;
-      if (user_off && user_cap >= 1) user_off[0] = 0;
-      c->total_bases = 0;
-      c->n_tiles = 0;
+  }
+  for (long long i = grid_tid(); i <= s.scan_tiles_cap; i += grid_threads()) s.scan_state[i] = 0ull;   // of the piece scan
+  const int tid = threadIdx.x;
+  for (int tile = (int)blockIdx.x; tile < s.h_tiles; tile += (int)gridDim.x) {   // block-uniform
+    unsigned long long run = 0;
+    for (int i = tid; i < tile; i += kBlock) run += s.hsum[i];
+    const long long per = 1ll << (s.h_shift - 5);
+    const long long w_end = min((n + 31) / 32, (tile + 1) * per);
+    bool first = true;
+    for (long long wb = tile * per; wb < w_end; wb += kBlock) {
+      const long long w = wb + tid;
+      unsigned bits = w < w_end ? s.hb[w] : 0u;
+      const unsigned lone = w < w_end ? s.hb_mask[w] : 0u, chain = bits & ~lone;
+      const int32_t* const hq = s.headq + 32 * w;
+      const unsigned q0 = chain ? (unsigned)hq[__ffs(chain) - 1] : 0u;
+      unsigned long long reads = __popc(lone) + q0;
+      for (unsigned c = chain & (chain - 1); c; c &= c - 1) reads += (unsigned)hq[__ffs(c) - 1];   // rare
+      if (first) {
+        run = block_sum<kBlock / 32>(run, tot[1]);
+        first = false;
+      }
+      unsigned long long all;
+      const unsigned long long e =
+          run + block_exclusive<kBlock / 32>(((unsigned long long)__popc(bits) << kHeadShift) | reads, tot[0], &all);
+      if (w < w_end) {
+        unsigned k = (unsigned)(e >> kHeadShift);
+        unsigned long long r = e & ((1ull << kHeadShift) - 1);
+        s.wp[w] = k;
+        for (; bits; bits &= bits - 1, ++k) {            // contigs in order of their smallest read
+          const int b = __ffs(bits) - 1;
+          const unsigned q = (lone >> b) & 1u ? 1u : (b == __ffs(chain) - 1 ? q0 : (unsigned)hq[b]);
+          s.qd[k] = (int32_t)q;
+          s.cbase[k] = r;
+          r += q;
+        }
+      }
+      run += all;
+      __syncthreads();                                   // tot is reused by the next words
+    }
+    if (tile == s.h_tiles - 1 && tid == 0) {
+      Counters* c = s.ctr;
+      unsigned C = (unsigned)(run >> kHeadShift);
+      unsigned long long W = run & ((1ull << kHeadShift) - 1);
+      if (W > (unsigned long long)n) {                   // contigs of more reads than there are: not a string graph
+        set_error(s.derr, DERR_KERNEL, K_SCAN_HEADS, (long long)W);
+        C = 0;
+        W = 0;
+      }
+      c->n_contigs = C;
+      s.cbase[C] = W;
+      c->n_walk = (unsigned)W;
+      if (C == 0) {                                      // no contigs: the piece scan has nothing to scan
+        s.contig_off[0] = 0;
+        if (user_off && user_cap >= 1) user_off[0] = 0;
+        c->total_bases = 0;
+        c->n_tiles = 0;
+      }
     }
   }
 }
@@ -189,14 +203,26 @@ __global__ void k_export_contig_off(Scratch s, int64_t* out, long long cap) {
 }  // namespace
 
 cudaError_t launch_offsets(const DevGraph& g, const Scratch& s, const Tuning& t, const LaunchEnv& env,
-                           int64_t* user_off, long long user_cap) {
+                           int64_t* user_off, long long user_cap, bool with_cycles) {
   if (g.n == 0) {
     k_contig_off<<<1, kBlock, 0, env.stream>>>(s);
     mark(env, "k_contig_off");
     return cudaGetLastError();
   }
   if (s.small) return launch_small(g, s, t, kStageOffsets, user_off, user_cap, env, env.pdl_first);
-  cudaError_t e = launch_k(k_heads, s.h_tiles, env, env.pdl_first, s, (long long)g.n, user_off, user_cap);
+  cudaError_t e = cudaSuccess;
+  if (with_cycles) {
+    // as many blocks as the closed chains can use, up to 2 candidates per read
+    const long long need = (g.n + kBlock / 2 - 1) / (kBlock / 2);
+    static const int heads_resident = resident_blocks(k_heads);
+    const long long most = std::min<long long>(env.coop_blocks, (long long)env.num_sms * heads_resident);
+    DevGraph gg = g;
+    Scratch sc = s;
+    void* args[] = {&gg, &sc, &with_cycles, &user_off, &user_cap};
+    e = coop((const void*)k_heads, (int)std::max(1LL, std::min(most, need)), args, env, env.pdl_first);
+  } else {
+    e = launch_k(k_heads, s.h_tiles, env, env.pdl_first, g, s, with_cycles, user_off, user_cap);
+  }
   if (e != cudaSuccess) return e;
   mark(env, "k_heads");
   static const int scatter_resident = resident_blocks(k_scatter);   // a persistent grid

@@ -11,6 +11,41 @@ namespace cg {
 
 namespace {
 
+constexpr long long kSpinLimit = 1ll << 22;   // barrier polls before giving up (~1 s with backoff)
+
+// Software grid barrier for kernels launched cooperatively (all blocks
+// co-resident). Bounded: a block that waits too long records DERR_TIMEOUT and
+// every block returns false from then on.
+__device__ bool grid_sync(Counters* c, DevError* e) {
+  __shared__ int ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ok = 1;
+    volatile unsigned* gen = &c->bar_gen;
+    unsigned g0 = *gen;
+    __threadfence();
+    unsigned arrived = atomicAdd(&c->bar_count, 1u);
+    if (arrived == gridDim.x - 1) {
+      c->bar_count = 0;
+      __threadfence();
+      atomicAdd(&c->bar_gen, 1u);
+    } else {
+      long long spins = 0;
+      while (*gen == g0) {
+        if (++spins > kSpinLimit || *(volatile int*)&e->err == DERR_TIMEOUT) {
+          set_error(e, DERR_TIMEOUT, K_JUMP, spins);
+          ok = 0;
+          break;
+        }
+        __nanosleep(spins < 64 ? 32 : 256);
+      }
+    }
+    __threadfence();
+  }
+  __syncthreads();
+  return ok != 0;
+}
+
 // Read m is the smallest read of a contig of q reads.
 __device__ __forceinline__ void mark_head(const Scratch& s, int32_t m, int32_t q) {
   atomicOr(&s.hb[m >> 5], 1u << (m & 31));
