@@ -33,7 +33,7 @@ namespace cg {
 namespace {
 
 constexpr int kTrTile = 2048;        // entries of one tile of the map: 64 words
-constexpr int kTrRows = 4;           // rows per thread of the row pass
+constexpr int kTrRows = 4;           // consecutive rows per thread of the row pass
 constexpr int kTrBatch = 120;        // listed rows a block takes at a time, at most
 constexpr int kTrAim = 960;          // entries a batch aims at: just under four per thread
 constexpr int kTrStage = 2048;       // entries of a batch staged in shared memory
@@ -51,55 +51,81 @@ __device__ __forceinline__ int32_t find_col(const int32_t* col, int32_t a, int32
   return lo < b && col[lo] == w ? lo : -1;
 }
 
+// Four consecutive values, by 16-byte loads and stores where `wide`.
+template <typename T>
+__device__ __forceinline__ void load4(const T* p, long long i, long long n, bool wide, T (&v)[4]) {
+  constexpr int kVec = 16 / sizeof(T);
+  if (wide && i + 4 <= n) {
+#pragma unroll
+    for (int k = 0; k < 4; k += kVec) {
+      const uint4 x = __ldg(reinterpret_cast<const uint4*>(p + i + k));
+      memcpy(&v[k], &x, 16);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = i + k < n ? p[i + k] : T(0);
+  }
+}
+__device__ __forceinline__ void load4_rows(const DevGraph& g, long long i, bool wide, int64_t (&v)[4]) {
+  if (g.rp64) {
+    load4(reinterpret_cast<const int64_t*>(g.row_ptr), i, g.n + 1, wide, v);
+  } else {
+    int32_t w[4];
+    load4(reinterpret_cast<const int32_t*>(g.row_ptr), i, g.n + 1, wide, w);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = w[k];
+  }
+}
+
 // Rows: offsets from 0 to m that never decrease, every read at least one base
 // long. Lists the rows with entries (read, first entry, entries), one
 // reservation per block, with a record per such read and a bit in a map of them.
-// Reads every row offset and length once, 12 B per read.
-__global__ void __launch_bounds__(kBlock, 6) k_tr_check(DevGraph g, TrBuffers t) {
+// Reads every row offset and length once, 12 B per read, four consecutive reads
+// per thread by 16-byte loads where the arrays allow.
+__global__ void __launch_bounds__(kBlock) k_tr_check(DevGraph g, TrBuffers t, bool wide_rows, bool wide_len) {
   __shared__ unsigned cnt, base;
-  const long long u0 = (long long)blockIdx.x * (kTrRows * kBlock) + threadIdx.x;
+  const long long u0 = ((long long)blockIdx.x * kBlock + threadIdx.x) * kTrRows;
   const int lane = threadIdx.x & 31;
   if (threadIdx.x == 0) cnt = 0;
   __syncthreads();
-  int64_t a[kTrRows], b[kTrRows];
-  int32_t len[kTrRows];
+  int64_t a[4] = {0, 0, 0, 0};
+  int32_t len[4] = {0, 0, 0, 0};
+  if (u0 <= g.n) load4_rows(g, u0, wide_rows, a);
+  if (u0 < g.n) load4(g.len, u0, g.n, wide_len, len);
+  int64_t next = __shfl_down_sync(0xffffffffu, a[0], 1);     // the offset after this thread's last row
+  if (lane == 31) next = u0 + 4 <= g.n ? rowp(g, u0 + 4) : 0;
+  unsigned full = 0;
 #pragma unroll
   for (int k = 0; k < kTrRows; ++k) {
-    const long long u = u0 + k * kBlock;
-    a[k] = u < g.n ? rowp(g, u) : 0;
-    b[k] = u < g.n ? rowp(g, u + 1) : 0;
-    len[k] = u < g.n ? g.len[u] : 1;
+    if (u0 + k >= g.n) continue;
+    const int64_t b = k + 1 < kTrRows ? a[k + 1 < kTrRows ? k + 1 : 0] : next;
+    if (a[k] < 0 || b < a[k] || b > g.m || len[k] < 1) set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, u0 + k);
+    else if (b > a[k]) full |= 1u << k;
   }
-  unsigned slot[kTrRows];
-#pragma unroll
-  for (int k = 0; k < kTrRows; ++k) {
-    const long long u = u0 + k * kBlock;
-    const bool ok = a[k] >= 0 && b[k] >= a[k] && b[k] <= g.m && len[k] >= 1;
-    if (!ok) {
-      set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, u);
-      b[k] = a[k];
-    }
-    const bool full = b[k] > a[k];
-    const unsigned bits = __ballot_sync(0xffffffffu, full);
-    if (lane == 0 && u < g.n) t.has[u >> 5] = bits;
-    slot[k] = 0;
-    if (bits) {                                        // warp-uniform
-      unsigned at = 0;
-      if (lane == 0) at = atomicAdd(&cnt, (unsigned)__popc(bits));
-      slot[k] = __shfl_sync(0xffffffffu, at, 0) + __popc(bits & ((1u << lane) - 1u));
-    }
+  // the bits of eight threads make a word of the map
+  unsigned bits = full << (4 * (lane & 7));
+  for (int o = 1; o < 8; o <<= 1) bits |= __shfl_xor_sync(0xffffffffu, bits, o);
+  if ((lane & 7) == 0 && u0 < g.n) t.has[u0 >> 5] = bits;
+  unsigned inc = __popc(full);
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned x = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += x;
   }
-  if (u0 == 0 && (rowp(g, 0) != 0 || rowp(g, g.n) != g.m)) set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, -1);
+  unsigned at = 0;
+  if (lane == 31 && inc) at = atomicAdd(&cnt, inc);
+  at = __shfl_sync(0xffffffffu, at, 31) + inc - __popc(full);
+  if (u0 == 0 && (a[0] != 0 || rowp(g, g.n) != g.m)) set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, -1);
   __syncthreads();
   if (threadIdx.x == 0) base = cnt ? atomicAdd(t.n_rows, cnt) : 0;
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < kTrRows; ++k) {
-    if (b[k] <= a[k]) continue;
-    const long long u = u0 + k * kBlock, at = (long long)base + slot[k];
-    if (at < t.rows_cap) t.rows[at] = make_int4((int)u, (int)a[k], (int)(b[k] - a[k]), 0);
+    if (!((full >> k) & 1u)) continue;
+    const int64_t b = k + 1 < kTrRows ? a[k + 1 < kTrRows ? k + 1 : 0] : next;
+    const long long u = u0 + k, slot = (long long)base + at++;
+    if (slot < t.rows_cap) t.rows[slot] = make_int4((int)u, (int)a[k], (int)(b - a[k]), 0);
     else set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, u);   // more rows with entries than entries: rows that overlap
-    t.info[u] = make_int4((int)a[k], 0, (int)b[k], len[k]);
+    t.info[u] = make_int4((int)a[k], 0, (int)b, len[k]);
   }
 }
 
@@ -234,7 +260,8 @@ __device__ __forceinline__ bool closes(unsigned cx, unsigned cy, unsigned cz, in
 // which are searched in place. What bounds it is the records, runs and columns
 // of the rows v, which lie at random (a sector or two each), and issuing the
 // searches, in warps whose lanes walk runs of unequal length. 3.38M entries of
-// 420 thousand rows, by events: 178 us, and 56 for the packing before it; a
+// 420 thousand rows, by events: 158 us (178 with the four searches one after
+// another), and 56 for the packing before it; a
 // thread per entry walking whole rows and searching u's row in memory took 283,
 // after 93 for mirrors found by a search of their own; eight lanes per row, four
 // rows of a warp in step, took 476, most of its lanes waiting for longer rows.
@@ -292,24 +319,28 @@ __global__ void __launch_bounds__(kBlock) k_tr_rows(DevGraph g, TrBuffers t, int
       for (; z < z1; z += 4) {
         uint2 q[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (z + k < z1) q[k] = t.ent[z + k];
+        for (int k = 0; k < 4; ++k) q[k] = z + k < z1 ? t.ent[z + k] : make_uint2(0u, 0u);
+        if (staged) {                                  // the four searches step together
+          int lo[4] = {s0, s0, s0, s0};                // the last column <= w, or the first one
+          for (int len = n; len > 1;) {
+            const int half = len >> 1;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          if (z + k >= z1) break;
-          const unsigned ez = q[k].x;
-          if (staged) {
-            int lo = s0;                               // the last column <= w, or the first one
-            for (int len = n; len > 1;) {
-              const int half = len >> 1;
-              if (key[lo + half] <= (ez | 3u)) lo += half;
-              len -= half;
-            }
-            const unsigned kx = key[lo];
-            if ((kx ^ ez) < 4u && closes(kx, cy, ez, suf[lo], sy, (int32_t)q[k].y, fuzz)) hit[lo] = 1;
-          } else {
-            const int32_t x = find_col(g.col, a, a + n, (int32_t)(ez >> 2));
-            if (x >= 0 && closes(g.code[x], cy, ez, g.suf[x], sy, (int32_t)q[k].y, fuzz)) t.trans[x] = 1;
+            for (int k = 0; k < 4; ++k)
+              if (key[lo[k] + half] <= (q[k].x | 3u)) lo[k] += half;
+            len -= half;
+          }
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const unsigned kx = key[lo[k]];
+            if (z + k < z1 && (kx ^ q[k].x) < 4u && closes(kx, cy, q[k].x, suf[lo[k]], sy, (int32_t)q[k].y, fuzz))
+              hit[lo[k]] = 1;
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            if (z + k >= z1) break;
+            const int32_t x = find_col(g.col, a, a + n, (int32_t)(q[k].x >> 2));
+            if (x >= 0 && closes(g.code[x], cy, q[k].x, g.suf[x], sy, (int32_t)q[k].y, fuzz)) t.trans[x] = 1;
           }
         }
       }
@@ -414,24 +445,44 @@ __device__ __forceinline__ unsigned kept_before(const TrBuffers& t, int64_t p) {
 }
 
 // The reduced graph: every kept entry to its place, and every row's offset;
-// nothing when the entries do not fit.
+// nothing when the entries do not fit. A thread takes four consecutive rows and
+// four consecutive entries at a time, whose words of the map are mostly the same
+// one (6.2M rows: 39 us by events, 41 with one of each). Offsets in and out may be loaded and stored by 16 bytes when `wide`.
 __global__ void __launch_bounds__(kBlock) k_tr_scatter(DevGraph g, TrBuffers t, long long cap, int64_t* row_ptr,
-                                                       int32_t* col, uint8_t* code, int32_t* suf) {
+                                                       int32_t* col, uint8_t* code, int32_t* suf, bool wide) {
   pdl_enter();
   if (failed(t.derr)) return;
   const unsigned long long total = *t.total;
   if ((long long)total > cap) return;
-  const long long most = max((long long)g.n + 1, (long long)g.m);
+  const long long most = max(((long long)g.n + 4) / 4, ((long long)g.m + 3) / 4);
   for (long long i = grid_tid(); i < most; i += grid_threads()) {
-    if (i <= g.n) {
-      const int64_t p = rowp(g, i);
-      row_ptr[i] = p < g.m ? (int64_t)kept_before(t, p) : (int64_t)total;
+    const long long r = 4 * i;
+    int64_t p[4] = {0, 0, 0, 0};
+    if (r <= g.n) load4_rows(g, r, wide, p);
+    unsigned keep = r < g.m ? (t.keep[r >> 5] >> (r & 31)) & 15u : 0u;   // of entries r .. r + 3
+    if (keep) {
+      unsigned o = kept_before(t, r);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (!((keep >> k) & 1u)) continue;
+        col[o] = g.col[r + k];
+        code[o] = g.code[r + k];
+        suf[o] = g.suf[r + k];
+        ++o;
+      }
     }
-    if (i < g.m && ((t.keep[i >> 5] >> (i & 31)) & 1u)) {
-      const unsigned o = kept_before(t, i);
-      col[o] = g.col[i];
-      code[o] = g.code[i];
-      suf[o] = g.suf[i];
+    if (r > g.n) continue;
+    int64_t o[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      o[k] = k > 0 && p[k] == p[k - 1] ? o[k - 1] : (p[k] < g.m ? (int64_t)kept_before(t, p[k]) : (int64_t)total);
+    if (wide && r + 4 <= g.n + 1) {
+      reinterpret_cast<longlong2*>(row_ptr + r)[0] = make_longlong2(o[0], o[1]);
+      reinterpret_cast<longlong2*>(row_ptr + r)[1] = make_longlong2(o[2], o[3]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (r + k <= g.n) row_ptr[r + k] = o[k];
     }
   }
 }
@@ -444,7 +495,8 @@ cudaError_t launch_transitive(const DevGraph& g, int fuzz, const TrBuffers& t, c
   cudaMemsetAsync(t.n_rows, 0, sizeof(unsigned), env.stream);
   cudaMemsetAsync(t.total, 0, sizeof(unsigned long long), env.stream);
   const long long blocks = std::max(1ll, ((long long)g.n + kTrRows * kBlock - 1) / (kTrRows * kBlock));
-  k_tr_check<<<(unsigned)blocks, kBlock, 0, env.stream>>>(g, t);
+  k_tr_check<<<(unsigned)blocks, kBlock, 0, env.stream>>>(g, t, (reinterpret_cast<uintptr_t>(g.row_ptr) & 15) == 0,
+                                                              (reinterpret_cast<uintptr_t>(g.len) & 15) == 0);
   mark(env, "k_tr_check");
   if (g.m > 0) {
     static const int pack_resident = resident_blocks(k_tr_pack), rows_resident = resident_blocks(k_tr_rows);
@@ -469,8 +521,9 @@ cudaError_t launch_transitive(const DevGraph& g, int fuzz, const TrBuffers& t, c
 
 cudaError_t launch_transitive_scatter(const DevGraph& g, const TrBuffers& t, long long cap, int64_t* row_ptr, int32_t* col,
                                       uint8_t* code, int32_t* suf, const LaunchEnv& env, bool chained) {
-  cudaError_t e = launch_k(k_tr_scatter, grid_for(std::max((long long)g.n + 1, (long long)g.m), env), env, chained, g, t,
-                           cap, row_ptr, col, code, suf);
+  const bool wide = ((reinterpret_cast<uintptr_t>(g.row_ptr) | reinterpret_cast<uintptr_t>(row_ptr)) & 15) == 0;
+  cudaError_t e = launch_k(k_tr_scatter, grid_for(std::max((long long)g.n + 4, (long long)g.m + 3) / 4, env), env, chained,
+                           g, t, cap, row_ptr, col, code, suf, wide);
   if (e != cudaSuccess) return e;
   mark(env, "k_tr_scatter");
   return cudaGetLastError();
