@@ -68,9 +68,9 @@ struct cg_graph {
   void* stage_reads = nullptr;
   int32_t* part_buf = nullptr;         // device copy of a host part assignment (cg_emit_part)
   int64_t part_buf_cap = 0;
-  StageExec execs[12];                 // mask, chains, offsets, emission, contig_off export, 2-bit emission; then for
+  StageExec execs[13];                 // mask, chains, offsets, emission, contig_off export, 2-bit emission; then for
                                        // contigs, 2-bit contigs and a share of them (Form): offsets + emission +
-                                       // export in one graph, all stages in one graph
+                                       // export in one graph, all stages in one graph; chains + per-read outputs
   int batch_k = 0;                     // graphs of a batch (0: a single graph)
   int64_t* batch_R = nullptr;          // device: first read of each graph, batch_k + 1 entries
   // a batch whose reads stay in pinned host memory: per graph its stream's
@@ -328,15 +328,18 @@ cg_status run_stage(cg_graph* g, int slot, uint64_t key, F&& launch) {
   return CG_OK;
 }
 
-cg_status run_mask(cg_graph* g) {
+// branch: the caller's device buffer for the branch bytes, or nullptr.
+cg_status run_mask(cg_graph* g, uint8_t* branch = nullptr) {
   cg_ctx* c = g->ctx;
   if (c->marks.on) {                   // a new run: per-kernel marks start over
     c->marks.n = 0;
     cudaEventRecord(c->marks.ev[0], c->stream);
   }
   StageTimer tm(c, 0);
-  cg_status st = run_stage(g, 0, 1, [&]() -> cg_status {
-    CK(cg::launch_mask(g->g, g->s, c->env), "mask kernels");
+  cg::Scratch s = g->s;
+  if (branch) s.branch = branch;       // nothing else reads the branch bytes
+  cg_status st = run_stage(g, 0, mix_key(1, (uint64_t)(uintptr_t)branch), [&]() -> cg_status {
+    CK(cg::launch_mask(g->g, s, c->env), "mask kernels");
     return CG_OK;
   });
   if (st != CG_OK) return st;
@@ -1202,9 +1205,11 @@ cg_status cg_mask_branches(cg_graph* g, uint8_t* is_branch, int mem, int64_t* n_
     return CG_OK;
   }
   g->want = 0;
-  st = run_mask(g);
+  // device bytes are written by the mask kernels themselves (they store eight at a time)
+  const bool in_place = is_branch && mem == CG_MEM_DEVICE && aligned(is_branch, 8);
+  st = run_mask(g, in_place ? is_branch : nullptr);
   if (st != CG_OK) return st;
-  if (is_branch && g->g.n > 0)
+  if (is_branch && !in_place && g->g.n > 0)
     CK(cudaMemcpyAsync(is_branch, g->s.branch, (size_t)g->g.n,
                        mem == CG_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, c->stream),
        "copy is_branch");
@@ -1232,11 +1237,27 @@ cg_status cg_chains(cg_graph* g, int32_t* chain_id, int32_t* rank, uint8_t* orie
     st = flush(g);
     if (st != CG_OK) return st;
   }
-  st = run_chains(g);
-  if (st != CG_OK) return st;
   const int64_t n = g->g.n;
   const bool want_reads = chain_id || rank || orient;
-  if (want_reads && n > 0) {
+  if (want_reads && n > 0 && mem == CG_MEM_DEVICE && defer_ok(c)) {
+    // the chain stage and the per-read outputs as one graph
+    if (g->stage < 1) {
+      st = run_mask(g);
+      if (st != CG_OK) return st;
+    }
+    uint64_t key = mix_key(mix_key((uint64_t)(uintptr_t)chain_id, (uint64_t)(uintptr_t)rank), (uint64_t)(uintptr_t)orient);
+    st = run_stage(g, 12, mix_key(key, (uint64_t)gt(g).ruler_log2), [&]() -> cg_status {
+      CK(cg::launch_chains(g->g, g->s, gt(g), c->env, false, true), "chain kernels");
+      CK(cg::launch_export_reads(g->g, g->s, chain_id, rank, orient, c->env, true), "export reads");
+      return CG_OK;
+    });
+    if (st != CG_OK) return st;
+    g->stage = 2;
+  } else {
+    st = run_chains(g);
+    if (st != CG_OK) return st;
+  }
+  if (want_reads && n > 0 && !(mem == CG_MEM_DEVICE && defer_ok(c))) {
     if (mem == CG_MEM_DEVICE) {
       CK(cg::launch_export_reads(g->g, g->s, chain_id, rank, orient, c->env), "export reads");
     } else {

@@ -272,8 +272,9 @@ cudaError_t launch_offsets(const DevGraph& g, const Scratch& s, const Tuning& t,
 cudaError_t launch_emit(const DevGraph& g, const Scratch& s, const Tuning& t, uint8_t* out, int64_t cap,
                         const LaunchEnv& env, long long t_begin = 0, long long t_end = 1ll << 62, int share = 0,
                         int n_shares = 1, bool after_layout = false);
+// after_chains: a launch_chains that left the closed chains comes right before on the stream.
 cudaError_t launch_export_reads(const DevGraph& g, const Scratch& s, int32_t* cid, int32_t* rank, uint8_t* orient,
-                                const LaunchEnv& env);
+                                const LaunchEnv& env, bool after_chains = false);
 // 2-bit spelling: cap = bytes of `out`, which must hold 16 * ceil(total / 64).
 // The 2-bit form of the tiles [t_begin, t_end) (tiles of tile_bytes bases; all by default).
 cudaError_t launch_emit2(const DevGraph& g, const Scratch& s, const Tuning& t, uint8_t* out, int64_t cap,
