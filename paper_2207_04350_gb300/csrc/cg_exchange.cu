@@ -185,7 +185,7 @@ __device__ __forceinline__ uint32_t word_checked(const uint32_t* words, const ui
 // stream read as 0. A warp per pair and one word per lane at a time took 124 us
 // for 33 MB, as seven of eight warps found nothing and the others waited for one
 // round trip per 128 bytes.
-constexpr int kPackPairs = 8;
+constexpr int kPackPairs = 8, kPackWords = 4;
 
 __global__ void __launch_bounds__(kBlock) k_x_pack(DevGraph g, Scratch s, XchgArgs x, const uint8_t* my_packed,
                                                    long long my_bytes, const int64_t* my_off, const uint32_t* mine,
@@ -215,15 +215,15 @@ __global__ void __launch_bounds__(kBlock) k_x_pack(DevGraph g, Scratch s, XchgAr
       uint32_t* dst = send + __shfl_sync(full, at, src);
       long long k = lane;
       if (w0 >= 0 && w0 + n <= safe) {
-        for (; k + 96 < n; k += 128) {
-          uint32_t lo[4], hi[4];
+        for (; k + 32 * (kPackWords - 1) < n; k += 32 * kPackWords) {
+          uint32_t lo[kPackWords], hi[kPackWords];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
+          for (int u = 0; u < kPackWords; ++u) {
             lo[u] = __ldg(mw + w0 + k + 32 * u);
             hi[u] = __ldg(mw + w0 + k + 32 * u + 1);
           }
 #pragma unroll
-          for (int u = 0; u < 4; ++u) dst[k + 32 * u] = __funnelshift_r(lo[u], hi[u], sh);
+          for (int u = 0; u < kPackWords; ++u) dst[k + 32 * u] = __funnelshift_r(lo[u], hi[u], sh);
         }
       }
       for (; k < n; k += 32)

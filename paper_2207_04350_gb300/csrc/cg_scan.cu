@@ -366,16 +366,24 @@ __global__ void k_sort_scatter(const unsigned long long* key_in, const int32_t* 
 // keys per lane are loaded before any is used. It sorts by wmax - weight, wmax
 // the largest weight there is, so that small weights (reads per contig) need
 // fewer passes than the bound kmax. Results in key[0], val[0]. The 3.1 Gb
-// graph's contigs, two passes: 40 us by events, and 100 for the ten launches above;
-// the line lies where a block's passes, growing with the contigs, meet them.
+// graph's 13,124 contigs by reads, one pass: 27 us by events (40 in two passes of
+// eight bits), and 100 for the ten launches above; by bases, three passes, 66 and
+// 136. The line lies where a block's passes, growing with the contigs, meet them.
 constexpr int kSortBlock = 1024;
 constexpr int kSortLoad = 8;
+constexpr int kSortBits = 10, kSortDigits = 1 << kSortBits;   // a digit per thread in the scan
+constexpr int kSortSmem = kSortBlock / 32 * kSortDigits * 4;  // counts per warp and digit
+
+__device__ __forceinline__ unsigned wide_digit(unsigned long long key, int pass) {
+  return (unsigned)((key >> (kSortBits * pass)) & (unsigned long long)(kSortDigits - 1));
+}
 
 __global__ void __launch_bounds__(kSortBlock) k_sort_block(const Scratch s, int C, int weight, unsigned long long kmax,
                                                            unsigned long long* key0, unsigned long long* key1,
                                                            int32_t* val0, int32_t* val1) {
   pdl_enter();
-  __shared__ unsigned cnt[kSortBlock / 32][256];
+  extern __shared__ __align__(16) unsigned char staged[];
+  unsigned(*const cnt)[kSortDigits] = reinterpret_cast<unsigned(*)[kSortDigits]>(staged);
   __shared__ unsigned long long red[kSortBlock / 32];
   __shared__ unsigned warp_tot[kSortBlock / 32];
   const unsigned full = 0xffffffffu;
@@ -393,7 +401,7 @@ __global__ void __launch_bounds__(kSortBlock) k_sort_block(const Scratch s, int 
   wmax = red[lane];
   for (int o = 16; o > 0; o >>= 1) wmax = max(wmax, __shfl_xor_sync(full, wmax, o));
   int passes = 1;
-  while (passes < 8 && (wmax >> (8 * passes)) != 0) ++passes;
+  while (passes < 7 && (wmax >> (kSortBits * passes)) != 0) ++passes;
   const int seg = (C + kSortBlock - 1) / kSortBlock * 32;          // keys per warp, whole rounds of 32
   const int i_begin = warp * seg, i_end = min(C, i_begin + seg);
   for (int pass = 0; pass < passes; ++pass) {
@@ -405,7 +413,7 @@ __global__ void __launch_bounds__(kSortBlock) k_sort_block(const Scratch s, int 
     // a key as sorted; the last pass stores kmax - weight
     auto load = [&](int i) -> unsigned long long { return pass == 0 ? wmax - weight_of(i) : kin[i]; };
     const unsigned long long shift = pass == passes - 1 ? kmax - wmax : 0ull;
-    for (int x = tid; x < (kSortBlock / 32) * 256; x += kSortBlock) (&cnt[0][0])[x] = 0;
+    for (int w = 0; w < kSortBlock / 32; ++w) cnt[w][tid] = 0;
     __syncthreads();
     for (int i0 = i_begin; i0 < i_begin + seg; i0 += 32 * kSortLoad) {   // warp-uniform
       unsigned long long k[kSortLoad];
@@ -413,14 +421,13 @@ __global__ void __launch_bounds__(kSortBlock) k_sort_block(const Scratch s, int 
       for (int j = 0; j < kSortLoad; ++j) k[j] = i0 + 32 * j + lane < i_end ? load(i0 + 32 * j + lane) : 0ull;
 #pragma unroll
       for (int j = 0; j < kSortLoad; ++j)
-        if (i0 + 32 * j + lane < i_end) atomicAdd(&cnt[warp][digit_of(k[j], pass)], 1u);
+        if (i0 + 32 * j + lane < i_end) atomicAdd(&cnt[warp][wide_digit(k[j], pass)], 1u);
     }
     __syncthreads();
     {                                                              // exclusive sums by digit, then by warp
-      const int d = tid >> 2, w0 = (tid & 3) * 8;
-      unsigned c[8], sum = 0;
-#pragma unroll
-      for (int w = 0; w < 8; ++w) { c[w] = cnt[w0 + w][d]; sum += c[w]; }
+      unsigned sum = 0;
+#pragma unroll 8
+      for (int w = 0; w < kSortBlock / 32; ++w) sum += cnt[w][tid];
       unsigned inc = sum;
       for (int o = 1; o < 32; o <<= 1) {
         const unsigned x = __shfl_up_sync(full, inc, o);
@@ -430,8 +437,12 @@ __global__ void __launch_bounds__(kSortBlock) k_sort_block(const Scratch s, int 
       __syncthreads();
       unsigned run = inc - sum;
       for (int w = 0; w < warp; ++w) run += warp_tot[w];
-#pragma unroll
-      for (int w = 0; w < 8; ++w) { cnt[w0 + w][d] = run; run += c[w]; }
+#pragma unroll 8
+      for (int w = 0; w < kSortBlock / 32; ++w) {
+        const unsigned c = cnt[w][tid];
+        cnt[w][tid] = run;
+        run += c;
+      }
     }
     __syncthreads();
     for (int i0 = i_begin; i0 < i_begin + seg; i0 += 32 * kSortLoad) {
@@ -446,12 +457,12 @@ __global__ void __launch_bounds__(kSortBlock) k_sort_block(const Scratch s, int 
 #pragma unroll
       for (int j = 0; j < kSortLoad; ++j) {
         const bool valid = i0 + 32 * j + lane < i_end;
-        const unsigned d = digit_of(k[j], pass);
+        const unsigned d = wide_digit(k[j], pass);
         // the lanes with this digit: a ballot per bit (a match instruction per 32
         // keys and phase made the two passes 48 us)
         unsigned peers = __ballot_sync(full, valid);
 #pragma unroll
-        for (int b = 0; b < 8; ++b) {
+        for (int b = 0; b < kSortBits; ++b) {
           const unsigned set = __ballot_sync(full, (d >> b) & 1u);
           peers &= (d >> b) & 1u ? set : ~set;
         }
@@ -481,11 +492,11 @@ __global__ void __launch_bounds__(kSortBlock) k_sort_block(const Scratch s, int 
 // key is above a raised key of a lower rank. When only the first is kept, the
 // least-loaded part stays so for a while, and takes every further contig that
 // leaves it below the second. The parts are those of the rule taken literally.
-// Up to 32 parts: a warp, a part per lane, ranked by P shuffles. More: a block,
 // G threads per part, each comparing its key with a G-th of the P keys in shared
-// memory. What bounds both is the chain of ranks and barriers of each round.
-// The 3.1 Gb graph's contigs into 72 parts: 121 us by events, and 776 one contig
-// at a time in one warp.
+// memory. What bounds it is the chain of ranks and barriers of each round. A few
+// parts, whose rounds would hand out that few contigs, take another way below.
+// The 3.1 Gb graph's contigs into 72 / 128 / 1024 parts: 125 / 90 / 305 us by
+// events, and 770 / 770 / 4851 one contig at a time in one warp.
 constexpr int kLptSmem = 160 << 10;  // bytes of weights and parts staged at a time; kMaxParts contigs at least
 
 // The smallest value of the lanes before this one.
@@ -520,55 +531,6 @@ __device__ __forceinline__ int lpt_run(const K* w, int n, K lowest, K second, K*
   return run;
 }
 
-// Rounds over the staged weights w[cur..n) for P <= 32, by one warp; `mine` is
-// the lane's key. Returns where it stopped: at n, or (unless `last`) with fewer
-// than P left. byrank: shared, 2 x 32 keys.
-template <typename K>
-__device__ __forceinline__ int lpt_rounds_warp(const K* w, short* to, int n, bool last, int P, int part_bits, K& mine,
-                                               K* byrank, int lane) {
-  const unsigned full = 0xffffffffu;
-  const K none = ~(K)0;
-  int cur = 0;
-  while (cur < n && (last || n - cur >= P)) {          // warp-uniform
-    const int cnt = min(P, n - cur);
-    int r = 0;
-#pragma unroll 8
-    for (int j = 0; j < P; ++j) r += __shfl_sync(full, mine, j) < mine;
-    if (lane >= P) r = 32;
-    const K raised = r < cnt ? mine + w[cur + r] : none;
-    const K top = __shfl_sync(full, mine, __ffs(__ballot_sync(full, r == cnt - 1)) - 1);
-    int kept = cnt;
-    if (__any_sync(full, r < cnt - 1 && raised < top)) {
-      if (lane < P) {
-        byrank[r] = mine;
-        byrank[32 + r] = raised;
-      }
-      __syncwarp();
-      const K old_key = lane < P ? byrank[lane] : none, new_key = lane < cnt ? byrank[32 + lane] : none;
-      const K before = warp_min_before(new_key, lane);
-      const unsigned bad = __ballot_sync(full, lane > 0 && lane < cnt && old_key > before);
-      if (bad) kept = __ffs(bad) - 1;
-      if (kept == 1) {
-        const K lowest = __shfl_sync(full, old_key, 0), second = __shfl_sync(full, old_key, 1);
-        K added;
-        const int run = lpt_run(w + cur, min(32, n - cur), lowest, second, &added, lane);
-        if (r == 0) mine += added;
-        if (lane < run) to[cur + lane] = (short)(lowest & (((K)1 << part_bits) - 1));
-        cur += run;
-        __syncwarp();
-        continue;
-      }
-      __syncwarp();
-    }
-    if (r < kept) {
-      to[cur + r] = (short)lane;
-      mine = raised;
-    }
-    cur += kept;
-  }
-  return cur;
-}
-
 template <typename K>
 __device__ __forceinline__ int keys_below(const K* keys, int n4, int g, int G, K mine);
 template <>
@@ -595,8 +557,21 @@ __device__ __forceinline__ int keys_below<unsigned long long>(const unsigned lon
   return r0 + r1;
 }
 
-// G threads per part (a power of two, 32 at most); P * G threads or more. Up to
-// 32 parts (G = 0): warp 0 assigns, the others only stage weights and write parts.
+// A barrier of the first `count` threads of the block, whole warps, and the same
+// with the or of a predicate over them.
+__device__ __forceinline__ void part_sync(int count) { asm volatile("barrier.cta.sync 1, %0;" ::"r"(count) : "memory"); }
+__device__ __forceinline__ bool part_sync_or(int count, bool x) {
+  int r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %2, 0;\n\tbarrier.cta.red.or.pred q, 1, %1, p;\n\tselp.s32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"(count), "r"((int)x)
+      : "memory");
+  return r != 0;
+}
+
+// G threads per part (a power of two): the first P * G threads, in whole warps,
+// assign, and the others only stage weights and write parts.
 template <typename K>
 __global__ void __launch_bounds__(kMaxParts) k_lpt_assign(const unsigned long long* key, const int32_t* val, long long C,
                                                           unsigned long long kmax, int P, int G, int part_bits,
@@ -612,9 +587,9 @@ __global__ void __launch_bounds__(kMaxParts) k_lpt_assign(const unsigned long lo
   const unsigned full = 0xffffffffu;
   const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, warp = tid >> 5;
   const K none = ~(K)0;
-  const int me = G ? tid / G : tid, g = G ? tid & (G - 1) : 0;
+  const int me = tid / G, g = tid & (G - 1);
   const bool act = me < P, lead = act && g == 0;
-  const int n4 = (P + 3) & ~3;
+  const int n4 = (P + 3) & ~3, A = (P * G + 31) & ~31;
   if (tid >= P && tid < n4) keys[tid] = none;              // the last vector's empty places
   K mine = act ? (K)me : none;
   for (long long c0 = 0; c0 < C;) {
@@ -624,61 +599,57 @@ __global__ void __launch_bounds__(kMaxParts) k_lpt_assign(const unsigned long lo
     __syncthreads();
     const bool last = c0 + n == C;
     int cur = 0;
-    if (G == 0) {
-      if (warp == 0) {
-        cur = lpt_rounds_warp(w, to, n, last, P, part_bits, mine, old_key, lane);
-        if (lane == 0) stop = cur;
-      }
-      __syncthreads();
-      cur = stop;
-    }
-    while (G && cur < n && (last || n - cur >= P)) {       // block-uniform
-      const int cnt = min(P, n - cur);
-      if (lead) keys[me] = mine;
-      __syncthreads();
-      int r = act ? keys_below<K>(keys, n4, g, G, mine) : 0;
-      for (int o = G >> 1; o > 0; o >>= 1) r += __shfl_xor_sync(full, r, o);
-      if (!act) r = P;
-      const K raised = r < cnt ? mine + w[cur + r] : none;
-      if (lead && r == cnt - 1) top = mine;
-      __syncthreads();
-      if (!__syncthreads_or(r < cnt - 1 && raised < top)) {
-        if (r < cnt) {
-          if (lead) to[cur + r] = (short)me;
-          mine = raised;
+    if (tid < A) {
+      while (cur < n && (last || n - cur >= P)) {            // the same for every thread of the parts
+        const int cnt = min(P, n - cur);
+        if (lead) keys[me] = mine;
+        part_sync(A);
+        int r = act ? keys_below<K>(keys, n4, g, G, mine) : 0;
+        for (int o = G >> 1; o > 0; o >>= 1) r += __shfl_xor_sync(full, r, o);
+        if (!act) r = P;
+        const K raised = r < cnt ? mine + w[cur + r] : none;
+        if (lead && r == cnt - 1) top = mine;
+        part_sync(A);
+        if (!part_sync_or(A, r < cnt - 1 && raised < top)) {
+          if (r < cnt) {
+            if (lead) to[cur + r] = (short)me;
+            mine = raised;
+          }
+          cur += cnt;
+          continue;
         }
-        cur += cnt;
-        continue;
-      }
-      if (lead) {
-        old_key[r] = mine;
-        if (r < cnt) new_key[r] = raised;
-      }
-      if (tid == 0) first_bad = cnt;
-      __syncthreads();
-      const K m = tid < cnt ? new_key[tid] : none;         // thread t now looks at rank t
-      K before = warp_min_before(m, lane);
-      if (lane == 31) warp_min[warp] = min(before, m);
-      __syncthreads();
-      for (int x = 0; x < warp; ++x) before = min(before, warp_min[x]);
-      if (tid > 0 && tid < cnt && old_key[tid] > before) atomicMin(&first_bad, tid);
-      __syncthreads();
-      const int kept = first_bad;
-      if (kept > 1) {
-        if (r < kept) {
-          if (lead) to[cur + r] = (short)me;
-          mine = raised;
+        if (lead) {
+          old_key[r] = mine;
+          if (r < cnt) new_key[r] = raised;
         }
-        cur += kept;
-      } else {                                             // every warp computes the run
-        K added;
-        const int run = lpt_run(w + cur, min(32, n - cur), old_key[0], old_key[1], &added, lane);
-        if (r == 0) mine += added;
-        if (tid < run) to[cur + tid] = (short)(old_key[0] & (((K)1 << part_bits) - 1));
-        cur += run;
+        if (tid == 0) first_bad = cnt;
+        part_sync(A);
+        const K m = tid < cnt ? new_key[tid] : none;         // thread t now looks at rank t
+        K before = warp_min_before(m, lane);
+        if (lane == 31) warp_min[warp] = min(before, m);
+        part_sync(A);
+        for (int x = 0; x < warp; ++x) before = min(before, warp_min[x]);
+        if (tid > 0 && tid < cnt && old_key[tid] > before) atomicMin(&first_bad, tid);
+        part_sync(A);
+        const int kept = first_bad;
+        if (kept > 1) {
+          if (r < kept) {
+            if (lead) to[cur + r] = (short)me;
+            mine = raised;
+          }
+          cur += kept;
+        } else {                                             // every warp computes the run
+          K added;
+          const int run = lpt_run(w + cur, min(32, n - cur), old_key[0], old_key[1], &added, lane);
+          if (r == 0) mine += added;
+          if (tid < run) to[cur + tid] = (short)(old_key[0] & (((K)1 << part_bits) - 1));
+          cur += run;
+        }
       }
+      if (tid == 0) stop = cur;
     }
     __syncthreads();
+    cur = stop;
 #pragma unroll 8
     for (int i = tid; i < cur; i += T) part[val[c0 + i]] = to[i];
     c0 += cur;
@@ -687,28 +658,140 @@ __global__ void __launch_bounds__(kMaxParts) k_lpt_assign(const unsigned long lo
   if (lead) psum[me] = (int64_t)(mine >> part_bits);
 }
 
-// As many contigs staged at a time as fit kLptSmem: all of them for most graphs,
-// since each chunk costs two round trips to memory.
-template <typename K>
-cudaError_t lpt_launch(const unsigned long long* key, const int32_t* val, long long C, unsigned long long kmax, int P, int G,
-                       int part_bits, int threads, int32_t* part, int64_t* psum, const LaunchEnv& env) {
-  const int per = (int)(sizeof(K) + sizeof(short)), most = kLptSmem / per / 64 * 64;
-  const int chunk = C < most ? (int)((C + 63) / 64 * 64) : most;
-  const size_t smem = (size_t)std::max(chunk, kMaxParts) * per;
-  cudaError_t e = cudaFuncSetAttribute(k_lpt_assign<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLptSmem);
+// Few parts, one contig after another, by one warp; the block's other warps only
+// stage weights and write parts. Up to 4 parts (M > 0) the keys are kept sorted in
+// registers, M of them: each contig goes to the first, whose raised key x moves to
+// its place among the others, R[j] = min(R[j+1], max(R[j], x)), all places at once,
+// so from one contig to the next it is an addition, a maximum and a minimum. Every
+// lane does the same, which spares the warp any exchange. With more parts a lane
+// holds one and the warp takes the smallest key with the redux unit. Either keeps
+// its keys relative to the smallest sum, which it lifts out after every few
+// contigs: no sum ever is further above the smallest than the largest weight, so
+// they fit 32 bits unless that weight (w0) is huge, and the warp then takes 64-bit
+// keys. Contigs of the 3.1 Gb graph by reads, 2 / 4 / 8 / 16 / 24 parts, by events:
+// sorted 232 / 265 / 397 us, a part per lane 330 for any number, in rounds 1612 /
+// 860 / 439 / 322 / 254 (by bases 385 at 16 and 358 at 20 parts, hence the line).
+constexpr int kLptSorted = 4, kLptWarp = 19;
+
+template <int M>
+__global__ void __launch_bounds__(kBlock) k_lpt_few(const unsigned long long* key, const int32_t* val, long long C,
+                                                    unsigned long long kmax, int P, int part_bits, int chunk,
+                                                    int32_t* part, int64_t* psum) {
+  pdl_enter();
+  extern __shared__ __align__(16) unsigned char staged[];
+  unsigned long long* const w = reinterpret_cast<unsigned long long*>(staged);
+  short* const to = reinterpret_cast<short*>(w + chunk);
+  const unsigned full = 0xffffffffu, none = ~0u;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const unsigned mask = (1u << part_bits) - 1u;
+  constexpr int kAhead = M ? 8 : 32;                   // contigs between two lifts
+  const unsigned long long w0 = kmax - key[0];         // the largest weight
+  const bool narrow = w0 < (1ull << 32) && ((kAhead + 1) * w0 + 1) << part_bits < (1ull << 32);
+  unsigned R[M ? M : 1];                               // sorted keys, or this lane's
+#pragma unroll
+  for (int j = 0; j < M; ++j) R[j] = j < P ? (unsigned)j : none;
+  if (M == 0) R[0] = lane < P ? (unsigned)lane : none;
+  unsigned long long lifted = 0;                       // taken out of every sum so far
+  unsigned long long wide = lane < P ? (unsigned long long)lane : ~0ull;   // this lane's key when 32 bits do not hold them
+  for (long long c0 = 0; c0 < C; c0 += chunk) {
+    const int n = (int)min((long long)chunk, C - c0);
+#pragma unroll 8
+    for (int i = tid; i < n; i += kBlock) w[i] = kmax - key[c0 + i];
+    __syncthreads();
+    if (tid < 32 && !narrow) {
+      for (int i0 = 0; i0 < n; i0 += 32) {
+        const unsigned long long wl = i0 + lane < n ? w[i0 + lane] << part_bits : 0ull;
+        unsigned got = 0;
+        for (int q = 0; q < min(32, n - i0); ++q) {
+          const unsigned long long wq = __shfl_sync(full, wl, q);
+          const unsigned hi = (unsigned)(wide >> 32), mhi = __reduce_min_sync(full, hi);
+          const unsigned mlo = __reduce_min_sync(full, hi == mhi ? (unsigned)wide : none);
+          const unsigned long long m = ((unsigned long long)mhi << 32) | mlo;
+          got = lane == q ? mlo & mask : got;
+          wide += wide == m ? wq : 0ull;
+        }
+        if (i0 + lane < n) to[i0 + lane] = (short)got;
+      }
+    } else if (tid < 32 && M == 0) {
+      for (int i0 = 0; i0 < n; i0 += kAhead) {
+        const unsigned wl = i0 + lane < n ? (unsigned)w[i0 + lane] << part_bits : 0u;
+        unsigned got = 0, m = 0;
+        for (int q = 0; q < min(32, n - i0); ++q) {
+          const unsigned wq = __shfl_sync(full, wl, q);
+          m = __reduce_min_sync(full, R[0]);
+          got = lane == q ? m & mask : got;
+          R[0] += R[0] == m ? wq : 0u;
+        }
+        if (i0 + lane < n) to[i0 + lane] = (short)got;
+        const unsigned lift = __reduce_min_sync(full, R[0]) & ~mask;
+        if (lane < P) R[0] -= lift;
+        lifted += lift >> part_bits;
+      }
+    } else if (tid < 32) {
+      for (int i0 = 0; i0 < n; i0 += kAhead) {
+        unsigned wi[kAhead], got[kAhead];
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) wi[k] = i0 + k < n ? (unsigned)w[i0 + k] << part_bits : 0u;
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) {             // past n a weight of 0 changes nothing
+          got[k] = R[0] & mask;
+          const unsigned x = R[0] + wi[k];
+#pragma unroll
+          for (int j = 0; j < M; ++j) {
+            const unsigned above = j + 1 < M ? R[j + 1 < M ? j + 1 : j] : none;
+            R[j] = min(above, j == 0 ? x : max(R[j], x));
+          }
+        }
+        if (lane == 0)
+#pragma unroll
+          for (int k = 0; k < kAhead; ++k)
+            if (i0 + k < n) to[i0 + k] = (short)got[k];
+        const unsigned lift = R[0] & ~mask;
+#pragma unroll
+        for (int j = 0; j < M; ++j) R[j] -= j < P ? lift : 0u;
+        lifted += lift >> part_bits;
+      }
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int i = tid; i < n; i += kBlock) part[val[c0 + i]] = to[i];
+    __syncthreads();
+  }
+  if (tid >= 32) return;
+  if (!narrow) {
+    if (lane < P) psum[lane] = (int64_t)(wide >> part_bits);
+  } else if (M == 0) {
+    if (lane < P) psum[lane] = (int64_t)(lifted + (R[0] >> part_bits));
+  } else if (lane == 0) {
+#pragma unroll
+    for (int j = 0; j < M; ++j)
+      if (j < P) psum[R[j] & mask] = (int64_t)(lifted + (R[j] >> part_bits));
+  }
+}
+
+// One block with the contigs' weights and parts staged: as many at a time as fit
+// kLptSmem, which is all of them for most graphs, since each chunk costs two round
+// trips to memory.
+int lpt_chunk(long long C, int weight_bytes) {
+  const int most = kLptSmem / (weight_bytes + (int)sizeof(short)) / 64 * 64;
+  return std::max(C < most ? (int)((C + 63) / 64 * 64) : most, kMaxParts);
+}
+
+template <typename... A, typename... B>
+cudaError_t lpt_launch(void (*kernel)(A...), int chunk, int weight_bytes, int threads, const LaunchEnv& env, B... args) {
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLptSmem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(1);
   cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
+  cfg.dynamicSmemBytes = (size_t)chunk * (size_t)(weight_bytes + (int)sizeof(short));
   cfg.stream = env.stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = env.pdl && !(env.marks && env.marks->on) ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k_lpt_assign<K>, key, val, C, kmax, P, G, part_bits, std::max(chunk, kMaxParts), part,
-                            psum);
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // One part takes every contig.
@@ -740,7 +823,10 @@ cudaError_t launch_partition(const Scratch& s, long long C, int weight, long lon
   int cur = 0;
   const bool small = C <= kSortBlockMax;
   if (small) {
-    k_sort_block<<<1, kSortBlock, 0, env.stream>>>(s, (int)C, weight, kmax, b.key[0], b.key[1], b.val[0], b.val[1]);
+    cudaError_t e = cudaFuncSetAttribute(k_sort_block, cudaFuncAttributeMaxDynamicSharedMemorySize, kSortSmem);
+    if (e != cudaSuccess) return e;
+    k_sort_block<<<1, kSortBlock, kSortSmem, env.stream>>>(s, (int)C, weight, kmax, b.key[0], b.key[1], b.val[0],
+                                                           b.val[1]);
     mark(env, "k_sort_block");
   } else {
     const long long tiles = (C + kSortTile - 1) / kSortTile;
@@ -768,14 +854,24 @@ cudaError_t launch_partition(const Scratch& s, long long C, int weight, long lon
   if (part_bits + bits > 63) return cudaErrorInvalidValue;
   // narrow: the largest key, max_weight << part_bits | (P - 1), stays below 2^32 - 1
   const bool narrow = (((unsigned long long)max_weight << part_bits) | (unsigned long long)(P - 1)) < 0xffffffffull;
-  // threads per part: as many as 512 threads allow (1024 from 129 parts on), and no more than there are vectors of keys
-  int G = 1;
-  while (2 * G * P <= (P > 128 ? kMaxParts : 512) && 2 * G <= (P + 3) / 4) G *= 2;
-  if (P <= 32) G = 0;
-  const int threads = std::max(256, (P * G + 31) & ~31);  // enough of them to stage the weights
-  cudaError_t e = narrow ? lpt_launch<uint32_t>(b.key[cur], b.val[cur], C, kmax, P, G, part_bits, threads, part, psum, env)
-                         : lpt_launch<unsigned long long>(b.key[cur], b.val[cur], C, kmax, P, G, part_bits, threads, part,
-                                                          psum, env);
+  const unsigned long long* const kk = b.key[cur];
+  const int32_t* const vv = b.val[cur];
+  cudaError_t e;
+  if (P <= kLptWarp) {
+    auto* const kernel = P <= 2 ? k_lpt_few<2> : P <= kLptSorted ? k_lpt_few<4> : k_lpt_few<0>;
+    const int chunk = lpt_chunk(C, 8);
+    e = lpt_launch(kernel, chunk, 8, kBlock, env, kk, vv, C, kmax, P, part_bits, chunk, part, psum);
+  } else {
+    // threads per part: as many as 512 threads allow, and no more than there are
+    // vectors of keys (72 parts: 161 us with one, 125 with four, 131 with eight)
+    int G = 1;
+    while (2 * G * P <= 512 && 2 * G <= (P + 3) / 4) G *= 2;
+    const int threads = std::max(256, (P * G + 31) & ~31);   // enough of them to stage the weights
+    const int chunk = lpt_chunk(C, narrow ? 4 : 8);
+    e = narrow ? lpt_launch(k_lpt_assign<uint32_t>, chunk, 4, threads, env, kk, vv, C, kmax, P, G, part_bits, chunk, part, psum)
+               : lpt_launch(k_lpt_assign<unsigned long long>, chunk, 8, threads, env, kk, vv, C, kmax, P, G, part_bits, chunk,
+                            part, psum);
+  }
   if (e != cudaSuccess) return e;
   mark(env, "k_lpt_assign");
   return cudaGetLastError();

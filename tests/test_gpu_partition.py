@@ -140,6 +140,15 @@ def test_uneven_and_many(ctx, sizes, parts):
     check(ctx, G, parts)
 
 
+def test_few_parts(ctx):
+    """Up to 19 parts one contig at a time: sorted keys, one per lane, and keys of
+    64 bits when a contig is too large for 32; 20 parts and up in rounds."""
+    G = structured(31, [400, 90, 50] + [2, 3, 5, 7, 20] * 60, lone=9)
+    check(ctx, G, list(range(1, 23)))
+    G = structured(32, [4000, 30, 20, 10, 5, 5, 3] + [2] * 40, min_len=40000, max_len=40000)
+    check(ctx, G, [2, 3, 4, 5, 8, 19, 20])
+
+
 def test_one_contig_of_80mb(ctx):
     """A contig of about 80 Mb with 3 and 32 parts: part sums beyond 32 bits
     once shifted above the part index, so the assignment takes wide keys."""
