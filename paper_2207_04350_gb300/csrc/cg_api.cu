@@ -1657,7 +1657,7 @@ cg_status cg_exchange_pack(cg_graph* g, int32_t n_shares, const int64_t* read_fi
     return fail(c, CG_EINVAL, "bad exchange buffers");
   Xchg X;
   st = x_count(g, n_shares, read_first, rank, true, X);
-  char* tmp = nullptr;
+  void* tmp = nullptr;
   if (st == CG_OK) {
     const int64_t words = Xchg::sum(X.send(), n_shares), pairs = X.pair0()[n_shares];
     if (4 * words > send_cap)
@@ -1665,12 +1665,14 @@ cg_status cg_exchange_pack(cg_graph* g, int32_t n_shares, const int64_t* read_fi
     else if (read_first[rank + 1] > read_first[rank] && !my_off)
       st = fail(c, CG_EINVAL, "my_off is required");
     else if (words > 0) {
-      const long long cap = (pairs + 2047) / 2048 + 1;   // the places of the pairs, and the scan's descriptors
-      tmp = (char*)dalloc(c, (size_t)pairs * 8 + (size_t)(cap + 1) * 8, &st);
+      // the places of the pairs, the first pairs of the chunks, and the scan's descriptors
+      const long long cap = (pairs + 2047) / 2048 + 1, chunks = (words + cg::kPackChunk - 1) / cg::kPackChunk;
+      long long* slot = (long long*)dalloc(c, (size_t)(pairs + chunks + cap + 1) * 8, &st);
+      tmp = slot;
       if (tmp) {
-        cudaError_t e = cg::launch_x_pack(g->g, g->s, X.x, my_packed, my_packed_bytes, my_off, X.mine, (long long*)tmp,
-                                          (unsigned long long*)(tmp + 8 * (size_t)pairs), cap,
-                                          reinterpret_cast<uint32_t*>(send_buf), pairs, c->env);
+        cudaError_t e = cg::launch_x_pack(g->g, g->s, X.x, my_packed, my_packed_bytes, my_off, X.mine, slot,
+                                          slot + pairs, (unsigned long long*)(slot + pairs + chunks), cap,
+                                          reinterpret_cast<uint32_t*>(send_buf), pairs, words, c->env);
         st = e != cudaSuccess ? cuda_fail(c, e, "exchange pack") : wait_and_read(g);
       }
     }

@@ -155,14 +155,21 @@ __global__ void __launch_bounds__(kBlock) k_x_sizes(Scratch s, XchgArgs x, uint3
 
 // Scan over all pairs: the words of the pieces this rank owns; every pair gets
 // its exclusive prefix, which is its offset in the send buffer, as the segments
-// lie end to end in the order of the shares.
+// lie end to end in the order of the shares. A pair that holds the first word of
+// a chunk of the buffer is that chunk's first pair.
 struct XPairLoad {
   const uint32_t* mine;
   __device__ unsigned long long operator()(long long i) const { return mine[i]; }
 };
 struct XPairStore {
+  const uint32_t* mine;
   long long* slot;
-  __device__ void item(long long i, unsigned long long e) const { slot[i] = (long long)e; }
+  long long* first;
+  __device__ void item(long long i, unsigned long long e) const {
+    slot[i] = (long long)e;
+    const unsigned long long z = e + mine[i];
+    for (unsigned long long c = (e + kPackChunk - 1) / kPackChunk; c * kPackChunk < z; ++c) first[c] = i;
+  }
   __device__ void last(long long, unsigned long long) const {}
 };
 
@@ -178,57 +185,87 @@ __device__ __forceinline__ uint32_t word_checked(const uint32_t* words, const ui
   return r;
 }
 
-// The pairs this rank owns, each warp looking at eight pairs: a piece's virtual
-// words W0 .. W0 + words - 1, each built from the rank's own stream (read v's
-// bases start at my_off[v - rf[rank]] there and at off[v] in the virtual stream)
-// with one funnel shift, four words per lane in flight; words outside the rank's
-// stream read as 0. A warp per pair and one word per lane at a time took 124 us
-// for 33 MB, as seven of eight warps found nothing and the others waited for one
-// round trip per 128 bytes.
-constexpr int kPackPairs = 8, kPackWords = 4;
+// The pairs this rank owns: a piece's virtual words W0 .. W0 + words - 1, each built
+// from the rank's own stream (read v's bases start at my_off[v - rf[rank]] there and
+// at off[v] in the virtual stream) with one funnel shift; words outside the rank's
+// stream read as 0. A warp takes kPackChunk words of the buffer at a time, whatever
+// pieces they belong to, from the chunk's first pair on: kPackWords words per lane in
+// flight, each lane stepping through the ends of the pieces in shared memory. Bound
+// by the chain of loads that finds a piece's source, then by memory: 41 MB packed
+// takes 22 us. With eight pairs per warp it took 41: reads of one rank often follow
+// one another on a walk, so that an eighth of the warps held all the words (32
+// pairs per warp: 92). Chunks of 1,024 words, or eight in flight: no faster.
+constexpr int kPackWords = 4;
 
 __global__ void __launch_bounds__(kBlock) k_x_pack(DevGraph g, Scratch s, XchgArgs x, const uint8_t* my_packed,
                                                    long long my_bytes, const int64_t* my_off, const uint32_t* mine,
-                                                   const long long* slot, uint32_t* send) {
+                                                   const long long* slot, const long long* first, uint32_t* send,
+                                                   long long n_words) {
   pdl_enter();
+  if (*(const volatile int*)&s.derr->err != 0) return;    // the scan gave up: slot and first are not whole
   const unsigned full = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
+  __shared__ long long s_end[kBlock], s_base[kBlock];     // per piece: its end in the buffer, the base that word 0 would start with
+  const int lane = threadIdx.x & 31, warp0 = threadIdx.x & ~31;
   const uint32_t* mw = reinterpret_cast<const uint32_t*>(my_packed);
   const long long my_first = x.rf[x.rank], n_pairs = x.pair0[x.n_shares], safe = my_bytes / 4 - 1;
-  for (long long i0 = (grid_tid() >> 5) * kPackPairs; i0 < n_pairs; i0 += (grid_threads() >> 5) * kPackPairs) {
-    const long long i = i0 + lane;
-    const bool look = lane < kPackPairs && i < n_pairs;
-    const uint32_t words = look ? mine[i] : 0u;
-    long long first = 0, at = 0;                          // first base in this rank's stream, place in the buffer
-    if (words) {
-      const int p = share_of_pair(x.pair0, x.n_shares, i);
-      const long long j = x.range[2 * p] + (i - x.pair0[p]);
-      const long long v = s.wread[j];
-      first = 16 * x_piece(s, j).W0 + my_off[v - my_first] - g.off[v];
-      at = slot[i];
-    }
-    for (unsigned m = __ballot_sync(full, words != 0); m; m &= m - 1) {   // warp-uniform
-      const int src = __ffs(m) - 1;
-      const long long b = __shfl_sync(full, first, src), w0 = b >> 4;     // floor, also below 0
-      const unsigned sh = (unsigned)(2 * (b & 15));
-      const long long n = (long long)__shfl_sync(full, words, src);
-      uint32_t* dst = send + __shfl_sync(full, at, src);
-      long long k = lane;
-      if (w0 >= 0 && w0 + n <= safe) {
-        for (; k + 32 * (kPackWords - 1) < n; k += 32 * kPackWords) {
-          uint32_t lo[kPackWords], hi[kPackWords];
+  const long long T = (grid_threads() >> 5) * kPackChunk;
+  for (long long a = (grid_tid() >> 5) * kPackChunk; a < n_words; a += T) {   // warp-uniform
+    const long long z = min(a + kPackChunk, n_words);
+    long long done = a;
+    for (long long i0 = first[a / kPackChunk]; done < z && i0 < n_pairs; i0 += 32) {
+      const long long i = i0 + lane, words = i < n_pairs ? (long long)mine[i] : 0ll;
+      const long long at = i < n_pairs ? slot[i] : z;
+      const bool have = words != 0 && at < z;
+      const unsigned own = __ballot_sync(full, have);
+      if (own == 0) continue;
+      bool inside = true;
+      if (have) {
+        const int p = share_of_pair(x.pair0, x.n_shares, i);
+        const long long j = x.range[2 * p] + (i - x.pair0[p]);
+        const long long v = s.wread[j];
+        const long long b = 16 * x_piece(s, j).W0 + my_off[v - my_first] - g.off[v];   // first base in this rank's stream
+        const int c = warp0 + __popc(own & ((1u << lane) - 1));
+        s_end[c] = at + words;
+        s_base[c] = b - 16 * at;
+        inside = b >= 0 && (b >> 4) + words <= safe;
+      }
+      inside = __all_sync(full, inside);
+      __syncwarp();
+      const long long end = min(z, __shfl_sync(full, at + words, 31 - __clz(own)));
+      int c = warp0;
+      long long e = s_end[c], f = s_base[c];
+      if (inside) {
+        for (long long k0 = done + lane; k0 < end; k0 += 32 * kPackWords) {
+          uint32_t lo[kPackWords], hi[kPackWords], sh[kPackWords];
 #pragma unroll
           for (int u = 0; u < kPackWords; ++u) {
-            lo[u] = __ldg(mw + w0 + k + 32 * u);
-            hi[u] = __ldg(mw + w0 + k + 32 * u + 1);
+            const long long k = min(k0 + 32 * u, end - 1);
+            while (k >= e) {
+              e = s_end[++c];
+              f = s_base[c];
+            }
+            const uint32_t* w = mw + ((f >> 4) + k);
+            sh[u] = (uint32_t)(2 * (f & 15));
+            lo[u] = __ldg(w);
+            hi[u] = __ldg(w + 1);
           }
 #pragma unroll
-          for (int u = 0; u < kPackWords; ++u) dst[k + 32 * u] = __funnelshift_r(lo[u], hi[u], sh);
+          for (int u = 0; u < kPackWords; ++u)
+            if (k0 + 32 * u < end) send[k0 + 32 * u] = __funnelshift_r(lo[u], hi[u], sh[u]);
+        }
+      } else {
+        for (long long k = done + lane; k < end; k += 32) {
+          while (k >= e) {
+            e = s_end[++c];
+            f = s_base[c];
+          }
+          const long long w = (f >> 4) + k;               // floor, also below 0
+          send[k] = __funnelshift_r(word_checked(mw, my_packed, my_bytes, w),
+                                    word_checked(mw, my_packed, my_bytes, w + 1), (unsigned)(2 * (f & 15)));
         }
       }
-      for (; k < n; k += 32)
-        dst[k] = __funnelshift_r(word_checked(mw, my_packed, my_bytes, w0 + k),
-                                 word_checked(mw, my_packed, my_bytes, w0 + k + 1), sh);
+      done = end;
+      __syncwarp();                                       // s_end and s_base are written again
     }
   }
 }
@@ -297,17 +334,18 @@ cudaError_t launch_x_sizes(const Scratch& s, const XchgArgs& x, int tile_bytes, 
 
 cudaError_t launch_x_pack(const DevGraph& g, const Scratch& s, const XchgArgs& x, const uint8_t* my_packed,
                           long long my_bytes, const int64_t* my_off, const uint32_t* mine, long long* slot,
-                          unsigned long long* state, long long state_cap, uint32_t* send, long long n_pairs,
-                          const LaunchEnv& env) {
-  if (n_pairs <= 0) return cudaSuccess;
+                          long long* first, unsigned long long* state, long long state_cap, uint32_t* send,
+                          long long n_pairs, long long n_words, const LaunchEnv& env) {
+  if (n_pairs <= 0 || n_words <= 0) return cudaSuccess;
   const long long tiles = (n_pairs + kTileItems - 1) / kTileItems;
   if (tiles > state_cap) return cudaErrorInvalidValue;
   cudaMemsetAsync(state, 0, (size_t)(state_cap + 1) * sizeof(unsigned long long), env.stream);
-  k_scan<<<scan_grid(tiles, env), kBlock, 0, env.stream>>>(XPairLoad{mine}, XPairStore{slot}, n_pairs, state, state_cap,
-                                                           s.derr, (int)K_SCAN_OFFSETS);
+  k_scan<<<scan_grid(tiles, env), kBlock, 0, env.stream>>>(XPairLoad{mine}, XPairStore{mine, slot, first}, n_pairs, state,
+                                                           state_cap, s.derr, (int)K_SCAN_OFFSETS);
   mark(env, "k_scan_exchange_pairs");
-  cudaError_t e = launch_k(k_x_pack, grid_for(32 * ((n_pairs + kPackPairs - 1) / kPackPairs), env), env, true, g, s, x,
-                           my_packed, my_bytes, my_off, mine, (const long long*)slot, send);
+  cudaError_t e = launch_k(k_x_pack, grid_for(32 * ((n_words + kPackChunk - 1) / kPackChunk), env), env, true, g, s, x,
+                           my_packed, my_bytes, my_off, mine, (const long long*)slot, (const long long*)first, send,
+                           n_words);
   if (e != cudaSuccess) return e;
   mark(env, "k_x_pack");
   return cudaGetLastError();

@@ -367,11 +367,13 @@ constexpr int kXchgTile = 1024;  // walk positions per tile of the receiver's sc
 cudaError_t launch_x_sizes(const Scratch& s, const XchgArgs& x, int tile_bytes, long long n, uint32_t* mine,
                            const LaunchEnv& env);
 // the sender: one exclusive scan over all pairs of `mine` (slot[i], the pair's
-// place in the send buffer), then the owned pieces' words
+// place in the send buffer; first[c], the pair that holds word c * kPackChunk of
+// it), then the owned pieces' n_words words
+constexpr int kPackChunk = 512;            // buffer words that a warp packs at a time
 cudaError_t launch_x_pack(const DevGraph& g, const Scratch& s, const XchgArgs& x, const uint8_t* my_packed,
                           long long my_bytes, const int64_t* my_off, const uint32_t* mine, long long* slot,
-                          unsigned long long* state, long long state_cap, uint32_t* send, long long n_pairs,
-                          const LaunchEnv& env);
+                          long long* first, unsigned long long* state, long long state_cap, uint32_t* send,
+                          long long n_pairs, long long n_words, const LaunchEnv& env);
 // the receiver: the source of every piece of its range (count of them) moved into
 // the receive buffer. state: n_shares x (state_cap + 1) words.
 cudaError_t launch_x_place(const Scratch& s, const XchgArgs& x, long long count, unsigned long long* state,

@@ -117,6 +117,18 @@ def test_many_shares_and_short_pieces(ctx, world, lens, mcr):
     assert all(np.array_equal(o, want.contig_off) for o in offs)
 
 
+@pytest.mark.parametrize("world,lens,lone", [
+    (2, (30_000, 90_000), 20),     # pieces over several chunks of 512 words that the sender's warps pack
+    (3, (8_100, 8_200), 100),      # pieces of about one chunk
+    (2, (17, 60), 40_000),         # hundreds of pieces in a chunk, most of a rank's pairs beside one another
+])
+def test_pieces_against_the_senders_chunks(ctx, world, lens, lone):
+    G = structured(world + 70, [60, 3, 2], min_len=lens[0], max_len=lens[1], lone=lone, align=1)
+    want = oracle.run(G, min_chain_reads=1)
+    shares, _, _ = _run_all(ctx, G, world, _bounds(G.n, world, 0.4), 1)
+    assert np.array_equal(np.concatenate(shares), want.bases)
+
+
 def test_exchange_refusals(ctx):
     import torch
     G = gen.generate("tiny-1Mb", threads=8)
