@@ -110,13 +110,12 @@ __global__ void __launch_bounds__(BT, 1024 / BT) k_emit(Scratch s, const uint8_t
   const int64_t* oo = s.out_off;
   const unsigned long long* ws = s.wsrc;
   const long long t_stop = min(ntiles, t_end);          // the layout tiles [t_begin, t_end) of this launch
-  // a warp spells `span` consecutive layout tiles at a time
-  const int span = emit_span(t_stop - t_begin, grid_threads() >> 5, emit_tile, tile_bytes, 8);
-  const long long n_spans = (t_stop - t_begin + span - 1) / span;
+  const SpanPlan plan(t_begin, t_stop, grid_threads() >> 5, emit_tile, tile_bytes);
+  const long long n_spans = plan.spans();
   TileQueue q(0);                                       // the warp's spans, from counters after the first
   for (; q.t < n_spans; q.next(0, n_spans)) {
     q.ask(s.tickets, 0, n_spans, lane);
-    const long long t = t_begin + q.t * span, t_hi = min(t + span, t_stop);
+    const long long t = plan.first(q.t), t_hi = plan.first(q.t + 1);
     const int lo = s.tile_seg[t], hi = s.tile_seg[t_hi];
     const long long tbase = t * (long long)tile_bytes;
     const long long tend = min(t_hi * (long long)tile_bytes, total);

@@ -186,19 +186,41 @@ inline unsigned long long emit_launch_key(const Tuning& t) {
 }
 
 // Layout tiles a spelling warp takes at once: emit_tile / layout tile when the
-// caller set one (at least one tile), else the largest span of at most 32 KiB
+// caller set one (at least one tile), else the largest span of at most max_bytes
 // that leaves every one of the launch's warps at least per_warp spans of the n
-// layout tiles (big outputs: 32 KiB spans, few per-span overheads; small ones:
-// one layout tile, enough spans to balance). The ASCII kernel asks for 8 per
-// warp; the 2-bit one, whose fixed cost per span weighs four times more
-// against its bytes, for 2.
+// layout tiles (big outputs: big spans, few per-span overheads; small ones: one
+// layout tile, enough spans to balance). The 2-bit kernel, whose fixed cost per
+// span weighs four times more against its bytes, asks for 2 per warp of at most
+// 32 KiB.
 __host__ __device__ inline int emit_span(long long n_tiles, long long warps, int emit_tile, int layout_tile,
-                                         int per_warp) {
+                                         int per_warp, int max_bytes) {
   if (emit_tile > 0) return emit_tile > layout_tile ? emit_tile / layout_tile : 1;
   int span = 1;
-  while (2 * span * layout_tile <= 32768 && n_tiles / (2 * span) >= per_warp * warps) span *= 2;
+  while (2 * span * layout_tile <= max_bytes && n_tiles / (2 * span) >= per_warp * warps) span *= 2;
   return span;
 }
+
+// The ASCII kernel's spans: of layout tiles [t0, t1), as many of emit_span's size
+// (4 per warp, at most 64 KiB) as leave one per warp, and the rest in eighths of
+// it, so that the warps end together although the spans are big. Against spans of
+// one size (8 per warp, at most 32 KiB), k_emit: 3.1 Gb 679 to 671 us, steps of
+// 500 Mb 205 to 201, 1 Gb 321 to 320, 2 Gb 560 to 555; at most 128 KiB, or 2 or 3
+// per warp, gave no more. The 2-bit kernel keeps one size: 141.3 us on 1.2 Gb with
+// or without halves at the end, 145.4 with quarters.
+struct SpanPlan {
+  long long t0, t1, big;       // big: how many spans of the full size
+  int span, small;
+  __device__ SpanPlan(long long t_begin, long long t_stop, long long warps, int emit_tile, int layout_tile)
+      : t0(t_begin), t1(max(t_begin, t_stop)) {
+    span = emit_span(t1 - t0, warps, emit_tile, layout_tile, 4, 65536);
+    small = emit_tile > 0 ? span : max(1, span / 8);
+    big = small == span ? 0 : max(0ll, (t1 - t0) / span - warps);
+  }
+  __device__ long long spans() const { return big + (t1 - t0 - big * span + small - 1) / small; }
+  __device__ long long first(long long i) const {        // first tile of span i; t1 past the last
+    return min(t1, t0 + (i < big ? i * span : big * span + (i - big) * small));
+  }
+};
 
 // CUDA events recorded after each kernel when timing is on.
 struct KernelMarks {

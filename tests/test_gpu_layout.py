@@ -5,6 +5,7 @@ more pieces than one look (256 tiles) of the look-back covers."""
 import numpy as np
 import pytest
 
+import gen
 import oracle
 from paper_2207_04350_gb300 import cg
 from tests._gpu import assert_parity, run_gpu
@@ -44,3 +45,26 @@ def test_heads_in_one_word(ctx):
     for mcr in (1, 2):
         assert_parity(run_gpu(ctx, G, min_chain_reads=mcr), oracle.run(G, min_chain_reads=mcr))
     assert np.count_nonzero(oracle.run(G).contig_off) == 3000
+
+
+@pytest.mark.parametrize("mb", [25, 90, 170])
+def test_spelling_spans(mb):
+    """Spans of 2, 8 and 16 tiles (on 608 warps) with smaller ones at the end,
+    whole and in shares that start at any tile."""
+    import torch
+    G = gen.generate(dict(gen.WORKLOADS["genome-3.1Gb"](), genome_len=mb * 1_000_000), threads=8)
+    want = oracle.run(G)
+    c = cg.cg_create(0)
+    try:
+        cg.cg_set_tuning(c, emit_blocks_per_sm=1, emit_block_threads=128)
+        assert_parity(run_gpu(c, G, inputs="device", outputs="device"), want)
+        g = cg.cg_load_graph(c, G)
+        for share in range(3):
+            first, n = cg.cg_emit_share(g, share, 3)
+            out = torch.full(((n + 15) // 16 * 16 + 16,), 7, dtype=torch.uint8, device="cuda")
+            cg.cg_emit_share(g, share, 3, None, out)
+            out = out.cpu().numpy()
+            assert np.array_equal(out[:n], want.bases[first:first + n]) and (out[n:] == 7).all()
+        g.close()
+    finally:
+        c.close()
