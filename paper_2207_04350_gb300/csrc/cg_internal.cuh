@@ -347,7 +347,7 @@ struct TrBuffers {
   int4* info;                  // n, set for rows with entries: first entry, first of the second run, end, read length
   unsigned* has;               // n bits: the read has entries
   uint2* ent;                  // m: each row in two runs by the end its entries leave through, (column << 2 | code, suffix)
-  uint8_t* trans;              // m: entry is transitive
+  uint8_t* trans;              // m: entry is transitive | code << 1
   int32_t* mir;                // m: the entry's mirror
   unsigned* keep;              // transitive_tiles(m) x 64 words: a bit per kept entry (its pair is not transitive)
   unsigned* before;            // per word: the kept entries before it in its tile

@@ -35,8 +35,10 @@ namespace {
 constexpr int kTrTile = 2048;        // entries of one tile of the map: 64 words
 constexpr int kTrRows = 4;           // consecutive rows per thread of the row pass
 constexpr int kTrBatch = 120;        // listed rows a block takes at a time, at most
-constexpr int kTrAim = 960;          // entries a batch aims at: just under four per thread
-constexpr int kTrStage = 2048;       // entries of a batch staged in shared memory
+constexpr int kTrAim = 960;          // entries a batch of the packing aims at: just under four per thread
+constexpr int kTrStage = 2048;       // entries of such a batch that are ranked in shared memory
+constexpr int kTrAimRows = 720;      // the same for the walks, just under three per thread: the less shared
+constexpr int kTrHold = 1536;        // memory the blocks of an SM hold, the more cache the random rows have
 
 __device__ __forceinline__ bool failed(const DevError* e) { return *(const volatile int*)&e->err != 0; }
 
@@ -164,9 +166,9 @@ __device__ __forceinline__ int find_row(const int4* row, int i) {
   return j;
 }
 
-// Rows per batch: as many as hold about kTrAim entries.
-__device__ __forceinline__ int batch_rows(long long m, long long R) {
-  return (int)max(1ll, min((long long)kTrBatch, kTrAim * R / max(m, 1ll)));
+// Rows per batch: as many as hold about `aim` entries.
+__device__ __forceinline__ int batch_rows(long long m, long long R, int aim) {
+  return (int)max(1ll, min((long long)kTrBatch, aim * R / max(m, 1ll)));
 }
 
 // Entries: columns in range, increasing in the row, not the row's own read and a
@@ -183,7 +185,7 @@ __global__ void __launch_bounds__(kBlock) k_tr_pack(DevGraph g, TrBuffers t) {
   if (__syncthreads_or(failed(t.derr))) return;
   const int tid = threadIdx.x, lane = tid & 31;
   const long long R = *t.n_rows;
-  const int rows = batch_rows(g.m, R);
+  const int rows = batch_rows(g.m, R, kTrAim);
   for (long long b0 = (long long)blockIdx.x * rows; b0 < R; b0 += (long long)gridDim.x * rows) {
     const int total = load_batch(t, b0, rows, R, row, warp_tot);
     constexpr int kPer = kTrStage / kBlock;
@@ -268,36 +270,36 @@ __device__ __forceinline__ bool closes(unsigned cx, unsigned cy, unsigned cz, in
 __global__ void __launch_bounds__(kBlock) k_tr_rows(DevGraph g, TrBuffers t, int fuzz) {
   pdl_enter();
   __shared__ int4 row[kTrBatch];                       // read, first entry, entries, first of the batch's entries
-  __shared__ unsigned key[kTrStage];                   // column << 2 | code
-  __shared__ int32_t suf[kTrStage];
-  __shared__ uint8_t row_of[kTrStage], hit[kTrStage];
+  __shared__ unsigned key[kTrHold];                    // column << 2 | code
+  __shared__ int32_t suf[kTrHold];
+  __shared__ uint8_t row_of[kTrHold], hit[kTrHold];
   __shared__ int warp_tot[kBlock / 32];
   if (__syncthreads_or(failed(t.derr))) return;
   const int tid = threadIdx.x;
   const long long R = *t.n_rows;
-  const int rows = batch_rows(g.m, R);
+  const int rows = batch_rows(g.m, R, kTrAimRows);
   for (long long b0 = (long long)blockIdx.x * rows; b0 < R; b0 += (long long)gridDim.x * rows) {
     const int total = load_batch(t, b0, rows, R, row, warp_tot);
     for (int i = tid; i < total; i += kBlock) {
       const int j = find_row(row, i);
       const int x = row[j].y + (i - row[j].w);
-      if (row[j].w + row[j].z <= kTrStage) {
+      if (row[j].w + row[j].z <= kTrHold) {
         key[i] = ((unsigned)g.col[x] << 2) | g.code[x];
         suf[i] = g.suf[x];
         row_of[i] = (uint8_t)j;
         hit[i] = 0;
       } else {
-        t.trans[x] = 0;
+        t.trans[x] = (uint8_t)(g.code[x] << 1);
       }
     }
     __syncthreads();
     for (int i = tid; i < total; i += kBlock) {
-      // entry i is staged when its whole row is: then it lies below kTrStage with row_of set
-      int j = i < kTrStage ? row_of[i] : kTrBatch;
-      if (j >= kTrBatch || i < row[j].w || i >= row[j].w + row[j].z || row[j].w + row[j].z > kTrStage)
+      // entry i is staged when its whole row is: then it lies below kTrHold with row_of set
+      int j = i < kTrHold ? row_of[i] : kTrBatch;
+      if (j >= kTrBatch || i < row[j].w || i >= row[j].w + row[j].z || row[j].w + row[j].z > kTrHold)
         j = find_row(row, i);
       const int u = row[j].x, a = row[j].y, n = row[j].z, s0 = row[j].w, y = a + (i - s0);
-      const bool staged = s0 + n <= kTrStage;
+      const bool staged = s0 + n <= kTrHold;
       const unsigned e = staged ? key[i] : ((unsigned)g.col[y] << 2) | g.code[y];
       const int32_t sy = staged ? suf[i] : g.suf[y];
       const int v = (int)(e >> 2);
@@ -309,11 +311,8 @@ __global__ void __launch_bounds__(kBlock) k_tr_rows(DevGraph g, TrBuffers t, int
       int z = cy & 2u ? iv.x : iv.y;
       if (u < v) {
         const int32_t back = find_col(g.col, iv.x, iv.z, u);
-        if (back < 0 || g.code[back] != (((cy & 1) << 1) | (cy >> 1))) {
-          set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, y);
-        } else {
-          t.mir[back] = y;
-        }
+        if (back >= 0) t.mir[back] = y;
+        else set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, y);
         t.mir[y] = back;
       }
       for (; z < z1; z += 4) {
@@ -340,24 +339,25 @@ __global__ void __launch_bounds__(kBlock) k_tr_rows(DevGraph g, TrBuffers t, int
           for (int k = 0; k < 4; ++k) {
             if (z + k >= z1) break;
             const int32_t x = find_col(g.col, a, a + n, (int32_t)(q[k].x >> 2));
-            if (x >= 0 && closes(g.code[x], cy, q[k].x, g.suf[x], sy, (int32_t)q[k].y, fuzz)) t.trans[x] = 1;
+            if (x >= 0 && closes(g.code[x], cy, q[k].x, g.suf[x], sy, (int32_t)q[k].y, fuzz))
+              t.trans[x] = (uint8_t)(1u | (g.code[x] << 1));
           }
         }
       }
     }
     __syncthreads();
-    for (int i = tid; i < min(total, kTrStage); i += kBlock) {
+    for (int i = tid; i < min(total, kTrHold); i += kBlock) {
       const int j = row_of[i];                         // set when i is staged
-      if (j < kTrBatch && i >= row[j].w && i < row[j].w + row[j].z && row[j].w + row[j].z <= kTrStage)
-        t.trans[row[j].y + (i - row[j].w)] = hit[i];
+      if (j < kTrBatch && i >= row[j].w && i < row[j].w + row[j].z && row[j].w + row[j].z <= kTrHold)
+        t.trans[row[j].y + (i - row[j].w)] = (uint8_t)(hit[i] | ((key[i] & 3u) << 1));
     }
     __syncthreads();
   }
 }
 
-// Per entry: its mirror must have been found; kept when neither is transitive. A block per
-// tile of the map writes the tile's words, the kept entries of the tile before
-// each word, and the tile's count.
+// Per entry: its mirror must have been found, with the ends of the pair exchanged;
+// kept when neither is transitive. A block per tile of the map writes the tile's
+// words, the kept entries of the tile before each word, and the tile's count.
 __global__ void __launch_bounds__(kBlock) k_tr_keep(long long m, const uint8_t* trans, const int32_t* mir, unsigned* keep,
                                                     unsigned* before, unsigned* tile_cnt, DevError* e) {
   pdl_enter();
@@ -366,21 +366,25 @@ __global__ void __launch_bounds__(kBlock) k_tr_keep(long long m, const uint8_t* 
   __shared__ unsigned cnt[kTrTile / 32];
   const long long tile = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long x0 = tile * kTrTile + threadIdx.x;
   uint8_t t[kPer];
   int32_t y[kPer];
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
-    const long long x = tile * kTrTile + k * kBlock + threadIdx.x;
+    const long long x = x0 + k * kBlock;
     t[k] = x < m ? trans[x] : 1;
     y[k] = x < m ? mir[x] : 0;
   }
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
     if (y[k] < 0) {                                    // an entry whose pair has no entry back
-      set_error(e, DERR_GRAPH, K_TRANSITIVE, tile * kTrTile + k * kBlock + threadIdx.x);
+      set_error(e, DERR_GRAPH, K_TRANSITIVE, x0 + k * kBlock);
       y[k] = 0;
     }
-    t[k] |= trans[y[k]];
+    const uint8_t back = trans[y[k]];
+    const bool pair = (back >> 1) == (((t[k] >> 1) & 1) << 1 | t[k] >> 2);   // the two ends, exchanged
+    if (x0 + k * kBlock < m && !pair) set_error(e, DERR_GRAPH, K_TRANSITIVE, x0 + k * kBlock);
+    t[k] = (t[k] | back) & 1;
   }
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {

@@ -131,6 +131,7 @@ def random_overlaps(seed, n, pairs, hub=0):
     (121, 2000, 0), (240, 3600, 0),             # batches of rows: 30 entries a row, so fewer rows than a batch holds
     (5000, 900, 0), (9000, 60, 0),              # mostly empty rows, batches that are not full
     (300, 12000, 0),                            # 80 entries a row
+    (2600, 4000, 1530), (2600, 4000, 1545),     # a row about as long as what the walks stage
     (2600, 4000, 2040), (2600, 4000, 2500),     # a row about as long as, and longer than, what is staged
 ])
 def test_row_shapes(ctx, n, pairs, hub):
@@ -159,6 +160,21 @@ def test_missing_or_foreign_mirrors(ctx):
     with pytest.raises(cg.CgError) as e:
         cg.cg_transitive_reduction(ctx, H)
     assert e.value.status == cg.CG_EGRAPH
+
+
+@pytest.mark.parametrize("hub", [0, 1600])
+@pytest.mark.parametrize("flip", [1, 2, 3])
+def test_pairs_whose_ends_disagree(ctx, hub, flip):
+    """One entry's code changed, seen from either read, in a row of any kind."""
+    G = random_overlaps(9, 1800, 4000, hub)
+    rows = np.repeat(np.arange(1800), np.diff(G.row_ptr))
+    for x in (0, np.flatnonzero(rows < G.col)[-1], G.m - 1):
+        H = type("R", (), dict(vars(G)))()
+        H.code = G.code.copy()
+        H.code[x] ^= flip
+        with pytest.raises(cg.CgError) as e:
+            cg.cg_transitive_reduction(ctx, H)
+        assert e.value.status == cg.CG_EGRAPH
 
 
 def test_invalid_and_capacity(ctx):
