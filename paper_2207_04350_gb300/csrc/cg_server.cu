@@ -14,7 +14,6 @@
 #include <cstdlib>
 #include <cstring>
 #include <deque>
-#include <iterator>
 #include <map>
 #include <mutex>
 #include <new>
@@ -36,9 +35,14 @@ int64_t now_ns() {
 // Host memory of one request's result. Pinned, so that the copy engines write it
 // while other batches run; the copies into pageable memory, freshly mapped and
 // zeroed for each request, were most of what a request took. Pinned blocks are
-// expensive to make, so released ones wait in the pool for the next request: at
-// most kPinnedMost bytes of them exist, waiting or in use, until the server stops,
-// and past that results lie in ordinary memory. Any thread may take and give.
+// expensive to make and to give back (cudaFreeHost waits for the device), so
+// released ones wait in the pool for the next request: at most kPinnedMost bytes of
+// them exist, waiting or in use, until the server stops, and past that results lie
+// in ordinary memory, written once before the copy. 2,000 requests of 42 Mb on
+// average, eight workers, all submitted at once: 2,110-2,170 requests a second; with
+// waiting blocks freed to make room for new ones 1,530, and with the ordinary memory
+// not written first either 700-920; with all results in ordinary memory 1,360-1,990.
+// Any thread may take and give.
 struct HostBuf {
   void* p = nullptr;
   size_t cap = 0;
@@ -51,7 +55,6 @@ class HostPool {
   // A block of at least `bytes`; p is null when there is no memory.
   HostBuf take(size_t bytes) {
     const size_t want = (bytes + 65535) & ~size_t(65535), make = want + want / 4;
-    std::vector<void*> drop;
     bool room = false;
     {
       std::lock_guard<std::mutex> lk(mu_);
@@ -61,17 +64,9 @@ class HostPool {
         idle_.erase(it);
         return b;
       }
-      // a new block; waiting ones that did not fit make room for it
-      while (held_ + make > kPinnedMost && !idle_.empty()) {
-        auto last = std::prev(idle_.end());
-        held_ -= last->first;
-        drop.push_back(last->second);
-        idle_.erase(last);
-      }
       room = held_ + make <= kPinnedMost;
       if (room) held_ += make;
     }
-    for (void* p : drop) cudaFreeHost(p);
     if (room) {
       void* p = nullptr;
       if (cudaHostAlloc(&p, make, cudaHostAllocPortable) == cudaSuccess) return HostBuf{p, make, true};
@@ -79,7 +74,9 @@ class HostPool {
       std::lock_guard<std::mutex> lk(mu_);
       held_ -= make;
     }
-    return HostBuf{std::malloc(bytes > 0 ? bytes : 1), bytes, false};
+    HostBuf b{std::malloc(bytes > 0 ? bytes : 1), bytes, false};
+    if (b.p) std::memset(b.p, 0, bytes);
+    return b;
   }
   void give(HostBuf& b) {
     if (b.p && b.pinned) {

@@ -93,3 +93,22 @@ def test_poll_and_timestamps(pool):
         srv.release(rid)
     finally:
         srv.stop()
+
+
+def test_results_past_the_pinned_memory():
+    """More unreleased results than the 1 GiB of pinned blocks: the rest lie in ordinary
+    memory, and blocks given back serve later requests of other sizes."""
+    big = gen.generate(dict(gen.WORKLOADS["genome-100Mb"](), genome_len=60_000_000), threads=8)
+    small = gen.generate("tiny-1Mb", threads=8)
+    want = {id(g): oracle.run(g, min_chain_reads=2) for g in (big, small)}
+    srv = cg.Server(0, hbm_budget_bytes=64 << 30, max_batch=4, workers=3)
+    try:
+        for _ in range(2):
+            asked = [big] * 20 + [small] * 4 + [big] * 2
+            ids = [srv.submit(g) for g in asked]
+            for rid, g in zip(ids, asked):                # all are there before any is released
+                _check(srv.wait(rid), want[id(g)])
+            for rid in ids:
+                srv.release(rid)
+    finally:
+        srv.stop()
