@@ -201,19 +201,21 @@ __host__ __device__ inline int emit_span(long long n_tiles, long long warps, int
 }
 
 // The ASCII kernel's spans: of layout tiles [t0, t1), as many of emit_span's size
-// (4 per warp, at most 64 KiB) as leave one per warp, and the rest in eighths of
-// it, so that the warps end together although the spans are big. Against spans of
-// one size (8 per warp, at most 32 KiB), k_emit: 3.1 Gb 679 to 671 us, steps of
-// 500 Mb 205 to 201, 1 Gb 321 to 320, 2 Gb 560 to 555; at most 128 KiB, or 2 or 3
-// per warp, gave no more. The 2-bit kernel keeps one size: 141.3 us on 1.2 Gb with
-// or without halves at the end, 145.4 with quarters.
+// (8 per warp, at most 64 KiB) as leave one per warp, and the rest in eighths of it
+// (of 8 KiB at least), so that the warps end together although the spans are big.
+// Against spans of one size of at most 32 KiB, k_emit on 3.1 Gb: 679 to 671 us;
+// whole steps: 3.1 Gb 830 to 822 us, 1.3 Gb 404 to 399, 512 graphs of 0.5-12 Mb 608
+// to 603. At most 128 KiB gave no more; 4 per warp made steps of 500 Mb 2% faster and
+// 1.2 Gb of lone reads 2.5% slower (288 to 294 us); halves at the end gave a third
+// of it. The 2-bit kernel keeps one size: 141.3 us on 1.2 Gb with or without halves
+// at the end, 145.4 with quarters.
 struct SpanPlan {
   long long t0, t1, big;       // big: how many spans of the full size
   int span, small;
   __device__ SpanPlan(long long t_begin, long long t_stop, long long warps, int emit_tile, int layout_tile)
       : t0(t_begin), t1(max(t_begin, t_stop)) {
-    span = emit_span(t1 - t0, warps, emit_tile, layout_tile, 4, 65536);
-    small = emit_tile > 0 ? span : max(1, span / 8);
+    span = emit_span(t1 - t0, warps, emit_tile, layout_tile, 8, 65536);
+    small = emit_tile > 0 ? span : min(span, max(span / 8, 8192 / layout_tile));
     big = small == span ? 0 : max(0ll, (t1 - t0) / span - warps);
   }
   __device__ long long spans() const { return big + (t1 - t0 - big * span + small - 1) / small; }

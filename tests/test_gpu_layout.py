@@ -47,9 +47,9 @@ def test_heads_in_one_word(ctx):
     assert np.count_nonzero(oracle.run(G).contig_off) == 3000
 
 
-@pytest.mark.parametrize("mb", [25, 90, 170])
+@pytest.mark.parametrize("mb", [50, 90, 330])
 def test_spelling_spans(mb):
-    """Spans of 2, 8 and 16 tiles (on 608 warps) with smaller ones at the end,
+    """Spans of 2, 4 and 16 tiles (on 608 warps) with smaller ones at the end,
     whole and in shares that start at any tile."""
     import torch
     G = gen.generate(dict(gen.WORKLOADS["genome-3.1Gb"](), genome_len=mb * 1_000_000), threads=8)
