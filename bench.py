@@ -32,9 +32,9 @@ METRIC = "contig Gbases/s & ms per graph (plain vs batched) vs HBM roofline; p50
 UNIT = "Gbases/s"
 PEAKS_FALLBACK = {"hbm_gbs": 6800.0}
 # DRAM bytes (read + write) per contig base of k_emit from one ncu capture
-# (--set full, the 3.1 Gb recipe on a 450 Mb genome: 552.2 MB for 481,446,585
+# (--set full, the 3.1 Gb recipe on a 450 Mb genome: 550.6 MB for 481,446,585
 # bases), valid only for the emission source it was taken on.
-EMIT_TRAFFIC = {"bytes_per_base": (128.766464e6 + 421.409280e6) / 481446585, "source_sha256_16": "81bd7d9611aecfe5"}
+EMIT_TRAFFIC = {"bytes_per_base": (129.027072e6 + 421.528576e6) / 481446585, "source_sha256_16": "148a0f9f1719bdd2"}
 
 
 def _reduce(x: float, world: int, op: str) -> float:
@@ -772,7 +772,7 @@ def run_ours(args, rank, world, local_rank):
               "kernel_ms": statistics.mean(tr_ms),
               "kernel_ms_by_name": {k: statistics.mean(v) for k, v in tr_kern.items()},
               "call_ms_two_calls": statistics.mean(tr_wall[1:]),
-              "note": "kernel_ms: one call's kernels (checks, mark, keep, row scan, scatter); the API's size query "
+              "note": "kernel_ms: one call's kernels (checks, packed rows, walks, keep, tiles, scatter); the API's size query "
                       "runs them once more"}
         del S, rd, Rf
 

@@ -361,10 +361,11 @@ typedef struct {
 CG_API cg_status cg_set_tuning(cg_ctx* ctx, const cg_tuning* t);
 CG_API cg_status cg_get_tuning(cg_ctx* ctx, cg_tuning* out);
 
-/* With graphs on (the default), each stage's kernel launches are captured
- * once into a CUDA graph per graph and set of buffers, sizes and launch
- * parameters, and replayed with one launch afterwards. Off: launched one by
- * one. Outputs are the same either way. */
+/* With graphs on (the default), a stage's kernel launches are captured into a
+ * CUDA graph per graph when the same buffers, sizes and launch parameters come
+ * a second time in a row, and replayed with one launch afterwards; a first use
+ * is launched one by one. Off: always launched one by one. Outputs are the same
+ * either way. */
 CG_API cg_status cg_set_graphs(cg_ctx* ctx, int enable);
 
 /* Programmatic dependent launch (on by default): a kernel that directly follows
