@@ -307,8 +307,8 @@ __global__ void __launch_bounds__(kBlock) k_tr_rows(DevGraph g, TrBuffers t, int
       const int4 iv = t.info[v];                       // first entry, first of the second run, end, length
       if (sy < 1 || sy > iv.w - 1) set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, y);
       // v is left through its other end: the first run when it was entered through end 1
-      const int z1 = cy & 2u ? iv.y : iv.z;
-      int z = cy & 2u ? iv.x : iv.y;
+      const unsigned z1 = (unsigned)(cy & 2u ? iv.y : iv.z);   // unsigned: z + 4 may pass the largest int
+      unsigned z = (unsigned)(cy & 2u ? iv.x : iv.y);
       if (u < v) {
         const int32_t back = find_col(g.col, iv.x, iv.z, u);
         if (back >= 0) t.mir[back] = y;
