@@ -175,8 +175,11 @@ __device__ __forceinline__ int batch_rows(long long m, long long R, int aim) {
 // read with entries; codes 0..3. Copies every row in two runs by the end its
 // entries leave through, each run in the row's order: 9 B read and 12 written per
 // entry. An entry's place in its run is the count of entries of that end before
-// it, from the ballots of the block's entries.
-__global__ void __launch_bounds__(kBlock) k_tr_pack(DevGraph g, TrBuffers t) {
+// it, from the ballots of the block's entries. Its loads wait on one another (row,
+// code, column), so that warps hide them: with eight blocks on an SM, at 32
+// registers, 51 us for 3.38M entries, with six 56; batches of 720 and 480 entries
+// 53 and 56.
+__global__ void __launch_bounds__(kBlock, 8) k_tr_pack(DevGraph g, TrBuffers t) {
   pdl_enter();
   __shared__ int4 row[kTrBatch];
   __shared__ unsigned zeros[kTrStage / 32];            // per word of staged entries: entries leaving through end 0
@@ -263,7 +266,7 @@ __device__ __forceinline__ bool closes(unsigned cx, unsigned cy, unsigned cz, in
 // of the rows v, which lie at random (a sector or two each), and issuing the
 // searches, in warps whose lanes walk runs of unequal length. 3.38M entries of
 // 420 thousand rows, by events: 158 us (178 with the four searches one after
-// another), and 56 for the packing before it; a
+// another), and 51 for the packing before it; a
 // thread per entry walking whole rows and searching u's row in memory took 283,
 // after 93 for mirrors found by a search of their own; eight lanes per row, four
 // rows of a warp in step, took 476, most of its lanes waiting for longer rows.
