@@ -779,31 +779,32 @@ cudaError_t launch_chains(const DevGraph& g, const Scratch& s, const Tuning& t, 
     cudaMemsetAsync(&s.ctr->n_rulers, 0, offsetof(Counters, n_contigs) - offsetof(Counters, n_rulers), env.stream);
   static const int succ_resident = resident_blocks(k_succ);   // persistent grids
   static const int final_resident = resident_blocks(k_final);
-  // a persistent grid, but no more blocks than the reads can use (a small
-  // graph's launches would otherwise spend their time starting idle blocks)
-  auto cap = [&](long long resident_grid, long long items_per_block) {
-    const long long need = (g.n + items_per_block - 1) / items_per_block;
+  // a persistent grid, but no more blocks than the candidates can use
+  const long long N = most_candidates(g);
+  auto cap = [&](long long resident_grid, long long items, long long items_per_block) {
+    const long long need = (items + items_per_block - 1) / items_per_block;
     return (int)std::max(1LL, std::min(resident_grid, need));
   };
-  cudaError_t e = launch_k(k_succ, cap((long long)env.num_sms * succ_resident, kBlock), env, after_mask, g, s,
-                           t.ruler_log2);
+  // k_succ also copies the words of a bitmap of the reads
+  cudaError_t e = launch_k(k_succ, cap((long long)env.num_sms * succ_resident, std::max(N, (long long)g.n / 32), kBlock),
+                           env, after_mask, g, s, t.ruler_log2);
   if (e != cudaSuccess) return e;
   mark(env, "k_succ");
-  e = launch_k(k_walk, grid_for(2 * g.n, env), env, true, s, t.ruler_log2, (int64_t)(2 * g.n + 1));
+  e = launch_k(k_walk, grid_for(2 * N, env), env, true, s, t.ruler_log2, (int64_t)(2 * g.n + 1));
   if (e != cudaSuccess) return e;
   mark(env, "k_walk");
-  e = launch_k(k_listwalk, grid_for(2 * g.n, env), env, true, s);
+  e = launch_k(k_listwalk, grid_for(N, env), env, true, s);   // a list per two oriented candidates, at most
   if (e != cudaSuccess) return e;
   mark(env, "k_listwalk");
   DevGraph gg = g;
   Scratch sc = s;
   void* args[] = {&gg, &sc};
-  e = coop((const void*)k_final, cap((long long)env.num_sms * final_resident, (long long)kBlock * kFinalItems), args, env,
-           true);
+  e = coop((const void*)k_final, cap((long long)env.num_sms * final_resident, N, (long long)kBlock * kFinalItems), args,
+           env, true);
   if (e != cudaSuccess) return e;
   mark(env, "k_final");
   if (leave_cycles) return cudaGetLastError();
-  e = coop((const void*)k_cycles, cap(env.coop_blocks, kBlock / 2), args, env, true);   // up to 2 candidates per read
+  e = coop((const void*)k_cycles, cap(env.coop_blocks, 2 * N, kBlock), args, env, true);
   if (e != cudaSuccess) return e;
   mark(env, "k_cycles");
   return cudaGetLastError();

@@ -497,6 +497,14 @@ inline cudaError_t coop(const void* fn, int blocks, void** args, const LaunchEnv
   return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
+// Candidates there can be, each with an entry of its own, and reads spelled. The
+// counts are on the device alone, and grids sized for all n reads start blocks by
+// the hundred that find nothing: the step of a 100 Mb genome (333 thousand reads,
+// 37 thousand entries) takes @@A@@ us so and @@B@@ with them. Every kernel loops over its
+// items, whatever its grid.
+inline long long most_candidates(const DevGraph& g) { return g.n < g.m ? g.n : g.m; }
+inline long long most_spelled(const DevGraph& g) { return g.min_chain <= 1 ? g.n : most_candidates(g); }
+
 inline int grid_for(long long n, const LaunchEnv& env, int per_sm = 8) {
   long long b = (n + kBlock - 1) / kBlock;
   long long cap = (long long)env.num_sms * per_sm;

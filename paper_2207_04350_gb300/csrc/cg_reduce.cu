@@ -265,11 +265,14 @@ __device__ __forceinline__ bool closes(unsigned cx, unsigned cy, unsigned cz, in
 // which are searched in place. What bounds it is the records, runs and columns
 // of the rows v, which lie at random (a sector or two each), and issuing the
 // searches, in warps whose lanes walk runs of unequal length. 3.38M entries of
-// 420 thousand rows, by events: 158 us (178 with the four searches one after
-// another), and 51 for the packing before it; a
+// 420 thousand rows, by events: 143 us (178 with the four searches one after
+// another; 157 with batches of 960 entries, 2,048 of them staged, and the mirror's
+// code read from its row instead of checked where the mirrors' flags are read). A
 // thread per entry walking whole rows and searching u's row in memory took 283,
 // after 93 for mirrors found by a search of their own; eight lanes per row, four
-// rows of a warp in step, took 476, most of its lanes waiting for longer rows.
+// rows of a warp in step, took 476, most of its lanes waiting for longer rows; the
+// runs of a warp's entries laid end to end, so that no lane waits, 139 to 160 by
+// the entries in flight, for as many instructions as without.
 __global__ void __launch_bounds__(kBlock) k_tr_rows(DevGraph g, TrBuffers t, int fuzz) {
   pdl_enter();
   __shared__ int4 row[kTrBatch];                       // read, first entry, entries, first of the batch's entries

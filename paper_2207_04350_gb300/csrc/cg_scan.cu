@@ -212,8 +212,8 @@ cudaError_t launch_offsets(const DevGraph& g, const Scratch& s, const Tuning& t,
   if (s.small) return launch_small(g, s, t, kStageOffsets, user_off, user_cap, env, env.pdl_first);
   cudaError_t e = cudaSuccess;
   if (with_cycles) {
-    // as many blocks as the closed chains can use, up to 2 candidates per read
-    const long long need = (g.n + kBlock / 2 - 1) / (kBlock / 2);
+    // as many blocks as the closed chains, of oriented candidates, or the tiles can use
+    const long long need = std::max((2 * most_candidates(g) + kBlock - 1) / kBlock, (long long)s.h_tiles);
     static const int heads_resident = resident_blocks(k_heads);
     const long long most = std::min<long long>(env.coop_blocks, (long long)env.num_sms * heads_resident);
     DevGraph gg = g;
@@ -226,13 +226,14 @@ cudaError_t launch_offsets(const DevGraph& g, const Scratch& s, const Tuning& t,
   if (e != cudaSuccess) return e;
   mark(env, "k_heads");
   static const int scatter_resident = resident_blocks(k_scatter);   // a persistent grid
-  const long long scatter_need = (g.n + (long long)kBlock * kScatterItems - 1) / ((long long)kBlock * kScatterItems);
+  const long long spelled = most_spelled(g), scatter_need = (spelled + kBlock * kScatterItems - 1) / (kBlock * kScatterItems);
   e = launch_k(k_scatter, (int)std::max(1LL, std::min((long long)env.num_sms * scatter_resident, scatter_need)), env,
                true, g, s);
   if (e != cudaSuccess) return e;
   mark(env, "k_scatter");
   PieceStore ps{s.out_off, s.contig_off, s.tile_seg, s.tiles_cap, t.tile_bytes, s.ctr, s.derr, user_off, user_cap};
-  e = launch_k(k_pieces, (int)std::min((long long)s.scan_tiles_cap, (long long)env.num_sms * 4), env, true, s, ps);
+  e = launch_k(k_pieces, (int)std::max(1LL, std::min((spelled + kPieceTile - 1) / kPieceTile, (long long)env.num_sms * 4)),
+               env, true, s, ps);
   if (e != cudaSuccess) return e;
   mark(env, "k_pieces");
   return cudaGetLastError();
