@@ -265,12 +265,11 @@ inline void mark(const LaunchEnv& env, const char* name) {
 // launchers of the single stages below use it for such graphs too.
 enum : int { kStageMask = 1, kStageChains = 2, kStageOffsets = 4 };
 // A small graph: one block beats ten kernels while a few reads and candidates per
-// thread are all there is. Steps in us, one block against ten kernels: 750 reads
-// 26.7 / 39.0, 5,000 31.5 / 44.0, 10,000 38.1 / 45.2, 20,000 51.7 / 49.6, 40,000
-// 84 / 56; with the lone reads spelled too, which one block also scatters, 2,500
-// 42.7 / 49.5 and 5,000 68.5 / 64.9. The bound on the entries is that of an
-// overlap graph of so many reads after the reduction; 8 entries a read would cost
-// what 20,000 reads do.
+// thread are all there is. Steps in us with a wait after each, one block against
+// nine kernels: 2,000 reads 37 / 48, 8,000 44 / 53, 16,250 56 / 57; with the lone
+// reads spelled too, which one block also scatters, 1,000 41 / 52, 3,000 54 / 61,
+// 4,000 62 / 64. The bound on the entries is that of an overlap graph of so many
+// reads after the reduction; 8 entries a read would cost what 20,000 reads do.
 constexpr int64_t kSmallReads = 16384, kSmallLoneReads = 4096, kSmallEntries = 8192;
 inline bool small_graph(int64_t n, int64_t m, int min_chain) {
   return n > 0 && n <= (min_chain <= 1 ? kSmallLoneReads : kSmallReads) && m <= kSmallEntries;
@@ -500,8 +499,9 @@ inline cudaError_t coop(const void* fn, int blocks, void** args, const LaunchEnv
 // Candidates there can be, each with an entry of its own, and reads spelled. The
 // counts are on the device alone, and grids sized for all n reads start blocks by
 // the hundred that find nothing: the step of a 100 Mb genome (333 thousand reads,
-// 37 thousand entries) takes @@A@@ us so and @@B@@ with them. Every kernel loops over its
-// items, whatever its grid.
+// 37 thousand entries) takes 90 us so and 95 with them, one of 20 Mb with its lone
+// reads 194 and 201. Smaller grids still, by what the walks mostly are, gave no
+// more. Every kernel loops over its items, whatever its grid.
 inline long long most_candidates(const DevGraph& g) { return g.n < g.m ? g.n : g.m; }
 inline long long most_spelled(const DevGraph& g) { return g.min_chain <= 1 ? g.n : most_candidates(g); }
 
