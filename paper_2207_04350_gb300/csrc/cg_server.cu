@@ -14,6 +14,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <deque>
+#include <iterator>
 #include <map>
 #include <mutex>
 #include <new>
@@ -34,15 +35,16 @@ int64_t now_ns() {
 
 // Host memory of one request's result. Pinned, so that the copy engines write it
 // while other batches run; the copies into pageable memory, freshly mapped and
-// zeroed for each request, were most of what a request took. Pinned blocks are
-// expensive to make and to give back (cudaFreeHost waits for the device), so
-// released ones wait in the pool for the next request: at most kPinnedMost bytes of
-// them exist, waiting or in use, until the server stops, and past that results lie
-// in ordinary memory, written once before the copy. 2,000 requests of 42 Mb on
-// average, eight workers, all submitted at once: 2,110-2,170 requests a second; with
-// waiting blocks freed to make room for new ones 1,530, and with the ordinary memory
-// not written first either 700-920; with all results in ordinary memory 1,360-1,990.
-// Any thread may take and give.
+// zeroed for each request, were most of what a request took. Making pinned memory
+// and giving it back stop the other workers' calls for many milliseconds, so the
+// server makes one stretch of kPinned bytes as it starts (30 ms), out of which
+// results are cut, first fit, and released ones joined again. Results that do not
+// fit lie in ordinary memory, written once before the copy. 2,000 requests of 42 Mb
+// on average, eight workers, all submitted at once: 1,850-2,340 requests a second,
+// and with 940-1,045 a second offered from the server's start on, p50 0.95 and p99
+// 4.9-6.7 ms. With a pinned block made for each request that found none waiting
+// 1,890-2,260, 1.0 and 43-138; with all results in ordinary memory 1,360-2,100, and
+// p50 1.3, p99 10-20 with a third as many offered. Any thread may take and give.
 struct HostBuf {
   void* p = nullptr;
   size_t cap = 0;
@@ -51,28 +53,35 @@ struct HostBuf {
 
 class HostPool {
  public:
-  static constexpr size_t kPinnedMost = size_t(1) << 30;
+  static constexpr size_t kPinned = size_t(1) << 30, kUnit = 65536;
+  // Less pinned memory, or none, when the host has not got it.
+  void make() {
+    for (size_t n = kPinned; n >= kPinned / 16 && !base_; n /= 2) {
+      void* p = nullptr;
+      if (cudaHostAlloc(&p, n, cudaHostAllocPortable) == cudaSuccess) {
+        base_ = static_cast<char*>(p);
+        free_[0] = n;
+      } else {
+        cudaGetLastError();
+      }
+    }
+  }
   // A block of at least `bytes`; p is null when there is no memory.
   HostBuf take(size_t bytes) {
-    const size_t want = (bytes + 65535) & ~size_t(65535), make = want + want / 4;
-    bool room = false;
+    const size_t want = bytes > 0 ? (bytes + kUnit - 1) / kUnit * kUnit : kUnit;
     {
       std::lock_guard<std::mutex> lk(mu_);
-      auto it = idle_.lower_bound(want);
-      if (it != idle_.end() && it->first <= 4 * want) {
-        HostBuf b{it->second, it->first, true};
-        idle_.erase(it);
-        return b;
+      for (auto it = free_.begin(); it != free_.end(); ++it) {
+        if (it->second < want) continue;
+        auto node = free_.extract(it);       // goes back as the rest of the stretch: nothing is allocated
+        char* const p = base_ + node.key();
+        if (node.mapped() > want) {
+          node.key() += want;
+          node.mapped() -= want;
+          free_.insert(std::move(node));
+        }
+        return HostBuf{p, want, true};
       }
-      room = held_ + make <= kPinnedMost;
-      if (room) held_ += make;
-    }
-    if (room) {
-      void* p = nullptr;
-      if (cudaHostAlloc(&p, make, cudaHostAllocPortable) == cudaSuccess) return HostBuf{p, make, true};
-      cudaGetLastError();
-      std::lock_guard<std::mutex> lk(mu_);
-      held_ -= make;
     }
     HostBuf b{std::malloc(bytes > 0 ? bytes : 1), bytes, false};
     if (b.p) std::memset(b.p, 0, bytes);
@@ -81,20 +90,35 @@ class HostPool {
   void give(HostBuf& b) {
     if (b.p && b.pinned) {
       std::lock_guard<std::mutex> lk(mu_);
-      idle_.emplace(b.cap, b.p);
+      const size_t at = static_cast<size_t>(static_cast<char*>(b.p) - base_);
+      size_t len = b.cap;
+      auto next = free_.lower_bound(at);
+      if (next != free_.end() && at + len == next->first) {
+        len += next->second;
+        next = free_.erase(next);
+      }
+      auto before = next == free_.begin() ? free_.end() : std::prev(next);
+      if (before != free_.end() && before->first + before->second == at) {
+        before->second += len;
+      } else {
+        try {
+          free_.emplace_hint(next, at, len);
+        } catch (const std::bad_alloc&) {    // the stretch is lost until the server stops
+        }
+      }
     } else {
       std::free(b.p);
     }
     b = HostBuf{};
   }
   ~HostPool() {
-    for (auto& kv : idle_) cudaFreeHost(kv.second);
+    if (base_) cudaFreeHost(base_);
   }
 
  private:
   std::mutex mu_;
-  std::multimap<size_t, void*> idle_;    // by size
-  size_t held_ = 0;                      // pinned bytes, waiting or in use
+  char* base_ = nullptr;
+  std::map<size_t, size_t> free_;        // free stretches: offset, length; no two adjoin
 };
 
 struct Request {
@@ -393,6 +417,7 @@ cg_status cg_server_start(int device, const cg_server_opts* opts, cg_server** ou
     uint64_t keep = ~0ull;   // freed buffers stay in the pool for the next batch
     cudaMemPoolSetAttribute(s->pool, cudaMemPoolAttrReleaseThreshold, &keep);
   }
+  s->results.make();
   for (int w = 0; w < opts->workers; ++w) {
     cg_ctx* c = nullptr;
     cudaStream_t st_w = nullptr;

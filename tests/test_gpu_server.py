@@ -96,8 +96,8 @@ def test_poll_and_timestamps(pool):
 
 
 def test_results_past_the_pinned_memory():
-    """More unreleased results than the 1 GiB of pinned blocks: the rest lie in ordinary
-    memory, and blocks given back serve later requests of other sizes."""
+    """More unreleased results than the 1 GiB of pinned memory holds: the rest lie in
+    ordinary memory, and what is given back serves later requests of other sizes."""
     big = gen.generate(dict(gen.WORKLOADS["genome-100Mb"](), genome_len=60_000_000), threads=8)
     small = gen.generate("tiny-1Mb", threads=8)
     want = {id(g): oracle.run(g, min_chain_reads=2) for g in (big, small)}
