@@ -27,6 +27,7 @@
 #include <algorithm>
 
 #include "cg_internal.cuh"
+#include "cg_search.h"
 
 namespace cg {
 
@@ -41,17 +42,6 @@ constexpr int kTrAimRows = 720;      // the same for the walks, just under three
 constexpr int kTrHold = 1536;        // memory the blocks of an SM hold, the more cache the random rows have
 
 __device__ __forceinline__ bool failed(const DevError* e) { return *(const volatile int*)&e->err != 0; }
-
-// Position of column w in the sorted row [a, b), or -1.
-__device__ __forceinline__ int32_t find_col(const int32_t* col, int32_t a, int32_t b, int32_t w) {
-  int32_t lo = a, hi = b;
-  while (lo < hi) {
-    const int32_t mid = (lo + hi) >> 1;
-    if (col[mid] < w) lo = mid + 1;
-    else hi = mid;
-  }
-  return lo < b && col[lo] == w ? lo : -1;
-}
 
 // Four consecutive values, by 16-byte loads and stores where `wide`.
 template <typename T>
