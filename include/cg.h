@@ -389,6 +389,8 @@ CG_API cg_status cg_set_host_direct(cg_ctx* ctx, int enable);
  * spec: "site:n[:ms]" entries separated by commas; the n-th time (from 1) this
  * context reaches `site` it fails as that step would: "alloc" (CG_ENOMEM),
  * "h2d" (an input copy, CG_ECUDA), "timeout" (a bounded device wait,
+ * CG_ETIMEOUT), "barrier" (the n-th stage's kernels start as after a device wait
+ * that gave up: they write no output, and the next waiting call returns
  * CG_ETIMEOUT), "kernel" (a kernel consistency check, CG_EKERNEL), "bad_graph"
  * (input validation, CG_EGRAPH). NULL or "" clears the plan. The CG_FAULT
  * environment variable gives the plan of every new context and server; a

@@ -281,6 +281,10 @@ const cg::Tuning& gt(cg_graph* g) {
 template <class F>
 cg_status run_stage(cg_graph* g, int slot, uint64_t key, F&& launch) {
   cg_ctx* c = g->ctx;
+  if (c->fault.hit("barrier")) {         // the error word as a barrier that gave up leaves it
+    const cg::DevError gone{cg::DERR_TIMEOUT, cg::K_JUMP, 0};
+    CK(cudaMemcpyAsync(c->derr, &gone, sizeof(gone), cudaMemcpyHostToDevice, c->stream), "set error word");
+  }
   if (!c->graphs) return launch();
   StageExec& e = g->execs[slot];
   key = mix_key(key, c->marks.on ? 1 : 2);

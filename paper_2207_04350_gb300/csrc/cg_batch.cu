@@ -76,6 +76,7 @@ __global__ void __launch_bounds__(kBlock) k_batch_copy(const CopySeg* __restrict
 __global__ void k_batch_ranges(Scratch s, int k, const int64_t* R, long long N, int64_t* first_contig,
                                int64_t* first_base) {
   const Counters* c = s.ctr;
+  if (gave_up(s.derr)) return;
   for (long long j = grid_tid(); j <= k; j += grid_threads()) {
     const long long r = R[j];
     long long ci;
@@ -169,6 +170,7 @@ __global__ void __launch_bounds__(kBlock) k_gather_pieces(Scratch s, int k, cons
                                                           const unsigned long long* slot, uint32_t* dst,
                                                           long long cap_words, long long t_begin, long long t_end) {
   long long j_begin = 0, W = *(const volatile unsigned*)&s.ctr->n_walk;
+  if (gave_up(s.derr)) return;
   if (t_end > 0) {
     const long long nt = *(const volatile unsigned*)&s.ctr->n_tiles;
     j_begin = t_begin > 0 ? (long long)s.tile_seg[min(t_begin, nt)] + 1 : 0;

@@ -88,7 +88,9 @@ __global__ void __launch_bounds__(BT, 1024 / BT) k_emit(Scratch s, const uint8_t
   pdl_enter();                 // the table needs nothing from the kernels before
   __syncthreads();
   const Counters* c = s.ctr;
+  const bool stop = gave_up(s.derr);
   const long long total = *(const volatile long long*)&c->total_bases;
+  if (stop) return;
   const long long ntiles = (total + tile_bytes - 1) / tile_bytes;
   if (n_shares > 1) {
     t_begin = (long long)share * ntiles / n_shares;

@@ -420,7 +420,9 @@ __global__ void __launch_bounds__(BT, BT >= 512 ? 2 : CG_EMIT2_MIN_BLOCKS * 256 
   pdl_enter();
   __shared__ PieceList lists[BT / 32];
   const Counters* c = s.ctr;
+  const bool stop = gave_up(s.derr);
   const long long total = *(const volatile long long*)&c->total_bases;
+  if (stop) return;
   const long long need = 16 * ((total + 63) / 64);
   if (need > cap_bytes) {
     if (grid_tid() == 0) set_error(s.derr, DERR_CAPACITY, K_EMIT, need);

@@ -72,6 +72,7 @@ __device__ __forceinline__ int share_of_pair(const long long* pair0, int n_share
 // k_x_sizes cleared.
 __global__ void __launch_bounds__(kMaxParts) k_x_ranges(Scratch s, XchgArgs x, int tile_bytes) {
   pdl_enter();
+  if (gave_up(s.derr)) return;
   __shared__ long long warp_tot[kMaxParts / 32];
   const int p = (int)threadIdx.x, lane = p & 31, warp = p >> 5;
   long long cnt = 0;
@@ -111,6 +112,7 @@ __global__ void __launch_bounds__(kMaxParts) k_x_ranges(Scratch s, XchgArgs x, i
 // in one share, which takes one addition for the warp.
 __global__ void __launch_bounds__(kBlock) k_x_sizes(Scratch s, XchgArgs x, uint32_t* mine) {
   pdl_enter();
+  if (gave_up(s.derr)) return;
   __shared__ unsigned long long send[kMaxParts], recv[kMaxParts];
   __shared__ long long pair0[kMaxParts + 1];
   __shared__ int64_t rf[kMaxParts + 1];
@@ -202,7 +204,7 @@ __global__ void __launch_bounds__(kBlock) k_x_pack(DevGraph g, Scratch s, XchgAr
                                                    const long long* slot, const long long* first, uint32_t* send,
                                                    long long n_words) {
   pdl_enter();
-  if (*(const volatile int*)&s.derr->err != 0) return;    // the scan gave up: slot and first are not whole
+  if (gave_up(s.derr)) return;                            // the scan did: slot and first are not whole
   const unsigned full = 0xffffffffu;
   __shared__ long long s_end[kBlock], s_base[kBlock];     // per piece: its end in the buffer, the base that word 0 would start with
   const int lane = threadIdx.x & 31, warp0 = threadIdx.x & ~31;
@@ -280,6 +282,7 @@ __global__ void __launch_bounds__(kBlock) k_x_place(Scratch s, XchgArgs x, unsig
   constexpr int kPer = kXchgTile / kBlock;
   __shared__ unsigned long long tot[kBlock / 32];
   __shared__ long long s_tile;
+  if (__syncthreads_or(gave_up(s.derr))) return;
   const int who = (int)blockIdx.y, tid = threadIdx.x;
   const long long j0 = x.range[2 * x.rank], count = x.range[2 * x.rank + 1] - j0 + 1;
   const long long tiles = (count + kXchgTile - 1) / kXchgTile;

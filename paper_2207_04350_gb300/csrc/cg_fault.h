@@ -4,7 +4,9 @@
 // A plan is "site:n[:ms]" entries separated by commas. The n-th time (from 1)
 // a context or server reaches `site`, the library behaves as if that step had
 // failed: an allocation ("alloc", CG_ENOMEM), an input copy ("h2d",
-// CG_ECUDA), a bounded device wait ("timeout", CG_ETIMEOUT), a kernel's
+// CG_ECUDA), a bounded device wait ("timeout", CG_ETIMEOUT), a device wait that
+// gave up before a stage's kernels ("barrier": the error word is set as such a wait
+// sets it, the kernels run, and the next wait reports CG_ETIMEOUT), a kernel's
 // consistency check ("kernel", CG_EKERNEL), input validation ("bad_graph",
 // CG_EGRAPH), server admission ("admit", CG_EBUSY), a server worker that
 // stalls for ms milliseconds before its batch ("queue_stall"), or a server

@@ -674,7 +674,7 @@ __global__ void k_cycles(DevGraph g, Scratch s) {
   pdl_enter();
   Counters* c = s.ctr;
   const unsigned C = *(volatile unsigned*)&c->n_cycle_reads;
-  if (C == 0) return;
+  if (C == 0 || __syncthreads_or(gave_up(s.derr))) return;
   close_cycles(g, s, C, grid_tid(), grid_threads(), [&] { return grid_sync(c, s.derr); });
 }
 
@@ -688,12 +688,12 @@ __global__ void __launch_bounds__(kBlock) k_export_reads(DevGraph g, Scratch s, 
                                                          int32_t* rank, uint8_t* orient) {
   pdl_enter();
   Counters* c = s.ctr;
-  if (with_cycles) {
-    const unsigned C = *(volatile unsigned*)&c->n_cycle_reads;   // the same for every block
-    if (C > 0) {
-      close_cycles(g, s, C, grid_tid(), grid_threads(), [&] { return grid_sync(c, s.derr); });
-      if (!grid_sync(c, s.derr)) return;
-    }
+  const bool stop = gave_up(s.derr);
+  const unsigned C = with_cycles ? *(volatile unsigned*)&c->n_cycle_reads : 0u;   // the same for every block
+  if (__syncthreads_or(stop)) return;
+  if (C > 0) {
+    close_cycles(g, s, C, grid_tid(), grid_threads(), [&] { return grid_sync(c, s.derr); });
+    if (!grid_sync(c, s.derr)) return;
   }
   const unsigned N = *(volatile unsigned*)&c->n_cand;
   for (long long v0 = 4 * grid_tid(); v0 < g.n; v0 += 4 * grid_threads()) {

@@ -11,7 +11,8 @@ constexpr int kBlock = 256;
 constexpr int kPieceTile = 1024; // walk positions per tile of the piece scan
 constexpr int kHeadShift = 31;   // heads-bitmap sums: the count of heads above, their contigs' reads below (both < 2^30)
 
-// First device-side error wins (atomicCAS from 0).
+// The first device-side error wins, except that a wait that gave up replaces any
+// other: what later kernels would read is then not whole.
 enum : int32_t {
   DERR_NONE = 0,
   DERR_GRAPH = 1,     // input check failed
@@ -409,11 +410,19 @@ cudaError_t launch_selftest_wait(unsigned long long* state, long long tiles, Dev
 
 // ---- device helpers ----
 __device__ __forceinline__ void set_error(DevError* e, int code, int where, long long index) {
-  if (atomicCAS(&e->err, 0, code) == 0) {
+  if (code == DERR_TIMEOUT ? atomicExch(&e->err, code) != code : atomicCAS(&e->err, 0, code) == 0) {
     e->where = where;
     e->index = index;
   }
 }
+
+// A bounded wait of this or of an earlier kernel gave up: its block, and those that
+// gave up with it, left out the rest of their work. Every kernel that uses what a
+// kernel with such a wait wrote (contig records, walk positions, offsets, slots) as
+// an index asks this first and returns: the values may never have been written. In
+// a kernel that waits itself the answer may change while it runs, so there a block
+// asks as one (__syncthreads_or).
+__device__ __forceinline__ bool gave_up(const DevError* e) { return *(const volatile int*)&e->err == DERR_TIMEOUT; }
 
 // Programmatic dependent launch (sm_90 and later): wait until the grid before this
 // one on the stream has completed and its writes are visible. Every kernel of the

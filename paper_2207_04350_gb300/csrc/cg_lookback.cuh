@@ -3,7 +3,7 @@
 // Tiles take tickets in order, publish their aggregate, then look back over
 // their predecessors with the whole block (256 descriptors at a time) until an
 // inclusive prefix is found. The wait on a predecessor is bounded; on timeout
-// the kernel records DERR_TIMEOUT and stops.
+// the kernel records DERR_TIMEOUT, and every tile that waits gives up with it.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -58,13 +58,13 @@ __device__ unsigned long long lookback(unsigned long long* state, long long tile
       none = min(none, near_none[k]);
     }
     if (none < first) {                                    // a tile before the nearest prefix has not published yet
-      if (++spins > kLookbackSpins) {
+      ++spins;
+      if (__syncthreads_or(tid == 0 && (spins > kLookbackSpins || ((spins & 63) == 0 && gave_up(derr))))) {
         if (tid == 0) set_error(derr, DERR_TIMEOUT, where, tile);
         return excl;
       }
       __nanosleep(spins < 32 ? 20 : 200);
-      __syncthreads();                                     // near_pre and near_none are written again
-      continue;
+      continue;                                            // near_pre and near_none are written again
     }
     unsigned long long v = tid <= first ? (w & kValMask) : 0ull;
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);

@@ -54,13 +54,13 @@ __global__ void __launch_bounds__(kBlock) k_heads(DevGraph g, Scratch s, bool wi
   pdl_enter();
   __shared__ unsigned long long tot[2][kBlock / 32];   // the prefix's sums, the words' sums
   const long long n = g.n;
-  if (with_cycles) {
+  const bool stop = gave_up(s.derr);
+  const unsigned cyc = with_cycles ? *(volatile unsigned*)&s.ctr->n_cycle_reads : 0u;   // the same for every block
+  if (__syncthreads_or(stop)) return;
+  if (cyc > 0) {
     Counters* c = s.ctr;
-    const unsigned C = *(volatile unsigned*)&c->n_cycle_reads;   // the same for every block
-    if (C > 0) {
-      close_cycles(g, s, C, grid_tid(), grid_threads(), [&] { return grid_sync(c, s.derr); });
-      if (!grid_sync(c, s.derr)) return;
-    }
+    close_cycles(g, s, cyc, grid_tid(), grid_threads(), [&] { return grid_sync(c, s.derr); });
+    if (!grid_sync(c, s.derr)) return;
   }
   for (long long i = grid_tid(); i <= s.scan_tiles_cap; i += grid_threads()) s.scan_state[i] = 0ull;   // of the piece scan
   const int tid = threadIdx.x;
@@ -134,7 +134,9 @@ __global__ void __launch_bounds__(kBlock) k_pieces(Scratch s, PieceStore ps) {
   __shared__ unsigned long long tot[kBlock / 32];
   __shared__ long long s_tile;
   const int tid = threadIdx.x;
+  const bool stop = gave_up(s.derr);
   const long long W = *(const volatile unsigned*)&s.ctr->n_walk;
+  if (__syncthreads_or(stop)) return;
   const long long tiles = (W + kPieceTile - 1) / kPieceTile;
   if (blockIdx.x == 0 && tid < kTicketSets) s.tickets[kTicketStride * tid] = 0ull;   // for a spelling right after
   if ((long long)blockIdx.x >= tiles) return;
@@ -174,7 +176,7 @@ __global__ void __launch_bounds__(kBlock) k_pieces(Scratch s, PieceStore ps) {
 
 __global__ void k_scatter(DevGraph g, Scratch s) {
   pdl_enter();
-  scatter_reads(g, s, grid_tid(), grid_threads());
+  scatter_reads(g, s, gave_up(s.derr), grid_tid(), grid_threads());
 }
 
 // An empty graph: no contigs, and the one offset 0.
@@ -193,6 +195,7 @@ __global__ void k_export_contig_off(Scratch s, int64_t* out, long long cap) {
   pdl_enter();
   Counters* c = s.ctr;
   long long C = *(volatile unsigned*)&c->n_contigs;
+  if (gave_up(s.derr)) return;
   if (C + 1 > cap) {
     if (grid_tid() == 0) set_error(s.derr, DERR_CAPACITY, K_CONTIG_OFF, C + 1);
     return;
@@ -325,7 +328,8 @@ struct HistStore {
 // in earlier rounds, in earlier warps of this round and in earlier lanes.
 __global__ void k_sort_scatter(const unsigned long long* key_in, const int32_t* val_in, unsigned long long* key_out,
                                int32_t* val_out, long long C, int pass, const unsigned long long* base,
-                               long long tiles) {
+                               long long tiles, const DevError* derr) {
+  if (gave_up(derr)) return;                         // the scan did: base is not whole
   __shared__ unsigned running[256];
   __shared__ unsigned wcnt[kBlock / 32][256];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -576,8 +580,10 @@ __device__ __forceinline__ bool part_sync_or(int count, bool x) {
 template <typename K>
 __global__ void __launch_bounds__(kMaxParts) k_lpt_assign(const unsigned long long* key, const int32_t* val, long long C,
                                                           unsigned long long kmax, int P, int G, int part_bits,
-                                                          int chunk, int32_t* part, int64_t* psum) {
+                                                          int chunk, int32_t* part, int64_t* psum,
+                                                          const DevError* derr) {
   pdl_enter();
+  if (gave_up(derr)) return;                               // a scan of the sort did: val is not whole
   __shared__ __align__(16) K keys[kMaxParts];              // by part
   __shared__ K old_key[kMaxParts], new_key[kMaxParts];     // by rank
   extern __shared__ __align__(16) unsigned char staged[];
@@ -677,8 +683,9 @@ constexpr int kLptSorted = 4, kLptWarp = 19;
 template <int M>
 __global__ void __launch_bounds__(kBlock) k_lpt_few(const unsigned long long* key, const int32_t* val, long long C,
                                                     unsigned long long kmax, int P, int part_bits, int chunk,
-                                                    int32_t* part, int64_t* psum) {
+                                                    int32_t* part, int64_t* psum, const DevError* derr) {
   pdl_enter();
+  if (gave_up(derr)) return;                           // a scan of the sort did: val is not whole
   extern __shared__ __align__(16) unsigned char staged[];
   unsigned long long* const w = reinterpret_cast<unsigned long long*>(staged);
   short* const to = reinterpret_cast<short*>(w + chunk);
@@ -845,7 +852,7 @@ cudaError_t launch_partition(const Scratch& s, long long C, int weight, long lon
                                                               b.state, b.state_cap, s.derr, K_SORT);
       mark(env, "k_scan_digits");
       k_sort_scatter<<<grid, kBlock, 0, env.stream>>>(b.key[cur], b.val[cur], b.key[cur ^ 1], b.val[cur ^ 1], C,
-                                                      pass, b.base, tiles);
+                                                      pass, b.base, tiles, s.derr);
       mark(env, "k_sort_scatter");
       cur ^= 1;
     }
@@ -861,7 +868,7 @@ cudaError_t launch_partition(const Scratch& s, long long C, int weight, long lon
   if (P <= kLptWarp) {
     auto* const kernel = P <= 2 ? k_lpt_few<2> : P <= kLptSorted ? k_lpt_few<4> : k_lpt_few<0>;
     const int chunk = lpt_chunk(C, 8);
-    e = lpt_launch(kernel, chunk, 8, kBlock, env, kk, vv, C, kmax, P, part_bits, chunk, part, psum);
+    e = lpt_launch(kernel, chunk, 8, kBlock, env, kk, vv, C, kmax, P, part_bits, chunk, part, psum, s.derr);
   } else {
     // threads per part: as many as 512 threads allow, and no more than there are
     // vectors of keys (72 parts: 161 us with one, 125 with four, 131 with eight)
@@ -869,9 +876,10 @@ cudaError_t launch_partition(const Scratch& s, long long C, int weight, long lon
     while (2 * G * P <= 512 && 2 * G <= (P + 3) / 4) G *= 2;
     const int threads = std::max(256, (P * G + 31) & ~31);   // enough of them to stage the weights
     const int chunk = lpt_chunk(C, narrow ? 4 : 8);
-    e = narrow ? lpt_launch(k_lpt_assign<uint32_t>, chunk, 4, threads, env, kk, vv, C, kmax, P, G, part_bits, chunk, part, psum)
+    e = narrow ? lpt_launch(k_lpt_assign<uint32_t>, chunk, 4, threads, env, kk, vv, C, kmax, P, G, part_bits, chunk, part, psum,
+                            s.derr)
                : lpt_launch(k_lpt_assign<unsigned long long>, chunk, 8, threads, env, kk, vv, C, kmax, P, G, part_bits, chunk,
-                            part, psum);
+                            part, psum, s.derr);
   }
   if (e != cudaSuccess) return e;
   mark(env, "k_lpt_assign");

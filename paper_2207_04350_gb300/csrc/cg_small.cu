@@ -252,7 +252,7 @@ __device__ void offsets_stage(const DevGraph& g, const Scratch& s, const PieceSt
   }
   if (tid < kTicketSets) s.tickets[kTicketStride * tid] = 0ull;   // for a spelling right after
   __syncthreads();
-  scatter_reads(g, s, tid, kThreads);
+  scatter_reads(g, s, false, tid, kThreads);
   __syncthreads();
   // piece offsets, four positions per thread at a time
   unsigned long long run = 0;

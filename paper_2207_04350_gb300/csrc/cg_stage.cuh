@@ -15,24 +15,27 @@ constexpr long long kSpinLimit = 1ll << 22;   // barrier polls before giving up 
 
 // Software grid barrier for kernels launched cooperatively (all blocks
 // co-resident). Bounded: a block that waits too long records DERR_TIMEOUT and
-// every block returns false from then on.
+// every block returns false from then on. A block that has seen that arrives at no
+// further barrier: an arrival of its own would let the others pass one that a block
+// still at work has not reached.
 __device__ bool grid_sync(Counters* c, DevError* e) {
   __shared__ int ok;
   __syncthreads();
   if (threadIdx.x == 0) {
-    ok = 1;
     volatile unsigned* gen = &c->bar_gen;
     unsigned g0 = *gen;
+    ok = !gave_up(e);
     __threadfence();
-    unsigned arrived = atomicAdd(&c->bar_count, 1u);
-    if (arrived == gridDim.x - 1) {
+    unsigned arrived = ok ? atomicAdd(&c->bar_count, 1u) : 0u;
+    if (!ok) {
+    } else if (arrived == gridDim.x - 1) {
       c->bar_count = 0;
       __threadfence();
       atomicAdd(&c->bar_gen, 1u);
     } else {
       long long spins = 0;
       while (*gen == g0) {
-        if (++spins > kSpinLimit || *(volatile int*)&e->err == DERR_TIMEOUT) {
+        if (++spins > kSpinLimit || gave_up(e)) {
           set_error(e, DERR_TIMEOUT, K_JUMP, spins);
           ok = 0;
           break;
@@ -313,14 +316,16 @@ struct PieceStore {
 // stage (each its own contig, whole and forward) and the candidates with a
 // contig in their record (chains long enough, and reads cut off by branch
 // reads when those are spelled alone). A thread takes two reads at a time and
-// issues each level of their dependent loads together, before any store.
+// issues each level of their dependent loads together, before any store. Nothing
+// with `stop` (gave_up).
 constexpr int kScatterItems = 2;
 
-__device__ __forceinline__ void scatter_reads(const DevGraph& g, const Scratch& s, long long tid, long long T) {
+__device__ __forceinline__ void scatter_reads(const DevGraph& g, const Scratch& s, bool stop, long long tid,
+                                              long long T) {
   Counters* c = s.ctr;
   const long long L1 = *(volatile unsigned*)&c->n_lone, NC = *(volatile unsigned*)&c->n_cand;
   const long long W = *(volatile unsigned*)&c->n_walk;
-  const long long total = L1 + NC;
+  const long long total = stop ? 0 : L1 + NC;
   for (long long k0 = tid; k0 < total; k0 += kScatterItems * T) {
     long long k[kScatterItems];
     int32_t v[kScatterItems];

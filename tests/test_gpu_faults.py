@@ -14,6 +14,11 @@ import pytest
 import gen
 import oracle
 from paper_2207_04350_gb300 import cg
+from tests._exchange import without_reads
+from tests._graphs import structured
+
+torch = pytest.importorskip("torch")
+I32, I64 = torch.int32, torch.int64
 
 pytestmark = pytest.mark.gpu
 
@@ -91,6 +96,60 @@ def test_injected_failure(tiny, site, at, status, sticky):
             assert e2.value.status == status
         else:
             exact(ctx, G, orc)                   # the same context goes on
+    finally:
+        ctx.close()
+    fresh = cg.cg_create(0)
+    try:
+        exact(fresh, G, orc)
+    finally:
+        fresh.close()
+
+
+# What each call that writes outputs is given: the load's flags, then the outputs' sizes
+# in bytes from (reads, contigs, bases), then the call.
+AFTER_A_TIMEOUT = {
+    "contigs": (0, lambda n, c, b: (8 * (c + 1), b + 16),
+                lambda g, o: cg.cg_emit_contigs(g, o[0].view(I64), o[1], want_counts=False)),
+    "contigs-after-chains": (0, lambda n, c, b: (8 * (c + 1), b + 16),
+                             lambda g, o: (cg.cg_chains(g, want_counts=False),
+                                           cg.cg_emit_contigs(g, o[0].view(I64), o[1], want_counts=False))),
+    "offsets": (0, lambda n, c, b: (8 * (c + 1),),
+                lambda g, o: cg.cg_emit_contigs(g, o[0].view(I64), None, want_counts=False)),
+    "2bit": (0, lambda n, c, b: (8 * (c + 1), 16 * (b // 64 + 1)),
+             lambda g, o: cg.cg_emit_contigs_2bit(g, o[0].view(I64), o[1], want_counts=False)),
+    "share": (0, lambda n, c, b: (8 * (c + 1), b + 16),
+              lambda g, o: cg.cg_emit_share(g, 0, 2, o[0].view(I64), o[1], want_range=False)),
+    "reads": (0, lambda n, c, b: (4 * n, 4 * n, n),
+              lambda g, o: cg.cg_chains(g, o[0].view(I32), o[1].view(I32), o[2], want_counts=False)),
+    "part": (0, lambda n, c, b: (4 * c, 8 * 24),
+             lambda g, o: cg.cg_partition_contigs(g, 24, part=o[0].view(I32), part_weight=o[1].view(I64))),
+    "exchange": (cg.NO_READS, lambda n, c, b: (), lambda g, o: cg.cg_exchange_sizes(g, 2, [0, g.n // 2, g.n], 0)),
+}
+
+
+@pytest.mark.parametrize("graphs", [True, False])
+@pytest.mark.parametrize("call", list(AFTER_A_TIMEOUT))
+def test_nothing_runs_on_after_a_wait_that_gave_up(tiny, call, graphs):
+    """A grid barrier that gave up leaves contig records unwritten, which the later
+    kernels would use as indices: with the error word as it leaves it, on a graph with
+    a chain long enough for the barrier and with closed chains, no output is written,
+    the next wait reports CG_ETIMEOUT and a fresh context is bit-exact."""
+    flags, sizes, run = AFTER_A_TIMEOUT[call]
+    G = structured(23, [30] * 800 + [6000] + [900] * 3, closed=[False] * 801 + [True] * 3)
+    orc = oracle.run(G, min_chain_reads=2)
+    out = [torch.full((b,), 0xA5, dtype=torch.uint8, device="cuda")
+           for b in sizes(G.n, len(orc.contig_off) - 1, len(orc.bases))]
+    ctx = cg.cg_create(0)
+    try:
+        cg.cg_set_graphs(ctx, graphs)
+        g = cg.cg_load_graph(ctx, without_reads(G) if flags & cg.NO_READS else G, flags=flags, min_chain_reads=2)
+        cg.cg_set_fault(ctx, "barrier:1")
+        with pytest.raises(cg.CgError) as e:
+            run(g, out)
+            cg.cg_sync(ctx)
+        assert e.value.status == cg.CG_ETIMEOUT
+        assert all(bool((t == 0xA5).all()) for t in out)
+        g.close()
     finally:
         ctx.close()
     fresh = cg.cg_create(0)
