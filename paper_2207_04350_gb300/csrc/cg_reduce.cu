@@ -500,8 +500,9 @@ cudaError_t launch_transitive(const DevGraph& g, int fuzz, const TrBuffers& t, c
   mark(env, "k_tr_check");
   if (g.m > 0) {
     static const int pack_resident = resident_blocks(k_tr_pack), rows_resident = resident_blocks(k_tr_rows);
-    // persistent grids; no more batches than rows with entries
-    const long long need = std::min((long long)g.n, (long long)g.m);
+    // persistent grids; no more batches than rows with entries, and one block for a
+    // graph that has entries but no reads: the row check has refused it by then
+    const long long need = std::max(1ll, std::min((long long)g.n, (long long)g.m));
     cudaError_t e = launch_k(k_tr_pack, (int)std::min(need, (long long)env.num_sms * pack_resident), env, true, g, t);
     if (e != cudaSuccess) return e;
     mark(env, "k_tr_pack");

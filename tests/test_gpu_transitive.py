@@ -162,6 +162,19 @@ def test_missing_or_foreign_mirrors(ctx):
     assert e.value.status == cg.CG_EGRAPH
 
 
+def test_entries_without_reads(ctx):
+    """Entries of a graph that has no reads: refused as an invalid graph, whatever the
+    offsets say, and the context goes on."""
+    G = random_overlaps(5, 200, 900)
+    for rp in ([0], [3], [G.m]):
+        H = type("R", (), dict(vars(G)))()
+        H.row_ptr, H.len, H.off, H.n = np.array(rp, np.int64), G.len[:0], G.off[:0], 0
+        with pytest.raises(cg.CgError) as e:
+            cg.cg_transitive_reduction(ctx, H)
+        assert e.value.status == cg.CG_EGRAPH
+        assert same_csr(cg.cg_transitive_reduction(ctx, G), oracle.transitive_reduction(G))
+
+
 @pytest.mark.parametrize("hub", [0, 1600])
 @pytest.mark.parametrize("flip", [1, 2, 3])
 def test_pairs_whose_ends_disagree(ctx, hub, flip):
