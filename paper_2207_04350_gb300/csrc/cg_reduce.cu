@@ -69,8 +69,8 @@ __device__ __forceinline__ void load4_rows(const DevGraph& g, long long i, bool 
   }
 }
 
-// Rows: offsets from 0 to m that never decrease, every read at least one base
-// long. Lists the rows with entries (read, first entry, entries), one
+// Rows: offsets from 0 to m that never decrease, no more entries in a row than
+// other reads, every read at least one base long. Lists the rows with entries (read, first entry, entries), one
 // reservation per block, with a record per such read and a bit in a map of them.
 // Reads every row offset and length once, 12 B per read, four consecutive reads
 // per thread by 16-byte loads where the arrays allow.
@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(kBlock) k_tr_check(DevGraph g, TrBuffers t, bo
   for (int k = 0; k < kTrRows; ++k) {
     if (u0 + k >= g.n) continue;
     const int64_t b = k + 1 < kTrRows ? a[k + 1 < kTrRows ? k + 1 : 0] : next;
-    if (a[k] < 0 || b < a[k] || b > g.m || len[k] < 1) set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, u0 + k);
+    if (!row_ok(a[k], b, g.m, g.n, len[k])) set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, u0 + k);
     else if (b > a[k]) full |= 1u << k;
   }
   // the bits of eight threads make a word of the map

@@ -1,5 +1,5 @@
-// cg_search.h - the search in a sorted row of a graph, for kernels and for host
-// code (which tests it on bounds that no test graph reaches).
+// cg_search.h - the check of a row of a graph and the search in a sorted one, for
+// kernels and for host code (which tests them on bounds that no test graph reaches).
 #pragma once
 
 #include <cstdint>
@@ -24,6 +24,14 @@ CG_HOST_DEVICE int32_t find_col(const Col& col, int32_t a, int32_t b, int32_t w)
     else hi = mid;
   }
   return lo < b && col[lo] == w ? lo : -1;
+}
+
+// Whether the row of entries [a, b) of a graph of m entries and n reads can be that
+// of a read of `len` bases: offsets in range and in order, at least one base, and no
+// more entries than there are other reads. The last keeps what a kernel counts over
+// one row far from the largest int, whatever offsets a malformed graph has.
+CG_HOST_DEVICE bool row_ok(int64_t a, int64_t b, int64_t m, int64_t n, int32_t len) {
+  return a >= 0 && b >= a && b <= m && b - a < n && len >= 1;
 }
 
 }  // namespace cg

@@ -1,7 +1,8 @@
-"""The reduction's search in a sorted row (csrc/cg_search.h), compiled for the
-host: every column of rows at the first, middle and last entries that the call
-accepts (2^31 - 1 of them), with a column reader that refuses any index outside
-the row. No graph of that size is made."""
+"""The reduction's search in a sorted row and its check of a row's offsets
+(csrc/cg_search.h), compiled for the host: every column of rows at the first,
+middle and last entries that the call accepts (2^31 - 1 of them), with a column
+reader that refuses any index outside the row, and offsets at the same bounds. No
+graph of that size is made."""
 import os
 import subprocess
 
@@ -26,6 +27,9 @@ struct Row {
   }
 };
 int main(int argc, char** argv) {
+  if (argc == 6)
+    return cg::row_ok(std::atoll(argv[1]), std::atoll(argv[2]), std::atoll(argv[3]), std::atoll(argv[4]),
+                      (int32_t)std::atoll(argv[5])) ? 0 : 1;
   const Row r{(int32_t)std::atoll(argv[1]), (int32_t)std::atoll(argv[2])};
   for (int32_t w = 0; w <= 2 * (r.b - r.a) + 4; ++w) {
     const bool in = w >= 3 && (w & 1) && (w - 3) / 2 < r.b - r.a;
@@ -55,3 +59,14 @@ def program(tmp_path_factory):
 def test_every_column_of_a_row(program, a, length):
     r = subprocess.run([program, str(a), str(a + length)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
+
+
+@pytest.mark.parametrize("a,b,m,n,length,ok", [
+    (0, 0, 0, 1, 1, True), (0, 3, 8, 4, 1, True), (5, 8, 8, 4, 9, True), (0, 3, 8, 4, 0, False),
+    (-1, 2, 8, 4, 1, False), (4, 3, 8, 4, 1, False), (6, 9, 8, 4, 1, False),
+    (0, 4, 8, 4, 1, False), (0, 1, 8, 1, 1, False),                     # as many entries as reads
+    (0, (1 << 31) - 1, (1 << 31) - 1, 1, 1, False), (0, (1 << 31) - 1, (1 << 31) - 1, (1 << 30) - 1, 1, False),
+    (1 << 30, (1 << 31) - 2, (1 << 31) - 1, (1 << 30) - 1, 1, True)])
+def test_rows_a_read_can_have(program, a, b, m, n, length, ok):
+    r = subprocess.run([program, str(a), str(b), str(m), str(n), str(length)])
+    assert (r.returncode == 0) == ok
