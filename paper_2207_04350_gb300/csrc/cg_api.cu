@@ -1918,8 +1918,10 @@ cg_status cg_transitive_reduction(cg_ctx* c, const cg_graph_desc* d, int32_t fuz
   G.len = (const int32_t*)in(d->len, (size_t)n * 4);
   cg::TrBuffers t{};
   const size_t tiles = (size_t)cg::transitive_tiles(m);
-  t.rows_cap = std::min(n, m);
+  t.rows_cap = cg::transitive_pieces(n, m);
   t.rows = (int4*)alloc((size_t)t.rows_cap * sizeof(int4));
+  t.units_cap = cg::transitive_units(n, m);
+  t.unit_first = (unsigned*)alloc((size_t)t.units_cap * sizeof(unsigned));
   t.info = (int4*)alloc((size_t)n * sizeof(int4));
   t.has = (unsigned*)alloc(((size_t)n + 31) / 32 * 4);
   t.ent = (uint2*)alloc((size_t)m * sizeof(uint2));
@@ -1929,7 +1931,7 @@ cg_status cg_transitive_reduction(cg_ctx* c, const cg_graph_desc* d, int32_t fuz
   t.before = (unsigned*)alloc(tiles * 64 * 4);
   t.tile_cnt = (unsigned*)alloc(tiles * 4);
   t.total = (unsigned long long*)alloc(16);
-  t.n_rows = t.total ? (unsigned*)(t.total + 1) : nullptr;
+  t.listed = t.total ? t.total + 1 : nullptr;
   t.derr = c->derr;
   // device outputs are written in place; an offset array that is not 8-byte aligned gets a copy
   const bool device_out = want && mem == CG_MEM_DEVICE;

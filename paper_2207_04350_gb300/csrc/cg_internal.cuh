@@ -343,9 +343,11 @@ struct SortBuffers {
 };
 // Buffers of the transitive reduction (m entries, n rows).
 struct TrBuffers {
-  int4* rows;                  // rows with entries: (read, first entry, entries)
-  long long rows_cap;          // at most min(n, m)
-  unsigned* n_rows;
+  int4* rows;                  // the list of rows with entries: (read, first entry, entries), long rows in pieces
+  long long rows_cap;          // transitive_pieces(n, m)
+  unsigned* unit_first;        // per unit of the list's weight, the first piece that starts in it
+  long long units_cap;         // transitive_units(n, m)
+  unsigned long long* listed;  // pieces listed << 33 | their half weights
   int4* info;                  // n, set for rows with entries: first entry, first of the second run, end, read length
   unsigned* has;               // n bits: the read has entries
   uint2* ent;                  // m: each row in two runs by the end its entries leave through, (column << 2 | code, suffix)
@@ -358,6 +360,8 @@ struct TrBuffers {
   DevError* derr;
 };
 long long transitive_tiles(long long m);
+long long transitive_pieces(long long n, long long m);
+long long transitive_units(long long n, long long m);
 // TransitiveReduction: checks, marks, keeps and counts (launch_transitive), then
 // writes the kept entries and the new row offsets, unless they are more than
 // `cap` (launch_transitive_scatter). After a failed check the later kernels do

@@ -8,12 +8,14 @@
 // both entries only when neither is transitive.
 //
 // Rows hold a few entries and most reads none, so the rows with entries are
-// listed first, and every row's entries are copied in two runs, those that leave
+// listed first, long ones in pieces, and the list is cut into batches of about as
+// many entries. Every row's entries are copied in two runs, those that leave
 // the read through its 5' end and those that leave through the other, each packed
-// into eight bytes. Then a block takes a batch of listed rows, stages them in
+// into eight bytes. Then a block takes a batch of the list, stages it in
 // shared memory and gives every entry (u->v) a thread, which walks the run of
 // v's row that leaves v through the other end: every entry of it is a walk u ->
-// v -> w, whose w is looked up in u's staged row. Everything after that is per
+// v -> w, whose w is looked up in u's staged row (in memory when u's row is listed
+// in pieces). Everything after that is per
 // entry: an entry is kept when neither it nor its mirror is transitive; the kept
 // entries are bits of one map over all entries with the count of those before
 // each word, and since entries lie in row order that count places both the kept
@@ -35,11 +37,36 @@ namespace {
 
 constexpr int kTrTile = 2048;        // entries of one tile of the map: 64 words
 constexpr int kTrRows = 4;           // consecutive rows per thread of the row pass
-constexpr int kTrBatch = 120;        // listed rows a block takes at a time, at most
-constexpr int kTrAim = 960;          // entries a batch of the packing aims at: just under four per thread
-constexpr int kTrStage = 2048;       // entries of such a batch that are ranked in shared memory
-constexpr int kTrAimRows = 720;      // the same for the walks, just under three per thread: the less shared
-constexpr int kTrHold = 1536;        // memory the blocks of an SM hold, the more cache the random rows have
+// The list of rows. A row of more than kTrPiece entries is listed as pieces of that
+// many, so that any piece fits the staging of a batch behind others. A piece weighs
+// its entries, kTrFloor at least: a batch is a run of the list of kTrPackUnits or
+// kTrWalkUnits units of weight, from the first piece that starts in it on, which
+// bounds both its entries and its pieces however long the rows are and whichever lie
+// side by side. Batches of so many rows as hold 960 or 720 entries on average, with
+// rows past the staging counted and searched in place by their block, took as long on
+// the 3.1 Gb graph; with a row of 10,000 / 50,000 entries among 200 thousand of 8
+// k_tr_pack took 4.1 / 103 ms (40 / 48 us now), and with 1,000 rows of 999 side by
+// side k_tr_rows 97 ms (5.4). With a floor of 8 a batch holds 6% fewer of the 3.1 Gb
+// graph's entries: 53.5 and 143 us for 51.5 and 141.
+constexpr int kTrPiece = 768;
+constexpr int kTrUnitLog2 = 7;       // a unit: 2^7 half weights, 256 entries
+constexpr int kTrPackUnits = 4;      // just under four entries per thread
+constexpr int kTrWalkUnits = 3;      // three: the less shared memory the blocks of an SM hold, the more cache the random rows have
+constexpr int kTrFloor = 6;          // entries that a piece counts as, at least
+constexpr int most_pieces(int units) { return ((units << kTrUnitLog2) - 1) / ((kTrFloor + 1) / 2) + 1; }
+constexpr int kTrPackRows = most_pieces(kTrPackUnits), kTrWalkRows = most_pieces(kTrWalkUnits);   // pieces of a batch, at most
+constexpr int kTrStage = 2048;       // entries of a batch of the packing, at most
+constexpr int kTrHold = 1536;        // of the walks
+static_assert((2 * kTrPackUnits << kTrUnitLog2) + kTrPiece <= kTrStage && (2 * kTrWalkUnits << kTrUnitLog2) + kTrPiece <= kTrHold,
+              "the units of a batch and a piece that starts in the last");
+static_assert(kTrPackRows <= 256 && kTrPackRows <= kBlock && kTrWalkRows <= 128, "find_row's steps, a thread per piece");
+constexpr int kTrPart = 1 << 30;     // flag beside the read: a piece of a row in pieces (reads stay below 2^30)
+constexpr int kTrHalfBits = 33;      // the list's counter: pieces above, half weights below
+constexpr unsigned long long kTrHalves = (1ull << kTrHalfBits) - 1;
+constexpr int kTrLocalBits = 20;     // the same of one block of the row pass, 1024 rows of one piece each at most
+static_assert(kBlock * kTrRows * (kTrPiece / 2) < 1 << kTrLocalBits && kBlock * kTrRows < 1 << (32 - kTrLocalBits), "");
+
+__device__ __forceinline__ int half_weight(int entries) { return (max(entries, kTrFloor) + 1) >> 1; }
 
 __device__ __forceinline__ bool failed(const DevError* e) { return *(const volatile int*)&e->err != 0; }
 
@@ -69,13 +96,52 @@ __device__ __forceinline__ void load4_rows(const DevGraph& g, long long i, bool 
   }
 }
 
+// Piece (u, first entry p, z entries) at place `slot` of the list, `half` half weights
+// before it; false when it does not fit: there are more pieces than the entries allow,
+// in rows that overlap, which the row check finds.
+__device__ __forceinline__ bool list_piece(const TrBuffers& t, unsigned slot, unsigned long long half, int u, int p, int z) {
+  if (slot >= (unsigned)t.rows_cap) {
+    set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, u & ~kTrPart);
+    return false;
+  }
+  t.rows[slot] = make_int4(u, p, z, 0);
+  unsigned unit = (unsigned)(half >> kTrUnitLog2);
+  int over = (int)((unsigned)half & ((1u << kTrUnitLog2) - 1u)) + half_weight(z) - (1 << kTrUnitLog2);
+  for (; over >= 0; over -= 1 << kTrUnitLog2) {        // units that start in the piece or right behind it
+    if (++unit >= (unsigned)t.units_cap) {
+      set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, u & ~kTrPart);
+      return false;
+    }
+    t.unit_first[unit] = slot + 1u;
+  }
+  return true;
+}
+
+// A row of more than kTrPiece entries, by one thread, with a reservation of its own.
+// Rows without end in an invalid graph are given up as soon as its error is set.
+__device__ __forceinline__ void list_long_row(const TrBuffers& t, int u, int a, int z) {
+  const int more = (z - 1) / kTrPiece, rest = z - more * kTrPiece;      // whole pieces before the last, its entries
+  unsigned long long at =
+      atomicAdd(t.listed, ((unsigned long long)(more + 1) << kTrHalfBits) +
+                              (unsigned long long)more * (kTrPiece / 2) + (unsigned long long)half_weight(rest));
+  for (int i = 0; i <= more; ++i) {
+    const int n = i < more ? kTrPiece : rest;
+    if (failed(t.derr) || !list_piece(t, (unsigned)(at >> kTrHalfBits), at & kTrHalves, u | kTrPart, a + i * kTrPiece, n))
+      return;
+    at += (1ull << kTrHalfBits) + (unsigned long long)half_weight(n);
+  }
+}
+
 // Rows: offsets from 0 to m that never decrease, no more entries in a row than
-// other reads, every read at least one base long. Lists the rows with entries (read, first entry, entries), one
-// reservation per block, with a record per such read and a bit in a map of them.
+// other reads, every read at least one base long. Lists the rows with entries (read,
+// first entry, entries; pieces of long ones), one reservation of places and weight
+// per block, and the first piece of every unit of weight, with a record per such read
+// and a bit in a map of them.
 // Reads every row offset and length once, 12 B per read, four consecutive reads
 // per thread by 16-byte loads where the arrays allow.
-__global__ void __launch_bounds__(kBlock) k_tr_check(DevGraph g, TrBuffers t, bool wide_rows, bool wide_len) {
-  __shared__ unsigned cnt, base;
+__global__ void __launch_bounds__(kBlock, 6) k_tr_check(DevGraph g, TrBuffers t, bool wide_rows, bool wide_len) {
+  __shared__ unsigned cnt;                             // of the block's rows of one piece: pieces << kTrLocalBits | half weights
+  __shared__ unsigned long long base;
   const long long u0 = ((long long)blockIdx.x * kBlock + threadIdx.x) * kTrRows;
   const int lane = threadIdx.x & 31;
   if (threadIdx.x == 0) cnt = 0;
@@ -86,48 +152,79 @@ __global__ void __launch_bounds__(kBlock) k_tr_check(DevGraph g, TrBuffers t, bo
   if (u0 < g.n) load4(g.len, u0, g.n, wide_len, len);
   int64_t next = __shfl_down_sync(0xffffffffu, a[0], 1);     // the offset after this thread's last row
   if (lane == 31) next = u0 + 4 <= g.n ? rowp(g, u0 + 4) : 0;
-  unsigned full = 0;
+  unsigned full = 0, mine = 0;
 #pragma unroll
   for (int k = 0; k < kTrRows; ++k) {
     if (u0 + k >= g.n) continue;
     const int64_t b = k + 1 < kTrRows ? a[k + 1 < kTrRows ? k + 1 : 0] : next;
-    if (!row_ok(a[k], b, g.m, g.n, len[k])) set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, u0 + k);
-    else if (b > a[k]) full |= 1u << k;
+    if (!row_ok(a[k], b, g.m, g.n, len[k])) {
+      set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, u0 + k);
+    } else if (b > a[k]) {
+      full |= 1u << k;
+      if (b - a[k] <= kTrPiece) mine += (1u << kTrLocalBits) + (unsigned)half_weight((int)(b - a[k]));
+    }
   }
   // the bits of eight threads make a word of the map
   unsigned bits = full << (4 * (lane & 7));
   for (int o = 1; o < 8; o <<= 1) bits |= __shfl_xor_sync(0xffffffffu, bits, o);
   if ((lane & 7) == 0 && u0 < g.n) t.has[u0 >> 5] = bits;
-  unsigned inc = __popc(full);
+  unsigned inc = mine;
   for (int o = 1; o < 32; o <<= 1) {
     const unsigned x = __shfl_up_sync(0xffffffffu, inc, o);
     if (lane >= o) inc += x;
   }
   unsigned at = 0;
   if (lane == 31 && inc) at = atomicAdd(&cnt, inc);
-  at = __shfl_sync(0xffffffffu, at, 31) + inc - __popc(full);
-  if (u0 == 0 && (a[0] != 0 || rowp(g, g.n) != g.m)) set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, -1);
+  at = __shfl_sync(0xffffffffu, at, 31) + inc - mine;
+  if (u0 == 0) {
+    if (a[0] != 0 || rowp(g, g.n) != g.m) set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, -1);
+    t.unit_first[0] = 0;
+  }
   __syncthreads();
-  if (threadIdx.x == 0) base = cnt ? atomicAdd(t.n_rows, cnt) : 0;
+  if (threadIdx.x == 0 && cnt)
+    base = atomicAdd(t.listed, ((unsigned long long)(cnt >> kTrLocalBits) << kTrHalfBits) + (cnt & ((1u << kTrLocalBits) - 1u)));
   __syncthreads();
-#pragma unroll
-  for (int k = 0; k < kTrRows; ++k) {
-    if (!((full >> k) & 1u)) continue;
-    const int64_t b = k + 1 < kTrRows ? a[k + 1 < kTrRows ? k + 1 : 0] : next;
-    const long long u = u0 + k, slot = (long long)base + at++;
-    if (slot < t.rows_cap) t.rows[slot] = make_int4((int)u, (int)a[k], (int)(b - a[k]), 0);
-    else set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, u);   // more rows with entries than entries: rows that overlap
-    t.info[u] = make_int4((int)a[k], 0, (int)b, len[k]);
+  const unsigned slot0 = (unsigned)(base >> kTrHalfBits);
+  const unsigned long long half0 = base & kTrHalves;
+  for (; full; full &= full - 1) {                     // few threads have more than one row to list
+    const int k = __ffs(full) - 1, u = (int)(u0 + k);
+    const int first = (int)(k == 0 ? a[0] : k == 1 ? a[1] : k == 2 ? a[2] : a[3]);
+    const int z = (int)(k == 0 ? a[1] : k == 1 ? a[2] : k == 2 ? a[3] : next) - first;
+    t.info[u] = make_int4(first, 0, first + z, k == 0 ? len[0] : k == 1 ? len[1] : k == 2 ? len[2] : len[3]);
+    if (z <= kTrPiece) {
+      list_piece(t, slot0 + (at >> kTrLocalBits), half0 + (at & ((1u << kTrLocalBits) - 1u)), u, first, z);
+      at += (1u << kTrLocalBits) + (unsigned)half_weight(z);
+    } else {
+      list_long_row(t, u, first, z);
+    }
   }
 }
 
-// A batch of listed rows: their records and the places of their entries in the
-// batch, row[j].w the first of row j. Returns the number of entries. Whole block.
-__device__ __forceinline__ int load_batch(const TrBuffers& t, long long b0, int rows, long long R, int4* row,
-                                          int* warp_tot) {
+// The list as batches of `units` units of weight: how many, and where one starts.
+struct TrList {
+  long long pieces, units;
+  int per;
+  const unsigned* unit_first;
+  __device__ TrList(const TrBuffers& t, int units_per_batch) : per(units_per_batch), unit_first(t.unit_first) {
+    const unsigned long long all = *t.listed;
+    pieces = (long long)(all >> kTrHalfBits);
+    units = (long long)((all & kTrHalves) >> kTrUnitLog2) + 1;
+  }
+  __device__ long long batches() const { return (units + per - 1) / per; }
+  __device__ long long first(long long batch) const {
+    return batch * per < units ? (long long)unit_first[batch * per] : pieces;
+  }
+};
+
+// A batch, pieces [r0, r1) of the list: their records and the places of their
+// entries in the batch, row[j].w the first of piece j. Returns the number of
+// entries; *parts: there are pieces of rows in pieces among them. Whole block.
+template <int kRows>
+__device__ __forceinline__ int load_batch(const TrBuffers& t, long long r0, long long r1, int4* row, int* warp_tot,
+                                          bool* parts) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   int4 mine = make_int4(0, 0, 0, 0);
-  if (tid < rows && b0 + tid < R) mine = t.rows[b0 + tid];
+  if (r0 + tid < r1) mine = t.rows[r0 + tid];          // at most kRows of them
   int inc = mine.z;
   for (int o = 1; o < 32; o <<= 1) {
     const int x = __shfl_up_sync(0xffffffffu, inc, o);
@@ -137,50 +234,68 @@ __device__ __forceinline__ int load_batch(const TrBuffers& t, long long b0, int 
   __syncthreads();
   int total = 0;
   mine.w = inc - mine.z;
-  for (int w = 0; w < (kTrBatch + 31) / 32; ++w) {
+  for (int w = 0; w < (kRows + 31) / 32; ++w) {
     if (w < warp) mine.w += warp_tot[w];
     total += warp_tot[w];
   }
-  if (tid < kTrBatch) row[tid] = mine;
-  __syncthreads();
+  if (tid < kRows) row[tid] = mine;
+  *parts = __syncthreads_or(mine.x & kTrPart) != 0;
   return total;
 }
 
-// The row of the batch's entry i (places past the last listed row start at the
-// batch's end).
+// The piece of the batch's entry i (places past the last piece start at the batch's
+// end).
+template <int kRows>
 __device__ __forceinline__ int find_row(const int4* row, int i) {
   int j = 0;
 #pragma unroll
-  for (int step = 64; step > 0; step >>= 1)
-    if (j + step < kTrBatch && row[j + step].w <= i) j += step;
+  for (int step = kRows > 128 ? 128 : 64; step > 0; step >>= 1)
+    if (((kRows & (kRows - 1)) == 0 || j + step < kRows) && row[j + step].w <= i) j += step;
   return j;
-}
-
-// Rows per batch: as many as hold about `aim` entries.
-__device__ __forceinline__ int batch_rows(long long m, long long R, int aim) {
-  return (int)max(1ll, min((long long)kTrBatch, aim * R / max(m, 1ll)));
 }
 
 // Entries: columns in range, increasing in the row, not the row's own read and a
 // read with entries; codes 0..3. Copies every row in two runs by the end its
 // entries leave through, each run in the row's order: 9 B read and 12 written per
 // entry. An entry's place in its run is the count of entries of that end before
-// it, from the ballots of the block's entries. Its loads wait on one another (row,
+// it, from the ballots of the block's entries; a piece of a long row adds those
+// of the rest of the row, counted by its block, a byte an entry. Its loads wait on one another (row,
 // code, column), so that warps hide them: with eight blocks on an SM, at 32
-// registers, 51 us for 3.38M entries, with six 56; batches of 720 and 480 entries
+// registers, 51 us for 3.36M entries, with six 56; batches of 720 and 480 entries
 // 53 and 56.
 __global__ void __launch_bounds__(kBlock, 8) k_tr_pack(DevGraph g, TrBuffers t) {
   pdl_enter();
-  __shared__ int4 row[kTrBatch];
+  __shared__ int4 row[kTrPackRows];
   __shared__ unsigned zeros[kTrStage / 32];            // per word of staged entries: entries leaving through end 0
   __shared__ int before[kTrStage / 32 + 1];            // the same before each word
+  __shared__ int rest_before[kTrPackRows], rest_all[kTrPackRows];   // pieces of long rows: entries of end 0 before the piece, in the row
   __shared__ int warp_tot[kBlock / 32];
   if (__syncthreads_or(failed(t.derr))) return;
   const int tid = threadIdx.x, lane = tid & 31;
-  const long long R = *t.n_rows;
-  const int rows = batch_rows(g.m, R, kTrAim);
-  for (long long b0 = (long long)blockIdx.x * rows; b0 < R; b0 += (long long)gridDim.x * rows) {
-    const int total = load_batch(t, b0, rows, R, row, warp_tot);
+  const TrList list(t, kTrPackUnits);
+  for (long long b = blockIdx.x; b < list.batches(); b += gridDim.x) {
+    bool parts;
+    const int total = load_batch<kTrPackRows>(t, list.first(b), list.first(b + 1), row, warp_tot, &parts);
+    if (parts) {
+      if (tid < kTrPackRows) rest_before[tid] = rest_all[tid] = 0;
+      __syncthreads();
+      for (int j = 0; j < kTrPackRows; ++j) {             // block-uniform
+        if (!(row[j].x & kTrPart)) continue;
+        const int4 iu = t.info[row[j].x & ~kTrPart];
+        unsigned zb = 0, za = 0;
+        for (unsigned y = (unsigned)iu.x + tid; y < (unsigned)iu.z; y += kBlock) {
+          const unsigned end0 = (g.code[y] & 1u) ^ 1u;
+          za += end0;
+          zb += y < (unsigned)row[j].y ? end0 : 0u;
+        }
+        za = __reduce_add_sync(0xffffffffu, za);
+        zb = __reduce_add_sync(0xffffffffu, zb);
+        if (lane == 0) {
+          atomicAdd(&rest_all[j], (int)za);
+          atomicAdd(&rest_before[j], (int)zb);
+        }
+      }
+    }
     constexpr int kPer = kTrStage / kBlock;
     unsigned cd[kPer];                                 // this thread's staged entries
 #pragma unroll
@@ -188,7 +303,7 @@ __global__ void __launch_bounds__(kBlock, 8) k_tr_pack(DevGraph g, TrBuffers t) 
       const int i = k * kBlock + tid;
       cd[k] = 4;
       if (i < total) {
-        const int j = find_row(row, i);
+        const int j = find_row<kTrPackRows>(row, i);
         cd[k] = g.code[row[j].y + (i - row[j].w)];
       }
       const unsigned z = __ballot_sync(0xffffffffu, i < total && (cd[k] & 1) == 0);
@@ -207,29 +322,26 @@ __global__ void __launch_bounds__(kBlock, 8) k_tr_pack(DevGraph g, TrBuffers t) 
       if (lane == 31) before[kTrStage / 32] = inc;
     }
     __syncthreads();
-    auto zeros_before = [&](int i) {                   // among the staged entries
+    auto zeros_before = [&](int i) {
       return before[i >> 5] + (i < kTrStage ? __popc(zeros[i >> 5] & ((1u << (i & 31)) - 1u)) : 0);
     };
     for (int i = tid; i < total; i += kBlock) {
-      const int j = find_row(row, i);
-      const int u = row[j].x, a = row[j].y, n = row[j].z, s0 = row[j].w, x = a + (i - s0);
+      const int j = find_row<kTrPackRows>(row, i);
+      const int u = row[j].x & ~kTrPart, n = row[j].z, s0 = row[j].w, x = row[j].y + (i - s0);
       const int32_t w = g.col[x];
       const unsigned c = g.code[x];
-      const bool ok = w >= 0 && w < g.n && w != u && c <= 3 && (i == s0 || g.col[x - 1] < w) &&
+      int a = row[j].y;                                // first entry of the row
+      // entries of end 0 before this one and in the row
+      int z = zeros_before(i) - zeros_before(s0), nz = zeros_before(s0 + n) - zeros_before(s0);
+      if (row[j].x & kTrPart) {
+        a = t.info[u].x;
+        z += rest_before[j];
+        nz = rest_all[j];
+        t.trans[x] = (uint8_t)(c << 1);                // the walks only set what they hit, from any block
+      }
+      const bool ok = w >= 0 && w < g.n && w != u && c <= 3 && (x == a || g.col[x - 1] < w) &&
                       ((t.has[w >> 5] >> (w & 31)) & 1u);
       if (!ok) set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, x);
-      int z, nz;                                       // entries of end 0 before this one and in the row
-      if (s0 + n <= kTrStage) {
-        z = zeros_before(i) - zeros_before(s0);
-        nz = zeros_before(s0 + n) - zeros_before(s0);
-      } else {
-        z = nz = 0;
-        for (int y = a; y < a + n; ++y) {
-          const int end0 = (g.code[y] & 1) == 0;
-          nz += end0;
-          z += y < x ? end0 : 0;
-        }
-      }
       if (i == s0) t.info[u].y = a + nz;
       const int at = (c & 1) == 0 ? a + z : a + nz + (x - a - z);
       t.ent[at] = make_uint2(((unsigned)w << 2) | (c & 3u), (unsigned)g.suf[x]);
@@ -251,11 +363,11 @@ __device__ __forceinline__ bool closes(unsigned cx, unsigned cy, unsigned cz, in
 // A block per batch of listed rows, a thread per entry y = (u->v): suffix in
 // [1, len-1]; from the smaller read's side, the pair's mirrors; and the entries
 // of u's row that a walk through v makes transitive. The look-ups are binary
-// searches in shared memory, except in rows past the staged entries of a batch,
-// which are searched in place. What bounds it is the records, runs and columns
+// searches in shared memory, except for the pieces of a long row, which search the
+// row in place. What bounds it is the records, runs and columns
 // of the rows v, which lie at random (a sector or two each), and issuing the
-// searches, in warps whose lanes walk runs of unequal length. 3.38M entries of
-// 420 thousand rows, by events: 143 us (178 with the four searches one after
+// searches, in warps whose lanes walk runs of unequal length. 3.36M entries of
+// 412 thousand rows, by events: 141 us (178 with the four searches one after
 // another; 157 with batches of 960 entries, 2,048 of them staged, and the mirror's
 // code read from its row instead of checked where the mirrors' flags are read). A
 // thread per entry walking whole rows and searching u's row in memory took 283,
@@ -263,41 +375,34 @@ __device__ __forceinline__ bool closes(unsigned cx, unsigned cy, unsigned cz, in
 // rows of a warp in step, took 476, most of its lanes waiting for longer rows; the
 // runs of a warp's entries laid end to end, so that no lane waits, 139 to 160 by
 // the entries in flight, for as many instructions as without.
-__global__ void __launch_bounds__(kBlock) k_tr_rows(DevGraph g, TrBuffers t, int fuzz) {
+__global__ void __launch_bounds__(kBlock, 6) k_tr_rows(DevGraph g, TrBuffers t, int fuzz) {
   pdl_enter();
-  __shared__ int4 row[kTrBatch];                       // read, first entry, entries, first of the batch's entries
+  __shared__ int4 row[kTrWalkRows];                       // read, first entry, entries, first of the batch's entries
   __shared__ unsigned key[kTrHold];                    // column << 2 | code
   __shared__ int32_t suf[kTrHold];
   __shared__ uint8_t row_of[kTrHold], hit[kTrHold];
   __shared__ int warp_tot[kBlock / 32];
   if (__syncthreads_or(failed(t.derr))) return;
   const int tid = threadIdx.x;
-  const long long R = *t.n_rows;
-  const int rows = batch_rows(g.m, R, kTrAimRows);
-  for (long long b0 = (long long)blockIdx.x * rows; b0 < R; b0 += (long long)gridDim.x * rows) {
-    const int total = load_batch(t, b0, rows, R, row, warp_tot);
+  const TrList list(t, kTrWalkUnits);
+  for (long long b = blockIdx.x; b < list.batches(); b += gridDim.x) {
+    bool parts;
+    const int total = load_batch<kTrWalkRows>(t, list.first(b), list.first(b + 1), row, warp_tot, &parts);
     for (int i = tid; i < total; i += kBlock) {
-      const int j = find_row(row, i);
+      const int j = find_row<kTrWalkRows>(row, i);
       const int x = row[j].y + (i - row[j].w);
-      if (row[j].w + row[j].z <= kTrHold) {
-        key[i] = ((unsigned)g.col[x] << 2) | g.code[x];
-        suf[i] = g.suf[x];
-        row_of[i] = (uint8_t)j;
-        hit[i] = 0;
-      } else {
-        t.trans[x] = (uint8_t)(g.code[x] << 1);
-      }
+      key[i] = ((unsigned)g.col[x] << 2) | g.code[x];
+      suf[i] = g.suf[x];
+      row_of[i] = (uint8_t)j;
+      hit[i] = 0;
     }
     __syncthreads();
     for (int i = tid; i < total; i += kBlock) {
-      // entry i is staged when its whole row is: then it lies below kTrHold with row_of set
-      int j = i < kTrHold ? row_of[i] : kTrBatch;
-      if (j >= kTrBatch || i < row[j].w || i >= row[j].w + row[j].z || row[j].w + row[j].z > kTrHold)
-        j = find_row(row, i);
-      const int u = row[j].x, a = row[j].y, n = row[j].z, s0 = row[j].w, y = a + (i - s0);
-      const bool staged = s0 + n <= kTrHold;
-      const unsigned e = staged ? key[i] : ((unsigned)g.col[y] << 2) | g.code[y];
-      const int32_t sy = staged ? suf[i] : g.suf[y];
+      const int j = row_of[i];
+      const int u = row[j].x & ~kTrPart, n = row[j].z, s0 = row[j].w, y = row[j].y + (i - s0);
+      const bool whole = (row[j].x & kTrPart) == 0;    // u's row is staged whole
+      const unsigned e = key[i];
+      const int32_t sy = suf[i];
       const int v = (int)(e >> 2);
       const unsigned cy = e & 3u;
       const int4 iv = t.info[v];                       // first entry, first of the second run, end, length
@@ -315,7 +420,7 @@ __global__ void __launch_bounds__(kBlock) k_tr_rows(DevGraph g, TrBuffers t, int
         uint2 q[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) q[k] = z + k < z1 ? t.ent[z + k] : make_uint2(0u, 0u);
-        if (staged) {                                  // the four searches step together
+        if (whole) {                                   // the four searches step together
           int lo[4] = {s0, s0, s0, s0};                // the last column <= w, or the first one
           for (int len = n; len > 1;) {
             const int half = len >> 1;
@@ -331,10 +436,11 @@ __global__ void __launch_bounds__(kBlock) k_tr_rows(DevGraph g, TrBuffers t, int
               hit[lo[k]] = 1;
           }
         } else {
+          const int4 iu = t.info[u];
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             if (z + k >= z1) break;
-            const int32_t x = find_col(g.col, a, a + n, (int32_t)(q[k].x >> 2));
+            const int32_t x = find_col(g.col, iu.x, iu.z, (int32_t)(q[k].x >> 2));
             if (x >= 0 && closes(g.code[x], cy, q[k].x, g.suf[x], sy, (int32_t)q[k].y, fuzz))
               t.trans[x] = (uint8_t)(1u | (g.code[x] << 1));
           }
@@ -342,10 +448,9 @@ __global__ void __launch_bounds__(kBlock) k_tr_rows(DevGraph g, TrBuffers t, int
       }
     }
     __syncthreads();
-    for (int i = tid; i < min(total, kTrHold); i += kBlock) {
-      const int j = row_of[i];                         // set when i is staged
-      if (j < kTrBatch && i >= row[j].w && i < row[j].w + row[j].z && row[j].w + row[j].z <= kTrHold)
-        t.trans[row[j].y + (i - row[j].w)] = (uint8_t)(hit[i] | ((key[i] & 3u) << 1));
+    for (int i = tid; i < total; i += kBlock) {
+      const int j = row_of[i];
+      if ((row[j].x & kTrPart) == 0) t.trans[row[j].y + (i - row[j].w)] = (uint8_t)(hit[i] | ((key[i] & 3u) << 1));
     }
     __syncthreads();
   }
@@ -490,19 +595,25 @@ __global__ void __launch_bounds__(kBlock) k_tr_scatter(DevGraph g, TrBuffers t, 
 }  // namespace
 
 long long transitive_tiles(long long m) { return (m + kTrTile - 1) / kTrTile; }
+// Pieces: a row gives one more than its whole multiples of kTrPiece. Units: a piece of
+// z entries weighs at most z / 2 + 4 halves.
+long long transitive_pieces(long long n, long long m) { return std::min(n, m) + m / kTrPiece; }
+long long transitive_units(long long n, long long m) {
+  return ((m / 2 + 1 + 4 * transitive_pieces(n, m)) >> kTrUnitLog2) + 2;
+}
 
 cudaError_t launch_transitive(const DevGraph& g, int fuzz, const TrBuffers& t, const LaunchEnv& env) {
-  cudaMemsetAsync(t.n_rows, 0, sizeof(unsigned), env.stream);
   cudaMemsetAsync(t.total, 0, sizeof(unsigned long long), env.stream);
+  cudaMemsetAsync(t.listed, 0, sizeof(unsigned long long), env.stream);
   const long long blocks = std::max(1ll, ((long long)g.n + kTrRows * kBlock - 1) / (kTrRows * kBlock));
   k_tr_check<<<(unsigned)blocks, kBlock, 0, env.stream>>>(g, t, (reinterpret_cast<uintptr_t>(g.row_ptr) & 15) == 0,
                                                               (reinterpret_cast<uintptr_t>(g.len) & 15) == 0);
   mark(env, "k_tr_check");
   if (g.m > 0) {
     static const int pack_resident = resident_blocks(k_tr_pack), rows_resident = resident_blocks(k_tr_rows);
-    // persistent grids; no more batches than rows with entries, and one block for a
-    // graph that has entries but no reads: the row check has refused it by then
-    const long long need = std::max(1ll, std::min((long long)g.n, (long long)g.m));
+    // persistent grids; no more batches than units, and one block for a graph that has
+    // entries but no reads: the row check has refused it by then
+    const long long need = std::max(1ll, t.units_cap);
     cudaError_t e = launch_k(k_tr_pack, (int)std::min(need, (long long)env.num_sms * pack_resident), env, true, g, t);
     if (e != cudaSuccess) return e;
     mark(env, "k_tr_pack");

@@ -100,14 +100,18 @@ def test_on_device_to_contigs(ctx):
     assert np.array_equal(off, orc.contig_off) and np.array_equal(bases, orc.bases)
 
 
-def random_overlaps(seed, n, pairs, hub=0):
+def random_overlaps(seed, n, pairs, hub=0, hubs=(0,), clique=0):
     """Overlaps of random pairs among n reads, codes at random, suffixes of 1 to 4
-    bases (so that many two-step walks add up); with `hub`, read 0 overlaps that
-    many others."""
+    bases (so that many two-step walks add up); with `hub`, each of the reads `hubs`
+    overlaps that many others, with `clique` the first so many reads all overlap."""
     rng = np.random.default_rng(seed)
     u, v = rng.integers(0, n, size=(2, pairs))
-    if hub:
-        u, v = np.concatenate([u, np.zeros(hub, np.int64)]), np.concatenate([v, np.arange(1, hub + 1)])
+    for h in hubs if hub else ():
+        others = np.delete(np.arange(n), h)[:hub]
+        u, v = np.concatenate([u, np.full(hub, h)]), np.concatenate([v, others])
+    if clique:
+        a, b = np.triu_indices(clique, 1)
+        u, v = np.concatenate([u, a]), np.concatenate([v, b])
     keep = u != v
     key = np.unique(np.minimum(u, v)[keep] * n + np.maximum(u, v)[keep])
     u, v = key // n, key % n
@@ -136,6 +140,19 @@ def random_overlaps(seed, n, pairs, hub=0):
 ])
 def test_row_shapes(ctx, n, pairs, hub):
     G = random_overlaps(n + hub, n, pairs, hub)
+    for fuzz in (0, 1):
+        assert same_csr(cg.cg_transitive_reduction(ctx, G, fuzz), oracle.transitive_reduction(G, fuzz))
+
+
+@pytest.mark.parametrize("n,pairs,hub,hubs,clique", [
+    (2600, 1500, 768, (0,), 0), (2600, 1500, 769, (0,), 0),     # as long as a piece, and one entry more
+    (2600, 1500, 1535, (7,), 0), (2600, 1500, 1536, (7,), 0), (2600, 1500, 1537, (7,), 0),   # two pieces
+    (3000, 1500, 2999, (0, 1, 2, 1500, 2999), 0),               # long rows side by side, the last read's too
+    (9000, 30, 8999, (4000,), 0),                               # a long row among rows of one entry
+    (1500, 0, 0, (), 150), (2000, 3000, 0, (), 400),            # rows of 149 and 400 entries side by side
+])
+def test_rows_in_pieces(ctx, n, pairs, hub, hubs, clique):
+    G = random_overlaps(n + hub, n, pairs, hub, hubs, clique)
     for fuzz in (0, 1):
         assert same_csr(cg.cg_transitive_reduction(ctx, G, fuzz), oracle.transitive_reduction(G, fuzz))
 
