@@ -248,7 +248,11 @@ CG_API cg_status cg_emit_contigs_2bit(cg_graph* g, int64_t* contig_off, int64_t 
  * call, host inputs are copied; the call waits for the GPU. An invalid R
  * (unsorted or repeated columns, bad offsets, codes, suffixes or mirrors)
  * gives CG_EGRAPH. S keeps R's reads, so a descriptor with S's arrays and R's
- * reads goes to cg_load_graph. */
+ * reads goes to cg_load_graph. Scratch from the context's memory: 16 bytes per
+ * read, 16 per read with entries (counted as min(n, m)) and 13.4 per entry, or,
+ * where that does not fit, 8 per read with entries, 5.4 per entry and an eighth
+ * per read, for a slower pass with the same results; CG_ENOMEM when that does
+ * not fit either. Host inputs and outputs have copies besides. */
 CG_API cg_status cg_transitive_reduction(cg_ctx* ctx, const cg_graph_desc* overlaps, int32_t fuzz, int64_t* row_ptr,
                                   int32_t* col, uint8_t* code, int32_t* suf, int64_t cap_entries, int mem,
                                   int64_t* n_entries);

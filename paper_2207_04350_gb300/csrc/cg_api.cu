@@ -1917,27 +1917,53 @@ cg_status cg_transitive_reduction(cg_ctx* c, const cg_graph_desc* d, int32_t fuz
   G.suf = (const int32_t*)in(d->suf, (size_t)m * 4);
   G.len = (const int32_t*)in(d->len, (size_t)n * 4);
   cg::TrBuffers t{};
-  const size_t tiles = (size_t)cg::transitive_tiles(m);
   t.rows_cap = cg::transitive_pieces(n, m);
-  t.rows = (int4*)alloc((size_t)t.rows_cap * sizeof(int4));
   t.units_cap = cg::transitive_units(n, m);
-  t.unit_first = (unsigned*)alloc((size_t)t.units_cap * sizeof(unsigned));
-  t.info = (int4*)alloc((size_t)n * sizeof(int4));
-  t.has = (unsigned*)alloc(((size_t)n + 31) / 32 * 4);
-  t.ent = (uint2*)alloc((size_t)m * sizeof(uint2));
-  t.trans = (uint8_t*)alloc((size_t)m);
-  t.mir = (int32_t*)alloc((size_t)m * 4);
-  t.keep = (unsigned*)alloc(tiles * 64 * 4);
-  t.before = (unsigned*)alloc(tiles * 64 * 4);
-  t.tile_cnt = (unsigned*)alloc(tiles * 4);
-  t.total = (unsigned long long*)alloc(16);
-  t.listed = t.total ? t.total + 1 : nullptr;
   t.derr = c->derr;
-  // device outputs are written in place; an offset array that is not 8-byte aligned gets a copy
-  const bool device_out = want && mem == CG_MEM_DEVICE;
-  int64_t* out_rp = row_ptr;
-  if (want && !(device_out && aligned(row_ptr, 8))) out_rp = (int64_t*)alloc((size_t)(n + 1) * 8);
+  // scratch in two allocations: what the walks need, and what places the kept entries
+  const size_t tiles = (size_t)cg::transitive_tiles(m);
+  std::vector<std::pair<void**, size_t>> parts;
+  auto part = [&](auto** p, size_t count) { parts.emplace_back(reinterpret_cast<void**>(p), count * sizeof(**p)); };
+  auto take = [&]() -> void* {
+    size_t bytes = 0;
+    for (auto& p : parts) bytes += (p.second + 15) & ~size_t(15);
+    char* const at = (char*)alloc(bytes);
+    size_t o = 0;
+    for (auto& p : parts) {
+      *p.first = at ? at + o : nullptr;
+      o += (p.second + 15) & ~size_t(15);
+    }
+    parts.clear();
+    return at;
+  };
+  part(&t.total, 1);
+  part(&t.listed, 1);
+  part(&t.keep, tiles * 64);
+  part(&t.before, tiles * 64);
+  part(&t.tile_cnt, tiles);
+  take();
   if (st != CG_OK) return done(st);
+  void* walks = nullptr;
+  for (const bool lean : {false, true}) {      // without the records and the two runs when they do not fit
+    st = CG_OK;
+    if (lean) {
+      part(&t.lean_rows, (size_t)t.rows_cap);
+    } else {
+      part(&t.rows, (size_t)t.rows_cap);
+      part(&t.info, (size_t)n);
+      part(&t.ent, (size_t)m);
+    }
+    part(&t.unit_first, (size_t)t.units_cap);
+    part(&t.has, ((size_t)n + 31) / 32);
+    part(&t.mir, (size_t)m);
+    part(&t.trans, (size_t)m);
+    walks = take();
+    if (walks || st != CG_ENOMEM) break;
+  }
+  if (st != CG_OK) return done(st);
+  // device outputs are written in place, in the same queue; others, and an offset array
+  // that is not 8-byte aligned, after the wait, in the walks' place
+  const bool device_out = want && mem == CG_MEM_DEVICE && aligned(row_ptr, 8);
   if (c->marks.on) {                   // per-kernel marks cover this call alone
     c->marks.n = 0;
     cudaEventRecord(c->marks.ev[0], c->stream);
@@ -1948,7 +1974,7 @@ cg_status cg_transitive_reduction(cg_ctx* c, const cg_graph_desc* d, int32_t fuz
   // with device outputs the whole call is queued before its one wait: the last
   // kernel writes nothing when a check failed or the entries do not fit
   if (e == cudaSuccess && device_out)
-    e = cg::launch_transitive_scatter(G, t, cap_entries, out_rp, col, code, suf, c->env, m > 0);
+    e = cg::launch_transitive_scatter(G, t, cap_entries, row_ptr, col, code, suf, c->env, m > 0);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->h_u64, t.total, 8, cudaMemcpyDeviceToHost, c->stream);
   if (e != cudaSuccess) return done(cuda_fail(c, e, "transitive reduction kernels"));
   st = wait_and_read(&probe);
@@ -1958,21 +1984,27 @@ cg_status cg_transitive_reduction(cg_ctx* c, const cg_graph_desc* d, int32_t fuz
   if (!want) return done(CG_OK);
   if (cap_entries < total) return done(fail(c, CG_EINVAL, "capacity %lld < %lld entries", (long long)cap_entries,
                                             (long long)total));
-  if (device_out && out_rp == row_ptr) return done(CG_OK);
-  const cudaMemcpyKind k = mem == CG_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
+  if (device_out) return done(CG_OK);
+  tmp.erase(std::find(tmp.begin(), tmp.end(), walks));
+  dfree(c, walks);
+  int64_t* const out_rp = (int64_t*)alloc((size_t)(n + 1) * 8);
+  int32_t *oc = col, *os = suf;
+  uint8_t* ok = code;
   if (mem == CG_MEM_HOST) {
-    int32_t* oc = (int32_t*)alloc((size_t)total * 4);
-    uint8_t* ok = (uint8_t*)alloc((size_t)total);
-    int32_t* os = (int32_t*)alloc((size_t)total * 4);
-    if (st != CG_OK) return done(st);
-    e = cg::launch_transitive_scatter(G, t, total, out_rp, oc, ok, os, c->env, false);
-    if (total > 0) {
-      if (e == cudaSuccess) e = cudaMemcpyAsync(col, oc, (size_t)total * 4, k, c->stream);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(code, ok, (size_t)total, k, c->stream);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(suf, os, (size_t)total * 4, k, c->stream);
-    }
+    oc = (int32_t*)alloc((size_t)total * 4);
+    ok = (uint8_t*)alloc((size_t)total);
+    os = (int32_t*)alloc((size_t)total * 4);
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(row_ptr, out_rp, (size_t)(n + 1) * 8, k, c->stream);
+  if (st != CG_OK) return done(st);
+  e = cg::launch_transitive_scatter(G, t, total, out_rp, oc, ok, os, c->env, false);
+  if (mem == CG_MEM_HOST && total > 0) {
+    if (e == cudaSuccess) e = cudaMemcpyAsync(col, oc, (size_t)total * 4, cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(code, ok, (size_t)total, cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(suf, os, (size_t)total * 4, cudaMemcpyDeviceToHost, c->stream);
+  }
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(row_ptr, out_rp, (size_t)(n + 1) * 8,
+                        mem == CG_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, c->stream);
   if (e != cudaSuccess) return done(cuda_fail(c, e, "write the reduced graph"));
   st = wait_and_read(&probe);
   return done(st);

@@ -348,6 +348,7 @@ struct TrBuffers {
   unsigned* unit_first;        // per unit of the list's weight, the first piece that starts in it
   long long units_cap;         // transitive_units(n, m)
   unsigned long long* listed;  // pieces listed << 33 | their half weights
+  int2* lean_rows;             // the list (read, first entry) without rows, info and ent, or nullptr
   int4* info;                  // n, set for rows with entries: first entry, first of the second run, end, read length
   unsigned* has;               // n bits: the read has entries
   uint2* ent;                  // m: each row in two runs by the end its entries leave through, (column << 2 | code, suffix)

@@ -21,6 +21,12 @@
 // each word, and since entries lie in row order that count places both the kept
 // entries and the new row offsets.
 //
+// Where the scratch for that does not fit the memory there is, the same kernels run
+// without the records and the two runs (kLean): the walks then read the graph's own
+// arrays, every entry of v's row, and need 8 bytes per read with entries and 5.4 per
+// entry in place of 16 per read, 16 per read with entries and 13.4 per entry. The call
+// on the 3.1 Gb overlap graph takes 374 us so (k_tr_rows 242) and 292 with them.
+//
 // Nothing waits for the host in between: an invalid graph sets the error word,
 // and every later kernel reads it first and returns. The kernels that follow
 // an entry to another row run only once all row offsets have passed.
@@ -99,12 +105,14 @@ __device__ __forceinline__ void load4_rows(const DevGraph& g, long long i, bool 
 // Piece (u, first entry p, z entries) at place `slot` of the list, `half` half weights
 // before it; false when it does not fit: there are more pieces than the entries allow,
 // in rows that overlap, which the row check finds.
+template <bool kLean>
 __device__ __forceinline__ bool list_piece(const TrBuffers& t, unsigned slot, unsigned long long half, int u, int p, int z) {
   if (slot >= (unsigned)t.rows_cap) {
     set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, u & ~kTrPart);
     return false;
   }
-  t.rows[slot] = make_int4(u, p, z, 0);
+  if constexpr (kLean) t.lean_rows[slot] = make_int2(u, p);
+  else t.rows[slot] = make_int4(u, p, z, 0);
   unsigned unit = (unsigned)(half >> kTrUnitLog2);
   int over = (int)((unsigned)half & ((1u << kTrUnitLog2) - 1u)) + half_weight(z) - (1 << kTrUnitLog2);
   for (; over >= 0; over -= 1 << kTrUnitLog2) {        // units that start in the piece or right behind it
@@ -119,6 +127,7 @@ __device__ __forceinline__ bool list_piece(const TrBuffers& t, unsigned slot, un
 
 // A row of more than kTrPiece entries, by one thread, with a reservation of its own.
 // Rows without end in an invalid graph are given up as soon as its error is set.
+template <bool kLean>
 __device__ __forceinline__ void list_long_row(const TrBuffers& t, int u, int a, int z) {
   const int more = (z - 1) / kTrPiece, rest = z - more * kTrPiece;      // whole pieces before the last, its entries
   unsigned long long at =
@@ -126,7 +135,7 @@ __device__ __forceinline__ void list_long_row(const TrBuffers& t, int u, int a, 
                               (unsigned long long)more * (kTrPiece / 2) + (unsigned long long)half_weight(rest));
   for (int i = 0; i <= more; ++i) {
     const int n = i < more ? kTrPiece : rest;
-    if (failed(t.derr) || !list_piece(t, (unsigned)(at >> kTrHalfBits), at & kTrHalves, u | kTrPart, a + i * kTrPiece, n))
+    if (failed(t.derr) || !list_piece<kLean>(t, (unsigned)(at >> kTrHalfBits), at & kTrHalves, u | kTrPart, a + i * kTrPiece, n))
       return;
     at += (1ull << kTrHalfBits) + (unsigned long long)half_weight(n);
   }
@@ -139,6 +148,7 @@ __device__ __forceinline__ void list_long_row(const TrBuffers& t, int u, int a, 
 // and a bit in a map of them.
 // Reads every row offset and length once, 12 B per read, four consecutive reads
 // per thread by 16-byte loads where the arrays allow.
+template <bool kLean>
 __global__ void __launch_bounds__(kBlock, 6) k_tr_check(DevGraph g, TrBuffers t, bool wide_rows, bool wide_len) {
   __shared__ unsigned cnt;                             // of the block's rows of one piece: pieces << kTrLocalBits | half weights
   __shared__ unsigned long long base;
@@ -190,12 +200,13 @@ __global__ void __launch_bounds__(kBlock, 6) k_tr_check(DevGraph g, TrBuffers t,
     const int k = __ffs(full) - 1, u = (int)(u0 + k);
     const int first = (int)(k == 0 ? a[0] : k == 1 ? a[1] : k == 2 ? a[2] : a[3]);
     const int z = (int)(k == 0 ? a[1] : k == 1 ? a[2] : k == 2 ? a[3] : next) - first;
-    t.info[u] = make_int4(first, 0, first + z, k == 0 ? len[0] : k == 1 ? len[1] : k == 2 ? len[2] : len[3]);
+    if constexpr (!kLean)
+      t.info[u] = make_int4(first, 0, first + z, k == 0 ? len[0] : k == 1 ? len[1] : k == 2 ? len[2] : len[3]);
     if (z <= kTrPiece) {
-      list_piece(t, slot0 + (at >> kTrLocalBits), half0 + (at & ((1u << kTrLocalBits) - 1u)), u, first, z);
+      list_piece<kLean>(t, slot0 + (at >> kTrLocalBits), half0 + (at & ((1u << kTrLocalBits) - 1u)), u, first, z);
       at += (1u << kTrLocalBits) + (unsigned)half_weight(z);
     } else {
-      list_long_row(t, u, first, z);
+      list_long_row<kLean>(t, u, first, z);
     }
   }
 }
@@ -219,12 +230,19 @@ struct TrList {
 // A batch, pieces [r0, r1) of the list: their records and the places of their
 // entries in the batch, row[j].w the first of piece j. Returns the number of
 // entries; *parts: there are pieces of rows in pieces among them. Whole block.
-template <int kRows>
-__device__ __forceinline__ int load_batch(const TrBuffers& t, long long r0, long long r1, int4* row, int* warp_tot,
-                                          bool* parts) {
+template <int kRows, bool kLean>
+__device__ __forceinline__ int load_batch(const DevGraph& g, const TrBuffers& t, long long r0, long long r1, int4* row,
+                                          int* warp_tot, bool* parts) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   int4 mine = make_int4(0, 0, 0, 0);
-  if (r0 + tid < r1) mine = t.rows[r0 + tid];          // at most kRows of them
+  if (r0 + tid < r1) {                                 // at most kRows of them
+    if constexpr (kLean) {
+      const int2 r = t.lean_rows[r0 + tid];
+      mine = make_int4(r.x, r.y, min((int)rowp(g, (r.x & ~kTrPart) + 1) - r.y, kTrPiece), 0);
+    } else {
+      mine = t.rows[r0 + tid];
+    }
+  }
   int inc = mine.z;
   for (int o = 1; o < 32; o <<= 1) {
     const int x = __shfl_up_sync(0xffffffffu, inc, o);
@@ -254,6 +272,14 @@ __device__ __forceinline__ int find_row(const int4* row, int i) {
   return j;
 }
 
+// A read with entries: its first one, the first of the second run (0 when there are no
+// runs), the end, the read's length.
+template <bool kLean>
+__device__ __forceinline__ int4 row_info(const DevGraph& g, const TrBuffers& t, int v) {
+  if constexpr (kLean) return make_int4((int)rowp(g, v), 0, (int)rowp(g, v + 1), g.len[v]);
+  else return t.info[v];
+}
+
 // Entries: columns in range, increasing in the row, not the row's own read and a
 // read with entries; codes 0..3. Copies every row in two runs by the end its
 // entries leave through, each run in the row's order: 9 B read and 12 written per
@@ -263,6 +289,7 @@ __device__ __forceinline__ int find_row(const int4* row, int i) {
 // code, column), so that warps hide them: with eight blocks on an SM, at 32
 // registers, 51 us for 3.36M entries, with six 56; batches of 720 and 480 entries
 // 53 and 56.
+template <bool kLean>
 __global__ void __launch_bounds__(kBlock, 8) k_tr_pack(DevGraph g, TrBuffers t) {
   pdl_enter();
   __shared__ int4 row[kTrPackRows];
@@ -275,8 +302,8 @@ __global__ void __launch_bounds__(kBlock, 8) k_tr_pack(DevGraph g, TrBuffers t) 
   const TrList list(t, kTrPackUnits);
   for (long long b = blockIdx.x; b < list.batches(); b += gridDim.x) {
     bool parts;
-    const int total = load_batch<kTrPackRows>(t, list.first(b), list.first(b + 1), row, warp_tot, &parts);
-    if (parts) {
+    const int total = load_batch<kTrPackRows, kLean>(g, t, list.first(b), list.first(b + 1), row, warp_tot, &parts);
+    if (!kLean && parts) {
       if (tid < kTrPackRows) rest_before[tid] = rest_all[tid] = 0;
       __syncthreads();
       for (int j = 0; j < kTrPackRows; ++j) {             // block-uniform
@@ -296,8 +323,8 @@ __global__ void __launch_bounds__(kBlock, 8) k_tr_pack(DevGraph g, TrBuffers t) 
         }
       }
     }
-    constexpr int kPer = kTrStage / kBlock;
-    unsigned cd[kPer];                                 // this thread's staged entries
+    constexpr int kPer = kLean ? 0 : kTrStage / kBlock;
+    unsigned cd[kTrStage / kBlock];                    // this thread's staged entries
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
       const int i = k * kBlock + tid;
@@ -310,7 +337,7 @@ __global__ void __launch_bounds__(kBlock, 8) k_tr_pack(DevGraph g, TrBuffers t) 
       if (lane == 0) zeros[(k * kBlock + tid) >> 5] = z;
     }
     __syncthreads();
-    if (tid < 32) {                                    // two words per lane
+    if (!kLean && tid < 32) {                          // two words per lane
       const int z0 = __popc(zeros[2 * lane]), z1 = __popc(zeros[2 * lane + 1]);
       int inc = z0 + z1;
       for (int o = 1; o < 32; o <<= 1) {
@@ -331,20 +358,27 @@ __global__ void __launch_bounds__(kBlock, 8) k_tr_pack(DevGraph g, TrBuffers t) 
       const int32_t w = g.col[x];
       const unsigned c = g.code[x];
       int a = row[j].y;                                // first entry of the row
-      // entries of end 0 before this one and in the row
-      int z = zeros_before(i) - zeros_before(s0), nz = zeros_before(s0 + n) - zeros_before(s0);
+      int z = 0, nz = 0;                               // entries of end 0 before this one and in the row
+      if constexpr (!kLean) {
+        z = zeros_before(i) - zeros_before(s0);
+        nz = zeros_before(s0 + n) - zeros_before(s0);
+      }
       if (row[j].x & kTrPart) {
-        a = t.info[u].x;
-        z += rest_before[j];
-        nz = rest_all[j];
+        a = row_info<kLean>(g, t, u).x;
+        if constexpr (!kLean) {
+          z += rest_before[j];
+          nz = rest_all[j];
+        }
         t.trans[x] = (uint8_t)(c << 1);                // the walks only set what they hit, from any block
       }
       const bool ok = w >= 0 && w < g.n && w != u && c <= 3 && (x == a || g.col[x - 1] < w) &&
                       ((t.has[w >> 5] >> (w & 31)) & 1u);
       if (!ok) set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, x);
-      if (i == s0) t.info[u].y = a + nz;
-      const int at = (c & 1) == 0 ? a + z : a + nz + (x - a - z);
-      t.ent[at] = make_uint2(((unsigned)w << 2) | (c & 3u), (unsigned)g.suf[x]);
+      if constexpr (!kLean) {
+        if (i == s0) t.info[u].y = a + nz;
+        const int at = (c & 1) == 0 ? a + z : a + nz + (x - a - z);
+        t.ent[at] = make_uint2(((unsigned)w << 2) | (c & 3u), (unsigned)g.suf[x]);
+      }
       if (w < u) t.mir[x] = -1;                        // found from the other side, or missing
     }
     __syncthreads();
@@ -375,6 +409,7 @@ __device__ __forceinline__ bool closes(unsigned cx, unsigned cy, unsigned cz, in
 // rows of a warp in step, took 476, most of its lanes waiting for longer rows; the
 // runs of a warp's entries laid end to end, so that no lane waits, 139 to 160 by
 // the entries in flight, for as many instructions as without.
+template <bool kLean>
 __global__ void __launch_bounds__(kBlock, 6) k_tr_rows(DevGraph g, TrBuffers t, int fuzz) {
   pdl_enter();
   __shared__ int4 row[kTrWalkRows];                       // read, first entry, entries, first of the batch's entries
@@ -387,7 +422,7 @@ __global__ void __launch_bounds__(kBlock, 6) k_tr_rows(DevGraph g, TrBuffers t, 
   const TrList list(t, kTrWalkUnits);
   for (long long b = blockIdx.x; b < list.batches(); b += gridDim.x) {
     bool parts;
-    const int total = load_batch<kTrWalkRows>(t, list.first(b), list.first(b + 1), row, warp_tot, &parts);
+    const int total = load_batch<kTrWalkRows, kLean>(g, t, list.first(b), list.first(b + 1), row, warp_tot, &parts);
     for (int i = tid; i < total; i += kBlock) {
       const int j = find_row<kTrWalkRows>(row, i);
       const int x = row[j].y + (i - row[j].w);
@@ -405,11 +440,12 @@ __global__ void __launch_bounds__(kBlock, 6) k_tr_rows(DevGraph g, TrBuffers t, 
       const int32_t sy = suf[i];
       const int v = (int)(e >> 2);
       const unsigned cy = e & 3u;
-      const int4 iv = t.info[v];                       // first entry, first of the second run, end, length
+      const int4 iv = row_info<kLean>(g, t, v);        // first entry, first of the second run, end, length
       if (sy < 1 || sy > iv.w - 1) set_error(t.derr, DERR_GRAPH, K_TRANSITIVE, y);
       // v is left through its other end: the first run when it was entered through end 1
-      const unsigned z1 = (unsigned)(cy & 2u ? iv.y : iv.z);   // unsigned: z + 4 may pass the largest int
-      unsigned z = (unsigned)(cy & 2u ? iv.x : iv.y);
+      // (of a row without runs, the entries that leave through it)
+      const unsigned z1 = (unsigned)(!kLean && (cy & 2u) ? iv.y : iv.z);   // unsigned: z + 4 may pass the largest int
+      unsigned z = (unsigned)(kLean || (cy & 2u) ? iv.x : iv.y);
       if (u < v) {
         const int32_t back = find_col(g.col, iv.x, iv.z, u);
         if (back >= 0) t.mir[back] = y;
@@ -418,8 +454,18 @@ __global__ void __launch_bounds__(kBlock, 6) k_tr_rows(DevGraph g, TrBuffers t, 
       }
       for (; z < z1; z += 4) {
         uint2 q[4];
+        bool use[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) q[k] = z + k < z1 ? t.ent[z + k] : make_uint2(0u, 0u);
+        for (int k = 0; k < 4; ++k) {
+          if constexpr (kLean) {
+            const unsigned cz = z + k < z1 ? g.code[z + k] : 0u;
+            use[k] = z + k < z1 && ((cz ^ (cy >> 1)) & 1u);
+            q[k] = use[k] ? make_uint2(((unsigned)g.col[z + k] << 2) | cz, (unsigned)g.suf[z + k]) : make_uint2(0u, 0u);
+          } else {
+            use[k] = z + k < z1;
+            q[k] = use[k] ? t.ent[z + k] : make_uint2(0u, 0u);
+          }
+        }
         if (whole) {                                   // the four searches step together
           int lo[4] = {s0, s0, s0, s0};                // the last column <= w, or the first one
           for (int len = n; len > 1;) {
@@ -432,14 +478,14 @@ __global__ void __launch_bounds__(kBlock, 6) k_tr_rows(DevGraph g, TrBuffers t, 
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             const unsigned kx = key[lo[k]];
-            if (z + k < z1 && (kx ^ q[k].x) < 4u && closes(kx, cy, q[k].x, suf[lo[k]], sy, (int32_t)q[k].y, fuzz))
+            if (use[k] && (kx ^ q[k].x) < 4u && closes(kx, cy, q[k].x, suf[lo[k]], sy, (int32_t)q[k].y, fuzz))
               hit[lo[k]] = 1;
           }
         } else {
-          const int4 iu = t.info[u];
+          const int4 iu = row_info<kLean>(g, t, u);
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            if (z + k >= z1) break;
+            if (!use[k]) continue;
             const int32_t x = find_col(g.col, iu.x, iu.z, (int32_t)(q[k].x >> 2));
             if (x >= 0 && closes(g.code[x], cy, q[k].x, g.suf[x], sy, (int32_t)q[k].y, fuzz))
               t.trans[x] = (uint8_t)(1u | (g.code[x] << 1));
@@ -602,32 +648,38 @@ long long transitive_units(long long n, long long m) {
   return ((m / 2 + 1 + 4 * transitive_pieces(n, m)) >> kTrUnitLog2) + 2;
 }
 
+template <bool kLean>
+static cudaError_t launch_transitive_walks(const DevGraph& g, int fuzz, const TrBuffers& t, const LaunchEnv& env) {
+  const long long blocks = std::max(1ll, ((long long)g.n + kTrRows * kBlock - 1) / (kTrRows * kBlock));
+  k_tr_check<kLean><<<(unsigned)blocks, kBlock, 0, env.stream>>>(g, t, (reinterpret_cast<uintptr_t>(g.row_ptr) & 15) == 0,
+                                                                 (reinterpret_cast<uintptr_t>(g.len) & 15) == 0);
+  mark(env, "k_tr_check");
+  if (g.m == 0) return cudaGetLastError();
+  static const int pack_resident = resident_blocks(k_tr_pack<kLean>), rows_resident = resident_blocks(k_tr_rows<kLean>);
+  // persistent grids; no more batches than units, and one block for a graph that has
+  // entries but no reads: the row check has refused it by then
+  const long long need = std::max(1ll, t.units_cap);
+  cudaError_t e = launch_k(k_tr_pack<kLean>, (int)std::min(need, (long long)env.num_sms * pack_resident), env, true, g, t);
+  if (e != cudaSuccess) return e;
+  mark(env, "k_tr_pack");
+  e = launch_k(k_tr_rows<kLean>, (int)std::min(need, (long long)env.num_sms * rows_resident), env, true, g, t, fuzz);
+  if (e != cudaSuccess) return e;
+  mark(env, "k_tr_rows");
+  return cudaGetLastError();
+}
+
 cudaError_t launch_transitive(const DevGraph& g, int fuzz, const TrBuffers& t, const LaunchEnv& env) {
   cudaMemsetAsync(t.total, 0, sizeof(unsigned long long), env.stream);
   cudaMemsetAsync(t.listed, 0, sizeof(unsigned long long), env.stream);
-  const long long blocks = std::max(1ll, ((long long)g.n + kTrRows * kBlock - 1) / (kTrRows * kBlock));
-  k_tr_check<<<(unsigned)blocks, kBlock, 0, env.stream>>>(g, t, (reinterpret_cast<uintptr_t>(g.row_ptr) & 15) == 0,
-                                                              (reinterpret_cast<uintptr_t>(g.len) & 15) == 0);
-  mark(env, "k_tr_check");
-  if (g.m > 0) {
-    static const int pack_resident = resident_blocks(k_tr_pack), rows_resident = resident_blocks(k_tr_rows);
-    // persistent grids; no more batches than units, and one block for a graph that has
-    // entries but no reads: the row check has refused it by then
-    const long long need = std::max(1ll, t.units_cap);
-    cudaError_t e = launch_k(k_tr_pack, (int)std::min(need, (long long)env.num_sms * pack_resident), env, true, g, t);
-    if (e != cudaSuccess) return e;
-    mark(env, "k_tr_pack");
-    e = launch_k(k_tr_rows, (int)std::min(need, (long long)env.num_sms * rows_resident), env, true, g, t, fuzz);
-    if (e != cudaSuccess) return e;
-    mark(env, "k_tr_rows");
-    const long long tiles = transitive_tiles(g.m);
-    e = launch_k(k_tr_keep, (int)tiles, env, true, (long long)g.m, t.trans, t.mir, t.keep, t.before, t.tile_cnt, t.derr);
-    if (e != cudaSuccess) return e;
-    mark(env, "k_tr_keep");
-    e = launch_kb(k_tr_tiles, 1, 1024, env, true, t.tile_cnt, tiles, t.total, t.derr);
-    if (e != cudaSuccess) return e;
-    mark(env, "k_tr_tiles");
-  }
+  cudaError_t e = t.lean_rows ? launch_transitive_walks<true>(g, fuzz, t, env) : launch_transitive_walks<false>(g, fuzz, t, env);
+  if (e != cudaSuccess || g.m == 0) return e;
+  const long long tiles = transitive_tiles(g.m);
+  e = launch_k(k_tr_keep, (int)tiles, env, true, (long long)g.m, t.trans, t.mir, t.keep, t.before, t.tile_cnt, t.derr);
+  if (e != cudaSuccess) return e;
+  mark(env, "k_tr_keep");
+  e = launch_kb(k_tr_tiles, 1, 1024, env, true, t.tile_cnt, tiles, t.total, t.derr);
+  if (e != cudaSuccess) return e;
+  mark(env, "k_tr_tiles");
   return cudaGetLastError();
 }
 

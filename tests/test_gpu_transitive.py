@@ -157,6 +157,35 @@ def test_rows_in_pieces(ctx, n, pairs, hub, hubs, clique):
         assert same_csr(cg.cg_transitive_reduction(ctx, G, fuzz), oracle.transitive_reduction(G, fuzz))
 
 
+@pytest.mark.parametrize("device", [False, True])
+@pytest.mark.parametrize("n,pairs,hub,hubs,clique", [
+    (200_000, 900, 0, (), 0), (20_000, 20_000, 0, (), 0), (300, 12000, 0, (), 0),
+    (3000, 1500, 2999, (0, 1, 1500, 2999), 0), (2000, 3000, 0, (), 400)])
+def test_scratch_within_a_tight_budget(n, pairs, hub, hubs, clique, device):
+    """With 12 bytes of scratch per read and 6 per entry (and the copies of host arrays),
+    too few for the rows' records and runs, the call gives the same."""
+    import torch
+    G = random_overlaps(n + hub, n, pairs, hub, hubs, clique)
+    want = oracle.transitive_reduction(G, 1)
+    k = len(want.col)
+    arrays = [4 * G.m, G.m, G.m, 4 * n, 8 * (n + 1), 8, 8 * (n // 2048 + 3)]
+    if not device:
+        arrays += [8 * (n + 1), 4 * G.m, G.m, 4 * G.m, 4 * n, 4 * k, k, 4 * k]
+    D = G
+    if device:
+        D = type("D", (), {})()
+        for f in ("row_ptr", "col", "code", "suf", "len", "off", "packed"):
+            setattr(D, f, torch.from_numpy(np.ascontiguousarray(getattr(G, f))).cuda())
+    ctx = cg.cg_create(0, hbm_budget_bytes=sum((b + 255) // 256 * 256 for b in arrays))
+    try:
+        S = cg.cg_transitive_reduction(ctx, D, 1, device=device)
+        for f in ("row_ptr", "col", "code", "suf"):
+            got = getattr(S, f)
+            assert np.array_equal(got.cpu().numpy() if device else got, getattr(want, f))
+    finally:
+        ctx.close()
+
+
 def test_missing_or_foreign_mirrors(ctx):
     """An entry whose pair lacks the entry back, seen from the smaller and from the
     larger read, and one that leads to a read without entries."""
