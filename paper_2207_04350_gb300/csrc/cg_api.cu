@@ -1577,13 +1577,12 @@ cg_status cg_emit_share(cg_graph* g, int32_t share, int32_t n_shares, int64_t* c
 }
 
 // ------------------------------------------------------------ read exchange
-// One exchange call: its device arrays (one allocation) and, on the host, what
-// the kernels counted.
+// One exchange call: its device arrays and, on the host, what the kernels counted.
 struct Xchg {
   cg::XchgArgs x{};
   std::vector<int64_t> counted;          // range (2 N), pair0 (N + 1), send words (N), receive words (N)
   uint32_t* mine = nullptr;
-  void* mem = nullptr;
+  void* mem = nullptr;                   // allocated, or nullptr: in the graph's scratch
   const int64_t* range() const { return counted.data(); }
   const int64_t* pair0() const { return counted.data() + 2 * x.n_shares; }
   const int64_t* send() const { return counted.data() + 3 * x.n_shares + 1; }
@@ -1594,6 +1593,15 @@ struct Xchg {
     return t;
   }
 };
+
+// Room for an exchange call's arrays: buffer k of the list ranking, 32 bytes per read,
+// which is free until the chains are ranked again; allocated (*own) for a graph with
+// too few reads. The calls need no memory of their own so.
+static void* x_room(cg_graph* g, int k, size_t bytes, void** own, cg_status* st) {
+  *own = nullptr;
+  if (bytes <= 2 * sizeof(int4) * (size_t)g->g.n) return g->s.pj[k];
+  return *own = dalloc(g->ctx, bytes, st);
+}
 
 // Checks the arguments, lays out the graph if needed and fills X; with want_mine
 // also every pair's words (X.mine). Waits once.
@@ -1612,9 +1620,8 @@ static cg_status x_count(cg_graph* g, int32_t n_shares, const int64_t* read_firs
   }
   const size_t N = (size_t)n_shares, counts = 5 * N + 1;
   const size_t pairs = want_mine ? (size_t)g->g.n + N : 0;    // a share's first piece may be the last of the one before
-  int64_t* d = (int64_t*)dalloc(c, (counts + N + 1) * 8 + pairs * 4, &st);
+  int64_t* d = (int64_t*)x_room(g, 0, (counts + N + 1) * 8 + pairs * 4, &X.mem, &st);
   if (!d) return st;
-  X.mem = d;
   X.x.n_shares = n_shares;
   X.x.rank = rank;
   X.x.range = (long long*)d;
@@ -1671,9 +1678,8 @@ cg_status cg_exchange_pack(cg_graph* g, int32_t n_shares, const int64_t* read_fi
     else if (words > 0) {
       // the places of the pairs, the first pairs of the chunks, and the scan's descriptors
       const long long cap = (pairs + 2047) / 2048 + 1, chunks = (words + cg::kPackChunk - 1) / cg::kPackChunk;
-      long long* slot = (long long*)dalloc(c, (size_t)(pairs + chunks + cap + 1) * 8, &st);
-      tmp = slot;
-      if (tmp) {
+      long long* slot = (long long*)x_room(g, 1, (size_t)(pairs + chunks + cap + 1) * 8, &tmp, &st);
+      if (slot) {
         cudaError_t e = cg::launch_x_pack(g->g, g->s, X.x, my_packed, my_packed_bytes, my_off, X.mine, slot,
                                           slot + pairs, (unsigned long long*)(slot + pairs + chunks), cap,
                                           reinterpret_cast<uint32_t*>(send_buf), pairs, words, c->env);
@@ -1700,14 +1706,14 @@ cg_status cg_emit_share_received(cg_graph* g, int32_t n_shares, const int64_t* r
     return fail(c, CG_EINVAL, "bad receive or output buffers");
   Xchg X;
   st = x_count(g, n_shares, read_first, rank, false, X);
-  unsigned long long* state = nullptr;
+  void* tmp = nullptr;
   if (st == CG_OK) {
     const int64_t words = Xchg::sum(X.recv(), n_shares), count = X.pair0()[rank + 1] - X.pair0()[rank];
     if (4 * words != recv_bytes)
       st = fail(c, CG_EINVAL, "received %lld bytes, the layout needs %lld", (long long)recv_bytes, (long long)(4 * words));
     else if (count > 0) {
       const long long cap = (count + cg::kXchgTile - 1) / cg::kXchgTile;
-      state = (unsigned long long*)dalloc(c, (size_t)n_shares * (size_t)(cap + 1) * 8, &st);
+      auto* state = (unsigned long long*)x_room(g, 1, (size_t)n_shares * (size_t)(cap + 1) * 8, &tmp, &st);
       if (state) {
         cudaError_t e = cg::launch_x_place(g->s, X.x, count, state, cap, c->env);
         if (e != cudaSuccess) st = cuda_fail(c, e, "exchange placement");
@@ -1738,7 +1744,7 @@ cg_status cg_emit_share_received(cg_graph* g, int32_t n_shares, const int64_t* r
       if (n_bases) *n_bases = std::max<int64_t>(0, std::min(total, t1 * tb) - t0 * tb);
     }
   }
-  dfree(c, state);
+  dfree(c, tmp);
   dfree(c, X.mem);
   return st;
 }

@@ -76,6 +76,36 @@ def _run_all(ctx, G, world, rf, mcr):
             g.close()
 
 
+def test_exchange_needs_no_more_memory_than_its_slots():
+    """On a context that holds the ranks' graphs and 8 bytes per piece besides, every
+    call of the exchange runs."""
+    G = structured(29, [1] * 500 + [30] * 400 + [2000] * 2, min_len=20, max_len=90)
+    W, n = 3, G.n
+    rf = _bounds(n, W, 0.3)
+
+    def fits(budget):
+        c = cg.cg_create(0, hbm_budget_bytes=budget)
+        try:
+            cg.cg_load_graph(c, without_reads(G), flags=cg.NO_READS, min_chain_reads=1).close()
+            return True
+        except cg.CgError as e:
+            assert e.status == cg.CG_ENOMEM
+            return False
+        finally:
+            c.close()
+    lo, hi = 0, 1 << 26                             # in units of 256 bytes
+    assert fits(hi << 8)
+    while hi - lo > 1:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if fits(mid << 8) else (mid, hi)
+    c = cg.cg_create(0, hbm_budget_bytes=W * (hi << 8) + 8 * (n + W) + 4096)
+    try:
+        shares, _, _ = _run_all(c, G, W, rf, 1)
+    finally:
+        c.close()
+    assert np.array_equal(np.concatenate(shares), oracle.run(G, min_chain_reads=1).bases)
+
+
 @pytest.mark.parametrize("world", [1, 2, 3, 4])
 @pytest.mark.parametrize("name", ["tiny-1Mb", "recipe-20Mb", "structured"])
 def test_exchange_gives_the_oracle_stream(ctx, name, world):
