@@ -395,7 +395,8 @@ CG_API cg_status cg_set_host_direct(cg_ctx* ctx, int enable);
  * "h2d" (an input copy, CG_ECUDA), "timeout" (a bounded device wait,
  * CG_ETIMEOUT), "barrier" (the n-th stage's kernels start as after a device wait
  * that gave up: they write no output, and the next waiting call returns
- * CG_ETIMEOUT), "kernel" (a kernel consistency check, CG_EKERNEL), "bad_graph"
+ * CG_ETIMEOUT), "capture" (the n-th capture of a stage into a graph, CG_ECUDA),
+ * "kernel" (a kernel consistency check, CG_EKERNEL), "bad_graph"
  * (input validation, CG_EGRAPH). NULL or "" clears the plan. The CG_FAULT
  * environment variable gives the plan of every new context and server; a
  * server also knows "admit" (cg_server_submit returns CG_EBUSY) and

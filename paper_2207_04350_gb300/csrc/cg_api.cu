@@ -49,7 +49,7 @@ struct cg_ctx {
 struct StageExec {
   cudaGraphExec_t exec = nullptr;
   uint64_t key = 0;
-  uint64_t seen = 0;                   // the key of the last stage launched without a graph (0: none)
+  uint64_t seen = 0;                   // the key of the stage's last use (0: none)
   unsigned long long kernels = 0;      // kernels in the graph
   int mark_end = 0;                    // per-kernel timing marks after the stage
 };
@@ -274,7 +274,8 @@ const cg::Tuning& gt(cg_graph* g) {
 // Runs one stage's launches. With graphs on, the launches are captured into a CUDA
 // graph per (stage, key) when the key comes a second time in a row, and replayed
 // with a single launch from then on; the key covers every host-side value the
-// launches bake in (buffers, sizes, tuning, timing marks). A stage that runs once,
+// launches bake in (buffers, sizes, tuning, timing marks). Two keys used in turn keep
+// the graph of the one that has it, and the other is launched. A stage that runs once,
 // as those of a graph that is loaded, spelled and freed do, is not worth a
 // capture: a first step on a 100 Mb genome takes 190 us with it and 134 without, a
 // 42 Mb request from load to free 546 and 458.
@@ -292,6 +293,7 @@ cg_status run_stage(cg_graph* g, int slot, uint64_t key, F&& launch) {
   key = mix_key(mix_key(key, (uint64_t)(uintptr_t)g->s.part), (uint64_t)(uint32_t)g->s.part_p);
   if (key == 0) key = 1;                 // 0: none seen yet
   if (e.exec && e.key == key) {
+    e.seen = key;
     c->launches += e.kernels;
     if (c->marks.on) c->marks.n = e.mark_end;
     CK(cudaGraphLaunch(e.exec, c->stream), "cudaGraphLaunch");
@@ -309,6 +311,7 @@ cg_status run_stage(cg_graph* g, int slot, uint64_t key, F&& launch) {
     e.exec = nullptr;
   }
   const unsigned long long l0 = c->launches;
+  if (c->fault.hit("capture")) return fail(c, CG_ECUDA, "injected: capture of a stage failed");
   CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal), "cudaStreamBeginCapture");
   cg_status st = launch();
   cudaGraph_t graph = nullptr;

@@ -6,7 +6,8 @@
 // failed: an allocation ("alloc", CG_ENOMEM), an input copy ("h2d",
 // CG_ECUDA), a bounded device wait ("timeout", CG_ETIMEOUT), a device wait that
 // gave up before a stage's kernels ("barrier": the error word is set as such a wait
-// sets it, the kernels run, and the next wait reports CG_ETIMEOUT), a kernel's
+// sets it, the kernels run, and the next wait reports CG_ETIMEOUT), the capture of a
+// stage's launches into a graph ("capture", CG_ECUDA), a kernel's
 // consistency check ("kernel", CG_EKERNEL), input validation ("bad_graph",
 // CG_EGRAPH), server admission ("admit", CG_EBUSY), a server worker that
 // stalls for ms milliseconds before its batch ("queue_stall"), or a server

@@ -98,7 +98,7 @@ struct Scratch {
                         //             length; smallest read id inside; last oriented read, 2v + o)
   int4* pj[2];          // sublist -> (next: -1 resolved, -2 unresolved; oriented reads to the list tail;
                         //             smallest read id to the tail; the list's last oriented read);
-                        //             jumping double buffers
+                        //             jumping double buffers; afterwards room for the read exchange (x_room)
   // per candidate
   int4* prd;            // n: (smallest read id of the chain, -1 in no contig; walk position;
                         //     bases this read adds to its contig; orientation 0 / 1, 255 in no contig)

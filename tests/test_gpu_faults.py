@@ -159,6 +159,38 @@ def test_nothing_runs_on_after_a_wait_that_gave_up(tiny, call, graphs):
         fresh.close()
 
 
+def test_a_stage_is_captured_when_it_comes_twice_in_a_row(tiny):
+    """Two output buffers used in turn are no reason to capture again: the first keeps
+    its graph and the other is launched, until one comes twice in a row."""
+    G, orc = tiny
+    out = [torch.zeros(len(orc.bases) + 16, dtype=torch.uint8, device="cuda") for _ in range(2)]
+    off = torch.zeros(len(orc.contig_off), dtype=I64, device="cuda")
+    ctx = cg.cg_create(0)
+    try:
+        g = cg.cg_load_graph(ctx, G)
+
+        def step(k):
+            out[k].zero_()
+            torch.cuda.synchronize()
+            cg.cg_mask_branches(g, want_count=False)
+            cg.cg_chains(g, want_counts=False)
+            cg.cg_emit_contigs(g, off, out[k], want_counts=False)
+            cg.cg_sync(ctx)
+            assert np.array_equal(out[k][:len(orc.bases)].cpu().numpy(), orc.bases)
+
+        step(0)
+        step(0)                                  # captured
+        cg.cg_set_fault(ctx, "capture:1")
+        for k in (1, 0, 1, 0, 0, 1, 0, 1):
+            step(k)
+        with pytest.raises(cg.CgError) as e:
+            step(1)                              # twice in a row: captured, which the plan fails
+        assert e.value.status == cg.CG_ECUDA
+        g.close()
+    finally:
+        ctx.close()
+
+
 def test_plan_from_environment(tiny):
     G, orc = tiny
     os.environ["CG_FAULT"] = "bad_graph:2"
