@@ -163,7 +163,11 @@ CG_API cg_status cg_batch_ranges(cg_graph* g, int64_t* first_contig, int64_t* fi
  * batch (continuous batching), so batches overlap on the device. Each
  * worker's device output buffers come from a stream-ordered memory pool, so
  * a growing batch never synchronises the device. Results stay in
- * server-owned host memory until cg_server_release. */
+ * server-owned host memory until cg_server_release: in pinned memory, which
+ * cg_server_start makes and cg_server_stop frees, 1 GiB of it or
+ * hbm_budget_bytes when that is less (half and so on down to a sixteenth, or
+ * none, when the host refuses it), and in ordinary memory, copied more slowly,
+ * when the results not yet released fill it. */
 typedef struct cg_server cg_server;
 typedef struct {
   int32_t max_batch;          /* requests per batch, >= 1 */

@@ -23,6 +23,7 @@
 
 #include "cg.h"
 #include "cg_fault.h"
+#include "cg_serve.h"
 #include <nvtx3/nvToolsExt.h>
 
 namespace {
@@ -37,7 +38,8 @@ int64_t now_ns() {
 // while other batches run; the copies into pageable memory, freshly mapped and
 // zeroed for each request, were most of what a request took. Making pinned memory
 // and giving it back stop the other workers' calls for many milliseconds, so the
-// server makes one stretch of kPinned bytes as it starts (30 ms), out of which
+// server makes one stretch of a GiB, or of its admission budget when that is less, as
+// it starts (30 ms a GiB), out of which
 // results are cut, first fit, and released ones joined again. Results that do not
 // fit lie in ordinary memory, written once before the copy. 2,000 requests of 42 Mb
 // on average, eight workers, all submitted at once: 1,850-2,340 requests a second,
@@ -53,16 +55,21 @@ struct HostBuf {
 
 class HostPool {
  public:
-  static constexpr size_t kPinned = size_t(1) << 30, kUnit = 65536;
-  // Less pinned memory, or none, when the host has not got it.
-  void make() {
-    for (size_t n = kPinned; n >= kPinned / 16 && !base_; n /= 2) {
+  static constexpr size_t kUnit = cg::kResultUnit;
+  // `want` bytes, or half of them and so on down to a sixteenth, or none, as the host
+  // gives them.
+  void make(size_t want) {
+    for (size_t n = want; n >= want / 16 && n >= kUnit && !base_; n = n / 2 / kUnit * kUnit) {
       void* p = nullptr;
-      if (cudaHostAlloc(&p, n, cudaHostAllocPortable) == cudaSuccess) {
-        base_ = static_cast<char*>(p);
-        free_[0] = n;
-      } else {
+      if (cudaHostAlloc(&p, n, cudaHostAllocPortable) != cudaSuccess) {
         cudaGetLastError();
+        continue;
+      }
+      base_ = static_cast<char*>(p);
+      try {
+        free_[0] = n;
+      } catch (const std::bad_alloc&) {      // results then lie in ordinary memory
+        return;
       }
     }
   }
@@ -417,7 +424,7 @@ cg_status cg_server_start(int device, const cg_server_opts* opts, cg_server** ou
     uint64_t keep = ~0ull;   // freed buffers stay in the pool for the next batch
     cudaMemPoolSetAttribute(s->pool, cudaMemPoolAttrReleaseThreshold, &keep);
   }
-  s->results.make();
+  s->results.make(cg::pinned_result_bytes(opts->hbm_budget_bytes));
   for (int w = 0; w < opts->workers; ++w) {
     cg_ctx* c = nullptr;
     cudaStream_t st_w = nullptr;

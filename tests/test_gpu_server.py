@@ -112,3 +112,22 @@ def test_results_past_the_pinned_memory():
                 srv.release(rid)
     finally:
         srv.stop()
+
+
+def test_results_past_the_pinned_memory_of_a_small_budget(pool):
+    """A budget of a few requests: the pinned memory is no larger, and results kept
+    beyond it lie in ordinary memory."""
+    graphs, want = pool
+    G, orc = graphs[-1], want[-1]
+    est = 2 * G.packed.nbytes + 400 * G.n + 16 * G.m + (1 << 20)
+    keep = 2 * int(3 * est) // len(orc.bases)
+    srv = cg.Server(0, hbm_budget_bytes=int(3 * est), max_batch=4, workers=2)
+    try:
+        for _ in range(2):
+            ids = [srv.submit(G) for _ in range(keep)]
+            for rid in ids:
+                _check(srv.wait(rid), orc)
+            for rid in ids:
+                srv.release(rid)
+    finally:
+        srv.stop()
