@@ -17,6 +17,7 @@ CPU oracle instead, on a bounded sample of the same workload.
 from __future__ import annotations
 
 import argparse
+import hashlib
 import json
 import os
 import statistics
@@ -32,9 +33,19 @@ METRIC = "contig Gbases/s & ms per graph (plain vs batched) vs HBM roofline; p50
 UNIT = "Gbases/s"
 PEAKS_FALLBACK = {"hbm_gbs": 6800.0}
 # DRAM bytes (read + write) per contig base of k_emit from one ncu capture
-# (--set full, the 3.1 Gb recipe on a 450 Mb genome: 550.6 MB for 481,446,585
-# bases), valid only for the emission source it was taken on.
-EMIT_TRAFFIC = {"bytes_per_base": (129.027072e6 + 421.528576e6) / 481446585, "source_sha256_16": "148a0f9f1719bdd2"}
+# (--set full, the 3.1 Gb recipe on a 450 Mb genome: 550.3 MB for 481,446,585
+# bases), valid only for the sources it was taken on: the kernel and the plan of its
+# spans, which decides how often pieces and tile-map entries are read again.
+EMIT_SOURCES = ("cg_emit.cu", "cg_spans.cuh")
+EMIT_TRAFFIC = {"bytes_per_base": (128.795136e6 + 421.527296e6) / 481446585, "source_sha256_16": "33fb9333015aa112"}
+
+
+def emit_source_sha256_16(csrc: str = os.path.join(ROOT, "paper_2207_04350_gb300", "csrc")) -> str:
+    h = hashlib.sha256()
+    for name in EMIT_SOURCES:
+        with open(os.path.join(csrc, name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
 
 
 def _reduce(x: float, world: int, op: str) -> float:
@@ -885,9 +896,7 @@ def run_ours(args, rank, world, local_rank):
         cpu["scaled_sample"] = cpu_baseline(args, cfg)
 
     B = bmin_bytes(G, W, total, n_contigs)
-    import hashlib
-    with open(os.path.join(ROOT, "paper_2207_04350_gb300", "csrc", "cg_emit.cu"), "rb") as f:
-        same_kernel = hashlib.sha256(f.read()).hexdigest()[:16] == EMIT_TRAFFIC["source_sha256_16"]
+    same_kernel = emit_source_sha256_16() == EMIT_TRAFFIC["source_sha256_16"]
     traffic = EMIT_TRAFFIC["bytes_per_base"] * total if same_kernel else None
     emit_bytes = total + (total + 3) // 4
     ach = emit_bytes / (ms_emit * 1e-3) / 1e9
@@ -925,7 +934,7 @@ def run_ours(args, rank, world, local_rank):
         "roofline": {"kernel": "k_emit (contig spelling)", "bound": "hbm", "achieved": ach, "peak": pk["hbm_gbs"],
                      "unit": "GB/s", "frac": ach / pk["hbm_gbs"], "traffic": traffic,
                      "traffic_note": "ncu dram bytes of a scaled capture (450 Mb recipe) x contig bases; null when "
-                                     "the kernel changed since",
+                                     "the kernel or the plan of its spans changed since",
                      "algorithmic_bytes_per_launch": emit_bytes, "bytes_per_unit": 1.25,
                      "units_per_launch": total, "ms_per_launch": ms_emit, "peak_kind": pk_kind + " (hbm_gbs, copy)"},
         "cpu_baseline": cpu,
