@@ -261,7 +261,7 @@ cudaError_t launch_gather_pieces(const Scratch& s, int k, const int64_t* PB, con
                                  const int64_t* bytes, const unsigned long long* slot, uint32_t* dst,
                                  long long cap_words, long long W, const LaunchEnv& env, long long t_begin = 0,
                                  long long t_end = 0);
-constexpr long long kSortBlockMax = 65536;   // contigs sorted by one block, without hist, base and state
+constexpr long long kSortBlockMax = 65536;   // contigs sorted by one block (k_sort_block), without hist, base and state
 // Buffers of the contig-weight sort (capacity: the number of contigs).
 struct SortBuffers {
   unsigned long long* key[2];

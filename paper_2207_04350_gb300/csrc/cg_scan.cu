@@ -373,7 +373,10 @@ __global__ void k_sort_scatter(const unsigned long long* key_in, const int32_t* 
 // fewer passes than the bound kmax. Results in key[0], val[0]. The 3.1 Gb
 // graph's 13,124 contigs by reads, one pass: 27 us by events (40 in two passes of
 // eight bits), and 100 for the ten launches above; by bases, three passes, 66 and
-// 136. The line lies where a block's passes, growing with the contigs, meet them.
+// 136. The line (kSortBlockMax) lies between where the block's passes, which grow with
+// the contigs, meet the launches by reads and by bases, block / launches: 32,000
+// contigs 40 / 99 and, in two passes, 89 / 138; 49,000 56 / 101 and 128 / 138; 65,000
+// 72 / 101 and 165 / 137; 98,000 102 / 102 and 240 / 139.
 constexpr int kSortBlock = 1024;
 constexpr int kSortLoad = 8;
 constexpr int kSortBits = 10, kSortDigits = 1 << kSortBits;   // a digit per thread in the scan
