@@ -39,14 +39,14 @@ int64_t now_ns() {
 // zeroed for each request, were most of what a request took. Making pinned memory
 // and giving it back stop the other workers' calls for many milliseconds, so the
 // server makes one stretch of a GiB, or of its admission budget when that is less, as
-// it starts (30 ms a GiB), out of which
-// results are cut, first fit, and released ones joined again. Results that do not
-// fit lie in ordinary memory, written once before the copy. 2,000 requests of 42 Mb
-// on average, eight workers, all submitted at once: 1,850-2,340 requests a second,
-// and with 940-1,045 a second offered from the server's start on, p50 0.95 and p99
-// 4.9-6.7 ms. With a pinned block made for each request that found none waiting
-// 1,890-2,260, 1.0 and 43-138; with all results in ordinary memory 1,360-2,100, and
-// p50 1.3, p99 10-20 with a third as many offered. Any thread may take and give.
+// it starts (30 ms a GiB), out of which results are cut, first fit, and released ones
+// joined again. Results that do not fit lie in ordinary memory, written once before
+// the copy. 2,000 requests of 42 Mb on average, eight workers: with 940-1,045 a second
+// offered from the server's start on, p50 0.95 and p99 4.9-6.7 ms; with a pinned block
+// made for each request that found none waiting 1.0 and 43-138; with all results in
+// ordinary memory p50 1.3, p99 10-20 with a third as many offered. All submitted at
+// once, requests a second: 1,810-2,340, 1,890-2,260 and 1,360-2,100, which differ by
+// less than the runs. Any thread may take and give.
 struct HostBuf {
   void* p = nullptr;
   size_t cap = 0;
