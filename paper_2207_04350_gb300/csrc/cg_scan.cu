@@ -497,14 +497,24 @@ __global__ void __launch_bounds__(kSortBlock) k_sort_block(const Scratch s, int 
 // levels the sums. So a round ranks the P keys, hands contig r to the part of
 // rank r and keeps the longest prefix for which that holds: all of it when every
 // raised key is above the largest old one, else up to the first rank whose old
-// key is above a raised key of a lower rank. When only the first is kept, the
-// least-loaded part stays so for a while, and takes every further contig that
-// leaves it below the second. The parts are those of the rule taken literally.
+// key is above a raised key of a lower rank. When that is few (lpt_few), or not all for
+// some rounds on end, a few parts lie below the others (which hold contigs larger than
+// a share, say) and take the next contigs among themselves for long: one warp then
+// hands kLptLeast contigs, and twice as many each further time in a row, to the
+// smallest of the kLptLow lowest keys one by one, while that is below the next key.
+// The parts are those of the rule taken literally.
 // G threads per part, each comparing its key with a G-th of the P keys in shared
 // memory. What bounds it is the chain of ranks and barriers of each round. A few
 // parts, whose rounds would hand out that few contigs, take another way below.
 // The 3.1 Gb graph's contigs into 72 / 128 / 1024 parts: 125 / 90 / 305 us by
-// events, and 770 / 770 / 4851 one contig at a time in one warp.
+// events, and 770 / 770 / 4851 one contig at a time in one warp. 20,000 contigs of a
+// few reads behind so many large ones that 2 / 10 / 18 / 24 parts of 72 / 72 / 128 /
+// 1024 lie below the others, whole call: 0.56 / 0.78 / 0.94 / 3.2 ms, 0.97 / 1.24 /
+// 1.44 / 13.2 in rounds of as few and 1.31 / 1.31 / 1.31 / 8.0 one at a time.
+constexpr int kLptLow = 64, kLptLeast = 48, kLptRun = 1024;
+// Below this a round costs more than as many contigs one by one (27 to 40 ns each): a
+// round is 0.65 us with up to 64 parts, 1.3 with 128, 16 with 1024.
+__device__ __forceinline__ int lpt_few(int P) { return P > 256 ? kLptLow : P > 128 ? 32 : min(24, 3 * P / 4); }
 constexpr int kLptSmem = 160 << 10;  // bytes of weights and parts staged at a time; kMaxParts contigs at least
 
 // The smallest value of the lanes before this one.
@@ -520,31 +530,46 @@ __device__ __forceinline__ K warp_min_before(K m, int lane) {
   return lane == 0 ? none : e;
 }
 
-// How many of the weights w[0..n), at most 32, the part with key `lowest` takes
-// one after another while it stays below `second`; their sum in *added. All
-// lanes of a warp.
-template <typename K>
-__device__ __forceinline__ int lpt_run(const K* w, int n, K lowest, K second, K* added, int lane) {
-  const unsigned full = 0xffffffffu;
-  const K wl = lane < n ? w[lane] : (K)0;
-  K sum = wl;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const K x = __shfl_up_sync(full, sum, o);
-    if (lane >= o) sum += x;
-  }
-  const unsigned ok = __ballot_sync(full, lane < n && (lane == 0 || lowest + (sum - wl) < second));
-  const int run = __popc(ok);                          // sums never decrease: the first `run` lanes
-  *added = __shfl_sync(full, sum, run - 1);
-  return run;
+// The smallest value of a warp's lanes, by the redux unit.
+__device__ __forceinline__ uint32_t warp_smallest(uint32_t x) { return __reduce_min_sync(0xffffffffu, x); }
+__device__ __forceinline__ unsigned long long warp_smallest(unsigned long long x) {
+  const unsigned hi = (unsigned)(x >> 32), mhi = __reduce_min_sync(0xffffffffu, hi);
+  return ((unsigned long long)mhi << 32) | __reduce_min_sync(0xffffffffu, hi == mhi ? (unsigned)x : ~0u);
 }
 
-template <typename K>
-__device__ __forceinline__ int keys_below(const K* keys, int n4, int g, int G, K mine);
-template <>
-__device__ __forceinline__ int keys_below<uint32_t>(const uint32_t* keys, int n4, int g, int G, uint32_t mine) {
-  int r0 = 0, r1 = 0;
+// Contigs of weights w[0..most) one after another to the smallest of a warp's keys, k0
+// and (kTwo) k1 of each lane, while that is below `limit`: the parts they go to in `to`,
+// how many they are returned. 32 at a time have their weights and parts in registers.
+template <bool kTwo, typename K>
+__device__ __forceinline__ int lpt_one_by_one(const K* w, short* to, int most, K& k0, K& k1, K limit, int part_bits,
+                                              int lane) {
+  const unsigned mask = (1u << part_bits) - 1u;
+  int q = 0;
+  for (bool low = true; low && q < most;) {
+    const int len = min(32, most - q);
+    const K wl = lane < len ? w[q + lane] : (K)0;
+    unsigned got = 0;
+    int i = 0;
 #pragma unroll 4
+    for (; i < len; ++i) {
+      const K wi = __shfl_sync(0xffffffffu, wl, i), m = warp_smallest(kTwo ? min(k0, k1) : k0);
+      low = m < limit;
+      if (!low) break;
+      got = lane == i ? (unsigned)m & mask : got;
+      k0 += k0 == m ? wi : (K)0;
+      if (kTwo) k1 += k1 == m ? wi : (K)0;
+    }
+    if (lane < i) to[q + lane] = (short)got;
+    q += i;
+  }
+  return q;
+}
+
+// How many of a g-th of the n4 keys are below `mine`.
+template <int kUnroll>
+__device__ __forceinline__ int keys_below(const uint32_t* keys, int n4, int g, int G, uint32_t mine) {
+  int r0 = 0, r1 = 0;
+#pragma unroll kUnroll
   for (int j = 4 * g; j < n4; j += 4 * G) {
     const uint4 x = *reinterpret_cast<const uint4*>(keys + j);
     r0 += (x.x < mine) + (x.y < mine);
@@ -552,11 +577,10 @@ __device__ __forceinline__ int keys_below<uint32_t>(const uint32_t* keys, int n4
   }
   return r0 + r1;
 }
-template <>
-__device__ __forceinline__ int keys_below<unsigned long long>(const unsigned long long* keys, int n4, int g, int G,
-                                                              unsigned long long mine) {
+template <int kUnroll>
+__device__ __forceinline__ int keys_below(const unsigned long long* keys, int n4, int g, int G, unsigned long long mine) {
   int r0 = 0, r1 = 0;
-#pragma unroll 4
+#pragma unroll kUnroll
   for (int j = 2 * g; j < n4; j += 2 * G) {
     const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(keys + j);
     r0 += x.x < mine;
@@ -579,9 +603,11 @@ __device__ __forceinline__ bool part_sync_or(int count, bool x) {
 }
 
 // G threads per part (a power of two): the first P * G threads, in whole warps,
-// assign, and the others only stage weights and write parts.
-template <typename K>
-__global__ void __launch_bounds__(kMaxParts) k_lpt_assign(const unsigned long long* key, const int32_t* val, long long C,
+// assign, and the others only stage weights and write parts. kUnroll: of the comparing
+// loop, which is a handful of steps with few parts (72 parts by reads: 171 us a call
+// with 1, 182 with 4; 1,024 parts 370 and 355).
+template <typename K, int kUnroll>
+__global__ void __launch_bounds__(kMaxParts, 1) k_lpt_assign(const unsigned long long* key, const int32_t* val, long long C,
                                                           unsigned long long kmax, int P, int G, int part_bits,
                                                           int chunk, int32_t* part, int64_t* psum,
                                                           const DevError* derr) {
@@ -593,7 +619,8 @@ __global__ void __launch_bounds__(kMaxParts) k_lpt_assign(const unsigned long lo
   K* const w = reinterpret_cast<K*>(staged);               // chunk weights
   short* const to = reinterpret_cast<short*>(w + chunk);   // and the parts they go to
   __shared__ K warp_min[32], top;
-  __shared__ int first_bad, stop;
+  __shared__ int first_bad, handed, stop;
+  __shared__ int again, run, bad_end;                      // rounds that kept a part on end, the next run, where the last one ended
   const unsigned full = 0xffffffffu;
   const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, warp = tid >> 5;
   const K none = ~(K)0;
@@ -601,6 +628,11 @@ __global__ void __launch_bounds__(kMaxParts) k_lpt_assign(const unsigned long lo
   const bool act = me < P, lead = act && g == 0;
   const int n4 = (P + 3) & ~3, A = (P * G + 31) & ~31;
   if (tid >= P && tid < n4) keys[tid] = none;              // the last vector's empty places
+  if (tid == 0) {
+    again = 0;
+    run = kLptLeast;
+    bad_end = -1;
+  }
   K mine = act ? (K)me : none;
   for (long long c0 = 0; c0 < C;) {
     const int n = (int)min((long long)chunk, C - c0);
@@ -614,7 +646,7 @@ __global__ void __launch_bounds__(kMaxParts) k_lpt_assign(const unsigned long lo
         const int cnt = min(P, n - cur);
         if (lead) keys[me] = mine;
         part_sync(A);
-        int r = act ? keys_below<K>(keys, n4, g, G, mine) : 0;
+        int r = act ? keys_below<kUnroll>(keys, n4, g, G, mine) : 0;
         for (int o = G >> 1; o > 0; o >>= 1) r += __shfl_xor_sync(full, r, o);
         if (!act) r = P;
         const K raised = r < cnt ? mine + w[cur + r] : none;
@@ -632,7 +664,10 @@ __global__ void __launch_bounds__(kMaxParts) k_lpt_assign(const unsigned long lo
           old_key[r] = mine;
           if (r < cnt) new_key[r] = raised;
         }
-        if (tid == 0) first_bad = cnt;
+        if (tid == 0) {
+          first_bad = cnt;
+          again = cur == bad_end ? again + 1 : 0;
+        }
         part_sync(A);
         const K m = tid < cnt ? new_key[tid] : none;         // thread t now looks at rank t
         K before = warp_min_before(m, lane);
@@ -642,19 +677,35 @@ __global__ void __launch_bounds__(kMaxParts) k_lpt_assign(const unsigned long lo
         if (tid > 0 && tid < cnt && old_key[tid] > before) atomicMin(&first_bad, tid);
         part_sync(A);
         const int kept = first_bad;
-        if (kept > 1) {
+        if (kept >= (again < 3 ? lpt_few(P) : max(lpt_few(P), min(24, P)))) {   // again: no full round for a while
           if (r < kept) {
             if (lead) to[cur + r] = (short)me;
             mine = raised;
           }
           cur += kept;
-        } else {                                             // every warp computes the run
-          K added;
-          const int run = lpt_run(w + cur, min(32, n - cur), old_key[0], old_key[1], &added, lane);
-          if (r == 0) mine += added;
-          if (tid < run) to[cur + tid] = (short)(old_key[0] & (((K)1 << part_bits) - 1));
-          cur += run;
+          if (tid == 0) {
+            run = kLptLeast;
+            bad_end = cur;
+          }
+          continue;
         }
+        if (warp == 0) {                                     // lane l: the parts of rank l and l + 32
+          K k0 = lane < P ? old_key[lane] : none, k1 = lane + 32 < P ? old_key[lane + 32] : none;
+          const K limit = P > kLptLow ? old_key[kLptLow] : none;
+          const int most = min(__shfl_sync(full, run, 0), n - cur);
+          const int q = P <= 32 ? lpt_one_by_one<false>(w + cur, to + cur, most, k0, k1, limit, part_bits, lane)
+                                : lpt_one_by_one<true>(w + cur, to + cur, most, k0, k1, limit, part_bits, lane);
+          new_key[lane] = k0;
+          new_key[lane + 32] = k1;
+          if (lane == 0) {
+            handed = q;
+            run = min(2 * run, kLptRun);
+            bad_end = cur + q;
+          }
+        }
+        part_sync(A);
+        if (act && r < kLptLow) mine = new_key[r];
+        cur += handed;
       }
       if (tid == 0) stop = cur;
     }
@@ -879,9 +930,10 @@ cudaError_t launch_partition(const Scratch& s, long long C, int weight, long lon
     while (2 * G * P <= 512 && 2 * G <= (P + 3) / 4) G *= 2;
     const int threads = std::max(256, (P * G + 31) & ~31);   // enough of them to stage the weights
     const int chunk = lpt_chunk(C, narrow ? 4 : 8);
-    e = narrow ? lpt_launch(k_lpt_assign<uint32_t>, chunk, 4, threads, env, kk, vv, C, kmax, P, G, part_bits, chunk, part, psum,
+    auto* const narrow_kernel = P <= 256 ? k_lpt_assign<uint32_t, 1> : k_lpt_assign<uint32_t, 4>;
+    e = narrow ? lpt_launch(narrow_kernel, chunk, 4, threads, env, kk, vv, C, kmax, P, G, part_bits, chunk, part, psum,
                             s.derr)
-               : lpt_launch(k_lpt_assign<unsigned long long>, chunk, 8, threads, env, kk, vv, C, kmax, P, G, part_bits, chunk,
+               : lpt_launch(k_lpt_assign<unsigned long long, 4>, chunk, 8, threads, env, kk, vv, C, kmax, P, G, part_bits, chunk,
                             part, psum, s.derr);
   }
   if (e != cudaSuccess) return e;

@@ -140,6 +140,19 @@ def test_uneven_and_many(ctx, sizes, parts):
     check(ctx, G, parts)
 
 
+@pytest.mark.parametrize("long_len", [40, 30000])            # keys of 32 bits, and of 64
+@pytest.mark.parametrize("P,big", [
+    (20, 18), (32, 29), (33, 32), (63, 62), (64, 60), (65, 1), (65, 64), (66, 2), (72, 71), (72, 70), (72, 40),
+    (97, 32), (128, 126), (128, 64), (128, 63), (1024, 1022), (1024, 961), (1024, 960), (1024, 900)])
+def test_a_few_parts_below_the_others(ctx, P, big, long_len):
+    """As many contigs far above the rest as leave 1 to 128 parts to take the small ones
+    one at a time, among them many of one weight, and more than one run of them."""
+    rng = np.random.default_rng(P * 7 + big)
+    sizes = list(90 + 3 * np.arange(big)) + list(2 + rng.geometric(0.3, size=900)) + [2] * 200
+    G = structured(P + big, [int(x) for x in sizes], min_len=8 if long_len == 40 else long_len, max_len=long_len)
+    check(ctx, G, [P])
+
+
 def test_few_parts(ctx):
     """Up to 19 parts one contig at a time: sorted keys, one per lane, and keys of
     64 bits when a contig is too large for 32; 20 parts and up in rounds."""
