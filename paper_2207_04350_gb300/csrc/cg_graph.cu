@@ -515,10 +515,11 @@ __global__ void k_listwalk(Scratch s) {
 // read id over that span, tail = the list's last oriented read. Sublists on
 // directed cycles keep next >= 0. Returns the buffer that holds the result, or -1
 // when a barrier gave up.
-__device__ __forceinline__ int jump_lists(const Scratch& s) {
+__device__ __forceinline__ int jump_lists(const Scratch& s, unsigned team) {
   Counters* c = s.ctr;
+  const long long T = (long long)team * blockDim.x;
   unsigned R = *(volatile unsigned*)&c->n_rulers;
-  for (long long i = grid_tid(); i < R; i += grid_threads()) {
+  for (long long i = grid_tid(); i < R; i += T) {
     const int4 rc = s.rec[i];
     s.pj[0][i] = make_int4(rc.x, rc.y, rc.z, rc.w);
   }
@@ -526,11 +527,11 @@ __device__ __forceinline__ int jump_lists(const Scratch& s) {
   while ((1u << rounds) < R + 1u && rounds < 31) ++rounds;
   ++rounds;
   int cur = 0;
-  if (!grid_sync(c, s.derr)) return -1;
+  if (!grid_sync(c, s.derr, team)) return -1;
   for (int r = 0; r < rounds; ++r) {
     int nxt = cur ^ 1;
     unsigned active = 0;
-    for (long long i = grid_tid(); i < R; i += grid_threads()) {
+    for (long long i = grid_tid(); i < R; i += T) {
       const int4 a = s.pj[cur][i];
       if (a.x >= 0) {
         const int4 b = s.pj[cur][a.x];
@@ -545,7 +546,7 @@ __device__ __forceinline__ int jump_lists(const Scratch& s) {
     active = __syncthreads_or(active);
     if (threadIdx.x == 0 && active) atomicOr(&c->round_flag[r], 1u);   // zeroed by the stage
     cur = nxt;
-    if (!grid_sync(c, s.derr)) return -1;
+    if (!grid_sync(c, s.derr, team)) return -1;
     if (*(volatile unsigned*)&c->round_flag[r] == 0) break;
   }
   return cur;
@@ -565,12 +566,14 @@ constexpr int kFinalItems = 2;
 // A list the list walk gave up on is jumped first, by the same (cooperative) grid:
 // a kernel of its own for that, which mostly found nothing to do, and one for the
 // closed chains (see k_heads) made the step of a 100 Mb genome 99.1 us, not 92.6.
-__global__ void __launch_bounds__(kBlock) k_final(DevGraph g, Scratch s) {
+// The jumping is the work of `team` blocks, or more for many sublists (coop_do).
+__global__ void __launch_bounds__(kBlock, 4) k_final(DevGraph g, Scratch s, unsigned team) {
   pdl_enter();
   Counters* c = s.ctr;
   int fb = 0;
   if (*(volatile unsigned*)&c->need_jump != 0) {   // the same for every block: written by the kernel before
-    fb = jump_lists(s);
+    team = coop_team(team, *(volatile unsigned*)&c->n_rulers);
+    fb = coop_do(s.derr, &c->jumped, team, [&] { return jump_lists(s, team); });
     if (fb < 0) return;
   }
   const long long N = *(volatile unsigned*)&c->n_cand;
@@ -675,7 +678,7 @@ __global__ void k_cycles(DevGraph g, Scratch s) {
   Counters* c = s.ctr;
   const unsigned C = *(volatile unsigned*)&c->n_cycle_reads;
   if (C == 0 || __syncthreads_or(gave_up(s.derr))) return;
-  close_cycles(g, s, C, grid_tid(), grid_threads(), [&] { return grid_sync(c, s.derr); });
+  close_cycles(g, s, C, grid_tid(), grid_threads(), [&] { return grid_sync(c, s.derr, gridDim.x); });
 }
 
 // Per-read chain outputs, four consecutive reads per thread: a candidate's record,
@@ -683,17 +686,20 @@ __global__ void k_cycles(DevGraph g, Scratch s) {
 // one-read contig). Every read is written once, in order; defaults for all reads
 // and then the candidates' records over them, in two kernels, took 18 us by
 // events for 1.25M reads, and this takes 13. with_cycles: the closed chains come first, on the same
-// (cooperative) grid, when there are any.
-__global__ void __launch_bounds__(kBlock) k_export_reads(DevGraph g, Scratch s, bool with_cycles, int32_t* cid,
-                                                         int32_t* rank, uint8_t* orient) {
+// (cooperative) grid, by `team` of its blocks or more, when there are any.
+__global__ void __launch_bounds__(kBlock, 6) k_export_reads(DevGraph g, Scratch s, bool with_cycles, unsigned team,
+                                                         int32_t* cid, int32_t* rank, uint8_t* orient) {
   pdl_enter();
   Counters* c = s.ctr;
   const bool stop = gave_up(s.derr);
   const unsigned C = with_cycles ? *(volatile unsigned*)&c->n_cycle_reads : 0u;   // the same for every block
   if (__syncthreads_or(stop)) return;
   if (C > 0) {
-    close_cycles(g, s, C, grid_tid(), grid_threads(), [&] { return grid_sync(c, s.derr); });
-    if (!grid_sync(c, s.derr)) return;
+    team = coop_team(team, 2ll * C);
+    auto sync = [&] { return grid_sync(c, s.derr, team); };
+    if (coop_do(s.derr, &c->closed, team, [&] {
+          return close_cycles(g, s, C, grid_tid(), (long long)team * kBlock, sync) && sync() ? 0 : -1;
+        }) < 0) return;
   }
   const unsigned N = *(volatile unsigned*)&c->n_cand;
   for (long long v0 = 4 * grid_tid(); v0 < g.n; v0 += 4 * grid_threads()) {
@@ -798,7 +804,8 @@ cudaError_t launch_chains(const DevGraph& g, const Scratch& s, const Tuning& t, 
   mark(env, "k_listwalk");
   DevGraph gg = g;
   Scratch sc = s;
-  void* args[] = {&gg, &sc};
+  unsigned team = (unsigned)env.coop_blocks;
+  void* args[] = {&gg, &sc, &team};
   e = coop((const void*)k_final, cap((long long)env.num_sms * final_resident, N, (long long)kBlock * kFinalItems), args,
            env, true);
   if (e != cudaSuccess) return e;
@@ -814,13 +821,18 @@ cudaError_t launch_export_reads(const DevGraph& g, const Scratch& s, int32_t* ci
                                 const LaunchEnv& env, bool after_chains) {
   static const int resident = resident_blocks(k_export_reads);
   const long long need = (g.n + 4 * kBlock - 1) / (4 * kBlock);
-  const int grid = (int)std::max(1LL, std::min(need, (long long)env.num_sms * resident));
   bool with_cycles = after_chains && !s.small;
+  // as many blocks as the reads or, two per SM, the closed chains can use
+  const long long team_need =
+      with_cycles ? std::min((2 * most_candidates(g) + kBlock - 1) / kBlock, (long long)env.coop_blocks) : 1;
+  const int grid = (int)std::min(std::max(need, team_need), (long long)env.num_sms * resident);
   DevGraph gg = g;
   Scratch sc = s;
-  void* args[] = {&gg, &sc, &with_cycles, &cid, &rank, &orient};
+  unsigned team = (unsigned)env.coop_blocks;
+  void* args[] = {&gg, &sc, &with_cycles, &team, &cid, &rank, &orient};
   cudaError_t e = with_cycles ? coop((const void*)k_export_reads, grid, args, env, true)
-                              : launch_k(k_export_reads, grid, env, after_chains, g, s, with_cycles, cid, rank, orient);
+                              : launch_k(k_export_reads, grid, env, after_chains, g, s, with_cycles, team, cid, rank,
+                                         orient);
   if (e != cudaSuccess) return e;
   mark(env, "k_export_reads");
   return cudaGetLastError();

@@ -47,6 +47,7 @@ struct Counters {
   unsigned int bar_count;      // grid barrier arrival counter
   unsigned int bar_gen;        // grid barrier generation
   unsigned int round_flag[64]; // "some pointer still moves" per jumping round
+  unsigned int jumped, closed; // what coop_do hands from its team to the other blocks: the jumping's result, the closed chains
   // offsets stage
   unsigned int n_contigs;
   unsigned int n_walk;         // walk positions = reads spelled

@@ -59,8 +59,8 @@ __global__ void __launch_bounds__(kBlock) k_heads(DevGraph g, Scratch s, bool wi
   if (__syncthreads_or(stop)) return;
   if (cyc > 0) {
     Counters* c = s.ctr;
-    close_cycles(g, s, cyc, grid_tid(), grid_threads(), [&] { return grid_sync(c, s.derr); });
-    if (!grid_sync(c, s.derr)) return;
+    auto sync = [&] { return grid_sync(c, s.derr, gridDim.x); };
+    if (!close_cycles(g, s, cyc, grid_tid(), grid_threads(), sync) || !sync()) return;
   }
   for (long long i = grid_tid(); i <= s.scan_tiles_cap; i += grid_threads()) s.scan_state[i] = 0ull;   // of the piece scan
   const int tid = threadIdx.x;

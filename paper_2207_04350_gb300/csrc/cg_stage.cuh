@@ -13,22 +13,21 @@ namespace {
 
 constexpr long long kSpinLimit = 1ll << 22;   // barrier polls before giving up (~1 s with backoff)
 
-// Software grid barrier for kernels launched cooperatively (all blocks
-// co-resident). Bounded: a block that waits too long records DERR_TIMEOUT and
-// every block returns false from then on. A block that has seen that arrives at no
-// further barrier: an arrival of its own would let the others pass one that a block
-// still at work has not reached.
-__device__ bool grid_sync(Counters* c, DevError* e) {
+// Software barrier over the first `blocks` blocks of a kernel launched cooperatively
+// (all blocks co-resident). Bounded: a block that waits too long records DERR_TIMEOUT
+// and gets false, as does every block that still waits then; such a block arrives at
+// no further barrier (an arrival of its own would let the others pass one that a block
+// still at work has not reached), so its caller returns.
+__device__ bool grid_sync(Counters* c, DevError* e, unsigned blocks) {
   __shared__ int ok;
   __syncthreads();
   if (threadIdx.x == 0) {
+    ok = 1;
     volatile unsigned* gen = &c->bar_gen;
     unsigned g0 = *gen;
-    ok = !gave_up(e);
     __threadfence();
-    unsigned arrived = ok ? atomicAdd(&c->bar_count, 1u) : 0u;
-    if (!ok) {
-    } else if (arrived == gridDim.x - 1) {
+    unsigned arrived = atomicAdd(&c->bar_count, 1u);
+    if (arrived == blocks - 1) {
       c->bar_count = 0;
       __threadfence();
       atomicAdd(&c->bar_gen, 1u);
@@ -47,6 +46,42 @@ __device__ bool grid_sync(Counters* c, DevError* e) {
   }
   __syncthreads();
   return ok != 0;
+}
+
+// Work of the first coop_team() blocks that all blocks use: a round of pointer jumping
+// costs its barrier, which grows with the blocks in it, until its items do. The team
+// returns a value of at least 0, or -1 when a barrier gave up; the others wait for it,
+// with the same limit, in a word that the stage zeroes, which they seldom look at (the
+// barrier's own words lie beside it). Whole grid; below 0: nothing to use.
+__device__ __forceinline__ unsigned coop_team(unsigned least, long long items) {
+  return (unsigned)min((long long)gridDim.x, max((long long)least, items / (2 * (long long)blockDim.x)));
+}
+template <class Work>
+__device__ __forceinline__ int coop_do(DevError* e, unsigned* word, unsigned team, Work work) {
+  __shared__ int got;
+  if (blockIdx.x < team) {
+    const int r = work();
+    if (r >= 0 && blockIdx.x == 0 && threadIdx.x == 0) {
+      __threadfence();
+      atomicExch(word, (unsigned)r + 1u);
+    }
+    return r;
+  }
+  if (threadIdx.x == 0) {
+    long long spins = 0;
+    unsigned x;
+    while ((x = *(volatile unsigned*)word) == 0u) {
+      if (++spins > kSpinLimit / 16 || gave_up(e)) {
+        set_error(e, DERR_TIMEOUT, K_JUMP, spins);
+        break;
+      }
+      __nanosleep(4000);
+    }
+    __threadfence();
+    got = (int)x - 1;
+  }
+  __syncthreads();
+  return got;
 }
 
 // Read m is the smallest read of a contig of q reads.
@@ -139,9 +174,9 @@ __device__ __forceinline__ int32_t piece_len(const DevGraph& g, const Scratch& s
 // smallest read), then cut the walk before (m,0) and rank by pointer jumping
 // again.
 // Over `threads` threads of which this is the tid-th; sync() is a barrier over them
-// all that makes their writes visible, false when it gave up.
+// all that makes their writes visible, false when it gave up: then so is the result.
 template <class Sync>
-__device__ __forceinline__ void close_cycles(const DevGraph& g, const Scratch& s, unsigned C, long long tid, long long threads,
+__device__ __forceinline__ bool close_cycles(const DevGraph& g, const Scratch& s, unsigned C, long long tid, long long threads,
                              Sync sync) {
   Counters* c = s.ctr;
   long long N = 2ll * C;
@@ -157,7 +192,7 @@ __device__ __forceinline__ void close_cycles(const DevGraph& g, const Scratch& s
   while ((1ll << rounds) < N + 1 && rounds < 31) ++rounds;
   ++rounds;
   int cur = 0;
-  if (!sync()) return;
+  if (!sync()) return false;
   for (int r = 0; r < rounds; ++r) {
     int nxt = cur ^ 1;
     for (long long i = tid; i < N; i += threads) {
@@ -168,7 +203,7 @@ __device__ __forceinline__ void close_cycles(const DevGraph& g, const Scratch& s
       s.c_ptr[nxt][u] = s.c_ptr[cur][p];
     }
     cur = nxt;
-    if (!sync()) return;
+    if (!sync()) return false;
   }
   // cut: on the walk copy, the oriented candidate before the start has no successor
   for (long long i = tid; i < N; i += threads) {
@@ -184,7 +219,7 @@ __device__ __forceinline__ void close_cycles(const DevGraph& g, const Scratch& s
     }
   }
   cur = 0;
-  if (!sync()) return;
+  if (!sync()) return false;
   for (int r = 0; r < rounds; ++r) {
     int nxt = cur ^ 1;
     for (long long i = tid; i < N; i += threads) {
@@ -200,7 +235,7 @@ __device__ __forceinline__ void close_cycles(const DevGraph& g, const Scratch& s
       }
     }
     cur = nxt;
-    if (!sync()) return;
+    if (!sync()) return false;
   }
   for (long long i = tid; i < N; i += threads) {
     const int32_t ci = s.cyc[i >> 1];
@@ -222,6 +257,7 @@ __device__ __forceinline__ void close_cycles(const DevGraph& g, const Scratch& s
     }
     if (rk == 0) atomicAdd(&c->n_cycles, 1u);
   }
+  return true;
 }
 
 // Block-wide exclusive prefix of one 64-bit value per thread; the sum of all in

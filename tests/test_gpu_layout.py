@@ -68,3 +68,14 @@ def test_spelling_spans(mb):
         g.close()
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("sizes,closed", [
+    ([200_000, 40], [False, False]), ([700_000], [False]),             # jumped by two blocks per SM, and by more of them
+    ([60_000, 300, 3], [True, False, True]), ([400_000], [True]),      # closed chains: by two per SM, and by all blocks
+    ([90_000, 90_000], [False, True])])
+def test_lists_that_a_part_of_the_grid_jumps(ctx, sizes, closed):
+    G = structured(len(sizes), sizes, closed=closed, lone=50)
+    want = oracle.run(G)
+    for outputs in ("host", "device"):                                 # chains alone, then per-read outputs with them
+        assert_parity(run_gpu(ctx, G, inputs="device", outputs=outputs), want)
