@@ -643,6 +643,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_final(DevGraph g, Scratch s, unsi
 #pragma unroll
     for (int j = 0; j < kFinalItems; ++j) {
       const long long ci = k0 + j * T;
+      int32_t reads = 0;                     // of the contig that v heads
       if (ok[j]) {
         int32_t len;
         if (g.pre) {   // x-drop form: l_v[post(e_in) : pre(e_out)], alpha / beta at the contig's ends
@@ -655,16 +656,14 @@ __global__ void __launch_bounds__(kBlock, 4) k_final(DevGraph g, Scratch s, unsi
           len = rk[j] == 0 ? L[j] : sin[j];
         }
         s.prd[ci] = make_int4(m[j], rk[j], len, o[j]);
-        if (v[j] == m[j]) {
-          mark_head(s, m[j], q[j]);
-          ++heads;
-        }
+        if (v[j] == m[j]) reads = q[j];
       } else if (in[j] && !cyc[j]) {
         s.prd[ci] = make_int4(-1, -1, 0, 255);
       } else if (!in[j] && ci < N && g.min_chain <= 1) {   // cut off by branch reads: its own contig
-        mark_head(s, v[j], 1);
-        ++heads;
+        reads = 1;
       }
+      mark_heads(s, v[j], reads);
+      heads += reads > 0;
       const unsigned slot = warp_append(&c->n_cycle_reads, cyc[j]);
       if (cyc[j]) s.cyc[slot] = (int32_t)ci;
     }
