@@ -196,15 +196,18 @@ inline void mark(const LaunchEnv& env, const char* name) {
 // The stages of a small graph, any of them in one kernel (cg_small.cu); the
 // launchers of the single stages below use it for such graphs too.
 enum : int { kStageMask = 1, kStageChains = 2, kStageOffsets = 4 };
-// A small graph: one block beats ten kernels while a few reads and candidates per
-// thread are all there is. Steps in us with a wait after each, one block against
-// nine kernels: 2,000 reads 37 / 48, 8,000 44 / 53, 16,250 56 / 57; with the lone
-// reads spelled too, which one block also scatters, 1,000 41 / 52, 3,000 54 / 61,
-// 4,000 62 / 64. The bound on the entries is that of an overlap graph of so many
-// reads after the reduction; 8 entries a read would cost what 20,000 reads do.
-constexpr int64_t kSmallReads = 16384, kSmallLoneReads = 4096, kSmallEntries = 8192;
+// A small graph: one block beats nine kernels while a few reads and candidates per
+// thread are all there is. Whole steps in us, one block against nine kernels, in
+// chains of 8 reads: 1,000 reads with 1,400 entries 116 / 126; 4,000 with 700 / 2,800 /
+// 4,200 / 7,000 134 / 139, 132 / 137, 140 / 139 and 157 / 142; 8,000 with 2,800 / 4,200
+// 141 / 143 and 147 / 140; 16,000 with 1,400 / 2,100 / 2,800 143 / 147, 149 / 149 and
+// 155 / 153; per-read outputs by as much. In one long chain, whose sublists the nine
+// follow one after another, the line lies at 7,000 entries, but a chain's length is not
+// known here. With the lone reads spelled too, which one block also scatters, 4,000
+// reads with 2,800 / 4,200 entries 134 / 136 and 144 / 140.
+constexpr int64_t kSmallReads = 16384, kSmallLoneReads = 4096, kSmallEntries = 3400;
 inline bool small_graph(int64_t n, int64_t m, int min_chain) {
-  return n > 0 && n <= (min_chain <= 1 ? kSmallLoneReads : kSmallReads) && m <= kSmallEntries;
+  return n > 0 && n <= (min_chain <= 1 ? kSmallLoneReads : kSmallReads) && m <= kSmallEntries - n / 9;
 }
 cudaError_t launch_small(const DevGraph& g, const Scratch& s, const Tuning& t, int stages, int64_t* user_off,
                          long long user_cap, const LaunchEnv& env, bool chained);

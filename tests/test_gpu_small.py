@@ -78,6 +78,12 @@ def test_read_counts(ctx, n, mcr):
     both(ctx, structured(n, [q] if q > 1 else [], lone=n - q if q > 1 else n), mcr)
 
 
+@pytest.mark.parametrize("n,m", [(3060, 3060), (3062, 3062), (8000, 2510), (8000, 2514), (16384, 1578), (16384, 1582)])
+def test_entry_counts(ctx, n, m):
+    """On either side of the line that falls with the reads."""
+    both(ctx, structured(m, [2] * (m // 2), lone=n - m), 2)
+
+
 @pytest.mark.parametrize("lone", [0, 20_000])
 @pytest.mark.parametrize("rp", [np.int32, np.int64])
 @pytest.mark.parametrize("mcr", [1, 2])
