@@ -76,6 +76,44 @@ def _run_all(ctx, G, world, rf, mcr):
             g.close()
 
 
+@pytest.mark.parametrize("world", [40, 300])
+def test_many_ranks(ctx, world):
+    """Ranks that own a piece in forty, or in three hundred: most pairs between two of a
+    rank's own are others', whole windows of them, up to the last."""
+    G = structured(37, [700, 300, 200, 90, 5], min_len=300, max_len=900, align=1)
+    rf = _bounds(G.n, world, 0.3)
+    shares, firsts = _run_some(ctx, G, world, rf, 2, sorted({0, 1, world // 3, world // 2, world - 2, world - 1}))
+    want = oracle.run(G, min_chain_reads=2).bases
+    for got, first in zip(shares, firsts):
+        assert np.array_equal(got, want[first:first + len(got)])
+
+
+def _run_some(ctx, G, world, rf, mcr, receivers):
+    """Every rank's segments, packed one rank after another by one graph, and the shares
+    of some of the ranks."""
+    import torch
+    g = cg.cg_load_graph(ctx, without_reads(G), flags=cg.NO_READS, min_chain_reads=mcr)
+    try:
+        segs = {r: [] for r in receivers}
+        for s, (stream, off) in enumerate(read_slices(G, rf)):
+            size = cg.cg_exchange_sizes(g, world, rf, s)[0]
+            send = torch.zeros(max(16, int(size.sum())), dtype=torch.uint8, device="cuda")
+            cg.cg_exchange_pack(g, world, rf, s, torch.from_numpy(stream).cuda(), torch.from_numpy(off).cuda(), send)
+            send, at = send.cpu().numpy(), np.concatenate([[0], np.cumsum(size)])
+            for r in receivers:
+                segs[r].append(send[at[r]:at[r + 1]])
+        shares, firsts = [], []
+        for r in receivers:
+            recv = torch.from_numpy(np.concatenate(segs[r])).cuda()
+            out = torch.zeros(1 << 21, dtype=torch.uint8, device="cuda")
+            first, n = cg.cg_emit_share_received(g, world, rf, r, recv, None, out)
+            shares.append(out[:n].cpu().numpy())
+            firsts.append(first)
+        return shares, firsts
+    finally:
+        g.close()
+
+
 def test_exchange_needs_no_more_memory_than_its_slots():
     """On a context that holds the ranks' graphs and 8 bytes per piece besides, every
     call of the exchange runs."""
