@@ -506,7 +506,7 @@ __global__ void __launch_bounds__(kSortBlock) k_sort_block(const Scratch s, int 
 // G threads per part, each comparing its key with a G-th of the P keys in shared
 // memory. What bounds it is the chain of ranks and barriers of each round. A few
 // parts, whose rounds would hand out that few contigs, take another way below.
-// The 3.1 Gb graph's contigs into 72 / 128 / 1024 parts: 125 / 90 / 305 us by
+// The 3.1 Gb graph's contigs into 72 / 128 / 1024 parts: 118 / 90 / 300 us by
 // events, and 770 / 770 / 4851 one contig at a time in one warp. 20,000 contigs of a
 // few reads behind so many large ones that 2 / 10 / 18 / 24 parts of 72 / 72 / 128 /
 // 1024 lie below the others, whole call: 0.56 / 0.78 / 0.94 / 3.2 ms, 0.97 / 1.24 /
