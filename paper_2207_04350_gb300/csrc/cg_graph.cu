@@ -567,7 +567,7 @@ constexpr int kFinalItems = 2;
 // a kernel of its own for that, which mostly found nothing to do, and one for the
 // closed chains (see k_heads) made the step of a 100 Mb genome 99.1 us, not 92.6.
 // The jumping is the work of `team` blocks, or more for many sublists (coop_do).
-// Three blocks per SM, 70 registers: with four it spills 32 bytes (500 Mb 11.8 us for
+// Three blocks per SM, 80 registers: with four it spills 32 bytes (500 Mb 11.8 us for
 // 10.2, 3.1 Gb 22.9 for 20.8).
 __global__ void __launch_bounds__(kBlock, 3) k_final(DevGraph g, Scratch s, unsigned team) {
   pdl_enter();
