@@ -71,6 +71,17 @@ def test_chains(ctx, sizes, closed, lone):
     both(ctx, G, 3)
 
 
+@pytest.mark.parametrize("sizes,closed", [
+    ([1400], [False]), ([1400], [True]), ([340] * 4, [True, False] * 2),      # as many entries as one block takes
+    ([3] * 600, [i % 7 == 0 for i in range(600)]), ([2] * 1400, [False] * 1400), ([1] * 900 + [7] * 150, [False] * 1050),
+])
+def test_chains_of_one_block(ctx, sizes, closed):
+    G = structured(sum(sizes), sizes, closed=closed)
+    assert G.m <= 3400 - G.n // 9
+    for mcr in (1, 2, 3):
+        both(ctx, G, mcr)
+
+
 @pytest.mark.parametrize("mcr", [1, 2])
 @pytest.mark.parametrize("n", [1, 32, 33, 1025, 4096, 4097, 16384, 16385])
 def test_read_counts(ctx, n, mcr):
